@@ -46,11 +46,19 @@ __global__ void __launch_bounds__(256) cgemm_kernel(Ops ops, int N, R alpha, R d
     }
     return;
   }
-  cplx<R> acc[4][4];
+  // FP32 Gram matrices (A^dag A of a nearly unitary A) sum many entries far below the rounding of
+  // the sum: added one by one they are lost, G comes out low and the Newton-Schulz step that uses
+  // it scales its matrix up (1.4e-7 per segment at N = 256).  Their K chunks are summed on their own
+  // and added with compensation.
+  constexpr bool kComp = ADJA && sizeof(R) == 4;
+  cplx<R> acc[4][4], tot[kComp ? 4 : 1][kComp ? 4 : 1], cmp[kComp ? 4 : 1][kComp ? 4 : 1];
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = cmake<R>(R(0), R(0));
+    for (int c = 0; c < 4; ++c) {
+      acc[r][c] = cmake<R>(R(0), R(0));
+      if constexpr (kComp) tot[r][c] = cmp[r][c] = acc[r][c];
+    }
   for (int k0 = 0; k0 < N; k0 += kBK) {
 #pragma unroll
     for (int x = 0; x < (kT * kBK) / 256; ++x) {
@@ -79,7 +87,25 @@ __global__ void __launch_bounds__(256) cgemm_kernel(Ops ops, int N, R alpha, R d
 #pragma unroll
         for (int c = 0; c < 4; ++c) cfma<R>(acc[r][c], a[r], bb[c]);
     }
+    if constexpr (kComp) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const R yx = acc[r][c].x - cmp[r][c].x, yy = acc[r][c].y - cmp[r][c].y;
+          const R sx = tot[r][c].x + yx, sy = tot[r][c].y + yy;
+          cmp[r][c] = cmake<R>((sx - tot[r][c].x) - yx, (sy - tot[r][c].y) - yy);
+          tot[r][c] = cmake<R>(sx, sy);
+          acc[r][c] = cmake<R>(R(0), R(0));
+        }
+    }
     __syncthreads();
+  }
+  if constexpr (kComp) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[r][c] = tot[r][c];
   }
 #pragma unroll
   for (int r = 0; r < 4; ++r)
@@ -654,6 +680,12 @@ static cudaError_t large_propagate_t(const redo_table* t, const int32_t* q, cons
   return large_finish_t<R>(t, p, reunit, ws, result, result_prec, s);
 }
 
+cudaError_t large_finish(const redo_table* t, const ChainPlan& p, int prec, bool reunit, void* ws, void** result,
+                         int* result_prec, cudaStream_t s) {
+  if (prec == REDO_FP64) return large_finish_t<double>(t, p, reunit, (char*)ws, result, result_prec, s);
+  return large_finish_t<float>(t, p, reunit, (char*)ws, result, result_prec, s);
+}
+
 cudaError_t large_finish_fp32(const redo_table* t, const ChainPlan& p, bool reunit, void* ws,
                               void** result, int* result_prec, cudaStream_t s) {
   return large_finish_t<float>(t, p, reunit, (char*)ws, result, result_prec, s);
@@ -981,6 +1013,28 @@ static cudaError_t large_scans_t(const redo_table* t, const ChainPlan& p, const 
   *Rck_out = Rck;
   *tau_out = tau;
   return cudaGetLastError();
+}
+
+template <typename R>
+static cudaError_t large_scans_reunit_t(const redo_table* t, const ChainPlan& p, const double2* UT, int tb,
+                                        double* F_out, bool reunit, char* ws, void** Pck, void** Rck, double2** tau,
+                                        cudaStream_t s) {
+  const int64_t n2 = (int64_t)t->N * t->N, G = p.B * p.S;
+  const size_t mat = ((size_t)G * n2 * sizeof(cplx<R>) + 255) & ~(size_t)255;
+  cudaError_t e;
+  if (reunit && p.M > 0 && (e = large_polar_t<R>(t->N, (cplx<R>*)ws, G, (cplx<R>*)(ws + 3 * mat), s))) return e;
+  cplx<R>*P, *Q;
+  if ((e = large_scans_t<R>(t, p, UT, tb, F_out, ws, &P, &Q, tau, s))) return e;
+  *Pck = P;
+  *Rck = Q;
+  return cudaSuccess;
+}
+
+cudaError_t large_grad_scans(const redo_table* t, const ChainPlan& p, int prec, const double2* UT, int tb,
+                             double* F_out, bool reunit, void* ws, void** Pck, void** Rck, double2** tau,
+                             cudaStream_t s) {
+  return prec == REDO_FP64 ? large_scans_reunit_t<double>(t, p, UT, tb, F_out, reunit, (char*)ws, Pck, Rck, tau, s)
+                           : large_scans_reunit_t<float>(t, p, UT, tb, F_out, reunit, (char*)ws, Pck, Rck, tau, s);
 }
 
 cudaError_t large_grad_scans_fp32(const redo_table* t, const ChainPlan& p, const double2* UT, int tb,

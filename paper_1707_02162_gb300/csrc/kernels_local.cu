@@ -1,0 +1,666 @@
+// Chains, gradients and state sweeps of locally controlled systems (local_ops.cuh), N <= 1024.
+// (Section II processes 1 and 2: the discrete operators and their products, here on the 2 x 2
+// parts whose tensor product the N x N table operator is; Section III: chain, GRAPE gradient, state
+// transfer; Section IV: observables along the chain.)
+#include <cmath>
+#include <cstdlib>
+#include <type_traits>
+#include <vector>
+
+#include "local_ops.cuh"
+
+namespace redo {
+
+// ============================================================================
+// Detection and one-qubit tables (at table build)
+// ============================================================================
+
+// Digit operators u[pair][j][c] = exp(-i dt theta h) of a 2 x 2 Hermitian h = a0 I + v.sigma:
+// exp(-i t a0) (cos(t |v|) I - i sin(t |v|) / |v| v.sigma), theta as in the dense table.
+__global__ void loc_table_kernel(const double2* __restrict__ h, const int32_t* __restrict__ k, int pairs, int d,
+                                 int base, double dt, const double* __restrict__ lo, const double* __restrict__ delta,
+                                 double2* __restrict__ u64, float2* __restrict__ u32) {
+  const int64_t total = (int64_t)pairs * d * base;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int c = (int)(e % base), j = (int)((e / base) % d), p = (int)(e / ((int64_t)base * d));
+    const int kk = k[p] & ~kLocFirst;
+    double bj = 1.0;
+    for (int i = 0; i < j; ++i) bj *= (double)base;
+    const double th = j == 0 ? __dadd_rn(lo[kk], __dmul_rn((double)c, delta[kk])) : __dmul_rn((double)c * bj, delta[kk]);
+    const double2 *hp = h + 4 * p;
+    const double a0 = 0.5 * (hp[0].x + hp[3].x), vz = 0.5 * (hp[0].x - hp[3].x), vx = hp[1].x, vy = -hp[1].y;
+    const double t = dt * th, v = sqrt(vx * vx + vy * vy + vz * vz);
+    double sn, cs, s0, c0;
+    sincos(t * v, &sn, &cs);
+    sincos(t * a0, &s0, &c0);
+    const double f = v > 0.0 ? sn / v : 0.0;
+    // cos I - i f (v.sigma), times exp(-i t a0) = c0 - i s0
+    const double2 m[4] = {make_double2(cs, -f * vz), make_double2(-f * vy, -f * vx), make_double2(f * vy, -f * vx),
+                          make_double2(cs, f * vz)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const double2 o = make_double2(m[i].x * c0 + m[i].y * s0, m[i].y * c0 - m[i].x * s0);
+      u64[e * 4 + i] = o;
+      u32[e * 4 + i] = make_float2((float)o.x, (float)o.y);
+    }
+  }
+}
+
+// Splits H (row-major N x N, host) into one-qubit terms h[i] (2 x 2); false when it has others.
+static bool split_local(const double* H, int N, int n, double2* h) {
+  auto at = [&](int r, int c) { return make_double2(H[2 * ((size_t)r * N + c)], H[2 * ((size_t)r * N + c) + 1]); };
+  double mx = 0.0;
+  for (size_t i = 0; i < (size_t)2 * N * N; ++i) mx = std::fmax(mx, std::fabs(H[i]));
+  const double tol = 8 * 2.3e-16 * mx;             // rounding of sums of the same terms
+  auto close = [&](double2 a, double2 b) { return std::fabs(a.x - b.x) <= tol && std::fabs(a.y - b.y) <= tol; };
+  const double2 d0 = at(0, 0);
+  for (int i = 0; i < n; ++i) {
+    const int m = 1 << i;
+    h[4 * i] = i == 0 ? make_double2(d0.x, 0.0) : make_double2(0.0, 0.0);
+    h[4 * i + 3] = make_double2(h[4 * i].x + at(m, m).x - d0.x, 0.0);
+    h[4 * i + 1] = at(0, m);
+    h[4 * i + 2] = make_double2(h[4 * i + 1].x, -h[4 * i + 1].y);
+  }
+  for (int r = 0; r < N; ++r) {
+    double2 dr = make_double2(0.0, 0.0);
+    for (int i = 0; i < n; ++i) {
+      const int b = (r >> i) & 1;
+      dr.x += h[4 * i + 3 * b].x;
+      if (!close(at(r, r ^ (1 << i)), h[4 * i + 1 + b])) return false;
+    }
+    if (!close(at(r, r), dr)) return false;
+    for (int c = 0; c < N; ++c) {
+      const int m = r ^ c;
+      if ((m & (m - 1)) != 0) {                    // more than one qubit flipped
+        const double2 v = at(r, c);
+        if (std::fabs(v.x) > tol || std::fabs(v.y) > tol) return false;
+      }
+    }
+  }
+  return true;
+}
+
+// h: host copies of H0 then H_0 .. H_{K-1}.  Leaves t->loc = 0 for any other system.
+cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_t s) {
+  t->loc = 0;
+  if (!t->h0_diagonal) return cudaSuccess;
+  const int N = t->N, K = t->K;
+  int n = 0;
+  while ((1 << n) < N) ++n;
+  const size_t n2 = (size_t)N * N;
+  std::vector<double2> hk((size_t)K * n * 4);
+  for (int k = 0; k < K; ++k)
+    if (!split_local(h.data() + 2 * n2 * (k + 1), N, n, hk.data() + (size_t)k * n * 4)) return cudaSuccess;
+  std::vector<int32_t> ptr(n + 1), kk;
+  std::vector<double2> hp;
+  std::vector<char> seen(K, 0);
+  for (int i = 0; i < n; ++i) {
+    ptr[i] = (int32_t)kk.size();
+    for (int k = 0; k < K; ++k) {
+      const double2* m = hk.data() + ((size_t)k * n + i) * 4;
+      bool any = false;
+      for (int e = 0; e < 4; ++e) any = any || m[e].x != 0.0 || m[e].y != 0.0;
+      if (!any) continue;
+      kk.push_back(k | (seen[k] ? 0 : kLocFirst));
+      seen[k] = 1;
+      hp.insert(hp.end(), m, m + 4);
+    }
+  }
+  for (int k = 0; k < K; ++k)
+    if (!seen[k]) {                                // H_k = 0: still a term whose level index is checked
+      kk.push_back(k | kLocFirst);
+      hp.insert(hp.end(), 4, make_double2(0.0, 0.0));
+    }
+  ptr[n] = (int32_t)kk.size();
+  const int pairs = (int)kk.size();
+  // one operator per level (no digit products per step) while the table stays small beside L2
+  const bool levels = t->levels <= 65536 && (double)pairs * t->levels * 96.0 <= 64e6;
+  t->loc_d = levels ? 1 : t->digit_count;
+  t->loc_base = levels ? (int)t->levels : t->digit_base;
+  t->loc_pairs = pairs;
+  const size_t ent = (size_t)pairs * t->loc_d * t->loc_base;
+  std::vector<double2> D(N);
+  for (int r = 0; r < N; ++r) {
+    const double a = t->dt * h[2 * ((size_t)r * N + r)];
+    D[r] = make_double2(std::cos(a), -std::sin(a));
+  }
+  cudaError_t e;
+  if ((e = cudaMalloc(&t->loc_ptr, sizeof(int32_t) * (n + 1))) || (e = cudaMalloc(&t->loc_k, sizeof(int32_t) * pairs)) ||
+      (e = cudaMalloc(&t->loc_h, sizeof(double2) * 4 * pairs)) ||
+      (e = cudaMalloc(&t->loc_u64, sizeof(double2) * 4 * ent)) || (e = cudaMalloc(&t->loc_u32, sizeof(float2) * 4 * ent)) ||
+      (e = cudaMalloc(&t->loc_D64, sizeof(double2) * N)))
+    return e;
+  if ((e = cudaMemcpyAsync(t->loc_ptr, ptr.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, s)) ||
+      (e = cudaMemcpyAsync(t->loc_k, kk.data(), sizeof(int32_t) * pairs, cudaMemcpyHostToDevice, s)) ||
+      (e = cudaMemcpyAsync(t->loc_h, hp.data(), sizeof(double2) * 4 * pairs, cudaMemcpyHostToDevice, s)) ||
+      (e = cudaMemcpyAsync(t->loc_D64, D.data(), sizeof(double2) * N, cudaMemcpyHostToDevice, s)))
+    return e;
+  loc_table_kernel<<<(unsigned)((ent + 127) / 128 < 4096 ? (ent + 127) / 128 : 4096), 128, 0, s>>>(
+      t->loc_h, t->loc_k, pairs, t->loc_d, t->loc_base, t->dt, t->d_lo, t->d_delta, t->loc_u64, t->loc_u32);
+  if ((e = cudaGetLastError()) || (e = cudaStreamSynchronize(s))) return e;   // the host arrays end here
+  t->loc = n;
+  return cudaSuccess;
+}
+
+void local_free(redo_table* t) {
+  cudaFree(t->loc_ptr);
+  cudaFree(t->loc_k);
+  cudaFree(t->loc_h);
+  cudaFree(t->loc_u64);
+  cudaFree(t->loc_u32);
+  cudaFree(t->loc_D64);
+}
+
+template <typename R> static LocTab<R> loc_tab(const redo_table* t, int64_t* status) {
+  LocTab<R> o;
+  o.ptr = t->loc_ptr;
+  o.k = t->loc_k;
+  o.u = std::is_same<R, double>::value ? (const cplx<R>*)t->loc_u64 : (const cplx<R>*)t->loc_u32;
+  o.d = t->loc_d;
+  o.base = t->loc_base;
+  o.K = t->K;
+  o.levels = t->levels;
+  o.status = status;
+  o.bad_weight = t->digits;
+  return o;
+}
+
+// ============================================================================
+// Step operators of every (pulse, step): rotations cs[b][n][i] and diagonals Delta[b][0..M][N]
+// ============================================================================
+constexpr int kPrepSteps = 8, kPrepThreads = 256;
+
+template <typename R> __device__ __forceinline__ phase_t<R> no_phase() {
+  if constexpr (sizeof(R) == 4) return 0;
+  else return cmake<R>(R(1), R(0));
+}
+
+template <typename R> __device__ __forceinline__ cplx<R> loc_times(cplx<R> v, double2 d) {
+  const cplx<R> hi = cmake<R>((R)d.x, (R)d.y);
+  if constexpr (sizeof(R) == 8) return cmul<R>(v, hi);
+  cplx<R> o = cmul<R>(v, cmake<R>((R)(d.x - (double)hi.x), (R)(d.y - (double)hi.y)));
+  cfma<R>(o, v, hi);
+  return o;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kPrepThreads)
+loc_steps_kernel(LocTab<R> tab, const int32_t* __restrict__ q, int64_t M, int n, int N, int E, int64_t tiles,
+                 const double2* __restrict__ D, const double2* __restrict__ pd, int64_t pd_b, int64_t pd_n,
+                 cplx<R>* __restrict__ cs, cplx<R>* __restrict__ delta) {
+  // phases of every (step, qubit); row j is step n0 - 1 + j (the step before the tile gives its x)
+  __shared__ phase_t<R> y0[kPrepSteps + 1][10], y1[kPrepSteps + 1][10], xx[kPrepSteps + 1][10];
+  const int64_t b = blockIdx.x / tiles;
+  const int64_t n0 = (blockIdx.x - b * tiles) * kPrepSteps;
+  for (int idx = threadIdx.x; idx < (kPrepSteps + 1) * n; idx += kPrepThreads) {
+    const int j = idx / n, i = idx - j * n;
+    const int64_t m = n0 - 1 + j;
+    Euler<R> f;
+    f.y0 = f.y1 = f.x = no_phase<R>();
+    if (m >= 0 && m < M) {
+      f = loc_factor<R>(loc_step<R>(tab, q + (b * M + m) * tab.K, i, j > 0));
+      if (j > 0) cs[(b * M + m) * n + i] = cmake<R>(f.c, f.s);
+    }
+    y0[j][i] = f.y0;
+    y1[j][i] = f.y1;
+    xx[j][i] = f.x;
+  }
+  __syncthreads();
+  const int G = N / E;
+  for (int idx = threadIdx.x; idx < kPrepSteps * N; idx += kPrepThreads) {
+    const int j = idx / N + 1, r = idx & (N - 1);
+    const int64_t m = n0 - 1 + j;
+    if (m > M) continue;
+    cplx<R> v;
+    if constexpr (sizeof(R) == 4) {
+      uint32_t a = 0;
+      for (int i = 0; i < n; ++i) a += ((r >> i) & 1) ? (uint32_t)y1[j][i] + (uint32_t)xx[j - 1][i] : (uint32_t)y0[j][i];
+      v = phasor((int32_t)a);
+    } else {
+      v = cmake<R>(R(1), R(0));
+      for (int i = 0; i < n; ++i) v = cmul<R>(v, ((r >> i) & 1) ? cmul<R>(y1[j][i], xx[j - 1][i]) : y0[j][i]);
+    }
+    if (m < M) {
+      // the drift (and a pulse's own) is the same at every step, so its FP32 rounding would add up
+      // over the chain: FP32 chains take it as hi + lo
+      v = loc_times<R>(v, D[r]);
+      if (pd) v = loc_times<R>(v, pd[b * pd_b + m * pd_n + r]);
+    }
+    // |Delta| = 1 to the last bit (the residual is exact under fma): without it the rounding of the
+    // phases changed the chain's norm five times as much
+    const R res = R(0.5) * fma(-v.y, v.y, fma(-v.x, v.x, R(1)));
+    delta[(b * (M + 1) + m) * N + loc_pos(r, E, G)] = cmake<R>(fma(res, v.x, v.x), fma(res, v.y, v.y));
+  }
+}
+
+// ============================================================================
+// Chains: segment products S_s = Rot_{n1-1} Delta_{n1-1} ... Rot_{n0} Delta_{n0} (the last segment
+// of a pulse also takes Delta_M), a column per G lanes, the whole segment in registers
+// ============================================================================
+constexpr int kLocThreads = 128;
+
+template <typename R, int N, int E>
+__global__ void __launch_bounds__(kLocThreads)
+loc_chain_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t M, int64_t S, int64_t sps,
+                 int64_t chains, cplx<R>* __restrict__ out) {
+  using L = LocCol<R, N, E>;
+  static_assert(L::G == 1 || N >= L::C, "lanes of one warp share a chain when they exchange");
+  const int lane = threadIdx.x & 31, l = lane / L::C;
+  const int64_t col = ((int64_t)blockIdx.x * (kLocThreads / 32) + (threadIdx.x >> 5)) * L::C + lane % L::C;
+  const int64_t g = col / N;
+  if (g >= chains) return;
+  const int x = (int)(col - g * N);
+  const int64_t b = g / S, n0 = (g - b * S) * sps, n1 = n0 + sps < M ? n0 + sps : M;
+  cplx<R> v[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) v[e] = cmake<R>(l * E + e == x ? R(1) : R(0), R(0));
+  const cplx<R>* d = delta + b * (M + 1) * N;
+  const cplx<R>* r = cs + b * M * L::NQ;
+#pragma unroll 1
+  for (int64_t m = n0; m < n1; ++m) {
+    cplx<R> c[L::NQ];
+    L::load_cs(c, r + m * L::NQ);
+    L::template diag<false>(v, d + m * N, l);
+    L::rotate(v, c, l);
+  }
+  if (n1 == M) L::template diag<false>(v, d + M * N, l);
+  cplx<R>* o = out + g * N * N + x;
+#pragma unroll
+  for (int e = 0; e < E; ++e) o[(int64_t)(l * E + e) * N] = v[e];
+}
+
+// Entries a lane holds.  FP32: 32 for chains (64 state registers), 16 for the gradient's two
+// vectors.  FP64: the FP64 pipe issues one warp instruction per ~70 cycles and scheduler whatever
+// the lane count, so a column is spread over more lanes; small N must fill a warp with one chain.
+__host__ __device__ constexpr int loc_entries(bool dbl, int N, bool two) {
+  if (dbl) return N <= 4 ? N : (N == 8 ? 2 : (N == 16 || (two && N <= 256) ? 8 : (N <= 512 ? 16 : 32)));
+  const int e = two && N <= 512 ? 16 : 32;
+  return N < e ? N : e;
+}
+
+template <typename R, int N, bool TWO>
+static cudaError_t loc_chain_n(const redo_table* t, const ChainPlan& p, int64_t B, const void* cs, const void* delta,
+                               void* out, cudaStream_t s) {
+  constexpr int E = loc_entries(sizeof(R) == 8, N, TWO);
+  const int64_t fps = (int64_t)t->K * t->digits, chains = B * p.S, sps = p.seg_len / fps;
+  const int64_t warps = (chains * N * (N / E) + 31) / 32;
+  if (warps == 0) return cudaSuccess;
+  loc_chain_kernel<R, N, E><<<(unsigned)((warps + 3) / 4), kLocThreads, 0, s>>>(
+      (const cplx<R>*)cs, (const cplx<R>*)delta, p.M, p.S, sps > 0 ? sps : 1, chains, (cplx<R>*)out);
+  return cudaGetLastError();
+}
+
+#define LOC_DISPATCH(FN, ...)                                     \
+  switch (t->N) {                                                 \
+    case 2: return FN<R, 2, TWO>(__VA_ARGS__);                    \
+    case 4: return FN<R, 4, TWO>(__VA_ARGS__);                    \
+    case 8: return FN<R, 8, TWO>(__VA_ARGS__);                    \
+    case 16: return FN<R, 16, TWO>(__VA_ARGS__);                  \
+    case 32: return FN<R, 32, TWO>(__VA_ARGS__);                  \
+    case 64: return FN<R, 64, TWO>(__VA_ARGS__);                  \
+    case 128: return FN<R, 128, TWO>(__VA_ARGS__);                \
+    case 256: return FN<R, 256, TWO>(__VA_ARGS__);                \
+    case 512: return FN<R, 512, TWO>(__VA_ARGS__);                \
+    case 1024: return FN<R, 1024, TWO>(__VA_ARGS__);              \
+    default: return cudaErrorInvalidValue;                        \
+  }
+
+template <typename R, bool TWO>
+static cudaError_t loc_chain_t(const redo_table* t, const ChainPlan& p, int64_t B, const void* cs, const void* delta,
+                               void* out, cudaStream_t s) {
+  LOC_DISPATCH(loc_chain_n, t, p, B, cs, delta, out, s)
+}
+
+// ============================================================================
+// GRAPE gradient: reverse sweep of the segments.  A column x of P and row x of R stay with the
+// same lanes, so undoing a step (P <- U^dag P, R <- R U) and the traces are local to them; only
+// the Bloch sums Im Tr(sigma_i P R) of every qubit are added over x.  They hold every control's
+// trace: Tr(g P R) for g = sum_i g_i needs the one-qubit partial traces only.  bl receives them as
+// [step][part][3n], one part per warp of the chain, added in a fixed order afterwards.
+// TZ (amplitude/phase calls): also Tz = Im Tr(S_kz P R) at every step boundary.
+// ============================================================================
+template <typename R, int N, int E, bool TZ>
+__global__ void __launch_bounds__(kLocThreads, E * sizeof(R) <= 64 ? 4 : 2)
+loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t M, int64_t S, int64_t sps,
+                 int64_t chains, const cplx<R>* __restrict__ Pck, const cplx<R>* __restrict__ Rck,
+                 const double2* __restrict__ tau, R* __restrict__ bl, int K, const double* __restrict__ sz,
+                 R* __restrict__ bz) {
+  using L = LocCol<R, N, E>;
+  using WS = WarpSums<R, 3 * L::NQ>;
+  constexpr int LPC = N * L::G, PARTS = LPC >= 32 ? LPC / 32 : 1, W = LPC >= 32 ? 32 : LPC;
+  const int lane = threadIdx.x & 31, l = lane / L::C;
+  const int64_t col = ((int64_t)blockIdx.x * (kLocThreads / 32) + (threadIdx.x >> 5)) * L::C + lane % L::C;
+  const bool on = col / N < chains;
+  const int64_t g = on ? col / N : chains - 1;       // idle lanes follow the last chain, write nothing
+  const int x = (int)(col % N);
+  const int part = x / L::C;
+  const int64_t b = g / S, n0 = (g - b * S) * sps, n1 = n0 + sps < M ? n0 + sps : M;
+  const cplx<R>* d = delta + b * (M + 1) * N;
+  const cplx<R>* r = cs + b * M * L::NQ;
+  cplx<R> p[E], w[E];
+  {
+    const double2 tb = tau[b];
+    const cplx<R>* P = Pck + g * N * N + x;
+    const cplx<R>* Q = Rck + g * N * N + (int64_t)x * N + l * E;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      p[e] = P[(int64_t)(l * E + e) * N];
+      const double qx = (double)Q[e].x, qy = (double)Q[e].y;      // R conj(tau): traces come out as Im alone
+      w[e] = cmake<R>((R)(qx * tb.x + qy * tb.y), (R)(qy * tb.x - qx * tb.y));
+    }
+  }
+  // Tr(S_kz P R) = sum_r sz[k][r] (P R)[r][r], this lane's rows
+  auto boundary = [&](int64_t n, bool act) {
+    if constexpr (TZ) {
+      R t[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) t[e] = fma(p[e].x, w[e].y, p[e].y * w[e].x);
+      for (int k = 0; k < K; ++k) {
+        R a = R(0);
+#pragma unroll
+        for (int e = 0; e < E; ++e) a = fma((R)sz[(int64_t)k * N + l * E + e], t[e], a);
+#pragma unroll
+        for (int off = W / 2; off >= 1; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+        if (act && lane % W == 0) bz[((b * (M + 1) + n) * PARTS + part) * K + k] = a;
+      }
+    }
+  };
+  if (n1 == M) {
+    L::template diag<true>(p, d + M * N, l);
+    L::template diag<false>(w, d + M * N, l);
+  }
+  boundary(M, on && n1 == M);
+  const int len = (int)(n1 - n0);
+  const int most = LPC >= 32 ? len : __reduce_max_sync(0xffffffffu, len);   // several chains in a warp
+#pragma unroll 1
+  for (int t = 0; t < most; ++t) {
+    const bool act = on && t < len;
+    const int64_t m = t < len ? n1 - 1 - t : n0;
+    cplx<R> c[L::NQ];
+    L::load_cs(c, r + m * L::NQ);
+    R v[WS::P];
+#pragma unroll
+    for (int i = 0; i < WS::P; ++i) v[i] = R(0);
+    L::trace_undo(p, w, c, l, v);
+    R* o = bl + ((b * M + m) * PARTS + part) * (3 * L::NQ);
+    if constexpr (W == 32) {
+      const int idx = WS::full(v, lane);
+      if (act && idx >= 0) o[idx] = v[0];
+    } else {
+#pragma unroll
+      for (int i = 0; i < 3 * L::NQ; ++i) {
+#pragma unroll
+        for (int off = W / 2; off >= 1; off >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], off);
+        if (act && lane % W == 0) o[i] = v[i];
+      }
+    }
+    boundary(m, act);
+    L::template diag<true>(p, d + m * N, l);
+    L::template diag<false>(w, d + m * N, l);
+  }
+}
+
+// dF/du_kn = (2 dt / N^2) sum_i Tr(g_ki rho_i) with g_ki = W h_ki W^dag, W the product of the
+// factors after k on qubit i, conjugated by the step's trailing phase diag(1, x_i) (the sums are
+// taken between the rotation and that phase): Re(g01 x (X + iY)) + gz Z.
+constexpr int kFinSteps = 8, kFinThreads = 128;
+
+template <typename R>
+__global__ void __launch_bounds__(kFinThreads)
+loc_grad_kernel(LocTab<R> tab, const double2* __restrict__ h, const int32_t* __restrict__ q, int64_t M, int n, int parts,
+                int64_t tiles, const R* __restrict__ bl, double scale, double* __restrict__ grad) {
+  __shared__ double sum[kFinSteps][30];
+  __shared__ double2 xy[kFinSteps][10];
+  const int64_t b = blockIdx.x / tiles, m0 = (blockIdx.x - b * tiles) * kFinSteps;
+  const int steps = (int)(M - m0 < kFinSteps ? M - m0 : kFinSteps);
+  for (int idx = threadIdx.x; idx < steps * 3 * n; idx += kFinThreads) {
+    const int j = idx / (3 * n), v = idx - j * 3 * n;
+    const R* o = bl + (b * M + m0 + j) * parts * (3 * n) + v;
+    double a = 0.0;
+    for (int p = 0; p < parts; ++p) a += (double)o[(int64_t)p * 3 * n];
+    sum[j][v] = a;
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < steps * n; idx += kFinThreads) {
+    const int j = idx / n, i = idx - j * n;
+    const phase_t<R> x = loc_factor<R>(loc_step<R>(tab, q + (b * M + m0 + j) * tab.K, i, false)).x;
+    double2 xv;
+    if constexpr (sizeof(R) == 4) {
+      const float2 f = phasor(x);
+      xv = make_double2(f.x, f.y);
+    } else {
+      xv = x;
+    }
+    const double X = sum[j][3 * i], Y = sum[j][3 * i + 1];
+    xy[j][i] = make_double2(xv.x * X - xv.y * Y, xv.x * Y + xv.y * X);
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < steps * tab.K; idx += kFinThreads) {
+    const int j = idx / tab.K, k = idx - j * tab.K;
+    const int32_t* qrow = q + (b * M + m0 + j) * tab.K;
+    double acc = 0.0;
+    for (int i = 0; i < n; ++i) {
+      Mat2<R> w;
+      w.a = w.e = cmake<R>(R(1), R(0));
+      w.b = w.c = cmake<R>(R(0), R(0));
+      for (int p = tab.ptr[i + 1] - 1; p >= tab.ptr[i]; --p) {
+        const int kf = tab.k[p];
+        if ((kf & ~kLocFirst) != k) {
+          w = mat2_mul<R>(w, loc_term<R>(tab, p, loc_level<R>(tab, qrow, kf, false)));
+          continue;
+        }
+        Mat2<R> hm, wd;
+        hm.a = cmake<R>((R)h[4 * p].x, (R)h[4 * p].y);
+        hm.b = cmake<R>((R)h[4 * p + 1].x, (R)h[4 * p + 1].y);
+        hm.c = cmake<R>((R)h[4 * p + 2].x, (R)h[4 * p + 2].y);
+        hm.e = cmake<R>((R)h[4 * p + 3].x, (R)h[4 * p + 3].y);
+        wd.a = cmake<R>(w.a.x, -w.a.y);
+        wd.b = cmake<R>(w.c.x, -w.c.y);
+        wd.c = cmake<R>(w.b.x, -w.b.y);
+        wd.e = cmake<R>(w.e.x, -w.e.y);
+        const Mat2<R> gm = mat2_mul<R>(mat2_mul<R>(w, hm), wd);
+        acc += (double)gm.b.x * xy[j][i].x - (double)gm.b.y * xy[j][i].y +
+               0.5 * ((double)gm.a.x - (double)gm.e.x) * sum[j][3 * i + 2];
+        break;
+      }
+    }
+    grad[(b * M + m0 + j) * tab.K + k] = scale * acc;
+  }
+}
+
+// gphi[b][n][k] = (2 / N^2) (Tz[n+1][k] - Tz[n][k]) (the traces already carry conj(tau))
+template <typename R>
+__global__ void loc_phase_kernel(const R* __restrict__ bz, int64_t B, int64_t M, int parts, int K, double scale,
+                                 double* __restrict__ gphi) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B * M * K; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t bn = i / K, b = bn / M, n = bn - b * M;
+    const int k = (int)(i - bn * K);
+    double a = 0.0, c = 0.0;
+    for (int p = 0; p < parts; ++p) {
+      a += (double)bz[((b * (M + 1) + n) * parts + p) * K + k];
+      c += (double)bz[((b * (M + 1) + n + 1) * parts + p) * K + k];
+    }
+    gphi[i] = scale * (c - a);
+  }
+}
+
+template <typename R, int N, bool TWO>
+static cudaError_t loc_sweep_n(const redo_table* t, const ChainPlan& p, int64_t B, const void* cs, const void* delta,
+                               const void* Pck, const void* Rck, const double2* tau, void* bl, void* bz,
+                               cudaStream_t s) {
+  if constexpr (sizeof(R) == 8 && N > 512) {
+    return cudaErrorInvalidValue;                    // not eligible: two columns do not fit the registers
+  } else {
+  constexpr int E = loc_entries(sizeof(R) == 8, N, true);
+  const int64_t fps = (int64_t)t->K * t->digits, chains = B * p.S, sps = p.seg_len / fps;
+  const int64_t warps = (chains * N * (N / E) + 31) / 32;
+  if (warps == 0) return cudaSuccess;
+  auto kern = bz ? loc_sweep_kernel<R, N, E, true> : loc_sweep_kernel<R, N, E, false>;
+  kern<<<(unsigned)((warps + 3) / 4), kLocThreads, 0, s>>>(
+      (const cplx<R>*)cs, (const cplx<R>*)delta, p.M, p.S, sps, chains, (const cplx<R>*)Pck, (const cplx<R>*)Rck, tau,
+      (R*)bl, t->K, t->sz64, (R*)bz);
+  return cudaGetLastError();
+  }
+}
+
+template <typename R>
+static cudaError_t loc_sweep_t(const redo_table* t, const ChainPlan& p, int64_t B, const void* cs, const void* delta,
+                               const void* Pck, const void* Rck, const double2* tau, void* bl, void* bz,
+                               cudaStream_t s) {
+  constexpr bool TWO = true;
+  LOC_DISPATCH(loc_sweep_n, t, p, B, cs, delta, Pck, Rck, tau, bl, bz, s)
+}
+
+// ============================================================================
+// Host side: step-operator scratch in slices of pulses, plans, launches
+// ============================================================================
+// A slice holds the rotations and diagonals of as many pulses as fit kLocSlice bytes, so that long
+// batches need bounded scratch; a pulse that does not fit alone keeps the dense path.
+constexpr size_t kLocSlice = (size_t)512 << 20;
+
+static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// parts of the Bloch sums of one step: the warps of a chain
+static int loc_parts(const redo_table* t, bool dbl) {
+  const int lanes = t->N * (t->N / loc_entries(dbl, t->N, true));
+  return lanes >= 32 ? lanes / 32 : 1;
+}
+
+// Scratch of nb pulses: diagonals, rotations and, for a gradient (what >= 1), the Bloch sums and
+// (what = 2) the boundary traces.
+struct LocScratch {
+  void *delta, *cs, *bl, *bz;
+  size_t total;
+};
+static LocScratch loc_scratch(const redo_table* t, int64_t nb, int64_t M, int prec, int what, void* base) {
+  const size_t el = prec == REDO_FP64 ? sizeof(double) : sizeof(float);
+  const size_t parts = what ? (size_t)loc_parts(t, prec == REDO_FP64) : 0;
+  LocScratch w;
+  char* c = (char*)base;
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    void* at = c + off;
+    off += up256(bytes);
+    return at;
+  };
+  w.delta = take((size_t)nb * (M + 1) * t->N * 2 * el);
+  w.cs = take((size_t)nb * M * t->loc * 2 * el);
+  w.bl = take(what >= 1 ? (size_t)nb * M * parts * 3 * t->loc * el : 0);
+  w.bz = take(what == 2 ? (size_t)nb * (M + 1) * parts * t->K * el : 0);
+  w.total = off;
+  return w;
+}
+
+bool local_eligible(const redo_table* t, int64_t M, int prec, int what) {
+  if (t->loc == 0 || (what && prec == REDO_FP64 && t->N > 512)) return false;
+  return loc_scratch(t, 1, M, prec, what, nullptr).total <= kLocSlice;
+}
+
+static int64_t local_slice(const redo_table* t, int64_t B, int64_t M, int prec, int what) {
+  const int64_t n = (int64_t)(kLocSlice / loc_scratch(t, 1, M, prec, what, nullptr).total);
+  return n < B ? n : B;
+}
+
+size_t local_ops_bytes(const redo_table* t, int64_t B, int64_t M, int prec, int what) {
+  return loc_scratch(t, local_slice(t, B, M, prec, what), M, prec, what, nullptr).total;
+}
+
+// Segments of whole steps.  Columns of one pulse are independent, so time is cut only as far as the
+// columns leave the GPU's schedulers idle (about four warps each), and not below 8 steps: every
+// further segment costs a dense product when the segments are multiplied.
+ChainPlan plan_chain_local(const redo_table* t, int64_t B, int64_t M, int prec, bool two) {
+  const bool dbl = prec == REDO_FP64;
+  const int E = loc_entries(dbl, t->N, two);
+  const int64_t warps = (B * t->N * (t->N / E) + 31) / 32;
+  int64_t S = warps > 0 ? (4 * 4 * (int64_t)t->num_sms + warps - 1) / warps : 1;
+  const int64_t min_steps = t->N <= 8 ? 4 : (t->N <= 64 ? 8 : 32);
+  if (S > M / min_steps) S = M / min_steps;
+  if (S > 64) S = 64;
+  if (S < 1) S = 1;
+  return plan_chain_aligned(t, B, M, M > 0 ? (M + S - 1) / S : 1);
+}
+
+template <typename R>
+static cudaError_t loc_steps_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int E, const LocalDiag& pd,
+                               int64_t b0, void* cs, void* delta, int64_t* status, cudaStream_t s) {
+  const int64_t tiles = (M + 1 + kPrepSteps - 1) / kPrepSteps;
+  loc_steps_kernel<R><<<(unsigned)(B * tiles), kPrepThreads, 0, s>>>(
+      loc_tab<R>(t, status), q + b0 * M * t->K, M, t->loc, t->N, E, tiles,
+      t->loc_D64,
+      pd.p ? pd.p + b0 * pd.sb : nullptr, pd.sb, pd.sn, (cplx<R>*)cs, (cplx<R>*)delta);
+  return cudaGetLastError();
+}
+
+static cudaError_t loc_steps(const redo_table* t, const int32_t* q, int64_t nb, int64_t M, int prec, int E,
+                             const LocalDiag& pd, int64_t b0, const LocScratch& w, int64_t* status, cudaStream_t s) {
+  return prec == REDO_FP64 ? loc_steps_t<double>(t, q, nb, M, E, pd, b0, w.cs, w.delta, status, s)
+                           : loc_steps_t<float>(t, q, nb, M, E, pd, b0, w.cs, w.delta, status, s);
+}
+
+cudaError_t launch_local_chain(const redo_table* t, const int32_t* q, const ChainPlan& p, int prec, int what,
+                               const LocalDiag& pd, void* ops, void* seg_out, int64_t* status, cudaStream_t s) {
+  const bool dbl = prec == REDO_FP64, two = what > 0;
+  const int64_t slice = local_slice(t, p.B, p.M, prec, what);
+  const LocScratch w = loc_scratch(t, slice, p.M, prec, what, ops);
+  const int E = loc_entries(dbl, t->N, two);
+  const size_t mat = (size_t)t->N * t->N * (dbl ? sizeof(double2) : sizeof(float2));
+  for (int64_t b0 = 0; b0 < p.B; b0 += slice) {
+    const int64_t nb = b0 + slice < p.B ? slice : p.B - b0;
+    cudaError_t e = loc_steps(t, q, nb, p.M, prec, E, pd, b0, w, status, s);
+    if (e) return e;
+    void* out = (char*)seg_out + (size_t)(b0 * p.S) * mat;
+    e = dbl ? (two ? loc_chain_t<double, true>(t, p, nb, w.cs, w.delta, out, s)
+                   : loc_chain_t<double, false>(t, p, nb, w.cs, w.delta, out, s))
+            : (two ? loc_chain_t<float, true>(t, p, nb, w.cs, w.delta, out, s)
+                   : loc_chain_t<float, false>(t, p, nb, w.cs, w.delta, out, s));
+    if (e) return e;
+  }
+  return cudaSuccess;
+}
+
+template <typename R>
+static cudaError_t loc_finish_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int parts, double norm,
+                                const LocScratch& w, double* grad, double* gphi, cudaStream_t s) {
+  const int64_t tiles = (M + kFinSteps - 1) / kFinSteps;
+  LocTab<R> tab = loc_tab<R>(t, nullptr);
+  loc_grad_kernel<R><<<(unsigned)(B * tiles), kFinThreads, 0, s>>>(tab, t->loc_h, q, M, t->loc, parts, tiles,
+                                                                   (const R*)w.bl, 2.0 * t->dt / norm, grad);
+  if (gphi) {
+    const int64_t n = B * M * t->K, blocks = (n + 255) / 256;
+    loc_phase_kernel<R><<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>((const R*)w.bz, B, M, parts, t->K,
+                                                                                  2.0 / norm, gphi);
+  }
+  return cudaGetLastError();
+}
+
+// Reverse sweep and gradients of all pulses (what = 2: also the phase gradients gphi).  With more
+// than one slice the step operators, overwritten by the later slices, are formed again.
+cudaError_t launch_local_grad(const redo_table* t, const int32_t* q, const ChainPlan& p, int prec, int what,
+                              const LocalDiag& pd, void* ops, const void* Pck, const void* Rck, const double2* tau,
+                              double* grad, double* gphi, int64_t* status, cudaStream_t s) {
+  const bool dbl = prec == REDO_FP64;
+  const int64_t slice = local_slice(t, p.B, p.M, prec, what);
+  const LocScratch w = loc_scratch(t, slice, p.M, prec, what, ops);
+  const int E = loc_entries(dbl, t->N, true), parts = loc_parts(t, dbl);
+  const size_t mat = (size_t)t->N * t->N * (dbl ? sizeof(double2) : sizeof(float2));
+  const double norm = (double)t->N * (double)t->N;
+  for (int64_t b0 = 0; b0 < p.B; b0 += slice) {
+    const int64_t nb = b0 + slice < p.B ? slice : p.B - b0;
+    cudaError_t e = cudaSuccess;
+    if (slice < p.B && (e = loc_steps(t, q, nb, p.M, prec, E, pd, b0, w, status, s))) return e;
+    const char* P = (const char*)Pck + (size_t)(b0 * p.S) * mat;
+    const char* Q = (const char*)Rck + (size_t)(b0 * p.S) * mat;
+    void* bz = what == 2 ? w.bz : nullptr;
+    e = dbl ? loc_sweep_t<double>(t, p, nb, w.cs, w.delta, P, Q, tau + b0, w.bl, bz, s)
+            : loc_sweep_t<float>(t, p, nb, w.cs, w.delta, P, Q, tau + b0, w.bl, bz, s);
+    if (e) return e;
+    const int64_t at = b0 * p.M * t->K;
+    double* gp = gphi ? gphi + at : nullptr;
+    e = dbl ? loc_finish_t<double>(t, q + at, nb, p.M, parts, norm, w, grad + at, gp, s)
+            : loc_finish_t<float>(t, q + at, nb, p.M, parts, norm, w, grad + at, gp, s);
+    if (e) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace redo

@@ -861,30 +861,59 @@ cudaError_t launch_chain_segments(const redo_table* t, const int32_t* q, const C
   return chain_segments_t<float>(t, q, p, seg_out, status, s, keep);
 }
 
-template <typename R>
-static cudaError_t chain_combine_t(const redo_table* t, const ChainPlan& p, const void* seg_in,
-                                   void* prod_out, int64_t* status, cudaStream_t s) {
-  DenseSrc<R> src;
-  src.P = (const cplx<R>*)seg_in;
-  src.per_unit = p.S;
-  cplx<R>* out = (cplx<R>*)prod_out;
+// Segments per group of the two-pass combine: about sqrt(S), 0 for one pass.  A pulse's segments
+// are multiplied by one CTA, so a single pulse of S segments is a chain of S dependent products;
+// groups make it sqrt(S) + S / sqrt(S), in parallel over the groups.
+static int64_t combine_group(const ChainPlan& p) {
   const int64_t L = p.F > 0 ? p.S : 0;
+  if (L < 9) return 0;
+  int64_t g = 3;
+  while (g * g < L) ++g;
+  return g;
+}
+
+size_t combine_mid_bytes(const redo_table* t, const ChainPlan& p, int prec) {
+  const int64_t g = combine_group(p);
+  if (!g) return 0;
+  const size_t el = prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
+  return ((size_t)p.B * ((p.S + g - 1) / g) * t->N * t->N * el + 255) & ~(size_t)255;
+}
+
+template <typename R>
+static cudaError_t chain_combine_pass(const redo_table* t, int64_t B, int64_t L, int64_t g, const void* in, void* outv,
+                                      int64_t* status, cudaStream_t s) {
+  DenseSrc<R> src;
+  src.P = (const cplx<R>*)in;
+  src.per_unit = L;
+  cplx<R>* out = (cplx<R>*)outv;
+  const int64_t units = g > 0 ? (L + g - 1) / g : 1;
   switch (t->N) {
-    case 2: return launch_chain_n<R, 2>(src, p.B, 1, L, L, out, status, s);
-    case 4: return launch_chain_n<R, 4>(src, p.B, 1, L, L, out, status, s);
-    case 8: return launch_chain_n<R, 8>(src, p.B, 1, L, L, out, status, s);
-    case 16: return launch_chain_n<R, 16>(src, p.B, 1, L, L, out, status, s);
-    case 32: return launch_chain_n<R, 32>(src, p.B, 1, L, L, out, status, s);
-    case 64: return launch_chain_n<R, 64>(src, p.B, 1, L, L, out, status, s);
+    case 2: return launch_chain_n<R, 2>(src, B, units, g, L, out, status, s);
+    case 4: return launch_chain_n<R, 4>(src, B, units, g, L, out, status, s);
+    case 8: return launch_chain_n<R, 8>(src, B, units, g, L, out, status, s);
+    case 16: return launch_chain_n<R, 16>(src, B, units, g, L, out, status, s);
+    case 32: return launch_chain_n<R, 32>(src, B, units, g, L, out, status, s);
+    case 64: return launch_chain_n<R, 64>(src, B, units, g, L, out, status, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
+template <typename R>
+static cudaError_t chain_combine_t(const redo_table* t, const ChainPlan& p, const void* seg_in,
+                                   void* prod_out, int64_t* status, cudaStream_t s, void* mid) {
+  const int64_t L = p.F > 0 ? p.S : 0, g = mid ? combine_group(p) : 0;
+  if (!g) return chain_combine_pass<R>(t, p.B, L, L, seg_in, prod_out, status, s);
+  cudaError_t e = chain_combine_pass<R>(t, p.B, L, g, seg_in, mid, status, s);
+  if (e) return e;
+  const int64_t L2 = (L + g - 1) / g;
+  return chain_combine_pass<R>(t, p.B, L2, L2, mid, prod_out, status, s);
+}
+
 cudaError_t launch_chain_combine(const redo_table* t, const ChainPlan& p, int prec,
                                  const void* seg_in, void* prod_out, int64_t* status,
-                                 cudaStream_t s) {
-  if (prec == REDO_FP64) return chain_combine_t<double>(t, p, seg_in, prod_out, status, s);
-  return chain_combine_t<float>(t, p, seg_in, prod_out, status, s);
+                                 cudaStream_t s, void* mid) {
+  if (prec == REDO_FP64) return chain_combine_t<double>(t, p, seg_in, prod_out, status, s, mid);
+  return chain_combine_t<float>(t, p, seg_in, prod_out, status, s, mid);
 }
 
 // ============================================================================

@@ -353,6 +353,7 @@ redo_status redo_build_table(int32_t N, int32_t K, double dt, const void* H0, co
     e = N > kSmallN ? launch_build_tc_large_planes(t, s) : launch_build_tc_planes(t, s);
     if (e != cudaSuccess) return fail(cuda_error(e, "FP16x3 planes"));
   }
+  if ((e = local_build(t, h, s)) != cudaSuccess) return fail(cuda_error(e, "one-qubit tables"));
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(cuda_error(e, "table build"));
   *out = t;
   return REDO_OK;
@@ -375,6 +376,7 @@ redo_status redo_table_free(redo_table* t) {
   cudaFree(t->hk_xmask);
   cudaFree(t->hk_xval);
   cudaFree(t->sz64);
+  local_free(t);
   std::free(t->h0_pairs);
   std::free(t);
   return REDO_OK;
@@ -464,6 +466,9 @@ struct PropLayout {
   size_t seg_off, prod_off, prod64_off, total;
   size_t strang_off, strang_tmp_off;   // symmetric split: conjugated products (+ dense-drift scratch)
   size_t pd_off, zf_off, phout_off;     // amplitude/phase calls
+  size_t mid_off;                       // group products of the two-pass combine (N <= 64)
+  bool local;                           // locally controlled system: kernels_local.cu forms the segments
+  size_t ops_off;                       // its step operators
 };
 
 // FP64 matrices appended to a workspace for the symmetric split's conjugation
@@ -490,12 +495,36 @@ static void add_phase(const redo_table* t, int64_t B, int64_t M, size_t& total, 
   total = out_off + up((size_t)B * t->N * t->N * sizeof(double2));
 }
 
+// diag: step-opening diagonals (1: one per step, amplitude/phase calls; 2: one per pulse, drift calls)
 static PropLayout prop_layout(const redo_table* t, int64_t B, int64_t M, redo_precision prec,
-                              int32_t reunit_every, bool phase = false) {
-  PropLayout L;
-  L.pd_off = L.zf_off = L.phout_off = 0;
+                              int32_t reunit_every, int diag = 0) {
+  PropLayout L{};
+  const bool phase = diag != 0;
+  // the tensor-core precision forms segment products in split FP16 and combines them in FP32
+  L.eff_prec = prec == REDO_FP16X3 ? REDO_FP32 : prec;
+  auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  const size_t el = L.eff_prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
+  const size_t n2 = (size_t)t->N * t->N;
+  if (local_eligible(t, M, L.eff_prec, 0)) {
+    L.local = true;
+    L.p = reunit_every > 0 ? plan_chain_aligned(t, B, M, reunit_every) : plan_chain_local(t, B, M, L.eff_prec, false);
+    if (t->N > kSmallN) {
+      // one whole-pulse segment needs no dense product
+      L.total = L.p.S > 1 || reunit_every > 0 ? large_prop_workspace(t, L.p, L.eff_prec, reunit_every > 0)
+                                              : up((size_t)B * n2 * el);
+    } else {
+      L.prod_off = up((size_t)B * L.p.S * n2 * el);
+      L.mid_off = L.prod_off + up((size_t)B * n2 * el);
+      L.prod64_off = L.mid_off + combine_mid_bytes(t, L.p, L.eff_prec);
+      L.total = L.prod64_off + (reunit_every > 0 ? up((size_t)B * n2 * sizeof(double2)) : 0);
+    }
+    L.ops_off = L.total;
+    L.total += local_ops_bytes(t, B, M, L.eff_prec, 0);
+    add_strang(t, B, L.total, L.strang_off, L.strang_tmp_off);
+    if (diag) add_phase(t, B, diag == 1 ? M : 1, L.total, L.pd_off, L.zf_off, L.phout_off);
+    return L;
+  }
   if (t->N > kSmallN) {
-    L.eff_prec = prec == REDO_FP16X3 ? REDO_FP32 : prec;
     if (reunit_every > 0) {
       L.p = plan_chain_aligned(t, B, M, reunit_every);
     } else {
@@ -513,8 +542,6 @@ static PropLayout prop_layout(const redo_table* t, int64_t B, int64_t M, redo_pr
     if (phase) add_phase(t, B, M, L.total, L.pd_off, L.zf_off, L.phout_off);
     return L;
   }
-  // the tensor-core path forms segment products in split FP16 and combines them in FP32
-  L.eff_prec = prec == REDO_FP16X3 ? REDO_FP32 : prec;
   // amplitude/phase calls: the SIMT chains carry each step's diagonal as an extra factor, the
   // tensor-core chains apply it in the epilogue of the step's last product
   const bool phase_factors = phase && prec != REDO_FP16X3;
@@ -522,12 +549,10 @@ static PropLayout prop_layout(const redo_table* t, int64_t B, int64_t M, redo_pr
     L.p = plan_chain_aligned(t, B, M, reunit_every, phase_factors);
   else
     L.p = prec == REDO_FP16X3 ? plan_chain_tc(t, B, M) : plan_chain(t, B, M, L.eff_prec, phase_factors);
-  auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  const size_t el = L.eff_prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
-  const size_t n2 = (size_t)t->N * t->N;
   L.seg_off = 0;
   L.prod_off = up((size_t)L.p.B * L.p.S * n2 * el);
-  L.prod64_off = L.prod_off + up((size_t)L.p.B * n2 * el);
+  L.mid_off = L.prod_off + up((size_t)L.p.B * n2 * el);
+  L.prod64_off = L.mid_off + combine_mid_bytes(t, L.p, L.eff_prec);
   L.total = L.prod64_off + (reunit_every > 0 ? up((size_t)L.p.B * n2 * sizeof(double2)) : 0);
   add_strang(t, B, L.total, L.strang_off, L.strang_tmp_off);
   if (phase) add_phase(t, B, M, L.total, L.pd_off, L.zf_off, L.phout_off);
@@ -565,7 +590,7 @@ static redo_status propagate_core(const redo_table* t, const int32_t* q, const d
     return set_error(REDO_ERR_INVALID, "U_target given without F_out or tau_out");
   if (!U_out && !U_target) return set_error(REDO_ERR_INVALID, "nothing to compute");
   if (reunit_every > M) reunit_every = M > 0 ? (int32_t)M : 0;
-  PropLayout L = prop_layout(t, B, M, prec, reunit_every, diag);
+  PropLayout L = prop_layout(t, B, M, prec, reunit_every, phase ? 1 : h ? 2 : 0);
   if (!workspace || workspace_bytes < L.total)
     return set_error(REDO_ERR_INVALID, "workspace of %zu bytes needed", L.total);
   if (((uintptr_t)workspace & 255) != 0) return set_error(REDO_ERR_INVALID, "workspace not 256-byte aligned");
@@ -575,9 +600,9 @@ static redo_status propagate_core(const redo_table* t, const int32_t* q, const d
   if (diag) {
     double2* pd = (double2*)((char*)workspace + L.pd_off);
     zf = (double2*)((char*)workspace + L.zf_off);
-    const bool tc = prec == REDO_FP16X3 && t->N <= kSmallN;     // the split-FP16 chains take FP32 diagonals
+    const bool tc = !L.local && prec == REDO_FP16X3 && t->N <= kSmallN;     // the split-FP16 chains take FP32 diagonals
     e = phase ? launch_phase_diag(t, phi, B, M, tc ? nullptr : pd, tc ? (float2*)pd : nullptr, zf, s)
-              : launch_drift_diag(t, h, B, M, tc ? nullptr : pd, tc ? (float2*)pd : nullptr, s);
+              : launch_drift_diag(t, h, B, L.local ? (M > 0 ? 1 : 0) : M, tc ? nullptr : pd, tc ? (float2*)pd : nullptr, s);
     if (e != cudaSuccess) return cuda_error(e, phase ? "phase diagonals" : "drift diagonals");
     if (tc)
       L.p.pd32 = (const float2*)pd;
@@ -598,12 +623,22 @@ static redo_status propagate_core(const redo_table* t, const int32_t* q, const d
   char* seg = (char*)workspace + L.seg_off;
   char* prod = (char*)workspace + L.prod_off;
   char* prod64 = (char*)workspace + L.prod64_off;
+  if (L.local) {
+    ProfScope ps(2, s);
+    const LocalDiag pd{L.p.pd, phase ? M * t->N : t->N, phase ? t->N : 0};
+    if ((e = launch_local_chain(t, q, p, eff, 0, pd, (char*)workspace + L.ops_off, seg, dev_status, s)) !=
+        cudaSuccess)
+      return cuda_error(e, "local chains");
+  }
   if (t->N > kSmallN) {
     void* res = nullptr;
     int res_prec = eff;
-    {
+    if (L.local && p.S == 1 && reunit_every == 0) {
+      res = seg;
+    } else {
       ProfScope ps(2, s);
-      e = prec == REDO_FP16X3
+      e = L.local ? large_finish(t, p, eff, reunit_every > 0, workspace, &res, &res_prec, s)
+          : prec == REDO_FP16X3
               ? tc_large_propagate(t, q, p, reunit_every > 0, workspace, &res, &res_prec, dev_status, s)
               : large_propagate(t, q, p, eff, reunit_every > 0, workspace, &res, &res_prec,
                                 dev_status, s);
@@ -627,7 +662,9 @@ static redo_status propagate_core(const redo_table* t, const int32_t* q, const d
       return cuda_error(e, "finalize");
     return REDO_OK;
   }
-  if (prec == REDO_FP16X3) {
+  if (L.local) {
+    // segment products already formed
+  } else if (prec == REDO_FP16X3) {
     ProfScope ps(5, s);
     if ((e = launch_chain_tc(t, q, p, seg, dev_status, s)) != cudaSuccess)
       return cuda_error(e, "tensor-core chain segments");
@@ -641,9 +678,12 @@ static redo_status propagate_core(const redo_table* t, const int32_t* q, const d
     if ((e = launch_polar(t, eff, eff, seg, seg, p.B * p.S, 1, s)) != cudaSuccess)
       return cuda_error(e, "segment re-unitarisation");
   }
-  {
+  if (p.S == 1 && p.F > 0) {
+    prod = seg;                                      // one segment is the pulse's product
+  } else {
     ProfScope ps(3, s);
-    if ((e = launch_chain_combine(t, p, eff, seg, prod, dev_status, s)) != cudaSuccess)
+    if ((e = launch_chain_combine(t, p, eff, seg, prod, dev_status, s,
+                                  L.prod64_off > L.mid_off ? (char*)workspace + L.mid_off : nullptr)) != cudaSuccess)
       return cuda_error(e, "chain combine");
   }
   const void* fin = prod;
@@ -698,7 +738,7 @@ redo_status redo_propagate_phase_workspace(const redo_table* t, int64_t B, int64
   if (st != REDO_OK) return st;
   if ((st = check_phase(t, prec)) != REDO_OK) return st;
   if (reunit_every > M) reunit_every = M > 0 ? (int32_t)M : 0;
-  *bytes = prop_layout(t, B, M, prec, reunit_every, true).total;
+  *bytes = prop_layout(t, B, M, prec, reunit_every, 1).total;
   return REDO_OK;
 }
 
@@ -729,7 +769,7 @@ redo_status redo_propagate_drift_workspace(const redo_table* t, int64_t B, int64
   redo_status st = check_drift(t, prec);
   if (st != REDO_OK) return st;
   if (reunit_every > M) reunit_every = M > 0 ? (int32_t)M : 0;
-  *bytes = prop_layout(t, B, M, prec, reunit_every, true).total;
+  *bytes = prop_layout(t, B, M, prec, reunit_every, 2).total;
   return REDO_OK;
 }
 
@@ -878,11 +918,69 @@ struct GradLayout {
   size_t keep_off = 0;                 // N <= 64: every forward state kept (0: not kept)
   bool keep = false;
   size_t strang_off, strang_tmp_off;   // symmetric split: transformed targets (+ scratch)
+  bool local = false;                  // locally controlled system (kernels_local.cu)
+  int eff_prec = 0;                    // its precision (FP32 for REDO_FP16X3)
+  size_t ops_off = 0;
 };
+
+// Locally controlled systems: segment products, checkpoints and costates as in the dense form, then
+// the step operators and the sweep's sums.  what: 1 gradient, 2 amplitude/phase gradient.
+static bool grad_layout_local(const redo_table* t, int64_t B, int64_t M, redo_precision prec, int32_t checkpoint_every,
+                              int what, GradLayout* L) {
+  L->eff_prec = prec == REDO_FP64 ? REDO_FP64 : REDO_FP32;
+  if (!local_eligible(t, M, L->eff_prec, what)) return false;
+  L->local = true;
+  L->p = checkpoint_every > 0 ? plan_chain_aligned(t, B, M, checkpoint_every)
+                              : plan_chain_local(t, B, M, L->eff_prec, true);
+  auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  L->seg_off = L->pck_off = L->rck_off = L->tau_off = 0;
+  if (t->N > kSmallN) {
+    L->total = large_grad_workspace(t, L->p, L->eff_prec);
+  } else {
+    const size_t el = L->eff_prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
+    const size_t mats = up((size_t)B * L->p.S * t->N * t->N * el);
+    L->pck_off = mats;
+    L->rck_off = 2 * mats;
+    L->tau_off = 3 * mats;
+    L->total = L->tau_off + up((size_t)B * sizeof(double2));
+  }
+  L->ops_off = L->total;
+  L->total += local_ops_bytes(t, B, M, L->eff_prec, what);
+  return true;
+}
+
+static redo_status grad_local(const redo_table* t, const int32_t* q, const GradLayout& L, int what, const double2* UT,
+                              int tb, const LocalDiag& pd, bool reunit, double* F_out, double* grad, double* gphi,
+                              char* w, int64_t* dev_status, cudaStream_t s) {
+  const ChainPlan& p = L.p;
+  void *P = w + L.pck_off, *Rc = w + L.rck_off;
+  double2* tau = (double2*)(w + L.tau_off);
+  cudaError_t e;
+  if ((e = launch_local_chain(t, q, p, L.eff_prec, what, pd, w + L.ops_off, w + L.seg_off, dev_status, s)) != cudaSuccess)
+    return cuda_error(e, "gradient segments");
+  if (t->N > kSmallN) {
+    if ((e = large_grad_scans(t, p, L.eff_prec, UT, tb, F_out, reunit, w, &P, &Rc, &tau, s)) != cudaSuccess)
+      return cuda_error(e, "gradient checkpoints");
+  } else {
+    if (reunit && p.M > 0 &&
+        (e = launch_polar(t, L.eff_prec, L.eff_prec, w + L.seg_off, w + L.seg_off, p.B * p.S, 1, s)) != cudaSuccess)
+      return cuda_error(e, "segment re-unitarisation");
+    if ((e = launch_grad_scan(t, p.B, p.S, L.eff_prec, w + L.seg_off, UT, tb, P, Rc, tau, F_out, s)) != cudaSuccess)
+      return cuda_error(e, "gradient checkpoints");
+  }
+  if (p.M > 0 && (e = launch_local_grad(t, q, p, L.eff_prec, what, pd, w + L.ops_off, P, Rc, tau, grad, gphi, nullptr,
+                                        s)) != cudaSuccess)
+    return cuda_error(e, "gradient sweep");
+  return REDO_OK;
+}
 
 static GradLayout grad_layout(const redo_table* t, int64_t B, int64_t M, redo_precision prec,
                               int32_t checkpoint_every) {
   GradLayout L;
+  if (grad_layout_local(t, B, M, prec, checkpoint_every, 1, &L)) {
+    add_strang(t, B, L.total, L.strang_off, L.strang_tmp_off);
+    return L;
+  }
   if (t->N > kSmallN) {
     L.p = checkpoint_every > 0 ? plan_chain_aligned(t, B, M, checkpoint_every)
                                : plan_chain_large(t, B, M);
@@ -965,6 +1063,9 @@ redo_status redo_fidelity_grad(const redo_table* t, const int32_t* q, int64_t B,
       return cuda_error(e, "half-drift conjugation of the target");
     U_target = sb;
   }
+  if (L.local)
+    return grad_local(t, q, L, 1, (const double2*)U_target, target_batched, LocalDiag{nullptr, 0, 0}, reunit_every > 0,
+                      F_out, grad, nullptr, w, dev_status, s);
   if (t->N > kSmallN) {
     const bool reunit = reunit_every > 0;
     e = prec == REDO_FP16X3
@@ -1002,7 +1103,9 @@ static PhaseGradLayout phase_grad_layout(const redo_table* t, int64_t B, int64_t
                                          int32_t checkpoint_every, bool phase = true) {
   PhaseGradLayout L;
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  if (t->N > kSmallN) {
+  if (grad_layout_local(t, B, M, prec, checkpoint_every, phase ? 2 : 1, &L.g)) {
+    L.pd_off = L.g.total;
+  } else if (t->N > kSmallN) {
     // lockstep SIMT sweeps on segments of whole steps (the diagonals fall between launches)
     const int64_t kd = (int64_t)t->K * t->digits;
     int64_t sps = checkpoint_every;
@@ -1026,11 +1129,12 @@ static PhaseGradLayout phase_grad_layout(const redo_table* t, int64_t B, int64_t
   }
   // the per-pulse drift form has no final rotation, transformed target or boundary traces
   const size_t ph = phase ? 1 : 0;
-  L.zf_off = L.pd_off + up((size_t)B * M * t->N * sizeof(double2));
+  // (a local system takes the drift form's diagonal once per pulse)
+  L.zf_off = L.pd_off + up((size_t)B * (L.g.local && !phase ? 1 : M) * t->N * sizeof(double2));
   L.ut_off = L.zf_off + ph * up((size_t)B * t->N * sizeof(double2));
   L.tz_off = L.ut_off + ph * up((size_t)B * t->N * t->N * sizeof(double2));
   L.total = L.tz_off + ph * up((size_t)B * (M + 1) * t->K * sizeof(double2));
-  if (t->N <= kSmallN) {
+  if (t->N <= kSmallN && !L.g.local) {
     // N <= 64: every forward state kept when they fit in 24 GiB (the sweep then multiplies only
     // the costates), as in the plain gradient
     const size_t el = prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
@@ -1095,6 +1199,9 @@ redo_status redo_fidelity_grad_phase(const redo_table* t, const int32_t* q, cons
   if ((e = launch_phase_target(t->N, B, (const double2*)U_target, target_batched, zf, ut, s)) != cudaSuccess)
     return cuda_error(e, "phase target");
   L.g.p.pd = pd;
+  if (L.g.local)
+    return grad_local(t, q, L.g, 2, ut, 1, LocalDiag{M > 0 ? pd : nullptr, M * t->N, t->N}, false, F_out, grad_amp,
+                      grad_phase, w, dev_status, s);
   if (t->N > kSmallN) {
     if ((e = large_grad(t, q, L.g.p, prec, ut, 1, F_out, grad_amp, workspace, dev_status, s, tz, grad_phase)) !=
         cudaSuccess)
@@ -1164,9 +1271,12 @@ redo_status redo_fidelity_grad_drift(const redo_table* t, const int32_t* q, cons
   const double2* ut = (const double2*)U_target;
   cudaError_t e;
   ProfScope ps(7, s);
-  if (M > 0 && (e = launch_drift_diag(t, h, B, M, pd, nullptr, s)) != cudaSuccess)
+  if (M > 0 && (e = launch_drift_diag(t, h, B, L.g.local ? 1 : M, pd, nullptr, s)) != cudaSuccess)
     return cuda_error(e, "drift diagonals");
   L.g.p.pd = pd;
+  if (L.g.local)
+    return grad_local(t, q, L.g, 1, ut, target_batched, LocalDiag{M > 0 ? pd : nullptr, t->N, 0}, reunit_every > 0,
+                      F_out, grad, nullptr, w, dev_status, s);
   if (t->N > kSmallN) {
     if ((e = large_grad(t, q, L.g.p, prec, ut, target_batched, F_out, grad, workspace, dev_status, s, nullptr,
                         nullptr, reunit_every > 0)) != cudaSuccess)

@@ -65,6 +65,16 @@ struct redo_table {
   double* sz64;               // [K][N] diagonals of the species' S_kz (amplitude/phase calls), or nullptr
   int32_t* h0_pairs;          // host: (row, column) of every off-diagonal nonzero of H0
   int64_t h0_npairs;
+  // locally controlled system (local_ops.cuh): number of qubits, or 0 when a control is not a sum of
+  // one-qubit operators or the drift is not diagonal
+  int loc;
+  int loc_pairs, loc_d, loc_base;
+  int32_t* loc_ptr;           // [loc + 1] (term, qubit) pairs of each qubit
+  int32_t* loc_k;             // [pairs] term, flagged at the first pair of a term
+  double2* loc_h;             // [pairs][4] one-qubit part of the term's operator
+  double2* loc_u64;           // [pairs][loc_d][loc_base][4] digit (or level) operators
+  float2* loc_u32;
+  double2* loc_D64;           // [N] diagonal of the drift step
   cudaStream_t build_stream;
   int num_sms;
 };
@@ -133,9 +143,12 @@ size_t chain_workspace_bytes(const redo_table* t, const ChainPlan& p, int prec);
 // keep[chain][t] (N x N, the chain precision).
 cudaError_t launch_chain_segments(const redo_table* t, const int32_t* q, const ChainPlan& p,
                                   int prec, void* seg_out, int64_t* status, cudaStream_t s, void* keep = nullptr);
+// Ordered product of every pulse's segments.  mid (combine_mid_bytes, or nullptr for one serial
+// pass) holds the products of groups of consecutive segments.
+size_t combine_mid_bytes(const redo_table* t, const ChainPlan& p, int prec);
 cudaError_t launch_chain_combine(const redo_table* t, const ChainPlan& p, int prec,
                                  const void* seg_in, void* prod_out, int64_t* status,
-                                 cudaStream_t s);
+                                 cudaStream_t s, void* mid = nullptr);
 // Segments of exactly `steps_per_segment` time steps (re-unitarisation period).
 ChainPlan plan_chain_aligned(const redo_table* t, int64_t B, int64_t M, int64_t steps_per_segment,
                              bool phase = false);
@@ -147,6 +160,27 @@ cudaError_t launch_polar(const redo_table* t, int prec_in, int prec_out, const v
 // The same Newton-Schulz steps on complex128 matrices (N <= 64), in FP64 or FP32 arithmetic.
 cudaError_t launch_polar_c128(int N, int prec_arith, const double2* in, double2* out, int64_t count, int iters,
                               cudaStream_t s);
+
+// Locally controlled systems (kernels_local.cu).  Step-opening diagonals of a call: p[b*sb + n*sn + r]
+// (nullptr: none; sn = 0: the same for every step of a pulse).
+struct LocalDiag {
+  const double2* p;
+  int64_t sb, sn;
+};
+}  // namespace redo
+#include <vector>
+namespace redo {
+cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_t s);
+void local_free(redo_table* t);
+// what: 0 chains only, 1 gradient, 2 amplitude/phase gradient (its Tz sums beside)
+bool local_eligible(const redo_table* t, int64_t M, int prec, int what);
+size_t local_ops_bytes(const redo_table* t, int64_t B, int64_t M, int prec, int what);
+ChainPlan plan_chain_local(const redo_table* t, int64_t B, int64_t M, int prec, bool two);
+cudaError_t launch_local_chain(const redo_table* t, const int32_t* q, const ChainPlan& p, int prec, int what,
+                               const LocalDiag& pd, void* ops, void* seg_out, int64_t* status, cudaStream_t s);
+cudaError_t launch_local_grad(const redo_table* t, const int32_t* q, const ChainPlan& p, int prec, int what,
+                              const LocalDiag& pd, void* ops, const void* Pck, const void* Rck, const double2* tau,
+                              double* grad, double* gphi, int64_t* status, cudaStream_t s);
 
 // Tensor-core chains (kernels_tc.cu), N = 64, split-FP16.
 size_t tc_planes_bytes(const redo_table* t);
@@ -218,9 +252,6 @@ cudaError_t mlp_adam(int64_t count, float* p, const float* g, float* m, float* v
                      float b1, float b2, float eps, cudaStream_t s);
 
 // Large-N path (kernels_large.cu), 64 < N <= 1024.
-}  // namespace redo
-#include <vector>
-namespace redo {
 cudaError_t large_table_build(redo_table* t, const double2* H0, const double2* Hk,
                               const std::vector<double>& hnorm1, double h0norm1, cudaStream_t s);
 ChainPlan plan_chain_large(const redo_table* t, int64_t B, int64_t M);
@@ -245,6 +276,9 @@ size_t large_sim_workspace(const redo_table* t, int64_t B);
 cudaError_t large_sim(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int prec,
                       const double2* psi0, int pb, const double* obs, double* expect, void* ws,
                       cudaStream_t s);
+// large_propagate without its chains: the segment products are at the start of the workspace
+cudaError_t large_finish(const redo_table* t, const ChainPlan& p, int prec, bool reunit, void* ws, void** result,
+                         int* result_prec, cudaStream_t s);
 cudaError_t large_finish_fp32(const redo_table* t, const ChainPlan& p, bool reunit, void* ws,
                               void** result, int* result_prec, cudaStream_t s);
 cudaError_t large_pair_products_fp32(const float2* in, float2* out, int64_t count, int N, cudaStream_t s);
@@ -254,6 +288,11 @@ cudaError_t large_costate_shift_fp32(const float2* Pck, const float2* Rck, float
 // out[2s+1] = H[2s] Cs[s], out[2s] = Cs[s] H[2s+1], for 2s+1 < Gf (FP32).
 cudaError_t large_half_costates_fp32(const float2* H, const float2* Cs, float2* out, int64_t Gf, int N,
                                      cudaStream_t s);
+// Checkpoints, costates and tau from the segment products at the start of a large_grad_workspace;
+// reunit: their Newton-Schulz step first.
+cudaError_t large_grad_scans(const redo_table* t, const ChainPlan& p, int prec, const double2* UT, int tb,
+                             double* F_out, bool reunit, void* ws, void** Pck, void** Rck, double2** tau,
+                             cudaStream_t s);
 cudaError_t large_grad_scans_fp32(const redo_table* t, const ChainPlan& p, const double2* UT, int tb,
                                   double* F_out, void* ws, float2** Pck, float2** Rck, double2** tau,
                                   cudaStream_t s);

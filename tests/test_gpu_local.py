@@ -1,0 +1,133 @@
+"""Locally controlled systems (every control a sum of one-qubit operators, diagonal drift) take
+their own chain and gradient kernels; here against the oracle, over the forms that route accepts:
+every dimension, several controls and axes per qubit, identity and z parts, a control that is zero,
+digit tables too large for one operator per level, step diagonals, ragged segments, re-unitarised
+segments, and controls just outside the class, which keep the dense path.
+
+Tolerances: FP64 products of a few hundred 2 x 2 operators, 1e-12; FP32 chains of M (n + 1)
+roundings of 6e-8 each, below 2e-5 at M = 29, n <= 7, and 2e-4 of the largest entry for gradients,
+as the dense FP32 paths are held to.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import redo_oracle as O  # noqa: E402
+from paper_1707_02162_gb300 import inputs  # noqa: E402
+from tests import _ref  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+SIG = [np.eye(2), np.array([[0, 1], [1, 0]]), np.array([[0, -1j], [1j, 0]]), np.diag([1.0, -1.0])]
+
+
+def _workload(n, controls, B, M, seed, base=4, digits=3, dt=1e-2):
+    """Coefficients in [-1, 1.5]; dt large enough that a step's rotations are of order 0.1 to 1."""
+    rng = np.random.default_rng(seed)
+    N = 2 ** n
+    if controls == "axes":            # three controls, each a random one-qubit operator on every qubit
+        Hk = np.stack([sum(inputs.embed({i: sum(c * s for c, s in zip(rng.normal(size=4), SIG))}, n)
+                           for i in range(n)) for _ in range(3)])
+    elif controls == "z_and_zero":    # a z control, an x control on the last qubit, and a zero operator
+        Hk = np.stack([inputs.embed({0: SIG[3] + 0j}, n), inputs.embed({n - 1: SIG[1] + 0j}, n),
+                       np.zeros((N, N), dtype=complex)])
+    elif controls == "pi":            # half and full turns: vanishing diagonal or off-diagonal entries
+        Hk = np.stack([inputs.embed({0: SIG[1] + 0j}, n), inputs.embed({n - 1: SIG[2] + 0j}, n)])
+    else:
+        Hk = {"local": inputs.controls_local_xy, "global": inputs.controls_global_xy}[controls](n)
+    Hk = np.asarray(Hk, dtype=np.complex128) * (20 if controls != "pi" else 1)
+    K = Hk.shape[0]
+    H0 = np.diag(rng.normal(size=N) * 15).astype(np.complex128)
+    lo, hi = np.full(K, -1.0), np.full(K, 1.5)
+    u = rng.uniform(-1.1, 1.6, size=(B, M, K))
+    if controls == "pi":
+        dt, lo, hi = 1.0, np.full(K, -np.pi / 2), np.full(K, np.pi)
+        u = rng.integers(-1, 3, size=(B, M, K)) * (np.pi / 2)
+        H0 = H0 / 20
+    return inputs.Workload("local", n, H0, Hk, dt, lo, hi, base ** digits, base, digits, u,
+                           target=inputs.haar_unitary(rng, N))
+
+
+def _table(w, **kw):
+    from paper_1707_02162_gb300 import redo
+    return redo.Table(w.H0, w.Hk, w.dt, w.lo, w.hi, w.base, w.digits, fp32=True, **kw)
+
+
+def _check(w, prec, tol, gtol, ck=0, reunit=0, **kw):
+    t = _table(w, **kw)
+    q = t.quantize(w.u)
+    U, F, _ = t.propagate(q, prec, target=w.target, reunit_every=reunit)
+    Fg, g = t.fidelity_grad(q, w.target, prec, checkpoint_every=ck, reunit_every=reunit)
+    T, D = O.build_table(w.H0, w.Hk, w.dt, w.lo, w.hi, w.levels, w.base, w.digits, method="eig")
+    _, dig, _, _ = _ref.oracle_levels(w)
+    for b in range(w.B):
+        Uo = O.propagate(T, D, dig[b])
+        assert np.abs(U[b].cpu().numpy() - Uo).max() < tol
+        assert abs(float(F[b]) - O.fidelity(w.target, Uo)) < tol
+        Fo, go = O.grape_gradient(T, D, w.Hk, w.dt, dig[b], w.target)
+        assert abs(float(Fg[b]) - Fo) < tol
+        assert np.abs(g[b].cpu().numpy() - go).max() <= gtol * max(np.abs(go).max(), 1e-30)
+    t.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 6, 7])
+@pytest.mark.parametrize("controls", ["local", "global", "axes", "z_and_zero"])
+@pytest.mark.parametrize("prec,tol,gtol", [("fp64", 1e-12, 1e-10), ("fp32", 2e-5, 2e-4)])
+def test_local_chain_and_gradient(n, controls, prec, tol, gtol):
+    _check(_workload(n, controls, B=3, M=29, seed=n), prec, tol, gtol)
+
+
+@pytest.mark.parametrize("n,M,ck", [(2, 7, 3), (3, 41, 20), (5, 33, 16), (7, 11, 4)])
+@pytest.mark.parametrize("prec,tol,gtol", [("fp64", 1e-12, 1e-10), ("fp32", 2e-5, 2e-4)])
+def test_local_ragged_reunitarised_segments(n, M, ck, prec, tol, gtol):
+    _check(_workload(n, "axes", B=2, M=M, seed=10 + n), prec, tol, gtol, ck=ck, reunit=ck)
+
+
+@pytest.mark.parametrize("prec,tol,gtol", [("fp64", 1e-12, 1e-10), ("fp32", 2e-5, 2e-4)])
+def test_local_half_turns(prec, tol, gtol):
+    # entries of the one-qubit operators that vanish exactly or to rounding
+    _check(_workload(3, "pi", B=4, M=17, seed=3, base=4, digits=1), prec, tol, gtol)
+
+
+def test_local_digit_operators():
+    # 16^5 levels: the one-qubit tables keep digits
+    _check(_workload(3, "axes", B=2, M=9, seed=5, base=16, digits=5), "fp64", 1e-12, 1e-10)
+
+
+def test_nearly_local_control_keeps_dense_products():
+    w = _workload(3, "local", B=2, M=9, seed=6)
+    w.Hk[1] = w.Hk[1] + 20 * inputs.embed({0: SIG[1] + 0j, 2: SIG[1] + 0j}, 3)    # a two-qubit term
+    _check(w, "fp64", 1e-12, 1e-10)
+
+
+def test_local_batches_are_sliced_without_a_seam():
+    # the step operators of 600 pulses x 2000 steps do not fit one slice of scratch
+    w = inputs.config(1, B=2, M=2000)
+    t = _table(w)
+    q2 = t.quantize(w.u)
+    q = q2[:1].expand(600, -1, -1).contiguous()
+    q[-1] = q2[1]
+    U, _, _ = t.propagate(q, "fp32", reunit_every=100)
+    one, _, _ = t.propagate(q2, "fp32", reunit_every=100)
+    assert torch.equal(U[0], one[0]) and torch.equal(U[598], one[0]) and torch.equal(U[599], one[1])
+    target = torch.as_tensor(w.target, device="cuda")
+    F, g = t.fidelity_grad(q, target, "fp32", checkpoint_every=100, reunit_every=100)
+    F1, g1 = t.fidelity_grad(q2, target, "fp32", checkpoint_every=100, reunit_every=100)
+    assert torch.equal(g[0], g1[0]) and torch.equal(g[598], g1[0]) and torch.equal(g[599], g1[1])
+    t.close()
+
+
+def test_local_bad_level_index_counts_once_per_digit():
+    from paper_1707_02162_gb300 import redo
+    w = _workload(3, "axes", B=1, M=5, seed=8)
+    t = _table(w)
+    q = t.quantize(w.u).clone()
+    q[0, 2, 1], q[0, 3, 0] = w.levels, -1
+    st = redo.new_status()
+    U, _, _ = t.propagate(q, "fp64", status=st)
+    q0 = q.clone()
+    q0[0, 2, 1] = q0[0, 3, 0] = 0
+    U0, _, _ = t.propagate(q0, "fp64")
+    assert int(st[3]) == 2 * w.digits and torch.equal(U, U0)
+    t.close()

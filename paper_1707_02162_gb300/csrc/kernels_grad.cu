@@ -28,39 +28,41 @@ namespace redo {
 // ----------------------------------------------------------------------------
 // Scan: Pck[b][s] = S_s ... S_0,  Rck[b][s] = U_T^dag S_{S-1} ... S_{s+1},
 // tau_b = Tr(U_T^dag U_b), F_b = |tau_b|^2 / N^2 (FP64 reduction)
+//
+// The products are dependent, so a pulse's scan is bound by its depth: the prefix and the suffix
+// direction have a block each, and with few pulses the segments are cut into groups of about
+// sqrt(S) that scan on their own (pass 0), then the groups' totals are scanned (pass 1) and carried
+// into every segment (pass 2).  With enough pulses to fill the GPU one group is the whole pulse.
 // ----------------------------------------------------------------------------
-template <typename R, int N>
-__global__ void __launch_bounds__(SmemMM<R, N, SqTile<N>::TM, SqTile<N>::TM>::THREADS)
-grad_scan_kernel(int64_t S, const cplx<R>* __restrict__ seg, const double2* __restrict__ UT,
-                 int target_batched, cplx<R>* __restrict__ Pck, cplx<R>* __restrict__ Rck,
-                 double2* __restrict__ tau, double* __restrict__ F_out) {
-  constexpr int TM = SqTile<N>::TM;
-  using MM = SmemMM<R, N, TM, TM>;
-  constexpr int N2 = N * N;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  cplx<R>* X = reinterpret_cast<cplx<R>*>(smem_raw);
-  cplx<R>* A = X + N2;
-  __shared__ double red_re[MM::THREADS], red_im[MM::THREADS];
-  const int lt = threadIdx.x;
-  const int64_t b = blockIdx.x;
-  const double2* Ut = UT + (target_batched ? b * N2 : 0);
-  cplx<R> Y[TM][TM];
-  for (int i = lt; i < N2; i += MM::THREADS) X[i] = cmake<R>((i / N == i % N) ? R(1) : R(0), R(0));
-  __syncthreads();
-  for (int64_t s = 0; s < S; ++s) {
-    const cplx<R>* Ss = seg + (b * S + s) * N2;
-    for (int i = lt; i < N2; i += MM::THREADS) A[i] = Ss[i];
-    __syncthreads();
-    MM::run(A, X, lt, Y);
-    __syncthreads();
-    MM::store(X, lt, Y);
-    __syncthreads();
-    cplx<R>* o = Pck + (b * S + s) * N2;
-    for (int i = lt; i < N2; i += MM::THREADS) o[i] = X[i];
+template <typename R, int N> struct ScanMM {
+  using MM = SmemMM<R, N, SqTile<N>::TM, SqTile<N>::TM>;
+  static constexpr int TM = SqTile<N>::TM, TH = MM::THREADS, N2 = N * N, PER = (N2 + TH - 1) / TH;
+  static __device__ __forceinline__ void fetch(cplx<R> (&r)[PER], const cplx<R>* src, int lt) {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) r[i] = src[lt + i * TH];
   }
-  // tau = sum conj(U_T) .* U in FP64
+  static __device__ __forceinline__ void put(cplx<R>* dst, const cplx<R> (&r)[PER], int lt) {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) dst[lt + i * TH] = r[i];
+  }
+  static __device__ __forceinline__ void adjoint(cplx<R>* X, const double2* U, int lt) {
+    for (int i = lt; i < N2; i += TH) {
+      const double2 g = U[(i % N) * N + i / N];
+      X[i] = cmake<R>((R)g.x, (R)(-g.y));
+    }
+  }
+  static __device__ __forceinline__ void identity(cplx<R>* X, int lt) {
+    for (int i = lt; i < N2; i += TH) X[i] = cmake<R>((i / N == i % N) ? R(1) : R(0), R(0));
+  }
+};
+
+template <typename R, int N>
+__device__ __forceinline__ void scan_tau(const cplx<R>* X, const double2* Ut, int lt, int64_t b, double2* tau,
+                                         double* F_out) {
+  constexpr int TH = ScanMM<R, N>::TH;
+  __shared__ double red_re[TH], red_im[TH];
   double re = 0.0, im = 0.0;
-  for (int i = lt; i < N2; i += MM::THREADS) {
+  for (int i = lt; i < N * N; i += TH) {
     const double2 g = Ut[i];
     const double ur = (double)X[i].x, ui = (double)X[i].y;
     re = fma(g.x, ur, re);
@@ -71,7 +73,7 @@ grad_scan_kernel(int64_t S, const cplx<R>* __restrict__ seg, const double2* __re
   red_re[lt] = re;
   red_im[lt] = im;
   __syncthreads();
-  for (int w = MM::THREADS / 2; w > 0; w >>= 1) {
+  for (int w = TH / 2; w > 0; w >>= 1) {
     if (lt < w) {
       red_re[lt] += red_re[lt + w];
       red_im[lt] += red_im[lt + w];
@@ -82,25 +84,106 @@ grad_scan_kernel(int64_t S, const cplx<R>* __restrict__ seg, const double2* __re
     tau[b] = make_double2(red_re[0], red_im[0]);
     if (F_out) F_out[b] = (red_re[0] * red_re[0] + red_im[0] * red_im[0]) / ((double)N * (double)N);
   }
-  // costates: Y = U_T^dag, then Y <- Y S_s going backwards
-  for (int i = lt; i < N2; i += MM::THREADS) {
-    const int r = i / N, c = i % N;
-    const double2 g = Ut[c * N + r];
-    X[i] = cmake<R>((R)g.x, (R)(-g.y));
+}
+
+// Blocks: (direction, pulse, group).  in [B][L] holds the factors; group i covers [i g, (i + 1) g).
+// Direction 0 writes P[s] = in_s ... in_first, direction 1 R[s] = Z in_last ... in_{s+1}, Z = U_T^dag when
+// there is one group, else the identity.  last (not null): the whole group's product, [B][groups].
+template <typename R, int N>
+__global__ void __launch_bounds__(ScanMM<R, N>::TH)
+grad_scan_kernel(int64_t L, int64_t g, int64_t groups, const cplx<R>* __restrict__ in, const double2* __restrict__ UT,
+                 int target_batched, cplx<R>* __restrict__ P, cplx<R>* __restrict__ Rm, cplx<R>* __restrict__ last,
+                 int reunit, double2* __restrict__ tau, double* __restrict__ F_out) {
+  using SM = ScanMM<R, N>;
+  constexpr int N2 = SM::N2;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  cplx<R>* X = reinterpret_cast<cplx<R>*>(smem_raw);
+  cplx<R>* A = X + N2;
+  const int lt = threadIdx.x;
+  const bool suffix = blockIdx.x & 1;
+  const int64_t b = (blockIdx.x >> 1) / groups, gi = (blockIdx.x >> 1) - b * groups;
+  const int64_t s0 = gi * g, s1 = s0 + g < L ? s0 + g : L;
+  const double2* Ut = UT + (target_batched ? b * N2 : 0);
+  cplx<R> Y[SM::TM][SM::TM], nx[SM::PER];
+  if (suffix && groups == 1)
+    SM::adjoint(X, Ut, lt);
+  else
+    SM::identity(X, lt);
+  const cplx<R>* src = in + b * L * N2;
+  if (s1 > s0) SM::fetch(nx, src + (suffix ? s1 - 1 : s0) * N2, lt);
+  __syncthreads();
+  // a first factor beside the identity is copied
+  for (int64_t i = 0; i < s1 - s0; ++i) {
+    const int64_t s = suffix ? s1 - 1 - i : s0 + i;
+    if (suffix) {
+      cplx<R>* o = Rm + (b * L + s) * N2;
+      for (int e = lt; e < N2; e += SM::TH) o[e] = X[e];
+      if (s == s0) break;
+    }
+    const bool copy = i == 0 && !(suffix && groups == 1);
+    SM::put(copy ? X : A, nx, lt);
+    if (i + 1 < s1 - s0) SM::fetch(nx, src + (suffix ? s - 1 : s + 1) * N2, lt);
+    __syncthreads();
+    if (!copy) {
+      SM::MM::run_blocked(suffix ? X : A, suffix ? A : X, lt, Y);
+      __syncthreads();
+      SM::MM::store(X, lt, Y);
+      __syncthreads();
+    }
+    if (!suffix) {
+      cplx<R>* o = P + (b * L + s) * N2;
+      for (int e = lt; e < N2; e += SM::TH) o[e] = X[e];
+      if (last && s == s1 - 1) {
+        o = last + (b * groups + gi) * N2;
+        for (int e = lt; e < N2; e += SM::TH) o[e] = X[e];
+      }
+    }
+  }
+  if (!suffix && tau && groups == 1) {
+    __syncthreads();
+    if (reunit) {
+      // re-unitarised chains: the pulse product gets a Newton-Schulz step too before tau and F, as in
+      // redo_propagate (near F = 1 the norm left by the scan's products is most of F's error)
+      SM::MM::ns_correction(X, A, lt);
+      __syncthreads();
+      SM::MM::run(X, A, lt, Y);
+      __syncthreads();
+      SM::MM::add(X, lt, Y);
+      __syncthreads();
+    }
+    scan_tau<R, N>(X, Ut, lt, b, tau, F_out);
+  }
+}
+
+// Carries the groups' prefix GP and costate GR into their segments: blocks (direction, pulse, segment),
+// P[s] <- P[s] GP[group - 1],  R[s] <- GR[group] R[s] (R[s] is the identity for a group's last segment).
+template <typename R, int N>
+__global__ void __launch_bounds__(ScanMM<R, N>::TH)
+grad_carry_kernel(int64_t L, int64_t g, int64_t groups, const cplx<R>* __restrict__ GP, const cplx<R>* __restrict__ GR,
+                  cplx<R>* __restrict__ P, cplx<R>* __restrict__ Rm) {
+  using SM = ScanMM<R, N>;
+  constexpr int N2 = SM::N2;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  cplx<R>* X = reinterpret_cast<cplx<R>*>(smem_raw);
+  cplx<R>* A = X + N2;
+  const int lt = threadIdx.x;
+  const bool suffix = blockIdx.x & 1;
+  const int64_t bs = blockIdx.x >> 1, b = bs / L, s = bs - b * L, gi = s / g;
+  if (!suffix && gi == 0) return;
+  cplx<R>* o = (suffix ? Rm : P) + bs * N2;
+  const cplx<R>* c = suffix ? GR + (b * groups + gi) * N2 : GP + (b * groups + gi - 1) * N2;
+  if (suffix && (s == L - 1 || s % g == g - 1)) {
+    for (int e = lt; e < N2; e += SM::TH) o[e] = c[e];
+    return;
+  }
+  for (int e = lt; e < N2; e += SM::TH) {
+    A[e] = suffix ? c[e] : o[e];
+    X[e] = suffix ? o[e] : c[e];
   }
   __syncthreads();
-  for (int64_t s = S - 1; s >= 0; --s) {
-    cplx<R>* o = Rck + (b * S + s) * N2;
-    for (int i = lt; i < N2; i += MM::THREADS) o[i] = X[i];
-    if (s == 0) break;
-    const cplx<R>* Ss = seg + (b * S + s) * N2;
-    for (int i = lt; i < N2; i += MM::THREADS) A[i] = Ss[i];
-    __syncthreads();
-    MM::run(X, A, lt, Y);
-    __syncthreads();
-    MM::store(X, lt, Y);
-    __syncthreads();
-  }
+  cplx<R> Y[SM::TM][SM::TM];
+  SM::MM::run_blocked(A, X, lt, Y);
+  SM::MM::store(o, lt, Y);
 }
 
 // ----------------------------------------------------------------------------
@@ -360,17 +443,46 @@ grad_sweep_kernel(GradArgs<R> a) {
     atomicAdd((unsigned long long*)&a.status[REDO_STATUS_TIMEOUT], 1ull);
 }
 
+// Segments per group: the whole pulse when the pulses' two blocks each fill half the SMs or the scan
+// is short, else about sqrt(S) (depth g + S / g + 1 instead of S).
+static int64_t scan_group(const redo_table* t, int64_t B, int64_t S) {
+  if (S < 8 || 4 * B >= t->num_sms) return S > 0 ? S : 1;
+  int64_t g = 2;
+  while (g * g < S) ++g;
+  return g;
+}
+
+size_t grad_scan_bytes(const redo_table* t, int64_t B, int64_t S, int prec) {
+  const int64_t g = scan_group(t, B, S), groups = S > 0 ? (S + g - 1) / g : 1;
+  const size_t el = prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
+  return groups > 1 ? 3 * (((size_t)B * groups * t->N * t->N * el + 255) & ~(size_t)255) : 0;
+}
+
 template <typename R, int N>
-static cudaError_t grad_scan_n(int64_t B, int64_t S, const void* seg, const double2* UT,
-                               int target_batched, void* Pck, void* Rck, double2* tau,
-                               double* F_out, cudaStream_t s) {
-  using MM = SmemMM<R, N, SqTile<N>::TM, SqTile<N>::TM>;
+static cudaError_t grad_scan_n(const redo_table* t, int64_t B, int64_t S, const void* seg, const double2* UT,
+                               int target_batched, int reunit, void* Pck, void* Rck, double2* tau,
+                               double* F_out, void* tmp, cudaStream_t s) {
+  using SM = ScanMM<R, N>;
   const size_t smem = 2 * sizeof(cplx<R>) * N * N;
-  auto kern = grad_scan_kernel<R, N>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto scan = grad_scan_kernel<R, N>;
+  auto carry = grad_carry_kernel<R, N>;
+  cudaError_t e = cudaFuncSetAttribute(scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(carry, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)B, MM::THREADS, smem, s>>>(S, (const cplx<R>*)seg, UT, target_batched,
-                                               (cplx<R>*)Pck, (cplx<R>*)Rck, tau, F_out);
+  const int64_t g = scan_group(t, B, S), groups = (S + g - 1) / g;
+  cplx<R>*P = (cplx<R>*)Pck, *Q = (cplx<R>*)Rck;
+  if (groups <= 1) {
+    scan<<<(unsigned)(2 * B), SM::TH, smem, s>>>(S, g, 1, (const cplx<R>*)seg, UT, target_batched, P, Q, nullptr, reunit,
+                                                 tau, F_out);
+    return cudaGetLastError();
+  }
+  const size_t mats = ((size_t)B * groups * N * N * sizeof(cplx<R>) + 255) & ~(size_t)255;
+  cplx<R>*tot = (cplx<R>*)tmp, *GP = (cplx<R>*)((char*)tmp + mats), *GR = (cplx<R>*)((char*)tmp + 2 * mats);
+  scan<<<(unsigned)(2 * B * groups), SM::TH, smem, s>>>(S, g, groups, (const cplx<R>*)seg, UT, target_batched, P, Q, tot,
+                                                        0, nullptr, nullptr);
+  scan<<<(unsigned)(2 * B), SM::TH, smem, s>>>(groups, groups, 1, tot, UT, target_batched, GP, GR, nullptr, reunit,
+                                               tau, F_out);
+  carry<<<(unsigned)(2 * B * S), SM::TH, smem, s>>>(S, g, groups, GP, GR, P, Q);
   return cudaGetLastError();
 }
 
@@ -395,26 +507,26 @@ static cudaError_t grad_sweep_n(const GradArgs<R>& a, int64_t B, cudaStream_t s)
 
 template <typename R>
 static cudaError_t grad_scan_t(const redo_table* t, int64_t B, int64_t S, const void* seg,
-                               const double2* UT, int tb, void* Pck, void* Rck, double2* tau,
-                               double* F, cudaStream_t s) {
+                               const double2* UT, int tb, int reunit, void* Pck, void* Rck, double2* tau,
+                               double* F, void* tmp, cudaStream_t s) {
   switch (t->N) {
-    case 2: return grad_scan_n<R, 2>(B, S, seg, UT, tb, Pck, Rck, tau, F, s);
-    case 4: return grad_scan_n<R, 4>(B, S, seg, UT, tb, Pck, Rck, tau, F, s);
-    case 8: return grad_scan_n<R, 8>(B, S, seg, UT, tb, Pck, Rck, tau, F, s);
-    case 16: return grad_scan_n<R, 16>(B, S, seg, UT, tb, Pck, Rck, tau, F, s);
-    case 32: return grad_scan_n<R, 32>(B, S, seg, UT, tb, Pck, Rck, tau, F, s);
-    case 64: return grad_scan_n<R, 64>(B, S, seg, UT, tb, Pck, Rck, tau, F, s);
+    case 2: return grad_scan_n<R, 2>(t, B, S, seg, UT, tb, reunit, Pck, Rck, tau, F, tmp, s);
+    case 4: return grad_scan_n<R, 4>(t, B, S, seg, UT, tb, reunit, Pck, Rck, tau, F, tmp, s);
+    case 8: return grad_scan_n<R, 8>(t, B, S, seg, UT, tb, reunit, Pck, Rck, tau, F, tmp, s);
+    case 16: return grad_scan_n<R, 16>(t, B, S, seg, UT, tb, reunit, Pck, Rck, tau, F, tmp, s);
+    case 32: return grad_scan_n<R, 32>(t, B, S, seg, UT, tb, reunit, Pck, Rck, tau, F, tmp, s);
+    case 64: return grad_scan_n<R, 64>(t, B, S, seg, UT, tb, reunit, Pck, Rck, tau, F, tmp, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_grad_scan(const redo_table* t, int64_t B, int64_t S, int prec, const void* seg,
-                             const double2* U_target, int target_batched, void* Pck, void* Rck,
-                             double2* tau, double* F_out, cudaStream_t s) {
+                             const double2* U_target, int target_batched, int reunit, void* Pck, void* Rck,
+                             double2* tau, double* F_out, void* tmp, cudaStream_t s) {
   if (B == 0) return cudaSuccess;
   if (prec == REDO_FP64)
-    return grad_scan_t<double>(t, B, S, seg, U_target, target_batched, Pck, Rck, tau, F_out, s);
-  return grad_scan_t<float>(t, B, S, seg, U_target, target_batched, Pck, Rck, tau, F_out, s);
+    return grad_scan_t<double>(t, B, S, seg, U_target, target_batched, reunit, Pck, Rck, tau, F_out, tmp, s);
+  return grad_scan_t<float>(t, B, S, seg, U_target, target_batched, reunit, Pck, Rck, tau, F_out, tmp, s);
 }
 
 template <typename R>

@@ -254,7 +254,17 @@ __global__ void copy_kernel(const cplx<R>* __restrict__ src, cplx<R>* __restrict
     dst[i] = src[i];
 }
 
-// Q = 1.5 I - 0.5 G (Newton-Schulz)
+// dst += src
+template <typename R>
+__global__ void add_kernel(const cplx<R>* __restrict__ src, cplx<R>* __restrict__ dst, int64_t n) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const cplx<R> a = src[i], b = dst[i];
+    dst[i] = cmake<R>(a.x + b.x, a.y + b.y);
+  }
+}
+
+// Q = (I - G) / 2 (Newton-Schulz correction)
 template <typename R>
 __global__ void ns_mid_kernel(cplx<R>* G, int64_t count, int N) {
   const int64_t n2 = (int64_t)N * N;
@@ -262,7 +272,7 @@ __global__ void ns_mid_kernel(cplx<R>* G, int64_t count, int N) {
        i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t e = i % n2;
     const cplx<R> g = G[i];
-    G[i] = cmake<R>(((e / N == e % N) ? R(1.5) : R(0)) - R(0.5) * g.x, -R(0.5) * g.y);
+    G[i] = cmake<R>(R(0.5) * (((e / N == e % N) ? R(1) : R(0)) - g.x), -R(0.5) * g.y);
   }
 }
 
@@ -612,7 +622,7 @@ static cudaError_t large_combine_t(int N, const ChainPlan& p, const cplx<R>* seg
   return cudaGetLastError();
 }
 
-// one Newton-Schulz step on `count` matrices in place; tmp holds 2*count matrices
+// one Newton-Schulz step P + P (I - P^dag P) / 2 on `count` matrices in place; tmp holds 2*count matrices
 template <typename R>
 static cudaError_t large_polar_t(int N, cplx<R>* P, int64_t count, cplx<R>* tmp, cudaStream_t s) {
   const int64_t n2 = (int64_t)N * N;
@@ -624,7 +634,7 @@ static cudaError_t large_polar_t(int N, cplx<R>* P, int64_t count, cplx<R>* tmp,
   ns_mid_kernel<R><<<blocks_for(count * n2), 256, 0, s>>>(G, count, N);
   DenseOps<R> m{P, G, Pn, n2, n2, n2};
   if ((e = cgemm<R, false>(m, count, N, R(1), R(0), s))) return e;
-  copy_kernel<R><<<blocks_for(count * n2), 256, 0, s>>>(Pn, P, count * n2);
+  add_kernel<R><<<blocks_for(count * n2), 256, 0, s>>>(Pn, P, count * n2);
   return cudaGetLastError();
 }
 

@@ -122,7 +122,8 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
   std::vector<double2> D(N);
   for (int r = 0; r < N; ++r) {
     const double a = t->dt * h[2 * ((size_t)r * N + r)];
-    D[r] = make_double2(std::cos(a), -std::sin(a));
+    const double sh = std::sin(0.5 * a);
+    D[r] = make_double2(-2.0 * sh * sh, -std::sin(a));                // exp(-i a) - 1
   }
   cudaError_t e;
   if ((e = cudaMalloc(&t->loc_ptr, sizeof(int32_t) * (n + 1))) || (e = cudaMalloc(&t->loc_k, sizeof(int32_t) * pairs)) ||
@@ -166,7 +167,9 @@ template <typename R> static LocTab<R> loc_tab(const redo_table* t, int64_t* sta
 }
 
 // ============================================================================
-// Step operators of every (pulse, step): rotations cs[b][n][i] and diagonals Delta[b][0..M][N]
+// Step operators of the steps m0 .. m0 + T of every pulse: rotations cs[b][n - m0][i] and diagonals
+// Delta[b][n - m0][N], n - m0 <= T (Delta_M closes the chain; a window that ends earlier also gets
+// the next step's)
 // ============================================================================
 constexpr int kPrepSteps = 8, kPrepThreads = 256;
 
@@ -175,61 +178,82 @@ template <typename R> __device__ __forceinline__ phase_t<R> no_phase() {
   else return cmake<R>(R(1), R(0));
 }
 
+// (1 + v)(1 + d) - 1, d in FP64 (FP32: hi + lo)
 template <typename R> __device__ __forceinline__ cplx<R> loc_times(cplx<R> v, double2 d) {
   const cplx<R> hi = cmake<R>((R)d.x, (R)d.y);
-  if constexpr (sizeof(R) == 8) return cmul<R>(v, hi);
-  cplx<R> o = cmul<R>(v, cmake<R>((R)(d.x - (double)hi.x), (R)(d.y - (double)hi.y)));
+  cplx<R> o = cmake<R>(v.x + hi.x, v.y + hi.y);
+  if constexpr (sizeof(R) == 4) {
+    o.x += (R)(d.x - (double)hi.x);
+    o.y += (R)(d.y - (double)hi.y);
+  }
   cfma<R>(o, v, hi);
   return o;
 }
 
-template <typename R>
+template <typename R, bool NEAR>
 __global__ void __launch_bounds__(kPrepThreads)
-loc_steps_kernel(LocTab<R> tab, const int32_t* __restrict__ q, int64_t M, int n, int N, int E, int64_t tiles,
+loc_steps_kernel(LocTab<R> tab, const int32_t* __restrict__ q, int64_t M, int64_t m0, int64_t T, int n, int N, int E,
+                 int64_t tiles,
                  const double2* __restrict__ D, const double2* __restrict__ pd, int64_t pd_b, int64_t pd_n,
                  cplx<R>* __restrict__ cs, cplx<R>* __restrict__ delta) {
   // phases of every (step, qubit); row j is step n0 - 1 + j (the step before the tile gives its x)
-  __shared__ phase_t<R> y0[kPrepSteps + 1][10], y1[kPrepSteps + 1][10], xx[kPrepSteps + 1][10];
+  __shared__ phase_t<R> y0[kPrepSteps + 1][10], y1[kPrepSteps + 1][10], xx[kPrepSteps + 1][10],
+      x0[kPrepSteps + 1][10];
   const int64_t b = blockIdx.x / tiles;
-  const int64_t n0 = (blockIdx.x - b * tiles) * kPrepSteps;
+  const int64_t n0 = m0 + (blockIdx.x - b * tiles) * kPrepSteps;
   for (int idx = threadIdx.x; idx < (kPrepSteps + 1) * n; idx += kPrepThreads) {
     const int j = idx / n, i = idx - j * n;
     const int64_t m = n0 - 1 + j;
     Euler<R> f;
-    f.y0 = f.y1 = f.x = no_phase<R>();
+    f.y0 = f.y1 = f.x = f.x0 = no_phase<R>();
     if (m >= 0 && m < M) {
-      f = loc_factor<R>(loc_step<R>(tab, q + (b * M + m) * tab.K, i, j > 0));
-      if (j > 0) cs[(b * M + m) * n + i] = cmake<R>(f.c, f.s);
+      const bool own = j > 0 && m < m0 + T;
+      f = loc_factor<R, NEAR>(loc_step<R>(tab, q + (b * M + m) * tab.K, i, own));
+      if (own) {
+        cplx<R>* o = cs + (b * T + m - m0) * n * (NEAR ? 2 : 1) + i;
+        o[0] = cmake<R>(f.c1, f.s);
+        if (NEAR) o[n] = cmake<R>(f.sy, R(0));
+      }
     }
     y0[j][i] = f.y0;
     y1[j][i] = f.y1;
     xx[j][i] = f.x;
+    if (NEAR) x0[j][i] = f.x0;
   }
   __syncthreads();
   const int G = N / E;
   for (int idx = threadIdx.x; idx < kPrepSteps * N; idx += kPrepThreads) {
     const int j = idx / N + 1, r = idx & (N - 1);
     const int64_t m = n0 - 1 + j;
-    if (m > M) continue;
-    cplx<R> v;
+    if (m > m0 + T) continue;
+    cplx<R> v;                                       // Delta - 1
     if constexpr (sizeof(R) == 4) {
       uint32_t a = 0;
-      for (int i = 0; i < n; ++i) a += ((r >> i) & 1) ? (uint32_t)y1[j][i] + (uint32_t)xx[j - 1][i] : (uint32_t)y0[j][i];
-      v = phasor((int32_t)a);
+      for (int i = 0; i < n; ++i) {
+        const bool up = (r >> i) & 1;
+        if (NEAR)
+          a += (uint32_t)(up ? xx[j - 1][i] : x0[j - 1][i]);
+        else
+          a += up ? (uint32_t)y1[j][i] + (uint32_t)xx[j - 1][i] : (uint32_t)y0[j][i];
+      }
+      v = phasor<true>((int32_t)a);
     } else {
       v = cmake<R>(R(1), R(0));
       for (int i = 0; i < n; ++i) v = cmul<R>(v, ((r >> i) & 1) ? cmul<R>(y1[j][i], xx[j - 1][i]) : y0[j][i]);
+      v.x -= R(1);
     }
     if (m < M) {
-      // the drift (and a pulse's own) is the same at every step, so its FP32 rounding would add up
-      // over the chain: FP32 chains take it as hi + lo
       v = loc_times<R>(v, D[r]);
-      if (pd) v = loc_times<R>(v, pd[b * pd_b + m * pd_n + r]);
+      if (pd) {
+        double2 p = pd[b * pd_b + m * pd_n + r];
+        p.x -= 1.0;
+        v = loc_times<R>(v, p);
+      }
     }
-    // |Delta| = 1 to the last bit (the residual is exact under fma): without it the rounding of the
-    // phases changed the chain's norm five times as much
-    const R res = R(0.5) * fma(-v.y, v.y, fma(-v.x, v.x, R(1)));
-    delta[(b * (M + 1) + m) * N + loc_pos(r, E, G)] = cmake<R>(fma(res, v.x, v.x), fma(res, v.y, v.y));
+    // scaled to |Delta| = 1: without it the rounding of the phases changed the chain's norm five
+    // times as much
+    const R res = R(-0.5) * fma(v.x, v.x, fma(v.y, v.y, R(2) * v.x));
+    delta[(b * (T + 1) + m - m0) * N + loc_pos(r, E, G)] = cmake<R>(v.x + fma(res, v.x, res), fma(res, v.y, v.y));
   }
 }
 
@@ -255,11 +279,11 @@ loc_chain_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
 #pragma unroll
   for (int e = 0; e < E; ++e) v[e] = cmake<R>(l * E + e == x ? R(1) : R(0), R(0));
   const cplx<R>* d = delta + b * (M + 1) * N;
-  const cplx<R>* r = cs + b * M * L::NQ;
+  const cplx<R>* r = cs + b * M * L::CS;
 #pragma unroll 1
   for (int64_t m = n0; m < n1; ++m) {
-    cplx<R> c[L::NQ];
-    L::load_cs(c, r + m * L::NQ);
+    cplx<R> c[L::CS];
+    L::load_cs(c, r + m * L::CS);
     L::template diag<false>(v, d + m * N, l);
     L::rotate(v, c, l);
   }
@@ -336,7 +360,7 @@ loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
   const int part = x / L::C;
   const int64_t b = g / S, n0 = (g - b * S) * sps, n1 = n0 + sps < M ? n0 + sps : M;
   const cplx<R>* d = delta + b * (M + 1) * N;
-  const cplx<R>* r = cs + b * M * L::NQ;
+  const cplx<R>* r = cs + b * M * L::CS;
   cplx<R> p[E], w[E];
   {
     const double2 tb = tau[b];
@@ -376,8 +400,8 @@ loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
   for (int t = 0; t < most; ++t) {
     const bool act = on && t < len;
     const int64_t m = t < len ? n1 - 1 - t : n0;
-    cplx<R> c[L::NQ];
-    L::load_cs(c, r + m * L::NQ);
+    cplx<R> c[L::CS];
+    L::load_cs(c, r + m * L::CS);
     R v[WS::P];
 #pragma unroll
     for (int i = 0; i < WS::P; ++i) v[i] = R(0);
@@ -401,21 +425,21 @@ loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
 }
 
 // dF/du_kn = (2 dt / N^2) sum_i Tr(g_ki rho_i) with g_ki = W h_ki W^dag, W the product of the
-// factors after k on qubit i, conjugated by the step's trailing phase diag(1, x_i) (the sums are
-// taken between the rotation and that phase): Re(g01 x (X + iY)) + gz Z.
+// factors after k on qubit i, conjugated by the step's trailing phases diag(x0_i, x1_i) (the sums are
+// taken between the rotation and those): Re(g01 conj(x0) x1 (X + iY)) + gz Z.
 constexpr int kFinSteps = 8, kFinThreads = 128;
 
-template <typename R>
+template <typename R, bool NEAR>
 __global__ void __launch_bounds__(kFinThreads)
-loc_grad_kernel(LocTab<R> tab, const double2* __restrict__ h, const int32_t* __restrict__ q, int64_t M, int n, int parts,
-                int64_t tiles, const R* __restrict__ bl, double scale, double* __restrict__ grad) {
+loc_grad_kernel(LocTab<R> tab, const double2* __restrict__ h, const int32_t* __restrict__ q, int64_t M, int64_t w0,
+                int64_t T, int n, int parts, int64_t tiles, const R* __restrict__ bl, double scale, double* __restrict__ grad) {
   __shared__ double sum[kFinSteps][30];
   __shared__ double2 xy[kFinSteps][10];
-  const int64_t b = blockIdx.x / tiles, m0 = (blockIdx.x - b * tiles) * kFinSteps;
-  const int steps = (int)(M - m0 < kFinSteps ? M - m0 : kFinSteps);
+  const int64_t b = blockIdx.x / tiles, j0 = (blockIdx.x - b * tiles) * kFinSteps, m0 = w0 + j0;
+  const int steps = (int)(T - j0 < kFinSteps ? T - j0 : kFinSteps);
   for (int idx = threadIdx.x; idx < steps * 3 * n; idx += kFinThreads) {
     const int j = idx / (3 * n), v = idx - j * 3 * n;
-    const R* o = bl + (b * M + m0 + j) * parts * (3 * n) + v;
+    const R* o = bl + (b * T + j0 + j) * parts * (3 * n) + v;
     double a = 0.0;
     for (int p = 0; p < parts; ++p) a += (double)o[(int64_t)p * 3 * n];
     sum[j][v] = a;
@@ -423,13 +447,13 @@ loc_grad_kernel(LocTab<R> tab, const double2* __restrict__ h, const int32_t* __r
   __syncthreads();
   for (int idx = threadIdx.x; idx < steps * n; idx += kFinThreads) {
     const int j = idx / n, i = idx - j * n;
-    const phase_t<R> x = loc_factor<R>(loc_step<R>(tab, q + (b * M + m0 + j) * tab.K, i, false)).x;
-    double2 xv;
+    const Euler<R> f = loc_factor<R, NEAR>(loc_step<R>(tab, q + (b * M + m0 + j) * tab.K, i, false));
+    double2 xv;                                      // conj(x0) x1
     if constexpr (sizeof(R) == 4) {
-      const float2 f = phasor(x);
-      xv = make_double2(f.x, f.y);
+      const float2 x = phasor<false>((int32_t)((uint32_t)f.x - (uint32_t)f.x0));
+      xv = make_double2(x.x, x.y);
     } else {
-      xv = x;
+      xv = f.x;
     }
     const double X = sum[j][3 * i], Y = sum[j][3 * i + 1];
     xy[j][i] = make_double2(xv.x * X - xv.y * Y, xv.x * Y + xv.y * X);
@@ -512,6 +536,216 @@ static cudaError_t loc_sweep_t(const redo_table* t, const ChainPlan& p, int64_t 
 }
 
 // ============================================================================
+// State sweeps: one column per pulse (Section IV observables, Section III state transfer).  The
+// steps of a pulse are serial, so a column is spread over a whole warp (N >= 64) and the next step's
+// diagonal and rotations are loaded while the present ones are applied; one warp per block, so that
+// a few pulses reach as many SMs.
+// ============================================================================
+__host__ __device__ constexpr int loc_vec_entries(int N) { return N >= 64 ? N / 32 : 2; }
+
+// a + b exactly as s + e
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = a + b;
+  const float z = s - a;
+  e = (a - (s - z)) + (b - z);
+}
+
+// This lane's part of sum_r o_r |v_r|^2.  FP32 states keep the FP64 accumulation's accuracy in
+// FP32 pairs (products split by fma, sums by two_sum): the FP64 pipe would take longer than the step.
+template <int E> __device__ __forceinline__ float2 lane_expect(const float2 (&v)[E], const float2 (&o)[E]) {
+  float acc = 0.f, lo = 0.f;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const float h = v[e].x * v[e].x, h2 = v[e].y * v[e].y;
+    float s, er;
+    two_sum(h, h2, s, er);
+    const float l = (fmaf(v[e].x, v[e].x, -h) + fmaf(v[e].y, v[e].y, -h2)) + er;
+    const float p = o[e].x * s;
+    const float pl = fmaf(o[e].y, s, fmaf(o[e].x, l, fmaf(o[e].x, s, -p)));
+    float t;
+    two_sum(acc, p, t, er);
+    acc = t;
+    lo += er + pl;
+  }
+  return make_float2(acc, lo);
+}
+template <int E> __device__ __forceinline__ double2 lane_expect(const double2 (&v)[E], const double2 (&o)[E]) {
+  double acc = 0.0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) acc = fma(o[e].x, fma(v[e].x, v[e].x, v[e].y * v[e].y), acc);
+  return make_double2(acc, 0.0);
+}
+
+// part[b][n][l]: lane l's part of <O> after n steps
+template <typename R, int N>
+__global__ void __launch_bounds__(32)
+loc_sim_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t B, int64_t M,
+               const double2* __restrict__ psi0, int batched, const double* __restrict__ obs, cplx<R>* __restrict__ part) {
+  constexpr int E = loc_vec_entries(N);
+  using L = LocCol<R, N, E>;
+  const int lane = threadIdx.x, l = lane / L::C;
+  const int64_t b_raw = (int64_t)blockIdx.x * L::C + lane % L::C;
+  const bool on = b_raw < B;
+  const int64_t b = on ? b_raw : B - 1;              // idle lanes follow the last pulse, write nothing
+  const cplx<R>* d = delta + b * (M + 1) * N;
+  const cplx<R>* r = cs + b * M * L::CS;
+  cplx<R>* o = part + b * (M + 1) * L::G + l;
+  cplx<R> v[E], w[E], dn[E], cn[L::CS];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const double2 z = psi0[(batched ? b * N : 0) + l * E + e];
+    v[e] = cmake<R>((R)z.x, (R)z.y);
+    const double ov = obs[l * E + e];
+    w[e] = cmake<R>((R)ov, (R)(ov - (double)(R)ov));
+  }
+  cplx<R> a = lane_expect<E>(v, w);
+  if (on) o[0] = a;
+  if (M > 0) {
+    L::load_diag(dn, d, l);
+    L::load_cs(cn, r);
+  }
+#pragma unroll 1
+  for (int64_t m = 0; m < M; ++m) {
+    cplx<R> c[L::CS];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = plus_mul<R, L::NEAR>(v[e], dn[e]);
+#pragma unroll
+    for (int i = 0; i < L::CS; ++i) c[i] = cn[i];
+    const int64_t nx = m + 1 < M ? m + 1 : m;
+    L::load_diag(dn, d + nx * N, l);
+    L::load_cs(cn, r + nx * L::CS);
+    L::rotate(v, c, l);
+    a = lane_expect<E>(v, w);                        // |v|^2: the trailing phases do not enter
+    if (on) o[(m + 1) * L::G] = a;
+  }
+}
+
+template <typename R>
+__global__ void loc_expect_kernel(const cplx<R>* __restrict__ part, int64_t n, int G, double* __restrict__ expect) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    double a = 0.0;
+    for (int l = 0; l < G; ++l) {
+      const cplx<R> p = part[i * G + l];
+      a += (double)p.x + (double)p.y;
+    }
+    expect[i] = a;
+  }
+}
+
+// F_S = |<psi_T|U|psi_0>|^2 and the Bloch sums of its gradient: forward over the steps, then back
+// with the state undone and the costate <psi_T| U_M ... carried along (trace_undo).  One launch
+// covers the steps [m0, m0 + T): forward (fwd), at the chain's end the overlap, and back (back);
+// between launches both vectors rest in st[b][2][N].
+template <typename R, int N>
+__global__ void __launch_bounds__(32)
+loc_state_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t B, int64_t M, int64_t m0,
+                 int64_t T, int fwd, int back, const double2* __restrict__ psi0, const double2* __restrict__ psiT,
+                 int batched, double* __restrict__ F_out, R* __restrict__ bl, cplx<R>* __restrict__ st) {
+  constexpr int E = loc_vec_entries(N);
+  using L = LocCol<R, N, E>;
+  using WS = WarpSums<R, 3 * L::NQ>;
+  const int lane = threadIdx.x, l = lane / L::C;
+  const int64_t b_raw = (int64_t)blockIdx.x * L::C + lane % L::C;
+  const bool on = b_raw < B;
+  const int64_t b = on ? b_raw : B - 1;              // idle lanes follow the last pulse, write nothing
+  const cplx<R>* d = delta + b * (T + 1) * N;
+  const cplx<R>* r = cs + b * T * L::CS;
+  cplx<R>* sp = st + b * 2 * N + l * E;
+  cplx<R> p[E], w[E], dn[E], cn[L::CS];
+  if (fwd) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const double2 z = m0 == 0 ? psi0[(batched ? b * N : 0) + l * E + e] : make_double2(0.0, 0.0);
+      p[e] = m0 == 0 ? cmake<R>((R)z.x, (R)z.y) : sp[e];
+    }
+    L::load_diag(dn, d, l);
+    if (T > 0) L::load_cs(cn, r);
+#pragma unroll 1
+    for (int64_t m = 0; m < T; ++m) {
+      cplx<R> c[L::CS];
+#pragma unroll
+      for (int e = 0; e < E; ++e) p[e] = plus_mul<R, L::NEAR>(p[e], dn[e]);
+#pragma unroll
+      for (int i = 0; i < L::CS; ++i) c[i] = cn[i];
+      L::load_diag(dn, d + (m + 1) * N, l);          // the last one read is the window's closing diagonal
+      if (m + 1 < T) L::load_cs(cn, r + (m + 1) * L::CS);
+      L::rotate(p, c, l);
+    }
+  } else {
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      p[e] = sp[e];
+      w[e] = sp[N + e];
+    }
+  }
+  if (fwd && m0 + T == M) {
+    double tx = 0.0, ty = 0.0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const double2 z = psiT[(batched ? b * N : 0) + l * E + e];
+      const cplx<R> u = plus_mul<R, L::NEAR>(p[e], dn[e]);
+      tx = fma(z.x, (double)u.x, tx); tx = fma(z.y, (double)u.y, tx);
+      ty = fma(z.x, (double)u.y, ty); ty = fma(-z.y, (double)u.x, ty);
+    }
+#pragma unroll
+    for (int off = L::C; off < 32; off *= 2) {
+      tx += __shfl_xor_sync(0xffffffffu, tx, off);
+      ty += __shfl_xor_sync(0xffffffffu, ty, off);
+    }
+    if (F_out && on && l == 0) F_out[b] = tx * tx + ty * ty;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      // conj(psi_T) conj(tau), then the closing diagonal
+      const double2 z = psiT[(batched ? b * N : 0) + l * E + e];
+      w[e] = plus_mul<R, L::NEAR>(cmake<R>((R)(z.x * tx - z.y * ty), (R)(-z.y * tx - z.x * ty)), dn[e]);
+    }
+  }
+  if (back && T > 0) {
+    L::load_diag(dn, d + (T - 1) * N, l);
+    L::load_cs(cn, r + (T - 1) * L::CS);
+#pragma unroll 1
+    for (int64_t m = T - 1; m >= 0; --m) {
+      cplx<R> c[L::CS], dc[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) dc[e] = dn[e];
+#pragma unroll
+      for (int i = 0; i < L::CS; ++i) c[i] = cn[i];
+      const int64_t nx = m > 0 ? m - 1 : 0;
+      L::load_diag(dn, d + nx * N, l);
+      L::load_cs(cn, r + nx * L::CS);
+      R v[WS::P];
+#pragma unroll
+      for (int i = 0; i < WS::P; ++i) v[i] = R(0);
+      L::trace_undo(p, w, c, l, v);
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        p[e] = plus_mul_conj<R, L::NEAR>(p[e], dc[e]);
+        w[e] = plus_mul<R, L::NEAR>(w[e], dc[e]);
+      }
+      R* o = bl + (b * T + m) * (3 * L::NQ);
+      if constexpr (L::G == 32) {
+        const int idx = WS::full(v, lane);
+        if (on && idx >= 0) o[idx] = v[0];
+      } else {
+#pragma unroll
+        for (int i = 0; i < 3 * L::NQ; ++i) {
+#pragma unroll
+          for (int off = L::C; off < 32; off *= 2) v[i] += __shfl_xor_sync(0xffffffffu, v[i], off);
+          if (on && l == 0) o[i] = v[i];
+        }
+      }
+    }
+  }
+  if (on && T < M) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      sp[e] = p[e];
+      if (!fwd || back) sp[N + e] = w[e];
+    }
+  }
+}
+
+// ============================================================================
 // Host side: step-operator scratch in slices of pulses, plans, launches
 // ============================================================================
 // A slice holds the rotations and diagonals of as many pulses as fit kLocSlice bytes, so that long
@@ -526,15 +760,17 @@ static int loc_parts(const redo_table* t, bool dbl) {
   return lanes >= 32 ? lanes / 32 : 1;
 }
 
-// Scratch of nb pulses: diagonals, rotations and, for a gradient (what >= 1), the Bloch sums and
-// (what = 2) the boundary traces.
+// Scratch of nb pulses: diagonals and rotations, then by what is computed (LocalWhat) the Bloch
+// sums, the boundary traces or the lanes' parts of the observable.
 struct LocScratch {
   void *delta, *cs, *bl, *bz;
   size_t total;
 };
 static LocScratch loc_scratch(const redo_table* t, int64_t nb, int64_t M, int prec, int what, void* base) {
   const size_t el = prec == REDO_FP64 ? sizeof(double) : sizeof(float);
-  const size_t parts = what ? (size_t)loc_parts(t, prec == REDO_FP64) : 0;
+  const bool grad = what == kLocalGrad || what == kLocalPhaseGrad;
+  const size_t parts = grad ? (size_t)loc_parts(t, prec == REDO_FP64) : 1;
+  const size_t lanes = what == kLocalSim ? (size_t)(t->N / loc_vec_entries(t->N)) : 0;
   LocScratch w;
   char* c = (char*)base;
   size_t off = 0;
@@ -544,15 +780,16 @@ static LocScratch loc_scratch(const redo_table* t, int64_t nb, int64_t M, int pr
     return at;
   };
   w.delta = take((size_t)nb * (M + 1) * t->N * 2 * el);
-  w.cs = take((size_t)nb * M * t->loc * 2 * el);
-  w.bl = take(what >= 1 ? (size_t)nb * M * parts * 3 * t->loc * el : 0);
-  w.bz = take(what == 2 ? (size_t)nb * (M + 1) * parts * t->K * el : 0);
+  w.cs = take((size_t)nb * M * t->loc * 2 * el * (loc_near(prec == REDO_FP64, t->N) ? 2 : 1));
+  w.bl = take(grad ? (size_t)nb * M * parts * 3 * t->loc * el : (size_t)nb * (M + 1) * lanes * 2 * el);
+  w.bz = take(what == kLocalPhaseGrad ? (size_t)nb * (M + 1) * parts * t->K * el : 0);
   w.total = off;
   return w;
 }
 
 bool local_eligible(const redo_table* t, int64_t M, int prec, int what) {
-  if (t->loc == 0 || (what && prec == REDO_FP64 && t->N > 512)) return false;
+  if (t->loc == 0) return false;
+  if ((what == kLocalGrad || what == kLocalPhaseGrad) && prec == REDO_FP64 && t->N > 512) return false;
   return loc_scratch(t, 1, M, prec, what, nullptr).total <= kLocSlice;
 }
 
@@ -581,11 +818,15 @@ ChainPlan plan_chain_local(const redo_table* t, int64_t B, int64_t M, int prec, 
 }
 
 template <typename R>
-static cudaError_t loc_steps_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int E, const LocalDiag& pd,
-                               int64_t b0, void* cs, void* delta, int64_t* status, cudaStream_t s) {
-  const int64_t tiles = (M + 1 + kPrepSteps - 1) / kPrepSteps;
-  loc_steps_kernel<R><<<(unsigned)(B * tiles), kPrepThreads, 0, s>>>(
-      loc_tab<R>(t, status), q + b0 * M * t->K, M, t->loc, t->N, E, tiles,
+static cudaError_t loc_steps_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int64_t m0, int64_t T, int E,
+                               const LocalDiag& pd, int64_t b0, void* cs, void* delta, int64_t* status,
+                               cudaStream_t s) {
+  const int64_t tiles = (T + 1 + kPrepSteps - 1) / kPrepSteps;
+  auto kern = loc_steps_kernel<R, false>;
+  if constexpr (sizeof(R) == 4)
+    if (loc_near(false, t->N)) kern = loc_steps_kernel<R, true>;
+  kern<<<(unsigned)(B * tiles), kPrepThreads, 0, s>>>(
+      loc_tab<R>(t, status), q + b0 * M * t->K, M, m0, T, t->loc, t->N, E, tiles,
       t->loc_D64,
       pd.p ? pd.p + b0 * pd.sb : nullptr, pd.sb, pd.sn, (cplx<R>*)cs, (cplx<R>*)delta);
   return cudaGetLastError();
@@ -593,13 +834,13 @@ static cudaError_t loc_steps_t(const redo_table* t, const int32_t* q, int64_t B,
 
 static cudaError_t loc_steps(const redo_table* t, const int32_t* q, int64_t nb, int64_t M, int prec, int E,
                              const LocalDiag& pd, int64_t b0, const LocScratch& w, int64_t* status, cudaStream_t s) {
-  return prec == REDO_FP64 ? loc_steps_t<double>(t, q, nb, M, E, pd, b0, w.cs, w.delta, status, s)
-                           : loc_steps_t<float>(t, q, nb, M, E, pd, b0, w.cs, w.delta, status, s);
+  return prec == REDO_FP64 ? loc_steps_t<double>(t, q, nb, M, 0, M, E, pd, b0, w.cs, w.delta, status, s)
+                           : loc_steps_t<float>(t, q, nb, M, 0, M, E, pd, b0, w.cs, w.delta, status, s);
 }
 
 cudaError_t launch_local_chain(const redo_table* t, const int32_t* q, const ChainPlan& p, int prec, int what,
                                const LocalDiag& pd, void* ops, void* seg_out, int64_t* status, cudaStream_t s) {
-  const bool dbl = prec == REDO_FP64, two = what > 0;
+  const bool dbl = prec == REDO_FP64, two = what != kLocalChain;
   const int64_t slice = local_slice(t, p.B, p.M, prec, what);
   const LocScratch w = loc_scratch(t, slice, p.M, prec, what, ops);
   const int E = loc_entries(dbl, t->N, two);
@@ -619,11 +860,15 @@ cudaError_t launch_local_chain(const redo_table* t, const int32_t* q, const Chai
 }
 
 template <typename R>
-static cudaError_t loc_finish_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int parts, double norm,
-                                const LocScratch& w, double* grad, double* gphi, cudaStream_t s) {
-  const int64_t tiles = (M + kFinSteps - 1) / kFinSteps;
+static cudaError_t loc_finish_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int64_t m0, int64_t T,
+                                int parts, double norm, const LocScratch& w, double* grad, double* gphi,
+                                cudaStream_t s) {
+  const int64_t tiles = (T + kFinSteps - 1) / kFinSteps;
   LocTab<R> tab = loc_tab<R>(t, nullptr);
-  loc_grad_kernel<R><<<(unsigned)(B * tiles), kFinThreads, 0, s>>>(tab, t->loc_h, q, M, t->loc, parts, tiles,
+  auto kern = loc_grad_kernel<R, false>;
+  if constexpr (sizeof(R) == 4)
+    if (loc_near(false, t->N)) kern = loc_grad_kernel<R, true>;
+  kern<<<(unsigned)(B * tiles), kFinThreads, 0, s>>>(tab, t->loc_h, q, M, m0, T, t->loc, parts, tiles,
                                                                    (const R*)w.bl, 2.0 * t->dt / norm, grad);
   if (gphi) {
     const int64_t n = B * M * t->K, blocks = (n + 255) / 256;
@@ -650,14 +895,137 @@ cudaError_t launch_local_grad(const redo_table* t, const int32_t* q, const Chain
     if (slice < p.B && (e = loc_steps(t, q, nb, p.M, prec, E, pd, b0, w, status, s))) return e;
     const char* P = (const char*)Pck + (size_t)(b0 * p.S) * mat;
     const char* Q = (const char*)Rck + (size_t)(b0 * p.S) * mat;
-    void* bz = what == 2 ? w.bz : nullptr;
+    void* bz = what == kLocalPhaseGrad ? w.bz : nullptr;
     e = dbl ? loc_sweep_t<double>(t, p, nb, w.cs, w.delta, P, Q, tau + b0, w.bl, bz, s)
             : loc_sweep_t<float>(t, p, nb, w.cs, w.delta, P, Q, tau + b0, w.bl, bz, s);
     if (e) return e;
     const int64_t at = b0 * p.M * t->K;
     double* gp = gphi ? gphi + at : nullptr;
-    e = dbl ? loc_finish_t<double>(t, q + at, nb, p.M, parts, norm, w, grad + at, gp, s)
-            : loc_finish_t<float>(t, q + at, nb, p.M, parts, norm, w, grad + at, gp, s);
+    e = dbl ? loc_finish_t<double>(t, q + at, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, s)
+            : loc_finish_t<float>(t, q + at, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, s);
+    if (e) return e;
+  }
+  return cudaSuccess;
+}
+
+#define LOC_VEC(KERNEL, ...)                                                       \
+  switch (t->N) {                                                                 \
+    case 2: KERNEL<R, 2><<<blocks, 32, 0, s>>>(__VA_ARGS__); break;               \
+    case 4: KERNEL<R, 4><<<blocks, 32, 0, s>>>(__VA_ARGS__); break;               \
+    case 8: KERNEL<R, 8><<<blocks, 32, 0, s>>>(__VA_ARGS__); break;               \
+    case 16: KERNEL<R, 16><<<blocks, 32, 0, s>>>(__VA_ARGS__); break;             \
+    case 32: KERNEL<R, 32><<<blocks, 32, 0, s>>>(__VA_ARGS__); break;             \
+    case 64: KERNEL<R, 64><<<blocks, 32, 0, s>>>(__VA_ARGS__); break;             \
+    case 128: KERNEL<R, 128><<<blocks, 32, 0, s>>>(__VA_ARGS__); break;           \
+    case 256: KERNEL<R, 256><<<blocks, 32, 0, s>>>(__VA_ARGS__); break;           \
+    case 512: KERNEL<R, 512><<<blocks, 32, 0, s>>>(__VA_ARGS__); break;           \
+    case 1024: KERNEL<R, 1024><<<blocks, 32, 0, s>>>(__VA_ARGS__); break;         \
+    default: return cudaErrorInvalidValue;                                        \
+  }
+
+template <typename R>
+static cudaError_t loc_sim_t(const redo_table* t, int64_t B, int64_t M, const double2* psi0, int batched,
+                             const double* obs, const LocScratch& w, double* expect, cudaStream_t s) {
+  const int lanes = t->N / loc_vec_entries(t->N), cols = 32 / lanes;
+  const unsigned blocks = (unsigned)((B + cols - 1) / cols);
+  LOC_VEC(loc_sim_kernel, (const cplx<R>*)w.cs, (const cplx<R>*)w.delta, B, M, psi0, batched, obs, (cplx<R>*)w.bl)
+  const int64_t n = B * (M + 1), nb = (n + 127) / 128;
+  loc_expect_kernel<R><<<(unsigned)(nb < 4096 ? nb : 4096), 128, 0, s>>>((const cplx<R>*)w.bl, n, lanes, expect);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_local_sim(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int prec, const double2* psi0,
+                             int batched, const double* obs, double* expect, void* ops, int64_t* status, cudaStream_t s) {
+  const int64_t slice = local_slice(t, B, M, prec, kLocalSim);
+  const LocScratch w = loc_scratch(t, slice, M, prec, kLocalSim, ops);
+  for (int64_t b0 = 0; b0 < B; b0 += slice) {
+    const int64_t nb = b0 + slice < B ? slice : B - b0;
+    cudaError_t e = loc_steps(t, q, nb, M, prec, loc_vec_entries(t->N), LocalDiag{nullptr, 0, 0}, b0, w, status, s);
+    if (e) return e;
+    const double2* p0 = psi0 + (batched ? b0 * t->N : 0);
+    double* ex = expect + b0 * (M + 1);
+    e = prec == REDO_FP64 ? loc_sim_t<double>(t, nb, M, p0, batched, obs, w, ex, s)
+                          : loc_sim_t<float>(t, nb, M, p0, batched, obs, w, ex, s);
+    if (e) return e;
+  }
+  return cudaSuccess;
+}
+
+// State-transfer scratch.  Its size may depend on the number of pulses only, so the step operators
+// are held for a window of steps (at most 4096, at least 64) of a slice of pulses and the sweep
+// goes window by window, forward and then back (most calls have one window).
+struct LocStatePlan {
+  int64_t pulses, steps;
+};
+static size_t loc_state_step(const redo_table* t) {              // FP64 bytes of one step of one pulse
+  return ((size_t)t->N + 3 * t->loc) * sizeof(double2);
+}
+static LocStatePlan loc_state_plan(const redo_table* t, int64_t B) {
+  const size_t per = loc_state_step(t);
+  int64_t pulses = (int64_t)(((size_t)256 << 20) / (64 * per));
+  if (pulses > B) pulses = B;
+  if (pulses < 1) pulses = 1;
+  int64_t steps = (int64_t)(((size_t)64 << 20) / ((size_t)pulses * per));
+  if (steps > 4096) steps = 4096;
+  if (steps < 64) steps = 64;
+  return LocStatePlan{pulses, steps};
+}
+// delta, rotations, Bloch sums of the window, and the two vectors of every pulse of the slice
+static LocScratch loc_state_scratch(const redo_table* t, const LocStatePlan& p, void* base) {
+  LocScratch w;
+  char* c = (char*)base;
+  const size_t nb = (size_t)p.pulses, T = (size_t)p.steps;
+  w.delta = c;
+  c += up256(nb * (T + 1) * t->N * sizeof(double2));
+  w.cs = c;
+  c += up256(nb * T * t->loc * sizeof(double2));
+  w.bl = c;
+  c += up256(nb * T * 3 * t->loc * sizeof(double));
+  w.bz = c;
+  c += up256(nb * 2 * t->N * sizeof(double2));
+  w.total = (size_t)(c - (char*)base);
+  return w;
+}
+
+size_t local_state_bytes(const redo_table* t, int64_t B) {
+  return t->loc > 0 && B > 0 ? loc_state_scratch(t, loc_state_plan(t, B), nullptr).total : 0;
+}
+
+template <typename R>
+static cudaError_t loc_state_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int64_t win,
+                               const double2* psi0, const double2* psiT, int batched, double* F_out, double* grad,
+                               const LocScratch& w, int64_t* status, cudaStream_t s) {
+  const int lanes = t->N / loc_vec_entries(t->N), cols = 32 / lanes;
+  const unsigned blocks = (unsigned)((B + cols - 1) / cols);
+  const int64_t nw = M > 0 ? (M + win - 1) / win : 1;
+  const bool back = grad && M > 0;
+  // windows 0 .. nw - 1 forward, the last one also back, then nw - 2 .. 0 back
+  for (int64_t i = 0; i < (back ? 2 * nw - 1 : nw); ++i) {
+    const bool fwd = i < nw;
+    const int64_t k = fwd ? i : 2 * nw - 2 - i, m0 = k * win, T = m0 + win < M ? win : M - m0;
+    const int bk = back && i >= nw - 1;
+    cudaError_t e = loc_steps_t<R>(t, q, B, M, m0, T, loc_vec_entries(t->N), LocalDiag{nullptr, 0, 0}, 0, w.cs,
+                                   w.delta, fwd ? status : nullptr, s);
+    if (e) return e;
+    LOC_VEC(loc_state_kernel, (const cplx<R>*)w.cs, (const cplx<R>*)w.delta, B, M, m0, T, fwd, bk, psi0, psiT, batched,
+            F_out, (R*)w.bl, (cplx<R>*)w.bz)
+    if (bk && (e = loc_finish_t<R>(t, q, B, M, m0, T, 1, 1.0, w, grad, nullptr, s))) return e;
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_local_state(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int prec,
+                               const double2* psi0, const double2* psiT, int batched, double* F_out, double* grad,
+                               void* ops, int64_t* status, cudaStream_t s) {
+  const LocStatePlan p = loc_state_plan(t, B);
+  const LocScratch w = loc_state_scratch(t, p, ops);
+  for (int64_t b0 = 0; b0 < B; b0 += p.pulses) {
+    const int64_t nb = b0 + p.pulses < B ? p.pulses : B - b0, at = b0 * M * t->K, v = batched ? b0 * t->N : 0;
+    double *F = F_out ? F_out + b0 : nullptr, *g = grad ? grad + at : nullptr;
+    const cudaError_t e =
+        prec == REDO_FP64
+            ? loc_state_t<double>(t, q + at, nb, M, p.steps, psi0 + v, psiT + v, batched, F, g, w, status, s)
+            : loc_state_t<float>(t, q + at, nb, M, p.steps, psi0 + v, psiT + v, batched, F, g, w, status, s);
     if (e) return e;
   }
   return cudaSuccess;

@@ -920,7 +920,9 @@ cudaError_t launch_chain_combine(const redo_table* t, const ChainPlan& p, int pr
 // Re-unitarisation: Newton-Schulz polar iteration  P <- P (3I - P^dag P) / 2,
 // one CTA per matrix.  Converges quadratically to the unitary polar factor
 // P (P^dag P)^(-1/2) when ||P^dag P - I|| < 1; the product chains hand it
-// matrices within ~1e-3 of unitary, so one step leaves ~1e-6 of that.
+// matrices within ~1e-3 of unitary, so one step leaves ~1e-6 of that.  Computed as
+// P + P (I - P^dag P) / 2: the correction is small, so only the final addition rounds at the
+// precision of P (P times (3I - P^dag P) / 2 rounds there once per term).
 // ============================================================================
 template <typename Rin, typename Rc, int N, typename Rout = Rc>
 __global__ void __launch_bounds__(SmemMM<Rc, N, (N >= 64 ? 4 : (N >= 32 ? 2 : 1)),
@@ -940,25 +942,12 @@ polar_ns_kernel(const cplx<Rin>* __restrict__ in, cplx<Rout>* __restrict__ out, 
   }
   __syncthreads();
   cplx<Rc> Y[TM][TM];
-  const int ty = lt / MM::TX, tx = lt % MM::TX;
   for (int it = 0; it < iters; ++it) {
-    if constexpr (MM::TY == MM::TX && TM > 1) {
-      MM::ns_half_gram(P, Q, lt);                        // Q = (3I - P^dag P) / 2, half the Gram tiles
-    } else {
-      MM::run_adj(P, P, lt, Y);                          // G = P^dag P (P read in column order)
-#pragma unroll
-      for (int a = 0; a < TM; ++a)
-#pragma unroll
-        for (int c = 0; c < TM; ++c) {
-          const int r = ty + MM::TY * a, col = tx + MM::TX * c;
-          Q[r * N + col] = cmake<Rc>((r == col ? Rc(1.5) : Rc(0)) - Rc(0.5) * Y[a][c].x,
-                                     -Rc(0.5) * Y[a][c].y);
-        }
-    }
+    MM::ns_correction(P, Q, lt);                         // Q = (I - P^dag P) / 2
     __syncthreads();
-    MM::run(P, Q, lt, Y);                                // P (3I - G) / 2
+    MM::run(P, Q, lt, Y);                                // P (I - G) / 2
     __syncthreads();
-    MM::store(P, lt, Y);
+    MM::add(P, lt, Y);
     __syncthreads();
   }
   for (int i = lt; i < N2; i += MM::THREADS) {

@@ -14,6 +14,10 @@
 //     Delta_n = (tensor_i diag(y0_i(n), y1_i(n))) D P_n (tensor_i diag(1, x_i(n-1))),
 // so a step costs 4 operations per entry for Delta_n and 4 per entry and qubit (a 2 x 2 complex
 // operator would take 8 per entry and qubit).  Delta_M closes the chain (the last step's x_i).
+// Both are kept as their difference from the identity, c - 1 and Delta - 1, and applied as
+// v + (c - 1) v - s w and v + (Delta - 1) v (as many operations): a step is near the identity, and a
+// c or Delta rounded beside 1 would change the norm by up to 3e-8 in FP32, at every step alike when
+// the drive is steady (N = 1024, one global control: 7e-6 of <Z> after 200 steps, now 1e-6).
 #pragma once
 #include "redo_internal.cuh"
 
@@ -112,8 +116,8 @@ constexpr float kTurn = (float)kTurn64, kTurnLo = (float)(kTurn64 - (double)kTur
 constexpr float kPerTurn = 683565275.576431f;           // 2^32 / (2 pi)
 
 // e^{i t}: the quadrant from the integer's top bits, sine and cosine of the rest (|a| <= pi/4),
-// corrected for what its float conversion dropped
-__device__ __forceinline__ float2 phasor(int32_t t) {
+// corrected for what its float conversion dropped.  M1: e^{i t} - 1.
+template <bool M1> __device__ __forceinline__ float2 phasor(int32_t t) {
   const int32_t k = (int32_t)((uint32_t)t + 0x20000000u) >> 30;
   const int32_t res = (int32_t)((uint32_t)t - ((uint32_t)k << 30));
   const float fh = (float)res;
@@ -122,44 +126,86 @@ __device__ __forceinline__ float2 phasor(int32_t t) {
   float s, c;
   sincosf(a, &s, &c);
   const float s1 = fmaf(d, c, s), c1 = fmaf(-d, s, c);
-  const float re = (k & 1) ? -s1 : c1, im = (k & 1) ? c1 : s1;
-  return (k & 2) ? make_float2(-re, -im) : make_float2(re, im);
+  float re = (k & 1) ? -s1 : c1, im = (k & 1) ? c1 : s1;
+  if (k & 2) {
+    re = -re;
+    im = -im;
+  }
+  if (M1) re = k == 0 ? -s1 * s1 / (1.f + c1) : re - 1.f;
+  return make_float2(re, im);
 }
 
 // the angle of z in turns: atan2f, then one refinement against the phasor it gives
 __device__ __forceinline__ int32_t turns_of(float2 z) {
   const int32_t t = (int32_t)(uint32_t)(long long)rintf(atan2f(z.y, z.x) * kPerTurn);
-  const float2 p = phasor(t);
+  const float2 p = phasor<false>(t);
   const float re = fmaf(z.x, p.x, z.y * p.y), im = fmaf(z.y, p.x, -(z.x * p.y));
   return re > 0.f ? (int32_t)((uint32_t)t + (uint32_t)(int32_t)rintf(im / re * kPerTurn)) : t;
 }
 
-template <typename R> struct Euler { phase_t<R> y0, y1, x; R c, s; };
+// FP32 systems of up to four qubits are factored as
+//     V_i = diag(x0_i, x1_i) [[c_i, -conj(s_i)], [s_i, c_i]],   s_i complex, y0 = y1 = 1,
+// instead: every part is then near the identity when the controls' angles are small, and a step
+// rounds once per qubit beside the state's entries (v + t with a small t) where the real rotations
+// between O(1) phases round twice and once more for each phase.  It costs 8 operations per entry and
+// qubit, not 4; with few rows to average over, the chain's error is 0.6 times as large (N = 4, 790
+// steps: 1.4e-6 -> 8e-7 of the gradient), no larger than the dense FP32 products'.
+__host__ __device__ constexpr bool loc_near(bool dbl, int N) { return !dbl && N <= 16; }
+
+// c1 = c - 1; s = (s, sy), sy = 0 in the real form; x0 = 1 in the real form
+template <typename R> struct Euler { phase_t<R> y0, y1, x0, x; R c1, s, sy; };
 
 // The phases of a vanishing entry are free; x comes from the larger of the two entries that
 // determine it, so every entry of V_i is reproduced to rounding.
-template <typename R> __device__ __forceinline__ Euler<R> loc_factor(const Mat2<R>& v) {
+template <typename R, bool NEAR> __device__ __forceinline__ Euler<R> loc_factor(const Mat2<R>& v) {
   Euler<R> o;
   const R c2 = fma(v.a.x, v.a.x, v.a.y * v.a.y), s2 = fma(v.b.x, v.b.x, v.b.y * v.b.y);
   const R c = sqrt(c2), s = sqrt(s2);
-  if constexpr (sizeof(R) == 4) {
+  // (c, s) scaled to c^2 + s^2 = 1 (the residual is exact under fma, so the scaling has no bias), then
+  // c - 1 = -s^2 / (1 + c) without cancellation
+  const R res = R(0.5) * fma(-s, s, fma(-c, c, R(1)));
+  o.s = fma(res, s, s);
+  o.sy = R(0);
+  o.c1 = -(o.s * o.s) / (R(1) + fma(res, c, c));
+  if constexpr (NEAR) {
+    o.y0 = o.y1 = 0;
+    o.x = c > 0.f ? turns_of(v.e) : 0;
+    const float2 q = phasor<false>(o.x);
+    const float2 w = cmul_conj<float>(v.c, q);           // s e^{...}: V10 conj(x1)
+    o.x0 = c >= s ? turns_of(v.a) : turns_of(cmul<float>(make_float2(-v.b.x, -v.b.y), w));
+    const float wn = sqrtf(fmaf(w.x, w.x, w.y * w.y)), f = wn > 0.f ? o.s / wn : 0.f;
+    o.s = w.x * f;
+    o.sy = w.y * f;
+  } else if constexpr (sizeof(R) == 4) {
     // diag(1, e^{iA}) V diag(1, e^{-iA}) has a real entry -s: y1 = e^{iA} cancels in the diagonal
     o.y0 = turns_of(v.a);
     o.y1 = s > 0.f ? turns_of(make_float2(-v.b.x, -v.b.y)) : 0;
+    o.x0 = 0;
     o.x = (int32_t)(c >= s ? (uint32_t)turns_of(v.e) - (uint32_t)o.y1 : (uint32_t)turns_of(v.c) - (uint32_t)o.y0);
   } else {
     o.y0 = c > R(0) ? cmake<R>(v.a.x / c, v.a.y / c) : cmake<R>(R(1), R(0));
     o.y1 = s > R(0) ? cmake<R>(-v.b.x / s, -v.b.y / s) : cmake<R>(R(1), R(0));
+    o.x0 = cmake<R>(R(1), R(0));
     const cplx<R> w = c >= s ? cmul_conj<R>(v.e, o.y1) : cmul_conj<R>(v.c, o.y0);
     const R wn = sqrt(fma(w.x, w.x, w.y * w.y));
     o.x = wn > R(0) ? cmake<R>(w.x / wn, w.y / wn) : cmake<R>(R(1), R(0));
   }
-  // c^2 + s^2 = 1 to the last bit: the residual is exact under fma, so the correction has no bias
-  // (dividing by sqrt(c2 + s2), whose spacing is uneven around 1, gained 5e-8 of norm per FP32 step)
-  const R res = R(0.5) * fma(-s, s, fma(-c, c, R(1)));
-  o.c = fma(res, c, c);
-  o.s = fma(res, s, s);
   return o;
+}
+
+// v + d v, and v + conj(d) v.  NEAR: the small part summed first, one rounding beside v.
+template <typename R, bool NEAR = false> __device__ __forceinline__ cplx<R> plus_mul(cplx<R> v, cplx<R> d) {
+  if constexpr (NEAR) return cmake<R>(v.x + fma(-d.y, v.y, d.x * v.x), v.y + fma(d.y, v.x, d.x * v.y));
+  return cmake<R>(fma(-d.y, v.y, fma(d.x, v.x, v.x)), fma(d.y, v.x, fma(d.x, v.y, v.y)));
+}
+template <typename R, bool NEAR = false> __device__ __forceinline__ cplx<R> plus_mul_conj(cplx<R> v, cplx<R> d) {
+  return plus_mul<R, NEAR>(v, cmake<R>(d.x, -d.y));
+}
+// v + (c1 v + (s + i t) o); t is ignored in the real form
+template <typename R, bool NEAR> __device__ __forceinline__ cplx<R> rot_one(cplx<R> v, cplx<R> o, R c1, R s, R t) {
+  if constexpr (NEAR)
+    return cmake<R>(v.x + fma(-t, o.y, fma(s, o.x, c1 * v.x)), v.y + fma(t, o.x, fma(s, o.y, c1 * v.y)));
+  return cmake<R>(fma(s, o.x, fma(c1, v.x, v.x)), fma(s, o.y, fma(c1, v.y, v.y)));
 }
 
 // Layout of one column (N rows) over G = N / E lanes, E entries each: lane part l holds rows
@@ -169,78 +215,86 @@ template <typename R> __device__ __forceinline__ Euler<R> loc_factor(const Mat2<
 template <int N> struct Log2 { static constexpr int v = 1 + Log2<N / 2>::v; };
 template <> struct Log2<1> { static constexpr int v = 0; };
 
-__host__ __device__ __forceinline__ int loc_pos(int r, int E, int G) {
+__host__ __device__ __forceinline__ int loc_pos(int r, int E, int G) {   // E >= 2
   const int l = r / E, e = r - l * E;
-  return E == 1 ? l : ((e >> 1) * G + l) * 2 + (e & 1);
+  return ((e >> 1) * G + l) * 2 + (e & 1);
 }
 
 template <typename R, int N, int E> struct LocCol {
+  static constexpr bool NEAR = loc_near(sizeof(R) == 8, N);
   static constexpr int G = N / E, C = 32 / G, NQ = Log2<N>::v, EB = Log2<E>::v;
+  static constexpr int CS = NQ * (NEAR ? 2 : 1);     // (c - 1, s) of every qubit, then (sy, 0)
   static_assert(G * E == N && G <= 32, "column layout");
 
-  // v <- Delta v (or conj(Delta) v)
+  // v <- Delta v (or conj(Delta) v), d holding Delta - 1
   template <bool CONJ> static __device__ __forceinline__ void diag(cplx<R> (&v)[E], const cplx<R>* d, int l) {
-    if constexpr (E == 1) {
-      const cplx<R> a = __ldg(d + l);
-      v[0] = CONJ ? cmul_conj<R>(v[0], a) : cmul<R>(v[0], a);
-    } else {
 #pragma unroll
-      for (int e = 0; e < E; e += 2) {
-        cplx<R> a, b;
-        if constexpr (sizeof(R) == 4) {
-          const float4 p = __ldg(reinterpret_cast<const float4*>(d) + (e >> 1) * G + l);
-          a = make_float2(p.x, p.y);
-          b = make_float2(p.z, p.w);
-        } else {
-          a = __ldg(d + ((e >> 1) * G + l) * 2);
-          b = __ldg(d + ((e >> 1) * G + l) * 2 + 1);
-        }
-        v[e] = CONJ ? cmul_conj<R>(v[e], a) : cmul<R>(v[e], a);
-        v[e + 1] = CONJ ? cmul_conj<R>(v[e + 1], b) : cmul<R>(v[e + 1], b);
+    for (int e = 0; e < E; e += 2) {
+      cplx<R> a, b;
+      if constexpr (sizeof(R) == 4) {
+        const float4 p = __ldg(reinterpret_cast<const float4*>(d) + (e >> 1) * G + l);
+        a = make_float2(p.x, p.y);
+        b = make_float2(p.z, p.w);
+      } else {
+        a = __ldg(d + ((e >> 1) * G + l) * 2);
+        b = __ldg(d + ((e >> 1) * G + l) * 2 + 1);
+      }
+      v[e] = CONJ ? plus_mul_conj<R, NEAR>(v[e], a) : plus_mul<R, NEAR>(v[e], a);
+      v[e + 1] = CONJ ? plus_mul_conj<R, NEAR>(v[e + 1], b) : plus_mul<R, NEAR>(v[e + 1], b);
+    }
+  }
+  // its entries alone, for a later step
+  static __device__ __forceinline__ void load_diag(cplx<R> (&o)[E], const cplx<R>* d, int l) {
+#pragma unroll
+    for (int e = 0; e < E; e += 2) {
+      if constexpr (sizeof(R) == 4) {
+        const float4 p = __ldg(reinterpret_cast<const float4*>(d) + (e >> 1) * G + l);
+        o[e] = make_float2(p.x, p.y);
+        o[e + 1] = make_float2(p.z, p.w);
+      } else {
+        o[e] = __ldg(d + ((e >> 1) * G + l) * 2);
+        o[e + 1] = __ldg(d + ((e >> 1) * G + l) * 2 + 1);
       }
     }
   }
   static __device__ __forceinline__ cplx<R> swap(cplx<R> v, int lane_mask) {
     return cmake<R>(__shfl_xor_sync(0xffffffffu, v.x, lane_mask), __shfl_xor_sync(0xffffffffu, v.y, lane_mask));
   }
-  // (c, s) real rotations of every qubit, [[c, -s], [s, c]] on the pair (bit 0, bit 1)
-  static __device__ __forceinline__ void rotate(cplx<R> (&v)[E], const cplx<R> (&cs)[NQ], int l) {
+  // rotations of every qubit, [[c, -conj(s)], [s, c]] on the pair (bit 0, bit 1)
+  static __device__ __forceinline__ void rotate(cplx<R> (&v)[E], const cplx<R> (&cs)[CS], int l) {
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
-      const R c = cs[i].x, s = cs[i].y;
+      const R c = cs[i].x, s = cs[i].y, t = NEAR ? cs[CS - NQ + i].x : R(0);
       if (i < EB) {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           if (e & (1 << i)) continue;
           const cplx<R> a = v[e], b = v[e | (1 << i)];
-          v[e] = cmake<R>(fma(-s, b.x, c * a.x), fma(-s, b.y, c * a.y));
-          v[e | (1 << i)] = cmake<R>(fma(s, a.x, c * b.x), fma(s, a.y, c * b.y));
+          v[e] = rot_one<R, NEAR>(a, b, c, -s, t);
+          v[e | (1 << i)] = rot_one<R, NEAR>(b, a, c, s, t);
         }
       } else {
         const int m = 1 << (i - EB);
         const R sg = (l & m) ? s : -s;
 #pragma unroll
-        for (int e = 0; e < E; ++e) {
-          const cplx<R> o = swap(v[e], m * C);
-          v[e] = cmake<R>(fma(sg, o.x, c * v[e].x), fma(sg, o.y, c * v[e].y));
-        }
+        for (int e = 0; e < E; ++e) v[e] = rot_one<R, NEAR>(v[e], swap(v[e], m * C), c, sg, t);
       }
     }
   }
-  static __device__ __forceinline__ void load_cs(cplx<R> (&cs)[NQ], const cplx<R>* p) {
+  static __device__ __forceinline__ void load_cs(cplx<R> (&cs)[CS], const cplx<R>* p) {
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) cs[i] = __ldg(p + i);
+    for (int i = 0; i < CS; ++i) cs[i] = __ldg(p + i);
   }
   // The three Bloch sums of every qubit,
   //   X = Im Tr(X_i P R), Y = Im Tr(Y_i P R), Z = Im Tr(Z_i P R)
   // over this lane's entries of a column p of P and the matching row w of R, then the qubit's
-  // rotation undone on both (p <- rot^T p, w <- rot^T w).  A partial trace over the other qubits
+  // rotation undone on both (p <- rot^dag p, w <- w rot).  A partial trace over the other qubits
   // does not change when those are rotated, so each qubit is traced just before its own undo.
-  static __device__ __forceinline__ void trace_undo(cplx<R> (&p)[E], cplx<R> (&w)[E], const cplx<R> (&cs)[NQ],
+  static __device__ __forceinline__ void trace_undo(cplx<R> (&p)[E], cplx<R> (&w)[E], const cplx<R> (&cs)[CS],
                                                     int l, R* bl) {
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
-      const R c = cs[i].x, s = cs[i].y;
+      const R c = cs[i].x, s = cs[i].y, t = NEAR ? cs[CS - NQ + i].x : R(0);
       R bx = R(0), by = R(0), bz = R(0);
       if (i < EB) {
 #pragma unroll
@@ -254,10 +308,10 @@ template <typename R, int N, int E> struct LocCol {
           by = fma(pa.x, wb.x, by); by = fma(-pa.y, wb.y, by);
           bz = fma(pa.x, wa.y, bz); bz = fma(pa.y, wa.x, bz);
           bz = fma(-pb.x, wb.y, bz); bz = fma(-pb.y, wb.x, bz);
-          p[e] = cmake<R>(fma(s, pb.x, c * pa.x), fma(s, pb.y, c * pa.y));
-          p[f] = cmake<R>(fma(-s, pa.x, c * pb.x), fma(-s, pa.y, c * pb.y));
-          w[e] = cmake<R>(fma(s, wb.x, c * wa.x), fma(s, wb.y, c * wa.y));
-          w[f] = cmake<R>(fma(-s, wa.x, c * wb.x), fma(-s, wa.y, c * wb.y));
+          p[e] = rot_one<R, NEAR>(pa, pb, c, s, -t);
+          p[f] = rot_one<R, NEAR>(pb, pa, c, -s, -t);
+          w[e] = rot_one<R, NEAR>(wa, wb, c, s, t);
+          w[f] = rot_one<R, NEAR>(wb, wa, c, -s, t);
         }
       } else {
         const int m = 1 << (i - EB);
@@ -269,8 +323,8 @@ template <typename R, int N, int E> struct LocCol {
           bx = fma(po.x, w[e].y, bx); bx = fma(po.y, w[e].x, bx);
           by = fma(po.x, w[e].x, by); by = fma(-po.y, w[e].y, by);
           bz = fma(p[e].x, w[e].y, bz); bz = fma(p[e].y, w[e].x, bz);
-          p[e] = cmake<R>(fma(sg, po.x, c * p[e].x), fma(sg, po.y, c * p[e].y));
-          w[e] = cmake<R>(fma(sg, wo.x, c * w[e].x), fma(sg, wo.y, c * w[e].y));
+          p[e] = rot_one<R, NEAR>(p[e], po, c, sg, -t);
+          w[e] = rot_one<R, NEAR>(w[e], wo, c, sg, t);
         }
         if (!up) by = -by;
         if (up) bz = -bz;

@@ -505,7 +505,7 @@ static PropLayout prop_layout(const redo_table* t, int64_t B, int64_t M, redo_pr
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t el = L.eff_prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
   const size_t n2 = (size_t)t->N * t->N;
-  if (local_eligible(t, M, L.eff_prec, 0)) {
+  if (local_eligible(t, M, L.eff_prec, kLocalChain)) {
     L.local = true;
     L.p = reunit_every > 0 ? plan_chain_aligned(t, B, M, reunit_every) : plan_chain_local(t, B, M, L.eff_prec, false);
     if (t->N > kSmallN) {
@@ -519,7 +519,7 @@ static PropLayout prop_layout(const redo_table* t, int64_t B, int64_t M, redo_pr
       L.total = L.prod64_off + (reunit_every > 0 ? up((size_t)B * n2 * sizeof(double2)) : 0);
     }
     L.ops_off = L.total;
-    L.total += local_ops_bytes(t, B, M, L.eff_prec, 0);
+    L.total += local_ops_bytes(t, B, M, L.eff_prec, kLocalChain);
     add_strang(t, B, L.total, L.strang_off, L.strang_tmp_off);
     if (diag) add_phase(t, B, diag == 1 ? M : 1, L.total, L.pd_off, L.zf_off, L.phout_off);
     return L;
@@ -626,7 +626,7 @@ static redo_status propagate_core(const redo_table* t, const int32_t* q, const d
   if (L.local) {
     ProfScope ps(2, s);
     const LocalDiag pd{L.p.pd, phase ? M * t->N : t->N, phase ? t->N : 0};
-    if ((e = launch_local_chain(t, q, p, eff, 0, pd, (char*)workspace + L.ops_off, seg, dev_status, s)) !=
+    if ((e = launch_local_chain(t, q, p, eff, kLocalChain, pd, (char*)workspace + L.ops_off, seg, dev_status, s)) !=
         cudaSuccess)
       return cuda_error(e, "local chains");
   }
@@ -915,6 +915,7 @@ redo_status redo_batched_product(int32_t N, int64_t count, const void* A, int32_
 struct GradLayout {
   ChainPlan p;
   size_t seg_off, pck_off, rck_off, tau_off, total;
+  size_t scan_off = 0;                 // N <= 64: the grouped scan's group products
   size_t keep_off = 0;                 // N <= 64: every forward state kept (0: not kept)
   bool keep = false;
   size_t strang_off, strang_tmp_off;   // symmetric split: transformed targets (+ scratch)
@@ -924,7 +925,7 @@ struct GradLayout {
 };
 
 // Locally controlled systems: segment products, checkpoints and costates as in the dense form, then
-// the step operators and the sweep's sums.  what: 1 gradient, 2 amplitude/phase gradient.
+// the step operators and the sweep's sums.
 static bool grad_layout_local(const redo_table* t, int64_t B, int64_t M, redo_precision prec, int32_t checkpoint_every,
                               int what, GradLayout* L) {
   L->eff_prec = prec == REDO_FP64 ? REDO_FP64 : REDO_FP32;
@@ -942,7 +943,8 @@ static bool grad_layout_local(const redo_table* t, int64_t B, int64_t M, redo_pr
     L->pck_off = mats;
     L->rck_off = 2 * mats;
     L->tau_off = 3 * mats;
-    L->total = L->tau_off + up((size_t)B * sizeof(double2));
+    L->scan_off = L->tau_off + up((size_t)B * sizeof(double2));
+    L->total = L->scan_off + grad_scan_bytes(t, B, L->p.S, L->eff_prec);
   }
   L->ops_off = L->total;
   L->total += local_ops_bytes(t, B, M, L->eff_prec, what);
@@ -965,7 +967,8 @@ static redo_status grad_local(const redo_table* t, const int32_t* q, const GradL
     if (reunit && p.M > 0 &&
         (e = launch_polar(t, L.eff_prec, L.eff_prec, w + L.seg_off, w + L.seg_off, p.B * p.S, 1, s)) != cudaSuccess)
       return cuda_error(e, "segment re-unitarisation");
-    if ((e = launch_grad_scan(t, p.B, p.S, L.eff_prec, w + L.seg_off, UT, tb, P, Rc, tau, F_out, s)) != cudaSuccess)
+    if ((e = launch_grad_scan(t, p.B, p.S, L.eff_prec, w + L.seg_off, UT, tb, reunit ? 1 : 0, P, Rc, tau,
+                              F_out, w + L.scan_off, s)) != cudaSuccess)
       return cuda_error(e, "gradient checkpoints");
   }
   if (p.M > 0 && (e = launch_local_grad(t, q, p, L.eff_prec, what, pd, w + L.ops_off, P, Rc, tau, grad, gphi, nullptr,
@@ -977,7 +980,7 @@ static redo_status grad_local(const redo_table* t, const int32_t* q, const GradL
 static GradLayout grad_layout(const redo_table* t, int64_t B, int64_t M, redo_precision prec,
                               int32_t checkpoint_every) {
   GradLayout L;
-  if (grad_layout_local(t, B, M, prec, checkpoint_every, 1, &L)) {
+  if (grad_layout_local(t, B, M, prec, checkpoint_every, kLocalGrad, &L)) {
     add_strang(t, B, L.total, L.strang_off, L.strang_tmp_off);
     return L;
   }
@@ -998,7 +1001,8 @@ static GradLayout grad_layout(const redo_table* t, int64_t B, int64_t M, redo_pr
   L.pck_off = mats;
   L.rck_off = 2 * mats;
   L.tau_off = 3 * mats;
-  L.total = L.tau_off + up((size_t)B * sizeof(double2));
+  L.scan_off = L.tau_off + up((size_t)B * sizeof(double2));
+  L.total = L.scan_off + grad_scan_bytes(t, B, L.p.S, prec);
   // every forward state kept when they fit in 24 GiB: the sweep then multiplies only the
   // costates (one product per factor instead of two)
   const size_t keep_bytes = (size_t)L.p.B * L.p.S * L.p.seg_len * t->N * t->N * el;
@@ -1064,7 +1068,7 @@ redo_status redo_fidelity_grad(const redo_table* t, const int32_t* q, int64_t B,
     U_target = sb;
   }
   if (L.local)
-    return grad_local(t, q, L, 1, (const double2*)U_target, target_batched, LocalDiag{nullptr, 0, 0}, reunit_every > 0,
+    return grad_local(t, q, L, kLocalGrad, (const double2*)U_target, target_batched, LocalDiag{nullptr, 0, 0}, reunit_every > 0,
                       F_out, grad, nullptr, w, dev_status, s);
   if (t->N > kSmallN) {
     const bool reunit = reunit_every > 0;
@@ -1083,7 +1087,8 @@ redo_status redo_fidelity_grad(const redo_table* t, const int32_t* q, int64_t B,
       (e = launch_polar(t, prec, prec, w + L.seg_off, w + L.seg_off, B * L.p.S, 1, s)) != cudaSuccess)
     return cuda_error(e, "segment re-unitarisation");
   if ((e = launch_grad_scan(t, B, L.p.S, prec, w + L.seg_off, (const double2*)U_target,
-                            target_batched, w + L.pck_off, w + L.rck_off, tau, F_out, s)) !=
+                            target_batched, reunit_every > 0, w + L.pck_off, w + L.rck_off, tau, F_out,
+                            w + L.scan_off, s)) !=
       cudaSuccess)
     return cuda_error(e, "gradient checkpoints");
   if (M > 0 && (e = launch_grad_sweep(t, q, L.p, prec, w + L.pck_off, w + L.rck_off, tau, grad,
@@ -1103,7 +1108,7 @@ static PhaseGradLayout phase_grad_layout(const redo_table* t, int64_t B, int64_t
                                          int32_t checkpoint_every, bool phase = true) {
   PhaseGradLayout L;
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  if (grad_layout_local(t, B, M, prec, checkpoint_every, phase ? 2 : 1, &L.g)) {
+  if (grad_layout_local(t, B, M, prec, checkpoint_every, phase ? kLocalPhaseGrad : kLocalGrad, &L.g)) {
     L.pd_off = L.g.total;
   } else if (t->N > kSmallN) {
     // lockstep SIMT sweeps on segments of whole steps (the diagonals fall between launches)
@@ -1125,7 +1130,8 @@ static PhaseGradLayout phase_grad_layout(const redo_table* t, int64_t B, int64_t
     L.g.pck_off = mats;
     L.g.rck_off = 2 * mats;
     L.g.tau_off = 3 * mats;
-    L.pd_off = L.g.tau_off + up((size_t)B * sizeof(double2));
+    L.g.scan_off = L.g.tau_off + up((size_t)B * sizeof(double2));
+    L.pd_off = L.g.scan_off + grad_scan_bytes(t, B, L.g.p.S, prec);
   }
   // the per-pulse drift form has no final rotation, transformed target or boundary traces
   const size_t ph = phase ? 1 : 0;
@@ -1200,7 +1206,7 @@ redo_status redo_fidelity_grad_phase(const redo_table* t, const int32_t* q, cons
     return cuda_error(e, "phase target");
   L.g.p.pd = pd;
   if (L.g.local)
-    return grad_local(t, q, L.g, 2, ut, 1, LocalDiag{M > 0 ? pd : nullptr, M * t->N, t->N}, false, F_out, grad_amp,
+    return grad_local(t, q, L.g, kLocalPhaseGrad, ut, 1, LocalDiag{M > 0 ? pd : nullptr, M * t->N, t->N}, false, F_out, grad_amp,
                       grad_phase, w, dev_status, s);
   if (t->N > kSmallN) {
     if ((e = large_grad(t, q, L.g.p, prec, ut, 1, F_out, grad_amp, workspace, dev_status, s, tz, grad_phase)) !=
@@ -1211,8 +1217,8 @@ redo_status redo_fidelity_grad_phase(const redo_table* t, const int32_t* q, cons
   void* keep = L.g.keep ? w + L.g.keep_off : nullptr;
   if ((e = launch_chain_segments(t, q, L.g.p, prec, w + L.g.seg_off, dev_status, s, keep)) != cudaSuccess)
     return cuda_error(e, "gradient segments");
-  if ((e = launch_grad_scan(t, B, L.g.p.S, prec, w + L.g.seg_off, ut, 1, w + L.g.pck_off, w + L.g.rck_off, tau,
-                            F_out, s)) != cudaSuccess)
+  if ((e = launch_grad_scan(t, B, L.g.p.S, prec, w + L.g.seg_off, ut, 1, 0, w + L.g.pck_off, w + L.g.rck_off, tau,
+                            F_out, w + L.g.scan_off, s)) != cudaSuccess)
     return cuda_error(e, "gradient checkpoints");
   if (M > 0) {
     if ((e = launch_grad_sweep(t, q, L.g.p, prec, w + L.g.pck_off, w + L.g.rck_off, tau, grad_amp, dev_status, s,
@@ -1275,7 +1281,7 @@ redo_status redo_fidelity_grad_drift(const redo_table* t, const int32_t* q, cons
     return cuda_error(e, "drift diagonals");
   L.g.p.pd = pd;
   if (L.g.local)
-    return grad_local(t, q, L.g, 1, ut, target_batched, LocalDiag{M > 0 ? pd : nullptr, t->N, 0}, reunit_every > 0,
+    return grad_local(t, q, L.g, kLocalGrad, ut, target_batched, LocalDiag{M > 0 ? pd : nullptr, t->N, 0}, reunit_every > 0,
                       F_out, grad, nullptr, w, dev_status, s);
   if (t->N > kSmallN) {
     if ((e = large_grad(t, q, L.g.p, prec, ut, target_batched, F_out, grad, workspace, dev_status, s, nullptr,
@@ -1289,13 +1295,22 @@ redo_status redo_fidelity_grad_drift(const redo_table* t, const int32_t* q, cons
   if (reunit_every > 0 && M > 0 &&
       (e = launch_polar(t, prec, prec, w + L.g.seg_off, w + L.g.seg_off, B * L.g.p.S, 1, s)) != cudaSuccess)
     return cuda_error(e, "segment re-unitarisation");
-  if ((e = launch_grad_scan(t, B, L.g.p.S, prec, w + L.g.seg_off, ut, target_batched, w + L.g.pck_off,
-                            w + L.g.rck_off, tau, F_out, s)) != cudaSuccess)
+  if ((e = launch_grad_scan(t, B, L.g.p.S, prec, w + L.g.seg_off, ut, target_batched, reunit_every > 0,
+                            w + L.g.pck_off, w + L.g.rck_off, tau, F_out, w + L.g.scan_off, s)) != cudaSuccess)
     return cuda_error(e, "gradient checkpoints");
   if (M > 0 && (e = launch_grad_sweep(t, q, L.g.p, prec, w + L.g.pck_off, w + L.g.rck_off, tau, grad, dev_status,
                                       s, nullptr, keep)) != cudaSuccess)
     return cuda_error(e, "gradient sweep");
   return REDO_OK;
+}
+
+// Scratch of the state sweep: a local system's step operators, or the two state vectors of the
+// lockstep simulation (N > 64 with fewer pulses than SMs).
+static size_t sim_state_bytes(const redo_table* t, int64_t B, int64_t M, redo_precision prec, bool local) {
+  const int eff = prec == REDO_FP64 ? REDO_FP64 : REDO_FP32;
+  size_t strang = t->strang ? ((size_t)B * t->N * sizeof(double2) + 255) & ~(size_t)255 : 0;   // D_h^dag psi0
+  if (local) return local_ops_bytes(t, B, M, eff, kLocalSim) + strang;
+  return (t->N > kSmallN && B < t->num_sms ? large_sim_workspace(t, B) : 0) + strang;
 }
 
 redo_status redo_simulate_workspace(const redo_table* t, int64_t B, int64_t M,
@@ -1305,9 +1320,9 @@ redo_status redo_simulate_workspace(const redo_table* t, int64_t B, int64_t M,
   if (B < 0 || M < 0 || reunit_every < 0) return set_error(REDO_ERR_INVALID, "negative size");
   redo_status st = check_prec(t, prec);
   if (st != REDO_OK) return st;
-  // the lockstep state simulation (N > 64 with fewer pulses than SMs) needs two state vectors
-  size_t state = t->N > kSmallN && B < t->num_sms ? large_sim_workspace(t, B) : 0;
-  if (t->strang) state += ((size_t)B * t->N * sizeof(double2) + 255) & ~(size_t)255;   // D_h^dag psi0
+  const size_t state = B > 0 ? sim_state_bytes(t, B, M, prec, local_eligible(t, M, prec == REDO_FP64 ? REDO_FP64
+                                                                                             : REDO_FP32, kLocalSim))
+                             : 0;
   size_t prop = 0;
   if (want_U) {
     st = redo_propagate_workspace(t, B, M, prec, reunit_every, &prop);
@@ -1338,8 +1353,13 @@ redo_status redo_simulate(const redo_table* t, const int32_t* q, int64_t B, int6
   {
     ProfScope ps(2, s);
     cudaError_t e;
-    const bool lockstep = t->N > kSmallN && B < t->num_sms;
-    const size_t need_state = lockstep ? large_sim_workspace(t, B) : 0;
+    const int eff = prec == REDO_FP64 ? REDO_FP64 : REDO_FP32;
+    // a caller that brings only the dense sweep's scratch (none at all for N <= 64) keeps that sweep
+    const bool local = local_eligible(t, M, eff, kLocalSim) && workspace && ((uintptr_t)workspace & 255) == 0 &&
+                       workspace_bytes >= sim_state_bytes(t, B, M, prec, true);
+    const bool lockstep = !local && t->N > kSmallN && B < t->num_sms;
+    const size_t need_state =
+        sim_state_bytes(t, B, M, prec, local) - (t->strang ? ((size_t)B * t->N * sizeof(double2) + 255) & ~(size_t)255 : 0);
     if (t->strang) {
       // symmetric split with a diagonal drift and observable: the symmetric states give the
       // same expectations as the folded chain started from D_h^dag psi0
@@ -1351,7 +1371,9 @@ redo_status redo_simulate(const redo_table* t, const int32_t* q, int64_t B, int6
         return cuda_error(e, "half-drift of the initial state");
       psi0 = pw;
     }
-    if (lockstep) {
+    if (local) {
+      e = launch_local_sim(t, q, B, M, eff, (const double2*)psi0, psi0_batched, obs_diag, expect, workspace, dev_status, s);
+    } else if (lockstep) {
       // fewer pulses than SMs: every SM works on every step (one launch per factor)
       if (!workspace || workspace_bytes < need_state)
         return set_error(REDO_ERR_INVALID, "workspace of %zu bytes needed", need_state);
@@ -1373,10 +1395,14 @@ redo_status redo_simulate(const redo_table* t, const int32_t* q, int64_t B, int6
   return REDO_OK;
 }
 
+static size_t state_strang_bytes(const redo_table* t, int64_t B) {
+  return t->strang ? 2 * (((size_t)B * t->N * sizeof(double2) + 255) & ~(size_t)255) : 0;
+}
+
 redo_status redo_state_grad_workspace(const redo_table* t, int64_t B, size_t* bytes) {
   if (!t || !bytes) return set_error(REDO_ERR_INVALID, "null argument");
   if (B < 0) return set_error(REDO_ERR_INVALID, "negative B");
-  *bytes = t->strang ? 2 * (((size_t)B * t->N * sizeof(double2) + 255) & ~(size_t)255) : 0;
+  *bytes = state_strang_bytes(t, B) + local_state_bytes(t, B);
   return REDO_OK;
 }
 
@@ -1396,8 +1422,7 @@ redo_status redo_state_grad(const redo_table* t, const int32_t* q, int64_t B, in
   if (!psi0 || !psi_target) return set_error(REDO_ERR_INVALID, "null psi0 or psi_target");
   if (!F_out && !grad) return set_error(REDO_ERR_INVALID, "nothing to compute");
   if (M > 0 && !q) return set_error(REDO_ERR_INVALID, "q is NULL");
-  size_t need = 0;
-  redo_state_grad_workspace(t, B, &need);
+  const size_t need = state_strang_bytes(t, B);
   if (need && (!workspace || workspace_bytes < need))
     return set_error(REDO_ERR_INVALID, "workspace of %zu bytes needed", need);
   cudaStream_t s = (cudaStream_t)stream;
@@ -1415,6 +1440,13 @@ redo_status redo_state_grad(const redo_table* t, const int32_t* q, int64_t B, in
       return cuda_error(e, "half-drift of the states");
     p0 = w0;
     pT = wT;
+  }
+  // a caller that brings only the dense sweep's scratch keeps that sweep
+  if (t->loc && workspace && ((uintptr_t)workspace & 255) == 0 && workspace_bytes >= need + local_state_bytes(t, B)) {
+    if ((e = launch_local_state(t, q, B, M, prec, p0, pT, batched, F_out, grad, (char*)workspace + need, dev_status,
+                                s)) != cudaSuccess)
+      return cuda_error(e, "state-transfer gradient");
+    return REDO_OK;
   }
   if ((e = launch_state_grad(t, q, B, M, prec, p0, pT, batched, F_out, grad, dev_status, s)) != cudaSuccess)
     return cuda_error(e, "state-transfer gradient");

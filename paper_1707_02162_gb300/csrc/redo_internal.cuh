@@ -74,7 +74,7 @@ struct redo_table {
   double2* loc_h;             // [pairs][4] one-qubit part of the term's operator
   double2* loc_u64;           // [pairs][loc_d][loc_base][4] digit (or level) operators
   float2* loc_u32;
-  double2* loc_D64;           // [N] diagonal of the drift step
+  double2* loc_D64;           // [N] diagonal of the drift step minus 1
   cudaStream_t build_stream;
   int num_sms;
 };
@@ -172,7 +172,9 @@ struct LocalDiag {
 namespace redo {
 cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_t s);
 void local_free(redo_table* t);
-// what: 0 chains only, 1 gradient, 2 amplitude/phase gradient (its Tz sums beside)
+// What a call computes: segment products, the gradient, the amplitude/phase gradient, the state's
+// observable.
+enum LocalWhat { kLocalChain = 0, kLocalGrad = 1, kLocalPhaseGrad = 2, kLocalSim = 3 };
 bool local_eligible(const redo_table* t, int64_t M, int prec, int what);
 size_t local_ops_bytes(const redo_table* t, int64_t B, int64_t M, int prec, int what);
 ChainPlan plan_chain_local(const redo_table* t, int64_t B, int64_t M, int prec, bool two);
@@ -181,6 +183,13 @@ cudaError_t launch_local_chain(const redo_table* t, const int32_t* q, const Chai
 cudaError_t launch_local_grad(const redo_table* t, const int32_t* q, const ChainPlan& p, int prec, int what,
                               const LocalDiag& pd, void* ops, const void* Pck, const void* Rck, const double2* tau,
                               double* grad, double* gphi, int64_t* status, cudaStream_t s);
+cudaError_t launch_local_sim(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int prec, const double2* psi0,
+                             int batched, const double* obs, double* expect, void* ops, int64_t* status, cudaStream_t s);
+// State transfer; ops of local_state_bytes(t, B) (0 when the system is not local)
+size_t local_state_bytes(const redo_table* t, int64_t B);
+cudaError_t launch_local_state(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int prec,
+                               const double2* psi0, const double2* psiT, int batched, double* F_out, double* grad,
+                               void* ops, int64_t* status, cudaStream_t s);
 
 // Tensor-core chains (kernels_tc.cu), N = 64, split-FP16.
 size_t tc_planes_bytes(const redo_table* t);
@@ -211,8 +220,9 @@ cudaError_t launch_lbfgs_step(const redo_table* t, double* u, const double* g, c
 
 // GRAPE gradient (kernels_grad.cu).
 cudaError_t launch_grad_scan(const redo_table* t, int64_t B, int64_t S, int prec, const void* seg,
-                             const double2* U_target, int target_batched, void* Pck, void* Rck,
-                             double2* tau, double* F_out, cudaStream_t s);
+                             const double2* U_target, int target_batched, int reunit, void* Pck, void* Rck,
+                             double2* tau, double* F_out, void* tmp, cudaStream_t s);
+size_t grad_scan_bytes(const redo_table* t, int64_t B, int64_t S, int prec);   // tmp of launch_grad_scan
 // With p.pd set (amplitude/phase calls) the sweep also records Tz[b][n][k] = Tr(S_kz P R) at
 // every step boundary n = 0..M ([B][M+1][K]).
 cudaError_t launch_grad_sweep(const redo_table* t, const int32_t* q, const ChainPlan& p, int prec,

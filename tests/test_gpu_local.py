@@ -114,7 +114,10 @@ def test_local_batches_are_sliced_without_a_seam():
     target = torch.as_tensor(w.target, device="cuda")
     F, g = t.fidelity_grad(q, target, "fp32", checkpoint_every=100, reunit_every=100)
     F1, g1 = t.fidelity_grad(q2, target, "fp32", checkpoint_every=100, reunit_every=100)
-    assert torch.equal(g[0], g1[0]) and torch.equal(g[598], g1[0]) and torch.equal(g[599], g1[1])
+    # (two pulses scan their segments in groups, so they agree with the large batch to rounding)
+    assert torch.equal(g[0], g[598])
+    for b, i in ((0, 0), (599, 1)):
+        assert (g[b] - g1[i]).abs().max().item() <= 2e-4 * g1[i].abs().max().item()
     t.close()
 
 
@@ -130,4 +133,79 @@ def test_local_bad_level_index_counts_once_per_digit():
     q0[0, 2, 1] = q0[0, 3, 0] = 0
     U0, _, _ = t.propagate(q0, "fp64")
     assert int(st[3]) == 2 * w.digits and torch.equal(U, U0)
+    t.close()
+
+
+def _states(rng, B, N):
+    v = rng.normal(size=(B, N)) + 1j * rng.normal(size=(B, N))
+    return torch.as_tensor(v / np.linalg.norm(v, axis=1, keepdims=True), device="cuda")
+
+
+def _dense_state_sweeps(t, q, prec, psi0, psiT, obs):
+    """The dense sweeps, which a call takes when it brings no scratch for the local ones (N <= 64)."""
+    from paper_1707_02162_gb300 import redo
+    B, M = q.shape[:2]
+    e = torch.empty((B, M + 1), dtype=torch.float64, device="cuda")
+    redo.redo_simulate(t.handle, q, prec, 0, psi0, obs, e, None, None)
+    F = torch.empty(B, dtype=torch.float64, device="cuda")
+    g = torch.empty((B, M, t.K), dtype=torch.float64, device="cuda")
+    redo.redo_state_grad(t.handle, q, prec, psi0, psiT, F, g, None)
+    return e, F, g
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("controls", ["local", "global", "axes"])
+@pytest.mark.parametrize("prec,tol,gtol", [("fp64", 1e-12, 1e-10), ("fp32", 2e-5, 2e-4)])
+def test_local_state_sweeps_match_the_dense_ones(n, controls, prec, tol, gtol):
+    w = _workload(n, controls, B=37, M=19, seed=20 + n)     # 37: a ragged last warp at every n
+    t = _table(w)
+    rng = np.random.default_rng(n)
+    psi0, psiT = _states(rng, w.B, w.N), _states(rng, w.B, w.N)
+    obs = torch.as_tensor(rng.normal(size=w.N), device="cuda")
+    q = t.quantize(w.u)
+    e, _ = t.simulate(q, psi0, obs, prec, want_U=False)
+    F, g = t.state_grad(q, psi0, psiT, prec)
+    eo, Fo, go = _dense_state_sweeps(t, q, "fp64", psi0, psiT, obs)
+    scale = float(obs.abs().max())
+    assert (e - eo).abs().max().item() < tol * scale
+    assert (F - Fo).abs().max().item() < tol
+    assert (g - go).abs().max().item() <= gtol * go.abs().max().item()
+    t.close()
+
+
+@pytest.mark.parametrize("n,M", [(7, 6), (9, 4), (10, 3)])
+@pytest.mark.parametrize("prec,tol,gtol", [("fp64", 1e-12, 1e-10), ("fp32", 2e-5, 2e-4)])
+def test_local_state_sweeps_large(n, M, prec, tol, gtol):
+    w = _workload(n, "global", B=2, M=M, seed=30 + n, base=4, digits=2)
+    t = _table(w)
+    rng = np.random.default_rng(n)
+    psi0, psiT = _states(rng, w.B, w.N), _states(rng, w.B, w.N)
+    obs = torch.as_tensor(rng.normal(size=w.N), device="cuda")
+    q = t.quantize(w.u)
+    e, _ = t.simulate(q, psi0, obs, prec, want_U=False)
+    F, g = t.state_grad(q, psi0, psiT, prec)
+    U, _, _ = t.propagate(q, "fp64")
+    psi = torch.einsum("bij,bj->bi", U, psi0)
+    assert (e[:, -1] - (psi.abs() ** 2) @ obs).abs().max().item() < tol * float(obs.abs().max())
+    a = (psiT.conj() * psi).sum(1)
+    assert (F - a.abs() ** 2).abs().max().item() < tol
+    from paper_1707_02162_gb300 import redo
+    go = torch.empty_like(g)
+    redo.redo_state_grad(t.handle, q, "fp64", psi0, psiT, None, go, None)      # the dense streamed sweep
+    assert (g - go).abs().max().item() <= gtol * go.abs().max().item()
+    t.close()
+
+
+def test_local_state_gradient_over_several_windows():
+    # 9001 steps: three windows of step operators, visited forward and then back
+    w = _workload(2, "axes", B=3, M=9001, seed=40, dt=1e-3)
+    t = _table(w)
+    rng = np.random.default_rng(40)
+    psi0, psiT = _states(rng, w.B, w.N), _states(rng, w.B, w.N)
+    q = t.quantize(w.u)
+    F, g = t.state_grad(q, psi0, psiT, "fp64")
+    F1, _ = t.state_grad(q, psi0, psiT, "fp64", want_grad=False)
+    _, Fo, go = _dense_state_sweeps(t, q, "fp64", psi0, psiT, torch.ones(w.N, dtype=torch.float64, device="cuda"))
+    assert (F - Fo).abs().max().item() < 1e-10 and torch.equal(F, F1)
+    assert (g - go).abs().max().item() <= 1e-8 * go.abs().max().item()
     t.close()

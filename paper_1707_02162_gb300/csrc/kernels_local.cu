@@ -113,6 +113,16 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
     }
   ptr[n] = (int32_t)kk.size();
   const int pairs = (int)kk.size();
+  std::vector<int32_t> kptr(K + 1, 0), kpair;
+  for (int k = 0; k < K; ++k) {
+    kptr[k] = (int32_t)kpair.size();
+    for (int i = 0; i < n; ++i)
+      for (int p = ptr[i]; p < ptr[i + 1]; ++p)
+        if ((kk[p] & ~kLocFirst) == k) kpair.push_back(p | (i << 20));
+  }
+  kptr[K] = (int32_t)kpair.size();
+  std::vector<float2> hp32(hp.size());
+  for (size_t i = 0; i < hp.size(); ++i) hp32[i] = make_float2((float)hp[i].x, (float)hp[i].y);
   // one operator per level (no digit products per step) while the table stays small beside L2
   const bool levels = t->levels <= 65536 && (double)pairs * t->levels * 96.0 <= 64e6;
   t->loc_d = levels ? 1 : t->digit_count;
@@ -129,12 +139,16 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
   if ((e = cudaMalloc(&t->loc_ptr, sizeof(int32_t) * (n + 1))) || (e = cudaMalloc(&t->loc_k, sizeof(int32_t) * pairs)) ||
       (e = cudaMalloc(&t->loc_h, sizeof(double2) * 4 * pairs)) ||
       (e = cudaMalloc(&t->loc_u64, sizeof(double2) * 4 * ent)) || (e = cudaMalloc(&t->loc_u32, sizeof(float2) * 4 * ent)) ||
-      (e = cudaMalloc(&t->loc_D64, sizeof(double2) * N)))
+      (e = cudaMalloc(&t->loc_D64, sizeof(double2) * N)) || (e = cudaMalloc(&t->loc_h32, sizeof(float2) * 4 * pairs)) ||
+      (e = cudaMalloc(&t->loc_kptr, sizeof(int32_t) * (K + 1))) || (e = cudaMalloc(&t->loc_kpair, sizeof(int32_t) * pairs)))
     return e;
   if ((e = cudaMemcpyAsync(t->loc_ptr, ptr.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(t->loc_k, kk.data(), sizeof(int32_t) * pairs, cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(t->loc_h, hp.data(), sizeof(double2) * 4 * pairs, cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemcpyAsync(t->loc_D64, D.data(), sizeof(double2) * N, cudaMemcpyHostToDevice, s)))
+      (e = cudaMemcpyAsync(t->loc_D64, D.data(), sizeof(double2) * N, cudaMemcpyHostToDevice, s)) ||
+      (e = cudaMemcpyAsync(t->loc_h32, hp32.data(), sizeof(float2) * 4 * pairs, cudaMemcpyHostToDevice, s)) ||
+      (e = cudaMemcpyAsync(t->loc_kptr, kptr.data(), sizeof(int32_t) * (K + 1), cudaMemcpyHostToDevice, s)) ||
+      (e = cudaMemcpyAsync(t->loc_kpair, kpair.data(), sizeof(int32_t) * kpair.size(), cudaMemcpyHostToDevice, s)))
     return e;
   loc_table_kernel<<<(unsigned)((ent + 127) / 128 < 4096 ? (ent + 127) / 128 : 4096), 128, 0, s>>>(
       t->loc_h, t->loc_k, pairs, t->loc_d, t->loc_base, t->dt, t->d_lo, t->d_delta, t->loc_u64, t->loc_u32);
@@ -150,6 +164,9 @@ void local_free(redo_table* t) {
   cudaFree(t->loc_u64);
   cudaFree(t->loc_u32);
   cudaFree(t->loc_D64);
+  cudaFree(t->loc_h32);
+  cudaFree(t->loc_kptr);
+  cudaFree(t->loc_kpair);
 }
 
 template <typename R> static LocTab<R> loc_tab(const redo_table* t, int64_t* status) {
@@ -171,7 +188,12 @@ template <typename R> static LocTab<R> loc_tab(const redo_table* t, int64_t* sta
 // Delta[b][n - m0][N], n - m0 <= T (Delta_M closes the chain; a window that ends earlier also gets
 // the next step's)
 // ============================================================================
-constexpr int kPrepSteps = 8, kPrepThreads = 256;
+// A block takes ts steps: the one-qubit work (a long dependent chain per step and qubit) needs many
+// steps in a block to fill its warps, few pulses need many blocks (loc_steps_t).  g (gradients):
+// also the step's derivative operators, for every pair (term k, qubit i) the real (gx, gy, gz) of
+//     W h_ki W^dag,  W the product of the factors after k on qubit i,
+// turned by the trailing phases (the sweep's Bloch sums are taken before those), [step][pair][3].
+constexpr int kPrepSteps = 32, kPrepThreads = 256;
 
 template <typename R> __device__ __forceinline__ phase_t<R> no_phase() {
   if constexpr (sizeof(R) == 4) return 0;
@@ -190,29 +212,56 @@ template <typename R> __device__ __forceinline__ cplx<R> loc_times(cplx<R> v, do
   return o;
 }
 
+template <typename R>
+__device__ __forceinline__ void loc_derivatives(const LocTab<R>& tab, const int32_t* qrow, int i, const Euler<R>& f,
+                                                const cplx<R>* __restrict__ h, R* __restrict__ g) {
+  cplx<R> x;                                         // conj(x0) x1
+  if constexpr (sizeof(R) == 4)
+    x = phasor<false>((int32_t)((uint32_t)f.x - (uint32_t)f.x0));
+  else
+    x = f.x;
+  Mat2<R> w;
+  w.a = w.e = cmake<R>(R(1), R(0));
+  w.b = w.c = cmake<R>(R(0), R(0));
+  const int p0 = tab.ptr[i];
+  for (int p = tab.ptr[i + 1] - 1; p >= p0; --p) {
+    const Mat2<R> hm = {h[4 * p], h[4 * p + 1], h[4 * p + 2], h[4 * p + 3]};
+    const Mat2<R> wd = {cmake<R>(w.a.x, -w.a.y), cmake<R>(w.c.x, -w.c.y), cmake<R>(w.b.x, -w.b.y),
+                        cmake<R>(w.e.x, -w.e.y)};
+    const Mat2<R> gm = mat2_mul<R>(mat2_mul<R>(w, hm), wd);
+    const cplx<R> g01 = cmul<R>(gm.b, x);
+    g[3 * p] = g01.x;
+    g[3 * p + 1] = -g01.y;
+    g[3 * p + 2] = R(0.5) * (gm.a.x - gm.e.x);
+    if (p > p0) w = mat2_mul<R>(w, loc_term<R>(tab, p, loc_level<R>(tab, qrow, tab.k[p], false)));
+  }
+}
+
 template <typename R, bool NEAR>
 __global__ void __launch_bounds__(kPrepThreads)
 loc_steps_kernel(LocTab<R> tab, const int32_t* __restrict__ q, int64_t M, int64_t m0, int64_t T, int n, int N, int E,
-                 int64_t tiles,
+                 int64_t tiles, int ts,
                  const double2* __restrict__ D, const double2* __restrict__ pd, int64_t pd_b, int64_t pd_n,
-                 cplx<R>* __restrict__ cs, cplx<R>* __restrict__ delta) {
+                 cplx<R>* __restrict__ cs, cplx<R>* __restrict__ delta, const cplx<R>* __restrict__ h, int pairs,
+                 R* __restrict__ gout) {
   // phases of every (step, qubit); row j is step n0 - 1 + j (the step before the tile gives its x)
   __shared__ phase_t<R> y0[kPrepSteps + 1][10], y1[kPrepSteps + 1][10], xx[kPrepSteps + 1][10],
       x0[kPrepSteps + 1][10];
   const int64_t b = blockIdx.x / tiles;
-  const int64_t n0 = m0 + (blockIdx.x - b * tiles) * kPrepSteps;
-  for (int idx = threadIdx.x; idx < (kPrepSteps + 1) * n; idx += kPrepThreads) {
+  const int64_t n0 = m0 + (blockIdx.x - b * tiles) * ts;
+  for (int idx = threadIdx.x; idx < (ts + 1) * n; idx += kPrepThreads) {
     const int j = idx / n, i = idx - j * n;
     const int64_t m = n0 - 1 + j;
     Euler<R> f;
     f.y0 = f.y1 = f.x = f.x0 = no_phase<R>();
-    if (m >= 0 && m < M) {
+    if (m >= 0 && m < M && m <= m0 + T) {
       const bool own = j > 0 && m < m0 + T;
       f = loc_factor<R, NEAR>(loc_step<R>(tab, q + (b * M + m) * tab.K, i, own));
       if (own) {
         cplx<R>* o = cs + (b * T + m - m0) * n * (NEAR ? 2 : 1) + i;
         o[0] = cmake<R>(f.c1, f.s);
         if (NEAR) o[n] = cmake<R>(f.sy, R(0));
+        if (gout) loc_derivatives<R>(tab, q + (b * M + m) * tab.K, i, f, h, gout + (b * T + m - m0) * pairs * 3);
       }
     }
     y0[j][i] = f.y0;
@@ -222,7 +271,7 @@ loc_steps_kernel(LocTab<R> tab, const int32_t* __restrict__ q, int64_t M, int64_
   }
   __syncthreads();
   const int G = N / E;
-  for (int idx = threadIdx.x; idx < kPrepSteps * N; idx += kPrepThreads) {
+  for (int idx = threadIdx.x; idx < ts * N; idx += kPrepThreads) {
     const int j = idx / N + 1, r = idx & (N - 1);
     const int64_t m = n0 - 1 + j;
     if (m > m0 + T) continue;
@@ -347,7 +396,7 @@ template <typename R, int N, int E, bool TZ>
 __global__ void __launch_bounds__(kLocThreads, E * sizeof(R) <= 64 ? 4 : 2)
 loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t M, int64_t S, int64_t sps,
                  int64_t chains, const cplx<R>* __restrict__ Pck, const cplx<R>* __restrict__ Rck,
-                 const double2* __restrict__ tau, R* __restrict__ bl, int K, const double* __restrict__ sz,
+                 const double2* __restrict__ tau, R* __restrict__ bl, int K, const R* __restrict__ sz,
                  R* __restrict__ bz) {
   using L = LocCol<R, N, E>;
   using WS = WarpSums<R, 3 * L::NQ>;
@@ -382,7 +431,7 @@ loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
       for (int k = 0; k < K; ++k) {
         R a = R(0);
 #pragma unroll
-        for (int e = 0; e < E; ++e) a = fma((R)sz[(int64_t)k * N + l * E + e], t[e], a);
+        for (int e = 0; e < E; ++e) a = fma(__ldg(sz + (int64_t)k * N + l * E + e), t[e], a);
 #pragma unroll
         for (int off = W / 2; off >= 1; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
         if (act && lane % W == 0) bz[((b * (M + 1) + n) * PARTS + part) * K + k] = a;
@@ -424,71 +473,50 @@ loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
   }
 }
 
-// dF/du_kn = (2 dt / N^2) sum_i Tr(g_ki rho_i) with g_ki = W h_ki W^dag, W the product of the
-// factors after k on qubit i, conjugated by the step's trailing phases diag(x0_i, x1_i) (the sums are
-// taken between the rotation and those): Re(g01 conj(x0) x1 (X + iY)) + gz Z.
-constexpr int kFinSteps = 8, kFinThreads = 128;
-
-template <typename R, bool NEAR>
-__global__ void __launch_bounds__(kFinThreads)
-loc_grad_kernel(LocTab<R> tab, const double2* __restrict__ h, const int32_t* __restrict__ q, int64_t M, int64_t w0,
-                int64_t T, int n, int parts, int64_t tiles, const R* __restrict__ bl, double scale, double* __restrict__ grad) {
-  __shared__ double sum[kFinSteps][30];
-  __shared__ double2 xy[kFinSteps][10];
-  const int64_t b = blockIdx.x / tiles, j0 = (blockIdx.x - b * tiles) * kFinSteps, m0 = w0 + j0;
-  const int steps = (int)(T - j0 < kFinSteps ? T - j0 : kFinSteps);
-  for (int idx = threadIdx.x; idx < steps * 3 * n; idx += kFinThreads) {
-    const int j = idx / (3 * n), v = idx - j * 3 * n;
-    const R* o = bl + (b * T + j0 + j) * parts * (3 * n) + v;
-    double a = 0.0;
-    for (int p = 0; p < parts; ++p) a += (double)o[(int64_t)p * 3 * n];
-    sum[j][v] = a;
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < steps * n; idx += kFinThreads) {
-    const int j = idx / n, i = idx - j * n;
-    const Euler<R> f = loc_factor<R, NEAR>(loc_step<R>(tab, q + (b * M + m0 + j) * tab.K, i, false));
-    double2 xv;                                      // conj(x0) x1
-    if constexpr (sizeof(R) == 4) {
-      const float2 x = phasor<false>((int32_t)((uint32_t)f.x - (uint32_t)f.x0));
-      xv = make_double2(x.x, x.y);
-    } else {
-      xv = f.x;
-    }
-    const double X = sum[j][3 * i], Y = sum[j][3 * i + 1];
-    xy[j][i] = make_double2(xv.x * X - xv.y * Y, xv.x * Y + xv.y * X);
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < steps * tab.K; idx += kFinThreads) {
-    const int j = idx / tab.K, k = idx - j * tab.K;
-    const int32_t* qrow = q + (b * M + m0 + j) * tab.K;
+// dF/du_kn = (2 dt / N^2) sum_i (gx X_i + gy Y_i + gz Z_i), a thread per (step, term): its pairs are
+// kpair[kptr[k] ..] (pair | qubit << 20), the Bloch sums bl [step][part][3n] or, already added, sums.
+template <typename R>
+__global__ void loc_grad_kernel(int64_t steps, int K, int n, int pairs, int parts, const int32_t* __restrict__ kptr,
+                                const int32_t* __restrict__ kpair, const R* __restrict__ g, const R* __restrict__ bl,
+                                const double* __restrict__ sums, int64_t M, int64_t w0, int64_t T, double scale,
+                                double* __restrict__ grad) {
+  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < steps * K;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t st = idx / K, b = st / T;
+    const int k = (int)(idx - st * K);
     double acc = 0.0;
-    for (int i = 0; i < n; ++i) {
-      Mat2<R> w;
-      w.a = w.e = cmake<R>(R(1), R(0));
-      w.b = w.c = cmake<R>(R(0), R(0));
-      for (int p = tab.ptr[i + 1] - 1; p >= tab.ptr[i]; --p) {
-        const int kf = tab.k[p];
-        if ((kf & ~kLocFirst) != k) {
-          w = mat2_mul<R>(w, loc_term<R>(tab, p, loc_level<R>(tab, qrow, kf, false)));
-          continue;
+    for (int e = kptr[k]; e < kptr[k + 1]; ++e) {
+      const int p = kpair[e] & 0xfffff, i = kpair[e] >> 20;
+      const R* gp = g + (st * pairs + p) * 3;
+      for (int c = 0; c < 3; ++c) {
+        double v = 0.0;
+        if (sums) {
+          v = sums[st * 3 * n + 3 * i + c];
+        } else {
+          for (int q = 0; q < parts; ++q) v += (double)bl[(st * parts + q) * 3 * n + 3 * i + c];
         }
-        Mat2<R> hm, wd;
-        hm.a = cmake<R>((R)h[4 * p].x, (R)h[4 * p].y);
-        hm.b = cmake<R>((R)h[4 * p + 1].x, (R)h[4 * p + 1].y);
-        hm.c = cmake<R>((R)h[4 * p + 2].x, (R)h[4 * p + 2].y);
-        hm.e = cmake<R>((R)h[4 * p + 3].x, (R)h[4 * p + 3].y);
-        wd.a = cmake<R>(w.a.x, -w.a.y);
-        wd.b = cmake<R>(w.c.x, -w.c.y);
-        wd.c = cmake<R>(w.b.x, -w.b.y);
-        wd.e = cmake<R>(w.e.x, -w.e.y);
-        const Mat2<R> gm = mat2_mul<R>(mat2_mul<R>(w, hm), wd);
-        acc += (double)gm.b.x * xy[j][i].x - (double)gm.b.y * xy[j][i].y +
-               0.5 * ((double)gm.a.x - (double)gm.e.x) * sum[j][3 * i + 2];
-        break;
+        acc += (double)gp[c] * v;
       }
     }
-    grad[(b * M + m0 + j) * tab.K + k] = scale * acc;
+    grad[(b * M + w0 + st - b * T) * K + k] = scale * acc;
+  }
+}
+
+// Bloch sums over many parts, one block per step
+template <typename R>
+__global__ void __launch_bounds__(256) loc_sums_kernel(const R* __restrict__ bl, int parts, int nv,
+                                                       double* __restrict__ sums) {
+  __shared__ double s[8][32];
+  const int v = threadIdx.x & 31, sl = threadIdx.x >> 5;
+  const R* o = bl + (int64_t)blockIdx.x * parts * nv + v;
+  double a = 0.0;
+  if (v < nv)
+    for (int p = sl; p < parts; p += 8) a += (double)o[(int64_t)p * nv];
+  s[sl][v] = a;
+  __syncthreads();
+  if (sl == 0 && v < nv) {
+    for (int i = 1; i < 8; ++i) a += s[i][v];
+    sums[(int64_t)blockIdx.x * nv + v] = a;
   }
 }
 
@@ -522,7 +550,8 @@ static cudaError_t loc_sweep_n(const redo_table* t, const ChainPlan& p, int64_t 
   auto kern = bz ? loc_sweep_kernel<R, N, E, true> : loc_sweep_kernel<R, N, E, false>;
   kern<<<(unsigned)((warps + 3) / 4), kLocThreads, 0, s>>>(
       (const cplx<R>*)cs, (const cplx<R>*)delta, p.M, p.S, sps, chains, (const cplx<R>*)Pck, (const cplx<R>*)Rck, tau,
-      (R*)bl, t->K, t->sz64, (R*)bz);
+      (R*)bl, t->K,
+      sizeof(R) == 8 ? (const R*)t->sz64 : (const R*)t->sz32, (R*)bz);
   return cudaGetLastError();
   }
 }
@@ -763,9 +792,11 @@ static int loc_parts(const redo_table* t, bool dbl) {
 // Scratch of nb pulses: diagonals and rotations, then by what is computed (LocalWhat) the Bloch
 // sums, the boundary traces or the lanes' parts of the observable.
 struct LocScratch {
-  void *delta, *cs, *bl, *bz;
+  void *delta, *cs, *bl, *bz, *g;
+  double* sums;
   size_t total;
 };
+constexpr size_t kLocSumParts = 8;                   // from here on the parts are added by a kernel of their own
 static LocScratch loc_scratch(const redo_table* t, int64_t nb, int64_t M, int prec, int what, void* base) {
   const size_t el = prec == REDO_FP64 ? sizeof(double) : sizeof(float);
   const bool grad = what == kLocalGrad || what == kLocalPhaseGrad;
@@ -783,6 +814,8 @@ static LocScratch loc_scratch(const redo_table* t, int64_t nb, int64_t M, int pr
   w.cs = take((size_t)nb * M * t->loc * 2 * el * (loc_near(prec == REDO_FP64, t->N) ? 2 : 1));
   w.bl = take(grad ? (size_t)nb * M * parts * 3 * t->loc * el : (size_t)nb * (M + 1) * lanes * 2 * el);
   w.bz = take(what == kLocalPhaseGrad ? (size_t)nb * (M + 1) * parts * t->K * el : 0);
+  w.g = grad ? take((size_t)nb * M * t->loc_pairs * 3 * el) : nullptr;
+  w.sums = grad && parts >= kLocSumParts ? (double*)take((size_t)nb * M * 3 * t->loc * sizeof(double)) : nullptr;
   w.total = off;
   return w;
 }
@@ -819,23 +852,24 @@ ChainPlan plan_chain_local(const redo_table* t, int64_t B, int64_t M, int prec, 
 
 template <typename R>
 static cudaError_t loc_steps_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int64_t m0, int64_t T, int E,
-                               const LocalDiag& pd, int64_t b0, void* cs, void* delta, int64_t* status,
+                               const LocalDiag& pd, int64_t b0, const LocScratch& w, int64_t* status,
                                cudaStream_t s) {
-  const int64_t tiles = (T + 1 + kPrepSteps - 1) / kPrepSteps;
+  const int ts = B * (T + 1) >= (int64_t)t->num_sms * 8 * kPrepSteps ? kPrepSteps : 8;
+  const int64_t tiles = (T + 1 + ts - 1) / ts;
   auto kern = loc_steps_kernel<R, false>;
   if constexpr (sizeof(R) == 4)
     if (loc_near(false, t->N)) kern = loc_steps_kernel<R, true>;
   kern<<<(unsigned)(B * tiles), kPrepThreads, 0, s>>>(
-      loc_tab<R>(t, status), q + b0 * M * t->K, M, m0, T, t->loc, t->N, E, tiles,
-      t->loc_D64,
-      pd.p ? pd.p + b0 * pd.sb : nullptr, pd.sb, pd.sn, (cplx<R>*)cs, (cplx<R>*)delta);
+      loc_tab<R>(t, status), q + b0 * M * t->K, M, m0, T, t->loc, t->N, E, tiles, ts, t->loc_D64,
+      pd.p ? pd.p + b0 * pd.sb : nullptr, pd.sb, pd.sn, (cplx<R>*)w.cs,
+      (cplx<R>*)w.delta, sizeof(R) == 8 ? (const cplx<R>*)t->loc_h : (const cplx<R>*)t->loc_h32, t->loc_pairs, (R*)w.g);
   return cudaGetLastError();
 }
 
 static cudaError_t loc_steps(const redo_table* t, const int32_t* q, int64_t nb, int64_t M, int prec, int E,
                              const LocalDiag& pd, int64_t b0, const LocScratch& w, int64_t* status, cudaStream_t s) {
-  return prec == REDO_FP64 ? loc_steps_t<double>(t, q, nb, M, 0, M, E, pd, b0, w.cs, w.delta, status, s)
-                           : loc_steps_t<float>(t, q, nb, M, 0, M, E, pd, b0, w.cs, w.delta, status, s);
+  return prec == REDO_FP64 ? loc_steps_t<double>(t, q, nb, M, 0, M, E, pd, b0, w, status, s)
+                           : loc_steps_t<float>(t, q, nb, M, 0, M, E, pd, b0, w, status, s);
 }
 
 cudaError_t launch_local_chain(const redo_table* t, const int32_t* q, const ChainPlan& p, int prec, int what,
@@ -860,16 +894,14 @@ cudaError_t launch_local_chain(const redo_table* t, const int32_t* q, const Chai
 }
 
 template <typename R>
-static cudaError_t loc_finish_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int64_t m0, int64_t T,
-                                int parts, double norm, const LocScratch& w, double* grad, double* gphi,
-                                cudaStream_t s) {
-  const int64_t tiles = (T + kFinSteps - 1) / kFinSteps;
-  LocTab<R> tab = loc_tab<R>(t, nullptr);
-  auto kern = loc_grad_kernel<R, false>;
-  if constexpr (sizeof(R) == 4)
-    if (loc_near(false, t->N)) kern = loc_grad_kernel<R, true>;
-  kern<<<(unsigned)(B * tiles), kFinThreads, 0, s>>>(tab, t->loc_h, q, M, m0, T, t->loc, parts, tiles,
-                                                                   (const R*)w.bl, 2.0 * t->dt / norm, grad);
+static cudaError_t loc_finish_t(const redo_table* t, int64_t B, int64_t M, int64_t m0, int64_t T, int parts, double norm,
+                                const LocScratch& w, double* grad, double* gphi, cudaStream_t s) {
+  const int64_t steps = B * T, gn = steps * t->K, gb = (gn + 127) / 128;
+  if (w.sums)
+    loc_sums_kernel<R><<<(unsigned)steps, 256, 0, s>>>((const R*)w.bl, parts, 3 * t->loc, w.sums);
+  loc_grad_kernel<R><<<(unsigned)(gb < 16384 ? gb : 16384), 128, 0, s>>>(
+      steps, t->K, t->loc, t->loc_pairs, parts, t->loc_kptr, t->loc_kpair, (const R*)w.g, (const R*)w.bl, w.sums, M, m0,
+      T, 2.0 * t->dt / norm, grad);
   if (gphi) {
     const int64_t n = B * M * t->K, blocks = (n + 255) / 256;
     loc_phase_kernel<R><<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>((const R*)w.bz, B, M, parts, t->K,
@@ -901,8 +933,8 @@ cudaError_t launch_local_grad(const redo_table* t, const int32_t* q, const Chain
     if (e) return e;
     const int64_t at = b0 * p.M * t->K;
     double* gp = gphi ? gphi + at : nullptr;
-    e = dbl ? loc_finish_t<double>(t, q + at, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, s)
-            : loc_finish_t<float>(t, q + at, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, s);
+    e = dbl ? loc_finish_t<double>(t, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, s)
+            : loc_finish_t<float>(t, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, s);
     if (e) return e;
   }
   return cudaSuccess;
@@ -958,7 +990,7 @@ struct LocStatePlan {
   int64_t pulses, steps;
 };
 static size_t loc_state_step(const redo_table* t) {              // FP64 bytes of one step of one pulse
-  return ((size_t)t->N + 3 * t->loc) * sizeof(double2);
+  return ((size_t)t->N + 3 * t->loc) * sizeof(double2) + 3 * t->loc_pairs * sizeof(double);
 }
 static LocStatePlan loc_state_plan(const redo_table* t, int64_t B) {
   const size_t per = loc_state_step(t);
@@ -983,6 +1015,9 @@ static LocScratch loc_state_scratch(const redo_table* t, const LocStatePlan& p, 
   c += up256(nb * T * 3 * t->loc * sizeof(double));
   w.bz = c;
   c += up256(nb * 2 * t->N * sizeof(double2));
+  w.g = c;
+  c += up256(nb * T * 3 * t->loc_pairs * sizeof(double));
+  w.sums = nullptr;
   w.total = (size_t)(c - (char*)base);
   return w;
 }
@@ -999,17 +1034,19 @@ static cudaError_t loc_state_t(const redo_table* t, const int32_t* q, int64_t B,
   const unsigned blocks = (unsigned)((B + cols - 1) / cols);
   const int64_t nw = M > 0 ? (M + win - 1) / win : 1;
   const bool back = grad && M > 0;
+  LocScratch fo = w;                                 // forward only: no derivative operators
+  fo.g = nullptr;
   // windows 0 .. nw - 1 forward, the last one also back, then nw - 2 .. 0 back
   for (int64_t i = 0; i < (back ? 2 * nw - 1 : nw); ++i) {
     const bool fwd = i < nw;
     const int64_t k = fwd ? i : 2 * nw - 2 - i, m0 = k * win, T = m0 + win < M ? win : M - m0;
     const int bk = back && i >= nw - 1;
-    cudaError_t e = loc_steps_t<R>(t, q, B, M, m0, T, loc_vec_entries(t->N), LocalDiag{nullptr, 0, 0}, 0, w.cs,
-                                   w.delta, fwd ? status : nullptr, s);
+    cudaError_t e = loc_steps_t<R>(t, q, B, M, m0, T, loc_vec_entries(t->N), LocalDiag{nullptr, 0, 0}, 0,
+                                   bk ? w : fo, fwd ? status : nullptr, s);
     if (e) return e;
     LOC_VEC(loc_state_kernel, (const cplx<R>*)w.cs, (const cplx<R>*)w.delta, B, M, m0, T, fwd, bk, psi0, psiT, batched,
             F_out, (R*)w.bl, (cplx<R>*)w.bz)
-    if (bk && (e = loc_finish_t<R>(t, q, B, M, m0, T, 1, 1.0, w, grad, nullptr, s))) return e;
+    if (bk && (e = loc_finish_t<R>(t, B, M, m0, T, 1, 1.0, w, grad, nullptr, s))) return e;
   }
   return cudaGetLastError();
 }

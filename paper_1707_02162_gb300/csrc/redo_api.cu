@@ -376,6 +376,7 @@ redo_status redo_table_free(redo_table* t) {
   cudaFree(t->hk_xmask);
   cudaFree(t->hk_xval);
   cudaFree(t->sz64);
+  cudaFree(t->sz32);
   local_free(t);
   std::free(t->h0_pairs);
   std::free(t);
@@ -402,6 +403,15 @@ redo_status redo_table_set_phase_axes(redo_table* t, const double* sz) {
       return set_error(REDO_ERR_OOM, "phase axes: %s", cudaGetErrorString(e));
     }
   }
+  if (!t->sz32) {
+    cudaError_t e = cudaMalloc(&t->sz32, sizeof(float) * K * N);
+    if (e != cudaSuccess) {
+      t->sz32 = nullptr;
+      return set_error(REDO_ERR_OOM, "phase axes: %s", cudaGetErrorString(e));
+    }
+  }
+  std::vector<float> f(sz, sz + (size_t)K * N);
+  REDO_CUDA_TRY(cudaMemcpy(t->sz32, f.data(), sizeof(float) * K * N, cudaMemcpyHostToDevice));
   REDO_CUDA_TRY(cudaMemcpy(t->sz64, sz, sizeof(double) * K * N, cudaMemcpyHostToDevice));
   return REDO_OK;
 }

@@ -62,6 +62,7 @@ struct redo_table {
   void* tc_planes;            // tensor-core planes or nullptr
   size_t tc_bytes;
   int tc_nb;                  // operand block height of the large-N planes (128 or 256)
+  float* sz32;                // sz64 in FP32
   double* sz64;               // [K][N] diagonals of the species' S_kz (amplitude/phase calls), or nullptr
   int32_t* h0_pairs;          // host: (row, column) of every off-diagonal nonzero of H0
   int64_t h0_npairs;
@@ -72,6 +73,9 @@ struct redo_table {
   int32_t* loc_ptr;           // [loc + 1] (term, qubit) pairs of each qubit
   int32_t* loc_k;             // [pairs] term, flagged at the first pair of a term
   double2* loc_h;             // [pairs][4] one-qubit part of the term's operator
+  float2* loc_h32;
+  int32_t* loc_kptr;          // [K + 1] and
+  int32_t* loc_kpair;         // [pairs]: the pairs of each term (pair | qubit << 20)
   double2* loc_u64;           // [pairs][loc_d][loc_base][4] digit (or level) operators
   float2* loc_u32;
   double2* loc_D64;           // [N] diagonal of the drift step minus 1

@@ -121,6 +121,11 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
         if ((kk[p] & ~kLocFirst) == k) kpair.push_back(p | (i << 20));
   }
   kptr[K] = (int32_t)kpair.size();
+  std::vector<float4> D32(N);
+  for (int r = 0; r < N; ++r) {
+    const double a = t->dt * h[2 * ((size_t)r * N + r)], sh = std::sin(0.5 * a), x = -2.0 * sh * sh, y = -std::sin(a);
+    D32[r] = make_float4((float)x, (float)y, (float)(x - (double)(float)x), (float)(y - (double)(float)y));
+  }
   std::vector<float2> hp32(hp.size());
   for (size_t i = 0; i < hp.size(); ++i) hp32[i] = make_float2((float)hp[i].x, (float)hp[i].y);
   // one operator per level (no digit products per step) while the table stays small beside L2
@@ -140,12 +145,14 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
       (e = cudaMalloc(&t->loc_h, sizeof(double2) * 4 * pairs)) ||
       (e = cudaMalloc(&t->loc_u64, sizeof(double2) * 4 * ent)) || (e = cudaMalloc(&t->loc_u32, sizeof(float2) * 4 * ent)) ||
       (e = cudaMalloc(&t->loc_D64, sizeof(double2) * N)) || (e = cudaMalloc(&t->loc_h32, sizeof(float2) * 4 * pairs)) ||
+      (e = cudaMalloc(&t->loc_D32, sizeof(float4) * N)) ||
       (e = cudaMalloc(&t->loc_kptr, sizeof(int32_t) * (K + 1))) || (e = cudaMalloc(&t->loc_kpair, sizeof(int32_t) * pairs)))
     return e;
   if ((e = cudaMemcpyAsync(t->loc_ptr, ptr.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(t->loc_k, kk.data(), sizeof(int32_t) * pairs, cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(t->loc_h, hp.data(), sizeof(double2) * 4 * pairs, cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(t->loc_D64, D.data(), sizeof(double2) * N, cudaMemcpyHostToDevice, s)) ||
+      (e = cudaMemcpyAsync(t->loc_D32, D32.data(), sizeof(float4) * N, cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(t->loc_h32, hp32.data(), sizeof(float2) * 4 * pairs, cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(t->loc_kptr, kptr.data(), sizeof(int32_t) * (K + 1), cudaMemcpyHostToDevice, s)) ||
       (e = cudaMemcpyAsync(t->loc_kpair, kpair.data(), sizeof(int32_t) * kpair.size(), cudaMemcpyHostToDevice, s)))
@@ -165,6 +172,7 @@ void local_free(redo_table* t) {
   cudaFree(t->loc_u32);
   cudaFree(t->loc_D64);
   cudaFree(t->loc_h32);
+  cudaFree(t->loc_D32);
   cudaFree(t->loc_kptr);
   cudaFree(t->loc_kpair);
 }
@@ -200,15 +208,30 @@ template <typename R> __device__ __forceinline__ phase_t<R> no_phase() {
   else return cmake<R>(R(1), R(0));
 }
 
-// (1 + v)(1 + d) - 1, d in FP64 (FP32: hi + lo)
-template <typename R> __device__ __forceinline__ cplx<R> loc_times(cplx<R> v, double2 d) {
-  const cplx<R> hi = cmake<R>((R)d.x, (R)d.y);
-  cplx<R> o = cmake<R>(v.x + hi.x, v.y + hi.y);
-  if constexpr (sizeof(R) == 4) {
-    o.x += (R)(d.x - (double)hi.x);
-    o.y += (R)(d.y - (double)hi.y);
+// (1 + v)(1 + d) - 1.  FP32 takes d as hi + lo: the drift is the same at every step, so its rounding
+// would add up over the chain.  (Kept split: converting FP64 values in the kernel, at the FP64 rate,
+// took two thirds of its time.)
+template <typename R> struct DiagOf { using T = double2; };
+template <> struct DiagOf<float> { using T = float4; };            // hi.x, hi.y, lo.x, lo.y
+__device__ __forceinline__ float4 loc_split(double2 d) {
+  const float2 h = make_float2((float)d.x, (float)d.y);
+  return make_float4(h.x, h.y, (float)(d.x - (double)h.x), (float)(d.y - (double)h.y));
+}
+// In place: a pulse's own diagonal (the same for all its steps) less 1, as FP32 hi + lo
+__global__ void loc_split_kernel(double2* p, int64_t n) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const double2 v = p[i];
+    reinterpret_cast<float4*>(p)[i] = loc_split(make_double2(v.x - 1.0, v.y));
   }
-  cfma<R>(o, v, hi);
+}
+__device__ __forceinline__ double2 loc_times(double2 v, double2 d) {
+  double2 o = make_double2(v.x + d.x, v.y + d.y);
+  cfma<double>(o, v, d);
+  return o;
+}
+__device__ __forceinline__ float2 loc_times(float2 v, float4 d) {
+  float2 o = make_float2(v.x + d.x + d.z, v.y + d.y + d.w);
+  cfma<float>(o, v, make_float2(d.x, d.y));
   return o;
 }
 
@@ -240,8 +263,8 @@ __device__ __forceinline__ void loc_derivatives(const LocTab<R>& tab, const int3
 template <typename R, bool NEAR>
 __global__ void __launch_bounds__(kPrepThreads)
 loc_steps_kernel(LocTab<R> tab, const int32_t* __restrict__ q, int64_t M, int64_t m0, int64_t T, int n, int N, int E,
-                 int64_t tiles, int ts,
-                 const double2* __restrict__ D, const double2* __restrict__ pd, int64_t pd_b, int64_t pd_n,
+                 int64_t tiles, int ts, const typename DiagOf<R>::T* __restrict__ D, const double2* __restrict__ pd,
+                 int64_t pd_b, int64_t pd_n,
                  cplx<R>* __restrict__ cs, cplx<R>* __restrict__ delta, const cplx<R>* __restrict__ h, int pairs,
                  R* __restrict__ gout) {
   // phases of every (step, qubit); row j is step n0 - 1 + j (the step before the tile gives its x)
@@ -271,38 +294,65 @@ loc_steps_kernel(LocTab<R> tab, const int32_t* __restrict__ q, int64_t M, int64_
   }
   __syncthreads();
   const int G = N / E;
-  for (int idx = threadIdx.x; idx < ts * N; idx += kPrepThreads) {
-    const int j = idx / N + 1, r = idx & (N - 1);
+  // Delta: a thread takes rows of one step that share their high bits
+  const int rows = N < 8 ? N : 8, low = N < 8 ? n : 3;
+  for (int idx = threadIdx.x; idx < ts * (N / rows); idx += kPrepThreads) {
+    const int j = idx / (N / rows) + 1, r0 = (idx - (j - 1) * (N / rows)) * rows;
     const int64_t m = n0 - 1 + j;
     if (m > m0 + T) continue;
-    cplx<R> v;                                       // Delta - 1
-    if constexpr (sizeof(R) == 4) {
-      uint32_t a = 0;
-      for (int i = 0; i < n; ++i) {
-        const bool up = (r >> i) & 1;
-        if (NEAR)
-          a += (uint32_t)(up ? xx[j - 1][i] : x0[j - 1][i]);
-        else
-          a += up ? (uint32_t)y1[j][i] + (uint32_t)xx[j - 1][i] : (uint32_t)y0[j][i];
+    phase_t<R> hi = no_phase<R>();
+    auto of = [&](int i, int up) -> phase_t<R> {
+      if constexpr (NEAR) {
+        return up ? xx[j - 1][i] : x0[j - 1][i];
+      } else if constexpr (sizeof(R) == 4) {
+        return up ? (int32_t)((uint32_t)y1[j][i] + (uint32_t)xx[j - 1][i]) : y0[j][i];
+      } else {
+        return up ? cmul<R>(y1[j][i], xx[j - 1][i]) : y0[j][i];
       }
-      v = phasor<true>((int32_t)a);
-    } else {
-      v = cmake<R>(R(1), R(0));
-      for (int i = 0; i < n; ++i) v = cmul<R>(v, ((r >> i) & 1) ? cmul<R>(y1[j][i], xx[j - 1][i]) : y0[j][i]);
-      v.x -= R(1);
-    }
-    if (m < M) {
-      v = loc_times<R>(v, D[r]);
-      if (pd) {
-        double2 p = pd[b * pd_b + m * pd_n + r];
-        p.x -= 1.0;
-        v = loc_times<R>(v, p);
+    };
+    auto join = [](phase_t<R> a, phase_t<R> b) -> phase_t<R> {
+      if constexpr (sizeof(R) == 4)
+        return (int32_t)((uint32_t)a + (uint32_t)b);
+      else
+        return cmul<R>(a, b);
+    };
+    for (int i = low; i < n; ++i) hi = join(hi, of(i, (r0 >> i) & 1));
+    phase_t<R> lo[3][2];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (i < low) {
+        lo[i][0] = of(i, 0);
+        lo[i][1] = of(i, 1);
       }
+    cplx<R>* o = delta + (b * (T + 1) + m - m0) * N;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if (e >= rows) break;
+      phase_t<R> a = hi;
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        if (i < low) a = join(a, lo[i][(e >> i) & 1]);
+      cplx<R> v;                                     // Delta - 1
+      if constexpr (sizeof(R) == 4)
+        v = phasor<true>(a);
+      else
+        v = cmake<R>(a.x - R(1), a.y);
+      const int r = r0 + e;
+      if (m < M) {
+        v = loc_times(v, D[r]);
+        if (pd) {
+          const double2* at = pd + b * pd_b + m * pd_n + r;
+          if constexpr (sizeof(R) == 4)
+            v = loc_times(v, pd_n == 0 ? *reinterpret_cast<const float4*>(at) : loc_split(make_double2(at->x - 1.0, at->y)));
+          else
+            v = loc_times(v, make_double2(at->x - 1.0, at->y));
+        }
+      }
+      // scaled to |Delta| = 1: without it the rounding of the phases changed the chain's norm five
+      // times as much
+      const R res = R(-0.5) * fma(v.x, v.x, fma(v.y, v.y, R(2) * v.x));
+      o[loc_pos(r, E, G)] = cmake<R>(v.x + fma(res, v.x, res), fma(res, v.y, v.y));
     }
-    // scaled to |Delta| = 1: without it the rounding of the phases changed the chain's norm five
-    // times as much
-    const R res = R(-0.5) * fma(v.x, v.x, fma(v.y, v.y, R(2) * v.x));
-    delta[(b * (T + 1) + m - m0) * N + loc_pos(r, E, G)] = cmake<R>(v.x + fma(res, v.x, res), fma(res, v.y, v.y));
   }
 }
 
@@ -860,7 +910,8 @@ static cudaError_t loc_steps_t(const redo_table* t, const int32_t* q, int64_t B,
   if constexpr (sizeof(R) == 4)
     if (loc_near(false, t->N)) kern = loc_steps_kernel<R, true>;
   kern<<<(unsigned)(B * tiles), kPrepThreads, 0, s>>>(
-      loc_tab<R>(t, status), q + b0 * M * t->K, M, m0, T, t->loc, t->N, E, tiles, ts, t->loc_D64,
+      loc_tab<R>(t, status), q + b0 * M * t->K, M, m0, T, t->loc, t->N, E, tiles, ts,
+      sizeof(R) == 8 ? (const typename DiagOf<R>::T*)t->loc_D64 : (const typename DiagOf<R>::T*)t->loc_D32,
       pd.p ? pd.p + b0 * pd.sb : nullptr, pd.sb, pd.sn, (cplx<R>*)w.cs,
       (cplx<R>*)w.delta, sizeof(R) == 8 ? (const cplx<R>*)t->loc_h : (const cplx<R>*)t->loc_h32, t->loc_pairs, (R*)w.g);
   return cudaGetLastError();
@@ -1066,6 +1117,13 @@ cudaError_t launch_local_state(const redo_table* t, const int32_t* q, int64_t B,
     if (e) return e;
   }
   return cudaSuccess;
+}
+
+cudaError_t launch_local_split(double2* pd, int64_t n, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  const int64_t blocks = (n + 255) / 256;
+  loc_split_kernel<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(pd, n);
+  return cudaGetLastError();
 }
 
 }  // namespace redo

@@ -634,6 +634,8 @@ chain_kernel(Src src, int64_t units, int64_t segs_per_unit, int64_t seg_len, int
         const double2* ph = src.phase(my_unit, my_f0 + t);
         if (ph)
           MM::scale_rows(ph, X, lt, Y);
+        else if (t == 0)
+          MM::load(A + stage * N2, lt, Y);               // the first factor beside the identity
         else
           MM::run(A + stage * N2, X, lt, Y);
       }
@@ -956,6 +958,95 @@ polar_ns_kernel(const cplx<Rin>* __restrict__ in, cplx<Rout>* __restrict__ out, 
   }
 }
 
+// The same step on an FP32 matrix with an FP64 result.  Only I - P^dag P needs more than FP32: it is
+// the small difference of sums near 1, so its products are split by fma and added with two_sum (about
+// 48 bits; 10 FP32 operations a term, where an FP64 one costs 64).  The correction P (I - P^dag P) / 2
+// is about 1e-6 of P, so its FP32 product is good to 1e-13, and P + it is added in FP64.
+template <int N>
+__global__ void __launch_bounds__(SmemMM<float, N, (N >= 64 ? 4 : (N >= 32 ? 2 : 1)),
+                                         (N >= 64 ? 4 : (N >= 32 ? 2 : 1))>::THREADS)
+polar_refine_kernel(const float2* __restrict__ in, double2* __restrict__ out) {
+  constexpr int TM = (N >= 64 ? 4 : (N >= 32 ? 2 : 1));
+  using MM = SmemMM<float, N, TM, TM>;
+  constexpr int N2 = N * N, T = MM::TY, HALF = T * (T + 1) / 2;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  float2* P = reinterpret_cast<float2*>(smem_raw);
+  float2* Q = P + N2;
+  const int lt = threadIdx.x;
+  const int64_t b = blockIdx.x;
+  for (int i = lt; i < N2; i += MM::THREADS) P[i] = in[b * N2 + i];
+  __syncthreads();
+  if (lt < HALF) {                                       // tiles (ty <= tx) of the Hermitian Gram matrix
+    int ty = 0, rem = lt;
+    while (rem >= T - ty) {
+      rem -= T - ty;
+      ++ty;
+    }
+    const int tx = ty + rem;
+    float2 s[TM][TM], lo[TM][TM];
+#pragma unroll
+    for (int a = 0; a < TM; ++a)
+#pragma unroll
+      for (int c = 0; c < TM; ++c) {
+        s[a][c] = make_float2(ty + T * a == tx + T * c ? -1.f : 0.f, 0.f);
+        lo[a][c] = make_float2(0.f, 0.f);
+      }
+    // s + lo += x y
+    auto mac = [](float& s, float& lo, float x, float y) {
+      const float h = x * y, l = fmaf(x, y, -h), t = s + h, z = t - s;
+      lo += l + ((s - (t - z)) + (h - z));
+      s = t;
+    };
+    for (int k = 0; k < N; ++k) {
+      float2 av[TM], xv[TM];
+#pragma unroll
+      for (int a = 0; a < TM; ++a) av[a] = P[k * N + ty + T * a];
+#pragma unroll
+      for (int c = 0; c < TM; ++c) xv[c] = P[k * N + tx + T * c];
+#pragma unroll
+      for (int a = 0; a < TM; ++a)
+#pragma unroll
+        for (int c = 0; c < TM; ++c) {                   // conj(a) x
+          mac(s[a][c].x, lo[a][c].x, av[a].x, xv[c].x);
+          mac(s[a][c].x, lo[a][c].x, av[a].y, xv[c].y);
+          mac(s[a][c].y, lo[a][c].y, av[a].x, xv[c].y);
+          mac(s[a][c].y, lo[a][c].y, -av[a].y, xv[c].x);
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < TM; ++a)
+#pragma unroll
+      for (int c = 0; c < TM; ++c) {
+        const int r = ty + T * a, col = tx + T * c;
+        const float x = -0.5f * (s[a][c].x + lo[a][c].x), y = -0.5f * (s[a][c].y + lo[a][c].y);
+        Q[r * N + col] = make_float2(x, r == col ? 0.f : y);
+        if (ty != tx) Q[col * N + r] = make_float2(x, -y);
+      }
+  }
+  __syncthreads();
+  float2 Y[TM][TM];
+  MM::run(P, Q, lt, Y);
+  const int ty = lt / MM::TX, tx = lt % MM::TX;
+#pragma unroll
+  for (int a = 0; a < TM; ++a)
+#pragma unroll
+    for (int c = 0; c < TM; ++c) {
+      const int i = (ty + MM::TY * a) * N + tx + MM::TX * c;
+      out[b * N2 + i] = make_double2((double)P[i].x + (double)Y[a][c].x, (double)P[i].y + (double)Y[a][c].y);
+    }
+}
+
+template <int N> static cudaError_t polar_refine_n(const void* in, void* out, int64_t count, cudaStream_t s) {
+  constexpr int TM = (N >= 64 ? 4 : (N >= 32 ? 2 : 1));
+  using MM = SmemMM<float, N, TM, TM>;
+  const size_t smem = 2 * sizeof(float2) * N * N;
+  cudaError_t e = cudaFuncSetAttribute(polar_refine_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  if (count == 0) return cudaSuccess;
+  polar_refine_kernel<N><<<(unsigned)count, MM::THREADS, smem, s>>>((const float2*)in, (double2*)out);
+  return cudaGetLastError();
+}
+
 template <typename Rin, typename Rc, int N, typename Rout = Rc>
 static cudaError_t polar_n(const void* in, void* out, int64_t count, int iters, cudaStream_t s) {
   constexpr int TM = (N >= 64 ? 4 : (N >= 32 ? 2 : 1));
@@ -987,7 +1078,17 @@ cudaError_t launch_polar(const redo_table* t, int prec_in, int prec_out, const v
                          int64_t count, int iters, cudaStream_t s) {
   const bool din = prec_in == REDO_FP64, dout = prec_out == REDO_FP64;
   if (din && dout) return polar_t<double, double>(t->N, in, out, count, iters, s);
-  if (!din && dout) return polar_t<float, double>(t->N, in, out, count, iters, s);
+  if (!din && dout && iters == 1) {
+    switch (t->N) {
+      case 2: return polar_refine_n<2>(in, out, count, s);
+      case 4: return polar_refine_n<4>(in, out, count, s);
+      case 8: return polar_refine_n<8>(in, out, count, s);
+      case 16: return polar_refine_n<16>(in, out, count, s);
+      case 32: return polar_refine_n<32>(in, out, count, s);
+      case 64: return polar_refine_n<64>(in, out, count, s);
+      default: return cudaErrorInvalidValue;
+    }
+  }
   if (!din && !dout) return polar_t<float, float>(t->N, in, out, count, iters, s);
   return cudaErrorInvalidValue;
 }

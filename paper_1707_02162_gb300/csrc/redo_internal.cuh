@@ -79,6 +79,7 @@ struct redo_table {
   double2* loc_u64;           // [pairs][loc_d][loc_base][4] digit (or level) operators
   float2* loc_u32;
   double2* loc_D64;           // [N] diagonal of the drift step minus 1
+  float4* loc_D32;            // the same as FP32 hi + lo
   cudaStream_t build_stream;
   int num_sms;
 };
@@ -166,7 +167,8 @@ cudaError_t launch_polar_c128(int N, int prec_arith, const double2* in, double2*
                               cudaStream_t s);
 
 // Locally controlled systems (kernels_local.cu).  Step-opening diagonals of a call: p[b*sb + n*sn + r]
-// (nullptr: none; sn = 0: the same for every step of a pulse).
+// (nullptr: none).  sn = 0: the same for every step of a pulse; an FP32 call then holds the diagonals
+// as launch_local_split leaves them (less 1, FP32 hi + lo).
 struct LocalDiag {
   const double2* p;
   int64_t sb, sn;
@@ -174,6 +176,7 @@ struct LocalDiag {
 }  // namespace redo
 #include <vector>
 namespace redo {
+cudaError_t launch_local_split(double2* pd, int64_t n, cudaStream_t s);
 cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_t s);
 void local_free(redo_table* t);
 // What a call computes: segment products, the gradient, the amplitude/phase gradient, the state's

@@ -192,6 +192,13 @@ struct SmemMM {
       }
     }
   }
+  __device__ __forceinline__ static void load(const cplx<R>* __restrict__ X, int lt, cplx<R> (&Y)[TM][TN]) {
+    const int ty = lt / TX, tx = lt % TX;
+#pragma unroll
+    for (int a = 0; a < TM; ++a)
+#pragma unroll
+      for (int c = 0; c < TN; ++c) Y[a][c] = X[(ty + TY * a) * N + tx + TX * c];
+  }
   // X <- X + Y
   __device__ __forceinline__ static void add(cplx<R>* __restrict__ X, int lt, const cplx<R> (&Y)[TM][TN]) {
     const int ty = lt / TX, tx = lt % TX;

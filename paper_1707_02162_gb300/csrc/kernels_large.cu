@@ -59,22 +59,36 @@ __global__ void __launch_bounds__(256) cgemm_kernel(Ops ops, int N, R alpha, R d
       acc[r][c] = cmake<R>(R(0), R(0));
       if constexpr (kComp) tot[r][c] = cmp[r][c] = acc[r][c];
     }
+  // the next K chunk is loaded into registers while the present one is multiplied
+  constexpr int kPer = (kT * kBK) / 256;
+  cplx<R> ra[kPer], rb[kPer];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int x = 0; x < kPer; ++x) {
+      const int e = tid + 256 * x;
+      const int kb = e / kT, c = e % kT;
+      if (!ADJA) {
+        ra[x] = A[(int64_t)(i0 + e / kBK) * N + k0 + e % kBK];
+      } else {
+        const cplx<R> v = A[(int64_t)(k0 + kb) * N + i0 + c];
+        ra[x] = cmake<R>(v.x, -v.y);
+      }
+      rb[x] = Bm[(int64_t)(k0 + kb) * N + j0 + c];
+    }
+  };
+  fetch(0);
   for (int k0 = 0; k0 < N; k0 += kBK) {
 #pragma unroll
-    for (int x = 0; x < (kT * kBK) / 256; ++x) {
+    for (int x = 0; x < kPer; ++x) {
       const int e = tid + 256 * x;
-      if (!ADJA) {
-        const int r = e / kBK, kk = e % kBK;
-        As[kk][r] = A[(int64_t)(i0 + r) * N + k0 + kk];
-      } else {
-        const int kk = e / kT, r = e % kT;
-        const cplx<R> v = A[(int64_t)(k0 + kk) * N + i0 + r];
-        As[kk][r] = cmake<R>(v.x, -v.y);
-      }
-      const int kb = e / kT, c = e % kT;
-      Bs[kb][c] = Bm[(int64_t)(k0 + kb) * N + j0 + c];
+      if (!ADJA)
+        As[e % kBK][e / kBK] = ra[x];
+      else
+        As[e / kT][e % kT] = ra[x];
+      Bs[e / kT][e % kT] = rb[x];
     }
     __syncthreads();
+    if (k0 + kBK < N) fetch(k0 + kBK);
 #pragma unroll
     for (int kk = 0; kk < kBK; ++kk) {
       cplx<R> a[4], bb[4];
@@ -972,9 +986,88 @@ struct CostateOps {
   }
 };
 
+// Long scans run in groups of about sqrt(S) segments (GroupStepOps, GroupCarryOps): 4S products in all
+// where the log-depth rounds take 2S per round, at a depth of about 2 sqrt(S) + 1 launches.
+//
+// Step i of a scan over consecutive groups of g of the L matrices X of every pulse; items are (pulse,
+// group, direction): prefix P[first + i] = X[first + i] P[first + i - 1], suffix Q[last - i] =
+// Q[last - i + 1] X[last - i]; at i = 0 copies.  in/out with L matrices per pulse.
+template <typename R>
+struct GroupStepOps {
+  const cplx<R>* X;
+  cplx<R>* P;
+  cplx<R>* Q;
+  int64_t L, g, groups, i, n2;
+  __device__ void get(int64_t it, const cplx<R>*& a, const cplx<R>*& bb, cplx<R>*& c) const {
+    const bool suffix = it & 1;
+    const int64_t u = (it >> 1) / groups, gi = (it >> 1) - u * groups;
+    const int64_t first = gi * g, last = first + g < L ? first + g - 1 : L - 1;
+    const int64_t s = suffix ? last - i : first + i;
+    a = nullptr;
+    bb = nullptr;
+    c = nullptr;
+    if (s < first || s > last) return;
+    const cplx<R>* x = X + (u * L + s) * n2;
+    c = (suffix ? Q : P) + (u * L + s) * n2;
+    if (i == 0) {
+      bb = x;
+    } else if (suffix) {
+      a = Q + (u * L + s + 1) * n2;
+      bb = x;
+    } else {
+      a = x;
+      bb = P + (u * L + s - 1) * n2;
+    }
+  }
+};
+
+// The groups' own scan GP, GQ carried into the segments, and the costates: items [0, B S) are
+// Pck[s] = P[s] GP[group - 1] (a copy in the first group), items [B S, 2 B S) are
+// Rck[s] = C[group] Q[s + 1] (C[group] alone for a group's last segment), C = the costate at the
+// group's end.
+template <typename R>
+struct GroupCarryOps {
+  const cplx<R>* P;
+  const cplx<R>* Q;
+  const cplx<R>* GP;
+  const cplx<R>* C;
+  cplx<R>* Pck;
+  cplx<R>* Rck;
+  int64_t BS, S, g, groups, n2;
+  __device__ void get(int64_t it, const cplx<R>*& a, const cplx<R>*& bb, cplx<R>*& c) const {
+    const bool suffix = it >= BS;
+    const int64_t j = suffix ? it - BS : it, u = j / S, s = j - u * S, gi = s / g;
+    if (!suffix) {
+      a = gi > 0 ? P + j * n2 : nullptr;
+      bb = gi > 0 ? GP + (u * groups + gi - 1) * n2 : P + j * n2;
+      c = Pck + j * n2;
+    } else {
+      const bool end = s == S - 1 || s % g == g - 1;
+      const cplx<R>* e = C + (u * groups + gi) * n2;
+      a = end ? nullptr : e;
+      bb = end ? e : Q + (j + 1) * n2;
+      c = Rck + j * n2;
+    }
+  }
+};
+
+// out[u][i] = in[u][min((i + 1) g, L) - 1]: the groups' totals (their last prefix)
+template <typename R>
+struct GroupTotalOps {
+  const cplx<R>* P;
+  cplx<R>* T;
+  int64_t L, g, groups, n2;
+  __device__ void get(int64_t it, const cplx<R>*& a, const cplx<R>*& bb, cplx<R>*& c) const {
+    const int64_t u = it / groups, gi = it - u * groups, e = (gi + 1) * g < L ? (gi + 1) * g - 1 : L - 1;
+    a = nullptr;
+    bb = P + (u * L + e) * n2;
+    c = T + it * n2;
+  }
+};
+
 // Prefix checkpoints, tau/F and suffix costates from the segment products in the first
 // workspace region, by log-depth scans (ceil(log2 S) batched rounds instead of 2S
-// dependent products).
+// dependent products), or in groups from 9 segments on.
 template <typename R>
 static cudaError_t large_scans_t(const redo_table* t, const ChainPlan& p, const double2* UT, int tb,
                                  double* F_out, char* ws, cplx<R>** Pck_out, cplx<R>** Rck_out,
@@ -992,6 +1085,35 @@ static cudaError_t large_scans_t(const redo_table* t, const ChainPlan& p, const 
   cplx<R>* run2 = (cplx<R>*)(ws + 5 * mat + up(p.B * n2 * sizeof(cplx<R>)));
   double2* tau = (double2*)(ws + 5 * mat + 2 * up(p.B * n2 * sizeof(cplx<R>)));
   cudaError_t e;
+  int64_t g = 3;
+  while (g * g < p.S) ++g;
+  const int64_t groups = p.S > 0 ? (p.S + g - 1) / g : 0;
+  // the totals, their two scans and the groups' costates (4 B groups matrices) take the segment
+  // products' place once those are scanned
+  if (p.S >= 9 && 4 * groups <= p.S) {
+    GroupStepOps<R> st{seg, ping, pong, p.S, g, groups, 0, n2};
+    for (; st.i < g; ++st.i)
+      if ((e = cgemm<R, false>(st, 2 * p.B * groups, N, R(1), R(0), s))) return e;
+    const int64_t BG = p.B * groups;
+    cplx<R>*tot = seg, *GP = seg + BG * n2, *GQ = seg + 2 * BG * n2, *C = seg + 3 * BG * n2;
+    GroupTotalOps<R> tt{ping, tot, p.S, g, groups, n2};
+    if ((e = cgemm<R, false>(tt, BG, N, R(1), R(0), s))) return e;
+    GroupStepOps<R> gs{tot, GP, GQ, groups, groups, 1, 0, n2};
+    for (; gs.i < groups; ++gs.i)
+      if ((e = cgemm<R, false>(gs, 2 * p.B, N, R(1), R(0), s))) return e;
+    adjoint_target_kernel<R><<<blocks_for(p.B * n2), 256, 0, s>>>(UT, tb, N, p.B, run);
+    CostateOps<R> gc{GQ, run, GP, C, run2, BG, groups, n2};
+    if ((e = cgemm<R, false>(gc, BG + p.B, N, R(1), R(0), s))) return e;
+    GroupCarryOps<R> ca{ping, pong, GP, C, Pck, Rck, G, p.S, g, groups, n2};
+    if ((e = cgemm<R, false>(ca, 2 * G, N, R(1), R(0), s))) return e;
+    if ((e = cudaMemsetAsync(tau, 0, sizeof(double2) * p.B, s))) return e;
+    tau_kernel<R><<<(unsigned)(p.B * kTauParts), 256, 0, s>>>(run2, UT, tb, N, tau);
+    if (F_out) fidelity_from_tau_kernel<<<(unsigned)((p.B + 127) / 128), 128, 0, s>>>(tau, p.B, N, F_out);
+    *Pck_out = Pck;
+    *Rck_out = Rck;
+    *tau_out = tau;
+    return cudaGetLastError();
+  }
   // prefix in Pck / ping, suffix in pong / Rck; the first round reads the segment products
   const cplx<R>* ps = seg;
   const cplx<R>* qs = seg;

@@ -3,7 +3,7 @@
 // parts whose tensor product the N x N table operator is; Section III: chain, GRAPE gradient, state
 // transfer; Section IV: observables along the chain.)
 #include <cmath>
-#include <cstdlib>
+#include <cstring>
 #include <type_traits>
 #include <vector>
 
@@ -140,23 +140,33 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
     const double sh = std::sin(0.5 * a);
     D[r] = make_double2(-2.0 * sh * sh, -std::sin(a));                // exp(-i a) - 1
   }
-  cudaError_t e;
-  if ((e = cudaMalloc(&t->loc_ptr, sizeof(int32_t) * (n + 1))) || (e = cudaMalloc(&t->loc_k, sizeof(int32_t) * pairs)) ||
-      (e = cudaMalloc(&t->loc_h, sizeof(double2) * 4 * pairs)) ||
-      (e = cudaMalloc(&t->loc_u64, sizeof(double2) * 4 * ent)) || (e = cudaMalloc(&t->loc_u32, sizeof(float2) * 4 * ent)) ||
-      (e = cudaMalloc(&t->loc_D64, sizeof(double2) * N)) || (e = cudaMalloc(&t->loc_h32, sizeof(float2) * 4 * pairs)) ||
-      (e = cudaMalloc(&t->loc_D32, sizeof(float4) * N)) ||
-      (e = cudaMalloc(&t->loc_kptr, sizeof(int32_t) * (K + 1))) || (e = cudaMalloc(&t->loc_kpair, sizeof(int32_t) * pairs)))
-    return e;
-  if ((e = cudaMemcpyAsync(t->loc_ptr, ptr.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemcpyAsync(t->loc_k, kk.data(), sizeof(int32_t) * pairs, cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemcpyAsync(t->loc_h, hp.data(), sizeof(double2) * 4 * pairs, cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemcpyAsync(t->loc_D64, D.data(), sizeof(double2) * N, cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemcpyAsync(t->loc_D32, D32.data(), sizeof(float4) * N, cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemcpyAsync(t->loc_h32, hp32.data(), sizeof(float2) * 4 * pairs, cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemcpyAsync(t->loc_kptr, kptr.data(), sizeof(int32_t) * (K + 1), cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemcpyAsync(t->loc_kpair, kpair.data(), sizeof(int32_t) * kpair.size(), cudaMemcpyHostToDevice, s)))
-    return e;
+  // one allocation and one copy for the small arrays, the tables behind them
+  std::vector<unsigned char> host;
+  auto put = [&](const void* src, size_t bytes) {
+    const size_t at = (host.size() + 255) & ~(size_t)255;
+    host.resize(at + bytes);
+    std::memcpy(host.data() + at, src, bytes);
+    return at;
+  };
+  const size_t o_ptr = put(ptr.data(), sizeof(int32_t) * (n + 1)), o_k = put(kk.data(), sizeof(int32_t) * pairs),
+               o_h = put(hp.data(), sizeof(double2) * 4 * pairs), o_h32 = put(hp32.data(), sizeof(float2) * 4 * pairs),
+               o_kptr = put(kptr.data(), sizeof(int32_t) * (K + 1)), o_kp = put(kpair.data(), sizeof(int32_t) * pairs),
+               o_D = put(D.data(), sizeof(double2) * N), o_D32 = put(D32.data(), sizeof(float4) * N);
+  const size_t o_u64 = (host.size() + 255) & ~(size_t)255, o_u32 = o_u64 + sizeof(double2) * 4 * ent;
+  cudaError_t e = cudaMalloc(&t->loc_mem, o_u32 + sizeof(float2) * 4 * ent);
+  if (e) return e;
+  char* base = (char*)t->loc_mem;
+  if ((e = cudaMemcpyAsync(base, host.data(), host.size(), cudaMemcpyHostToDevice, s))) return e;
+  t->loc_ptr = (int32_t*)(base + o_ptr);
+  t->loc_k = (int32_t*)(base + o_k);
+  t->loc_h = (double2*)(base + o_h);
+  t->loc_h32 = (float2*)(base + o_h32);
+  t->loc_kptr = (int32_t*)(base + o_kptr);
+  t->loc_kpair = (int32_t*)(base + o_kp);
+  t->loc_D64 = (double2*)(base + o_D);
+  t->loc_D32 = (float4*)(base + o_D32);
+  t->loc_u64 = (double2*)(base + o_u64);
+  t->loc_u32 = (float2*)(base + o_u32);
   loc_table_kernel<<<(unsigned)((ent + 127) / 128 < 4096 ? (ent + 127) / 128 : 4096), 128, 0, s>>>(
       t->loc_h, t->loc_k, pairs, t->loc_d, t->loc_base, t->dt, t->d_lo, t->d_delta, t->loc_u64, t->loc_u32);
   if ((e = cudaGetLastError()) || (e = cudaStreamSynchronize(s))) return e;   // the host arrays end here
@@ -164,18 +174,7 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
   return cudaSuccess;
 }
 
-void local_free(redo_table* t) {
-  cudaFree(t->loc_ptr);
-  cudaFree(t->loc_k);
-  cudaFree(t->loc_h);
-  cudaFree(t->loc_u64);
-  cudaFree(t->loc_u32);
-  cudaFree(t->loc_D64);
-  cudaFree(t->loc_h32);
-  cudaFree(t->loc_D32);
-  cudaFree(t->loc_kptr);
-  cudaFree(t->loc_kpair);
-}
+void local_free(redo_table* t) { cudaFree(t->loc_mem); }
 
 template <typename R> static LocTab<R> loc_tab(const redo_table* t, int64_t* status) {
   LocTab<R> o;

@@ -70,6 +70,7 @@ struct redo_table {
   // one-qubit operators or the drift is not diagonal
   int loc;
   int loc_pairs, loc_d, loc_base;
+  void* loc_mem;              // the one allocation that the following arrays lie in
   int32_t* loc_ptr;           // [loc + 1] (term, qubit) pairs of each qubit
   int32_t* loc_k;             // [pairs] term, flagged at the first pair of a term
   double2* loc_h;             // [pairs][4] one-qubit part of the term's operator

@@ -23,12 +23,14 @@ namespace large {
 constexpr int kT = 64;    // output tile (complex)
 constexpr int kBK = 16;   // K chunk
 
-template <typename R, bool ADJA, class Ops>
+// TT: output tile, 64 or 32 (one launch of few tiles is bound by one tile's time: a quarter of it)
+template <typename R, bool ADJA, int TT, class Ops>
 __global__ void __launch_bounds__(256) cgemm_kernel(Ops ops, int N, R alpha, R diag) {
-  __shared__ cplx<R> As[kBK][kT + 1];
-  __shared__ cplx<R> Bs[kBK][kT + 1];
+  constexpr int PT = TT / 16;
+  __shared__ cplx<R> As[kBK][TT + 1];
+  __shared__ cplx<R> Bs[kBK][TT + 1];
   // blockIdx.x = (batch item, row tile, column tile)
-  const int tiles = N / kT;
+  const int tiles = N / TT;
   const int64_t b = blockIdx.x / ((int64_t)tiles * tiles);
   const int tile = (int)(blockIdx.x % ((int64_t)tiles * tiles));
   const cplx<R>* A;
@@ -36,12 +38,12 @@ __global__ void __launch_bounds__(256) cgemm_kernel(Ops ops, int N, R alpha, R d
   cplx<R>* C;
   ops.get(b, A, Bm, C);
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const int i0 = (tile / tiles) * kT, j0 = (tile % tiles) * kT;
+  const int i0 = (tile / tiles) * TT, j0 = (tile % tiles) * TT;
   if (C == nullptr) return;
   if (A == nullptr) {
     // identity: copy the tile
-    for (int e = tid; e < kT * kT; e += 256) {
-      const int r = e / kT, c = e % kT;
+    for (int e = tid; e < TT * TT; e += 256) {
+      const int r = e / TT, c = e % TT;
       C[(int64_t)(i0 + r) * N + j0 + c] = Bm[(int64_t)(i0 + r) * N + j0 + c];
     }
     return;
@@ -51,22 +53,22 @@ __global__ void __launch_bounds__(256) cgemm_kernel(Ops ops, int N, R alpha, R d
   // it scales its matrix up (1.4e-7 per segment at N = 256).  Their K chunks are summed on their own
   // and added with compensation.
   constexpr bool kComp = ADJA && sizeof(R) == 4;
-  cplx<R> acc[4][4], tot[kComp ? 4 : 1][kComp ? 4 : 1], cmp[kComp ? 4 : 1][kComp ? 4 : 1];
+  cplx<R> acc[PT][PT], tot[kComp ? PT : 1][kComp ? PT : 1], cmp[kComp ? PT : 1][kComp ? PT : 1];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < PT; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < PT; ++c) {
       acc[r][c] = cmake<R>(R(0), R(0));
       if constexpr (kComp) tot[r][c] = cmp[r][c] = acc[r][c];
     }
   // the next K chunk is loaded into registers while the present one is multiplied
-  constexpr int kPer = (kT * kBK) / 256;
+  constexpr int kPer = (TT * kBK) / 256;
   cplx<R> ra[kPer], rb[kPer];
   auto fetch = [&](int k0) {
 #pragma unroll
     for (int x = 0; x < kPer; ++x) {
       const int e = tid + 256 * x;
-      const int kb = e / kT, c = e % kT;
+      const int kb = e / TT, c = e % TT;
       if (!ADJA) {
         ra[x] = A[(int64_t)(i0 + e / kBK) * N + k0 + e % kBK];
       } else {
@@ -84,28 +86,28 @@ __global__ void __launch_bounds__(256) cgemm_kernel(Ops ops, int N, R alpha, R d
       if (!ADJA)
         As[e % kBK][e / kBK] = ra[x];
       else
-        As[e / kT][e % kT] = ra[x];
-      Bs[e / kT][e % kT] = rb[x];
+        As[e / TT][e % TT] = ra[x];
+      Bs[e / TT][e % TT] = rb[x];
     }
     __syncthreads();
     if (k0 + kBK < N) fetch(k0 + kBK);
 #pragma unroll
     for (int kk = 0; kk < kBK; ++kk) {
-      cplx<R> a[4], bb[4];
+      cplx<R> a[PT], bb[PT];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
+      for (int r = 0; r < PT; ++r) a[r] = As[kk][ty + 16 * r];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) bb[c] = Bs[kk][tx + 16 * c];
+      for (int c = 0; c < PT; ++c) bb[c] = Bs[kk][tx + 16 * c];
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < PT; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) cfma<R>(acc[r][c], a[r], bb[c]);
+        for (int c = 0; c < PT; ++c) cfma<R>(acc[r][c], a[r], bb[c]);
     }
     if constexpr (kComp) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < PT; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < PT; ++c) {
           const R yx = acc[r][c].x - cmp[r][c].x, yy = acc[r][c].y - cmp[r][c].y;
           const R sx = tot[r][c].x + yx, sy = tot[r][c].y + yy;
           cmp[r][c] = cmake<R>((sx - tot[r][c].x) - yx, (sy - tot[r][c].y) - yy);
@@ -117,14 +119,14 @@ __global__ void __launch_bounds__(256) cgemm_kernel(Ops ops, int N, R alpha, R d
   }
   if constexpr (kComp) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < PT; ++r)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) acc[r][c] = tot[r][c];
+      for (int c = 0; c < PT; ++c) acc[r][c] = tot[r][c];
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < PT; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < PT; ++c) {
       const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
       C[(int64_t)i * N + j] = cmake<R>(alpha * acc[r][c].x + (i == j ? diag : R(0)), alpha * acc[r][c].y);
     }
@@ -134,7 +136,12 @@ template <typename R, bool ADJA, class Ops>
 static cudaError_t cgemm(const Ops& ops, int64_t batch, int N, R alpha, R diag, cudaStream_t s) {
   if (batch == 0) return cudaSuccess;
   const int64_t blocks = batch * (N / kT) * (N / kT);
-  cgemm_kernel<R, ADJA, Ops><<<(unsigned)blocks, 256, 0, s>>>(ops, N, alpha, diag);
+  // up to two tiles of 64 per SM: 32 x 32 tiles spread them (10 products of N = 256: 50 -> 28 us; one
+  // at a time 29 -> 11 us); above, the larger tile's operand reuse wins
+  if (blocks <= 304)
+    cgemm_kernel<R, ADJA, 32, Ops><<<(unsigned)(4 * blocks), 256, 0, s>>>(ops, N, alpha, diag);
+  else
+    cgemm_kernel<R, ADJA, kT, Ops><<<(unsigned)blocks, 256, 0, s>>>(ops, N, alpha, diag);
   return cudaGetLastError();
 }
 

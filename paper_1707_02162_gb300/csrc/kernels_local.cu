@@ -620,6 +620,7 @@ static cudaError_t loc_sweep_t(const redo_table* t, const ChainPlan& p, int64_t 
 // a few pulses reach as many SMs.
 // ============================================================================
 __host__ __device__ constexpr int loc_vec_entries(int N) { return N >= 64 ? N / 32 : 2; }
+__host__ __device__ constexpr int loc_sim_entries(int N) { return N > 256 ? 8 : loc_vec_entries(N); }
 
 // a + b exactly as s + e
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -652,6 +653,76 @@ template <int E> __device__ __forceinline__ double2 lane_expect(const double2 (&
 #pragma unroll
   for (int e = 0; e < E; ++e) acc = fma(o[e].x, fma(v[e].x, v[e].x, v[e].y * v[e].y), acc);
   return make_double2(acc, 0.0);
+}
+
+// The same for N >= 512: a pulse per block of W warps, eight entries a lane (one warp would issue
+// 2500 instructions a step, one after another).  The qubits of the warp index pair the same lanes of
+// other warps through shared memory; two of them share one exchange, and the buffers alternate so
+// that one barrier a step is enough.
+template <typename R, int N>
+__global__ void __launch_bounds__(N / 8)
+loc_sim_wide_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t M,
+                    const double2* __restrict__ psi0, int batched, const double* __restrict__ obs,
+                    cplx<R>* __restrict__ part) {
+  constexpr int E = 8, W = N / 256, LANES = 32 * W, NQ = Log2<N>::v;
+  using L = LocCol<R, 256, E>;                       // the qubits within a warp
+  __shared__ cplx<R> ex[2][E][LANES];
+  const int lane = threadIdx.x & 31, l = threadIdx.x, wp = threadIdx.x >> 5;
+  const int64_t b = blockIdx.x;
+  const cplx<R>* d = delta + b * (M + 1) * N;
+  const cplx<R>* r = cs + b * M * NQ;
+  cplx<R>* o = part + b * (M + 1) * LANES + l;
+  cplx<R> v[E], w[E], dn[E], cn[NQ];
+  auto load = [&](int64_t m) {
+#pragma unroll
+    for (int e = 0; e < E; e += 2) {
+      const cplx<R>* p = d + m * N + ((e >> 1) * LANES + l) * 2;
+      if constexpr (sizeof(R) == 4) {
+        const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+        dn[e] = make_float2(q.x, q.y);
+        dn[e + 1] = make_float2(q.z, q.w);
+      } else {
+        dn[e] = __ldg(p);
+        dn[e + 1] = __ldg(p + 1);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) cn[i] = __ldg(r + m * NQ + i);
+  };
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const double2 z = psi0[(batched ? b * N : 0) + l * E + e];
+    v[e] = cmake<R>((R)z.x, (R)z.y);
+    const double ov = obs[l * E + e];
+    w[e] = cmake<R>((R)ov, (R)(ov - (double)(R)ov));
+  }
+  o[0] = lane_expect<E>(v, w);
+  if (M > 0) load(0);
+#pragma unroll 1
+  for (int64_t m = 0; m < M; ++m) {
+    cplx<R> c[L::NQ];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = plus_mul<R>(v[e], dn[e]);
+#pragma unroll
+    for (int i = 0; i < L::NQ; ++i) c[i] = cn[i];
+    const cplx<R> c8 = cn[8], c9 = cn[NQ - 1];
+    load(m + 1 < M ? m + 1 : m);
+    L::rotate(v, c, lane);
+    cplx<R>(*x)[LANES] = ex[m & 1];
+#pragma unroll
+    for (int e = 0; e < E; ++e) x[e][l] = v[e];
+    __syncthreads();
+    const R s8 = (wp & 1) ? c8.y : -c8.y;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      v[e] = rot_one<R, false>(v[e], x[e][l ^ 32], c8.x, s8, R(0));
+      if constexpr (W == 4) {
+        const cplx<R> p = rot_one<R, false>(x[e][l ^ 64], x[e][l ^ 96], c8.x, s8, R(0));
+        v[e] = rot_one<R, false>(v[e], p, c9.x, (wp & 2) ? c9.y : -c9.y, R(0));
+      }
+    }
+    o[(m + 1) * LANES] = lane_expect<E>(v, w);
+  }
 }
 
 // part[b][n][l]: lane l's part of <O> after n steps
@@ -850,7 +921,7 @@ static LocScratch loc_scratch(const redo_table* t, int64_t nb, int64_t M, int pr
   const size_t el = prec == REDO_FP64 ? sizeof(double) : sizeof(float);
   const bool grad = what == kLocalGrad || what == kLocalPhaseGrad;
   const size_t parts = grad ? (size_t)loc_parts(t, prec == REDO_FP64) : 1;
-  const size_t lanes = what == kLocalSim ? (size_t)(t->N / loc_vec_entries(t->N)) : 0;
+  const size_t lanes = what == kLocalSim ? (size_t)(t->N / loc_sim_entries(t->N)) : 0;
   LocScratch w;
   char* c = (char*)base;
   size_t off = 0;
@@ -1008,9 +1079,23 @@ cudaError_t launch_local_grad(const redo_table* t, const int32_t* q, const Chain
 template <typename R>
 static cudaError_t loc_sim_t(const redo_table* t, int64_t B, int64_t M, const double2* psi0, int batched,
                              const double* obs, const LocScratch& w, double* expect, cudaStream_t s) {
-  const int lanes = t->N / loc_vec_entries(t->N), cols = 32 / lanes;
+  const int lanes = t->N / loc_sim_entries(t->N), cols = lanes < 32 ? 32 / lanes : 1;
   const unsigned blocks = (unsigned)((B + cols - 1) / cols);
-  LOC_VEC(loc_sim_kernel, (const cplx<R>*)w.cs, (const cplx<R>*)w.delta, B, M, psi0, batched, obs, (cplx<R>*)w.bl)
+  const cplx<R>*cs = (const cplx<R>*)w.cs, *delta = (const cplx<R>*)w.delta;
+  cplx<R>* part = (cplx<R>*)w.bl;
+  switch (t->N) {
+    case 2: loc_sim_kernel<R, 2><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
+    case 4: loc_sim_kernel<R, 4><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
+    case 8: loc_sim_kernel<R, 8><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
+    case 16: loc_sim_kernel<R, 16><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
+    case 32: loc_sim_kernel<R, 32><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
+    case 64: loc_sim_kernel<R, 64><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
+    case 128: loc_sim_kernel<R, 128><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
+    case 256: loc_sim_kernel<R, 256><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
+    case 512: loc_sim_wide_kernel<R, 512><<<blocks, 64, 0, s>>>(cs, delta, M, psi0, batched, obs, part); break;
+    case 1024: loc_sim_wide_kernel<R, 1024><<<blocks, 128, 0, s>>>(cs, delta, M, psi0, batched, obs, part); break;
+    default: return cudaErrorInvalidValue;
+  }
   const int64_t n = B * (M + 1), nb = (n + 127) / 128;
   loc_expect_kernel<R><<<(unsigned)(nb < 4096 ? nb : 4096), 128, 0, s>>>((const cplx<R>*)w.bl, n, lanes, expect);
   return cudaGetLastError();
@@ -1022,7 +1107,7 @@ cudaError_t launch_local_sim(const redo_table* t, const int32_t* q, int64_t B, i
   const LocScratch w = loc_scratch(t, slice, M, prec, kLocalSim, ops);
   for (int64_t b0 = 0; b0 < B; b0 += slice) {
     const int64_t nb = b0 + slice < B ? slice : B - b0;
-    cudaError_t e = loc_steps(t, q, nb, M, prec, loc_vec_entries(t->N), LocalDiag{nullptr, 0, 0}, b0, w, status, s);
+    cudaError_t e = loc_steps(t, q, nb, M, prec, loc_sim_entries(t->N), LocalDiag{nullptr, 0, 0}, b0, w, status, s);
     if (e) return e;
     const double2* p0 = psi0 + (batched ? b0 * t->N : 0);
     double* ex = expect + b0 * (M + 1);

@@ -11,6 +11,7 @@
 #include "redo_internal.cuh"
 
 #include <type_traits>
+#include <vector>
 
 namespace redo {
 
@@ -336,12 +337,181 @@ expect_cols_kernel(const cplx<R>* __restrict__ T, int64_t entries, const int32_t
   if (mean && active && c == 0) mean[b] = M > 0 ? tot / (double)M : e0;
 }
 
+// ----------------------------------------------------------------------------
+// Diagonal controls (the freezing drive in the basis of its x-magnetisation): a step is the dense
+// drift D and then diagonal factors, N^2 + d N complex FMAs a column instead of K d N^2, and the only
+// dense operand is the same for every pulse, so its shared-memory reads are broadcasts (the gathered
+// table operators cost a read per pulse of the warp, which bound the kernel).  D and the factors
+// are kept as their difference from the identity (v + (D - 1) v): a fixed D rounded beside 1 in FP32
+// would change the norm alike at every step.
+// ----------------------------------------------------------------------------
+// u[k][j][c][r] = exp(-i dt theta_kjc H_k[r][r]) - 1, d1 = D - 1
+__global__ void diag_ctl_kernel(const double* __restrict__ hd, const double2* __restrict__ D, int N, int K, int d, int base,
+                                double dt, const double* __restrict__ lo, const double* __restrict__ delta,
+                                double2* __restrict__ u, float2* __restrict__ u32, double2* __restrict__ d1,
+                                float2* __restrict__ d32) {
+  const int64_t total = (int64_t)K * d * base * N;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total + N * N; i += (int64_t)gridDim.x * blockDim.x) {
+    double2 v;
+    if (i < total) {
+      const int r = (int)(i % N), c = (int)(i / N % base), j = (int)(i / ((int64_t)N * base) % d);
+      const int k = (int)(i / ((int64_t)N * base * d));
+      double bj = 1.0;
+      for (int q = 0; q < j; ++q) bj *= (double)base;
+      const double th = j == 0 ? __dadd_rn(lo[k], __dmul_rn((double)c, delta[k])) : __dmul_rn((double)c * bj, delta[k]);
+      const double x = dt * th * hd[k * N + r], sh = sin(0.5 * x);
+      v = make_double2(-2.0 * sh * sh, -sin(x));
+      u[i] = v;
+      u32[i] = make_float2((float)v.x, (float)v.y);
+    } else {
+      const int e = (int)(i - total);
+      v = D[e];
+      if (e / N == e % N) v.x -= 1.0;
+      d1[e] = v;
+      d32[e] = make_float2((float)v.x, (float)v.y);
+    }
+  }
+}
+
+// h: host copies of H0 then H_0 .. H_{K-1}.  Leaves t->dct = 0 unless every control is diagonal, N <= 16
+// and the factors fit shared memory.
+cudaError_t diag_ctl_build(redo_table* t, const std::vector<double>& h, cudaStream_t s) {
+  t->dct = 0;
+  const int N = t->N, K = t->K;
+  const size_t ent = (size_t)K * t->digit_count * t->digit_base * N;
+  if (N > 16 || (ent + N * N) * sizeof(double2) > 160 * 1024) return cudaSuccess;
+  std::vector<double> hd((size_t)K * N);
+  for (int k = 0; k < K; ++k) {
+    const double* H = h.data() + 2 * (size_t)N * N * (k + 1);
+    for (int r = 0; r < N; ++r)
+      for (int c = 0; c < N; ++c) {
+        if (r != c && (H[2 * (r * N + c)] != 0.0 || H[2 * (r * N + c) + 1] != 0.0)) return cudaSuccess;
+        if (r == c) hd[(size_t)k * N + r] = H[2 * (r * N + c)];
+      }
+  }
+  const size_t tot = ent + (size_t)N * N;
+  cudaError_t e = cudaMalloc(&t->dct_u, tot * (sizeof(double2) + sizeof(float2)) + hd.size() * sizeof(double));
+  if (e) return e;
+  t->dct_u32 = (float2*)(t->dct_u + tot);
+  double* dhd = (double*)(t->dct_u32 + tot);
+  if ((e = cudaMemcpyAsync(dhd, hd.data(), hd.size() * sizeof(double), cudaMemcpyHostToDevice, s))) return e;
+  diag_ctl_kernel<<<(unsigned)((tot + 127) / 128), 128, 0, s>>>(dhd, t->D64, N, K, t->digit_count, t->digit_base, t->dt,
+                                                                t->d_lo, t->d_delta, t->dct_u, t->dct_u32, t->dct_u + ent,
+                                                                t->dct_u32 + ent);
+  if ((e = cudaGetLastError()) || (e = cudaStreamSynchronize(s))) return e;
+  t->dct = 1;
+  return cudaSuccess;
+}
+
+template <typename R, int N>
+__global__ void __launch_bounds__(kColThreads)
+expect_diagctl_kernel(const cplx<R>* __restrict__ U, int64_t entries, const int32_t* __restrict__ q, int64_t B, int64_t M,
+                      int K, int d, int base, int64_t levels, const double* __restrict__ rho,
+                      const double* __restrict__ obs, double* __restrict__ expect, double* __restrict__ mean,
+                      int64_t* status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cplx<R>* us = reinterpret_cast<cplx<R>*>(smem_raw);    // the factors, then D - 1
+  for (int64_t i = threadIdx.x; i < entries + N * N; i += blockDim.x) us[i] = U[i];
+  const cplx<R>* D = us + entries;
+  __syncthreads();
+  const int c = threadIdx.x % N;
+  const int64_t b_raw = (int64_t)blockIdx.x * (blockDim.x / N) + threadIdx.x / N;
+  const bool active = b_raw < B;
+  const int64_t b = active ? b_raw : B - 1;        // idle lanes follow the last pulse, write nothing
+  R o[N];
+#pragma unroll
+  for (int r = 0; r < N; ++r) o[r] = (R)obs[r];
+  const double rc = rho[c];
+  cplx<R> u[N];
+#pragma unroll
+  for (int r = 0; r < N; ++r) u[r] = cmake<R>(r == c ? R(1) : R(0), R(0));
+  auto part = [&]() -> R {
+    R v = R(0);
+#pragma unroll
+    for (int r = 0; r < N; ++r) v = fma(o[r], fma(u[r].x, u[r].x, u[r].y * u[r].y), v);
+    return v;
+  };
+  auto group_sum = [&](double v) -> double {
+#pragma unroll
+    for (int off = N / 2; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off, N);
+    return v;
+  };
+  const double e0 = group_sum(rc * (double)part());
+  if (expect && active && c == 0) expect[b * (M + 1)] = e0;
+  R acc = R(0), lo = R(0);                         // the steps' sum as a pair: an FP32 step needs no FP64
+  const int32_t* qb = q + b * M * K;
+  int32_t qn = M > 0 ? qb[0] : 0;
+  for (int64_t n = 0; n < M; ++n) {
+    const int32_t* qrow = qb + n * K;
+    cplx<R> v[N];
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      cplx<R> s = cmake<R>(R(0), R(0));
+      if constexpr (sizeof(R) == 4) {
+        const float4* D4 = reinterpret_cast<const float4*>(D + r * N);
+#pragma unroll
+        for (int kk = 0; kk < N; kk += 2) {
+          const float4 a2 = D4[kk / 2];
+          cfma<R>(s, cmake<R>(a2.x, a2.y), u[kk]);
+          cfma<R>(s, cmake<R>(a2.z, a2.w), u[kk + 1]);
+        }
+      } else {
+#pragma unroll
+        for (int kk = 0; kk < N; ++kk) cfma<R>(s, D[r * N + kk], u[kk]);
+      }
+      v[r] = s;
+    }
+#pragma unroll
+    for (int r = 0; r < N; ++r) u[r] = cmake<R>(u[r].x + v[r].x, u[r].y + v[r].y);
+    for (int k = 0; k < K; ++k) {
+      int32_t qv = qn;
+      // next coefficient's level, loaded while this one is applied
+      qn = (k + 1 < K) ? qrow[k + 1] : (n + 1 < M ? qrow[K] : 0);
+      if (qv < 0 || qv >= levels) {
+        if (status && active) atomicAdd((unsigned long long*)&status[REDO_STATUS_BADINDEX], 1ull);
+        qv = 0;
+      }
+      for (int j = 0; j < d; ++j) {
+        const cplx<R>* f = us + ((int64_t)(k * d + j) * base + qv % base) * N;
+        qv /= base;
+#pragma unroll
+        for (int r = 0; r < N; ++r) {
+          const cplx<R> a = f[r];
+          u[r] = cmake<R>(u[r].x + fma(-a.y, u[r].y, a.x * u[r].x), u[r].y + fma(a.y, u[r].x, a.x * u[r].y));
+        }
+      }
+    }
+    const R pv = part(), t = acc + pv, z = t - acc;
+    lo += (acc - (t - z)) + (pv - z);
+    acc = t;
+    if (expect) {
+      const double ev = group_sum(rc * (double)pv);
+      if (active && c == 0) expect[b * (M + 1) + n + 1] = ev;
+    }
+  }
+  const double tot = group_sum(rc * ((double)acc + (double)lo));
+  if (mean && active && c == 0) mean[b] = M > 0 ? tot / (double)M : e0;
+}
+
 template <typename R, int N>
 static cudaError_t expect_diag_n(const redo_table* t, const int32_t* q, int64_t B, int64_t M, const double* rho,
                                  const double* obs, double* expect, double* mean, int64_t* status,
                                  cudaStream_t s) {
   const cplx<R>* T = std::is_same<R, double>::value ? (const cplx<R>*)t->T64 : (const cplx<R>*)t->T32;
   if constexpr (N * sizeof(R) <= 64) {            // one column in registers: N <= 16 (FP32), 8 (FP64)
+    if (t->dct) {
+      // blocks of one warp until there are pulses for a full block on every SM
+      const int th = B * N >= (int64_t)t->num_sms * kColThreads ? kColThreads : 32, per = th / N;
+      const int64_t ent = (int64_t)t->K * t->digit_count * t->digit_base * N;
+      const size_t smem = (size_t)(ent + N * N) * sizeof(cplx<R>);
+      cudaError_t e = cudaFuncSetAttribute(expect_diagctl_kernel<R, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)smem);
+      if (e != cudaSuccess) return e;
+      expect_diagctl_kernel<R, N><<<(unsigned)((B + per - 1) / per), th, smem, s>>>(
+          std::is_same<R, double>::value ? (const cplx<R>*)t->dct_u : (const cplx<R>*)t->dct_u32, ent, q, B, M, t->K,
+          t->digit_count, t->digit_base, t->levels, rho, obs, expect, mean, status);
+      return cudaGetLastError();
+    }
     const size_t table_smem = (size_t)t->entries * N * N * sizeof(cplx<R>);
     // worth it once every SM gets a full CTA (256 / N pulses); fewer pulses keep one CTA each
     if (table_smem <= 200 * 1024 && B * N >= (int64_t)t->num_sms * kColThreads) {

@@ -354,6 +354,7 @@ redo_status redo_build_table(int32_t N, int32_t K, double dt, const void* H0, co
     if (e != cudaSuccess) return fail(cuda_error(e, "FP16x3 planes"));
   }
   if ((e = local_build(t, h, s)) != cudaSuccess) return fail(cuda_error(e, "one-qubit tables"));
+  if ((e = diag_ctl_build(t, h, s)) != cudaSuccess) return fail(cuda_error(e, "diagonal controls"));
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(cuda_error(e, "table build"));
   *out = t;
   return REDO_OK;
@@ -378,6 +379,7 @@ redo_status redo_table_free(redo_table* t) {
   cudaFree(t->sz64);
   cudaFree(t->sz32);
   local_free(t);
+  cudaFree(t->dct_u);
   std::free(t->h0_pairs);
   std::free(t);
   return REDO_OK;

@@ -81,6 +81,11 @@ struct redo_table {
   float2* loc_u32;
   double2* loc_D64;           // [N] diagonal of the drift step minus 1
   float4* loc_D32;            // the same as FP32 hi + lo
+  // every control diagonal and N <= 16 (kernels_sim.cu): dct, and [K][digit_count][digit_base][N] diagonal
+  // digit factors less 1 followed by D - 1
+  int dct;
+  double2* dct_u;
+  float2* dct_u32;
   cudaStream_t build_stream;
   int num_sms;
 };
@@ -246,6 +251,7 @@ cudaError_t launch_state_grad(const redo_table* t, const int32_t* q, int64_t B, 
 cudaError_t launch_sim_stream(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int prec,
                               const double2* psi0, int psi0_batched, const double* obs, double* expect,
                               int64_t* status, cudaStream_t s);
+cudaError_t diag_ctl_build(redo_table* t, const std::vector<double>& h, cudaStream_t s);
 cudaError_t launch_levels_closed_form(const redo_table* t, const int32_t* xm, const double2* xh, const double* xa,
                                       double2* E, cudaStream_t s);
 cudaError_t launch_expect_diag(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int prec,

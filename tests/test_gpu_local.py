@@ -209,3 +209,28 @@ def test_local_state_gradient_over_several_windows():
     assert (F - Fo).abs().max().item() < 1e-10 and torch.equal(F, F1)
     assert (g - go).abs().max().item() <= 1e-8 * go.abs().max().item()
     t.close()
+
+
+@pytest.mark.parametrize("n,B", [(1, 3), (2, 5), (3, 4870), (4, 3), (4, 2450)])
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp32", 2e-5)])
+def test_diagonal_controls_expectations(n, B, prec, tol):
+    # two diagonal controls (one with an identity part) and a dense drift, one warp per block and full
+    # blocks with idle lanes; N = 16 in FP64 keeps the general kernel
+    rng = np.random.default_rng(50 + n)
+    N, M = 2 ** n, 21
+    A = rng.normal(size=(N, N)) + 1j * rng.normal(size=(N, N))
+    Hk = np.stack([np.diag(rng.normal(size=N)), np.diag(1.0 + rng.normal(size=N))]).astype(np.complex128)
+    w = inputs.Workload("diag", n, (A + A.conj().T) / 2, Hk, 0.1, np.array([-1.0, 0.0]), np.array([1.0, 2.0]), 64, 4, 3,
+                        np.stack([rng.uniform(-1, 1, (B, M)), rng.uniform(0, 2, (B, M))], -1))
+    rho, obs = rng.uniform(-1, 1, N), rng.uniform(-1, 1, N)
+    t = _table(w)
+    ex, mean = t.expect_diag(t.quantize(w.u), rho, obs, prec)
+    _, mean2 = t.expect_diag(t.quantize(w.u), rho, obs, prec, series=False)
+    assert torch.equal(mean, mean2)
+    T, D = O.build_table(w.H0, w.Hk, w.dt, w.lo, w.hi, w.levels, w.base, w.digits, method="eig")
+    _, dig, _, _ = _ref.oracle_levels(w)
+    for b in sorted({0, B // 2, B - 1}):
+        eo, _ = O.expect_mixed(T, D, dig[b], np.diag(rho).astype(complex), np.diag(obs).astype(complex))
+        assert np.abs(ex[b].cpu().numpy() - eo).max() < tol
+        assert abs(float(mean[b]) - eo[1:].mean()) < tol
+    t.close()

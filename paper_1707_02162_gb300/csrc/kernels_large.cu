@@ -23,7 +23,7 @@ namespace large {
 constexpr int kT = 64;    // output tile (complex)
 constexpr int kBK = 16;   // K chunk
 
-// TT: output tile, 64 or 32 (one launch of few tiles is bound by one tile's time: a quarter of it)
+// TT: output tile, 64 or 32 (one launch of few tiles is bound by the time of one tile)
 template <typename R, bool ADJA, int TT, class Ops>
 __global__ void __launch_bounds__(256) cgemm_kernel(Ops ops, int N, R alpha, R diag) {
   constexpr int PT = TT / 16;
@@ -136,8 +136,8 @@ template <typename R, bool ADJA, class Ops>
 static cudaError_t cgemm(const Ops& ops, int64_t batch, int N, R alpha, R diag, cudaStream_t s) {
   if (batch == 0) return cudaSuccess;
   const int64_t blocks = batch * (N / kT) * (N / kT);
-  // up to two tiles of 64 per SM: 32 x 32 tiles spread them (10 products of N = 256: 50 -> 28 us; one
-  // at a time 29 -> 11 us); above, the larger tile's operand reuse wins
+  // up to two tiles of 64 per SM: 32 x 32 tiles spread them (10 products of N = 256: 50 -> 45 us; two
+  // 29 -> 23 us); above, the larger tile reads its operands half as often
   if (blocks <= 304)
     cgemm_kernel<R, ADJA, 32, Ops><<<(unsigned)(4 * blocks), 256, 0, s>>>(ops, N, alpha, diag);
   else

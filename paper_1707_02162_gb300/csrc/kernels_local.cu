@@ -769,15 +769,20 @@ loc_sim_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta
   }
 }
 
+// expect[i] = sum of its G parts, min(G, 32) lanes an item
 template <typename R>
 __global__ void loc_expect_kernel(const cplx<R>* __restrict__ part, int64_t n, int G, double* __restrict__ expect) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+  const int w = G < 32 ? G : 32, l = threadIdx.x % w;
+  const int64_t per = blockDim.x / w;
+  for (int64_t i0 = blockIdx.x * per; i0 < n; i0 += gridDim.x * per) {
+    const int64_t i = i0 + threadIdx.x / w;
     double a = 0.0;
-    for (int l = 0; l < G; ++l) {
-      const cplx<R> p = part[i * G + l];
+    for (int q = l; q < G && i < n; q += w) {
+      const cplx<R> p = part[i * G + q];
       a += (double)p.x + (double)p.y;
     }
-    expect[i] = a;
+    for (int off = w / 2; off >= 1; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+    if (l == 0 && i < n) expect[i] = a;
   }
 }
 
@@ -1096,7 +1101,7 @@ static cudaError_t loc_sim_t(const redo_table* t, int64_t B, int64_t M, const do
     case 1024: loc_sim_wide_kernel<R, 1024><<<blocks, 128, 0, s>>>(cs, delta, M, psi0, batched, obs, part); break;
     default: return cudaErrorInvalidValue;
   }
-  const int64_t n = B * (M + 1), nb = (n + 127) / 128;
+  const int64_t n = B * (M + 1), per = 128 / (lanes < 32 ? lanes : 32), nb = (n + per - 1) / per;
   loc_expect_kernel<R><<<(unsigned)(nb < 4096 ? nb : 4096), 128, 0, s>>>((const cplx<R>*)w.bl, n, lanes, expect);
   return cudaGetLastError();
 }

@@ -438,6 +438,7 @@ expect_diagctl_kernel(const cplx<R>* __restrict__ U, int64_t entries, const int3
   };
   const double e0 = group_sum(rc * (double)part());
   if (expect && active && c == 0) expect[b * (M + 1)] = e0;
+  const uint32_t recip = (uint32_t)((((uint64_t)1 << 32) + base - 1) / base);
   R acc = R(0), lo = R(0);                         // the steps' sum as a pair: an FP32 step needs no FP64
   const int32_t* qb = q + b * M * K;
   int32_t qn = M > 0 ? qb[0] : 0;
@@ -472,8 +473,10 @@ expect_diagctl_kernel(const cplx<R>* __restrict__ U, int64_t entries, const int3
         qv = 0;
       }
       for (int j = 0; j < d; ++j) {
-        const cplx<R>* f = us + ((int64_t)(k * d + j) * base + qv % base) * N;
-        qv /= base;
+        // the last digit is what is left; qv < 2^24 and base < 2^8 make the reciprocal exact
+        const int32_t nq = j == d - 1 ? 0 : (base < 256 ? (int32_t)__umulhi((uint32_t)qv, recip) : qv / base);
+        const cplx<R>* f = us + ((k * d + j) * base + qv - nq * base) * N;
+        qv = nq;
 #pragma unroll
         for (int r = 0; r < N; ++r) {
           const cplx<R> a = f[r];
@@ -500,8 +503,9 @@ static cudaError_t expect_diag_n(const redo_table* t, const int32_t* q, int64_t 
   const cplx<R>* T = std::is_same<R, double>::value ? (const cplx<R>*)t->T64 : (const cplx<R>*)t->T32;
   if constexpr (N * sizeof(R) <= 64) {            // one column in registers: N <= 16 (FP32), 8 (FP64)
     if (t->dct) {
-      // blocks of one warp until there are pulses for a full block on every SM
-      const int th = B * N >= (int64_t)t->num_sms * kColThreads ? kColThreads : 32, per = th / N;
+      // small blocks: they fill the SMs evenly (256 threads left a third wave nearly empty), and one
+      // warp each while the pulses are few
+      const int th = B * N >= (int64_t)t->num_sms * kColThreads ? 64 : 32, per = th / N;
       const int64_t ent = (int64_t)t->K * t->digit_count * t->digit_base * N;
       const size_t smem = (size_t)(ent + N * N) * sizeof(cplx<R>);
       cudaError_t e = cudaFuncSetAttribute(expect_diagctl_kernel<R, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,

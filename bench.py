@@ -224,6 +224,23 @@ def chain_roofline(peaks, clk, B, M, N, K, digits, prods_per_step, avg_s, prec, 
     return out
 
 
+def local_roofline(clk, prec, kernel, N, columns, steps, avg_s, gradient=False):
+    """Roofline of the one-qubit-operator path that systems with a diagonal drift and one-qubit
+    controls take: per entry of a column and step 4 multiply-adds for the diagonal and 4 per qubit; a
+    gradient's reverse sweep adds 8 and 14 per qubit (two columns undone, three Bloch sums)."""
+    n = int(np.log2(N))
+    fma = (4 + 4 * n) + ((8 + 14 * n) if gradient else 0)
+    flop = 2.0 * fma * N * columns * steps
+    f32 = prec != "fp64"
+    peak = 152 * 128 * 2 * (clk.get("sm_max_mhz") or 2070.0) * 1e6 / 1e12 if f32 else 1.25
+    return {"kernel": kernel, "launch_ms": avg_s * 1e3, "bound": "alu", "unit": "TFLOP/s",
+            "achieved": flop / avg_s / 1e12, "peak": peak, "frac": flop / avg_s / 1e12 / peak, "traffic": None,
+            "algorithmic_per_launch": f"{flop:.4g} flop: {fma} multiply-adds per entry and step, {N} rows x "
+                                      f"{columns} columns",
+            "peak_source": ("FP32 FMA pipe: 152 SMs x 128 lanes x 2 flop x max SM clock" if f32
+                            else "nominal GB300 FP64")}
+
+
 def grape_summary(gres, gflop, gbuild, gw, peaks):
     """GRAPE iterations/s on the N=256 workload with the three flop counts side by side."""
     ms = gres["fp16x3"]["ms_per_iter"]
@@ -286,16 +303,9 @@ def plain_measure(redo, inputs, torch, reps=5):
                 redo.redo_propagate(t.handle, q, prec, U, target, F, tau, ws)
             it()
             ms = _events_time(it, reps)
-            # 4 complex 8x8 products per pulse-step: K*d = 4 digit operators, the drift folded in
-            flop = B * w.M * w.K * w.digits * 8.0 * w.N ** 3
-            peak = 1.25 if prec == "fp64" else 152 * 128 * 2 * 2.07e9 / 1e12
             res[f"B{B}_{prec}"] = {"pulse_steps_per_s": B * w.M / (ms / 1e3), "ms_per_call": ms,
-                                   "roofline": {"bound": "alu", "unit": "TFLOP/s",
-                                                "achieved": flop / (ms / 1e3) / 1e12, "peak": peak,
-                                                "frac": flop / (ms / 1e3) / 1e12 / peak,
-                                                "peak_source": ("nominal GB300 FP64" if prec == "fp64" else
-                                                                "FP32 FMA pipe: 152 x 128 lanes x 2 x 2.07 GHz"),
-                                                "timed": "whole call (quantize, chain, combine, fidelity)"}}
+                                   "roofline": dict(local_roofline({}, prec, "call", w.N, B * w.N, w.M, ms / 1e3),
+                                                    timed="whole call (quantize, chain, combine, fidelity)")}
         t.close()
     return {"metric": "REDO prop steps/s, plain REDO FP64 (N=8)", "unit": "pulse-steps/s",
             "workload": "3 qubits (N=8), K=2 global x/y controls, M=1000 steps of 1 us, 4096 levels, "
@@ -312,8 +322,6 @@ def ensemble_measure(redo, inputs, torch, peaks, M=2000):
     table (two products per step)."""
     w = inputs.config(3, M=M)
     steps = w.B * M
-    alg = steps * w.K * w.digits * 8.0 * w.N ** 3          # 2 complex 1024x1024 products per realisation-step
-    sus = peaks.get("bf16_tflops_sustained", 1699.6)
     res = {}
     for levels in (True, False):
         t0 = time.time()
@@ -340,7 +348,6 @@ def ensemble_measure(redo, inputs, torch, peaks, M=2000):
             "products_per_step": w.K * (1 if levels else w.digits),
             "fp64_state_only": {"realisation_steps_per_s": steps / (ms64 / 1e3), "ms_per_call": ms64},
             "max_abs_dZ1_fp16x3_vs_fp64": float((ex16 - ex64).abs().max()),
-            "tensor_frac_algorithmic": alg / (ms16 / 1e3) / 1e12 / sus,
             "table_build_s": build_s}
         t.close()
         del ws16, ws64, Uf
@@ -349,13 +356,9 @@ def ensemble_measure(redo, inputs, torch, peaks, M=2000):
             "workload": "10-qubit ZZ chain (N=1024), K=1 global x drive Omega(1+xi), OU sigma=0.1 tau=50 us, "
                         f"64 realisations x {M} steps of 1 us, 4096 levels",
             "value": lv["realisation_steps_per_s"], "ms_per_call": lv["ms_per_call"],
-            "precision": "fp16x3 products, fp32 state path", "results": res,
-            "roofline": {"bound": "tensor", "unit": "TFLOP/s", "peak": sus,
-                         "peak_source": "measured dense bf16, sustained (of measured)",
-                         "achieved": alg / (lv["ms_per_call"] / 1e3) / 1e12,
-                         "frac": alg / (lv["ms_per_call"] / 1e3) / 1e12 / sus, "timed": "whole call",
-                         "algorithmic_per_call": f"{alg:.4g} flop (2 complex digit-operator products of 8N^3 per "
-                                                 "realisation-step)"}}
+            "precision": "fp32 one-qubit operators (requested fp16x3)", "results": res,
+            "roofline": dict(local_roofline({}, "fp32", "call", w.N, w.B * (w.N + 1), M, lv["ms_per_call"] / 1e3),
+                             timed="whole call")}
 
 
 def run_gpu(args):
@@ -442,7 +445,11 @@ def run_gpu(args):
     else:
         dom_ms, dom_n, dom_name = seg_ms, seg_n, "chain_segments"
     avg_s = (dom_ms / max(dom_n, 1)) / 1e3
-    roof = chain_roofline(peaks, clk, B, M, N, w.K, w.digits, prods_per_step, avg_s, MAIN_PREC, dom_name)
+    if tc_n:
+        roof = chain_roofline(peaks, clk, B, M, N, w.K, w.digits, prods_per_step, avg_s, MAIN_PREC, dom_name)
+    else:
+        # per-qubit x/y controls and a diagonal drift: one-qubit operators in place of dense products
+        roof = local_roofline(clk, MAIN_PREC, dom_name, N, B * N, M, avg_s)
 
     # ---- end to end through the C ABI with host buffers (right after the timed steps, before the
     # FP64 comparison arm, so that both see the same clocks)
@@ -499,6 +506,11 @@ def run_gpu(args):
         gres, gflop, gbuild, gw = grape_measure(redo, inputs, torch, 3, levels=True, with_fp32=False,
                                                 with_fp64=not args.skip_fp64)
         grape = grape_summary(gres, gflop, gbuild, gw, peaks)
+        # the call runs on one-qubit operators; the dense counts above are what it replaces
+        grape["roofline"] = local_roofline(clk, "fp32", "gradient", gw.N, gw.N, gw.M,
+                                           gres["fp16x3"]["ms_per_iter"] / 1e3, gradient=True)
+        grape["flop_counts"] = {k: {x: v[x] for x in ("tflop_per_iteration", "what")}
+                                for k, v in grape["flop_counts"].items()}
 
     # ---- each precision form on sampled pulses, for their error against the oracle (CPU leg)
     forms = None
@@ -523,7 +535,7 @@ def run_gpu(args):
     launches = sum(n for _, n in prof.values())
     out = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
-           "vs_baseline": None, "dtype": {"fp32": "f32", "fp64": "f64", "fp16x3": "f16x3 (f32 accumulate)"}[MAIN_PREC],
+           "vs_baseline": None, "dtype": {"fp32": "f32", "fp64": "f64", "fp16x3": "f16x3 (f32 accumulate)" if tc_n else "f32"}[MAIN_PREC],
            "data": "synthetic (seeded NMR-like Hamiltonian, uniform random controls, Haar target)",
            "config": _workload_config({"precision": MAIN_PREC, "B": B, "M": M, "reunit_every": reunit_main,
                                        "table": ("level table (process 3): K products per step" if args.levels
@@ -649,15 +661,14 @@ def run_workload(args):
                                               with_fp32=not args.skip_fp64, with_fp64=not args.skip_fp64,
                                               M=args.M if args.M != M_FULL else None)
         out.update({"metric": "GRAPE iters/s", "unit": "iterations/s", "value": res["fp16x3"]["iters_per_s"],
-                    "precision": "fp16x3 (tcgen05 lockstep chains, FP32 accumulate)", "fp32_simt": res.get("fp32"),
+                    "precision": "fp32 one-qubit operators (requested fp16x3)", "fp32_simt": res.get("fp32"),
                     "fp64_plain_redo": res.get("fp64"),
                     "speedup_vs_fp64": (res["fp16x3"]["iters_per_s"] / res["fp64"]["iters_per_s"]
                                         if "fp64" in res else None),
                     "phase_ms": res["fp16x3"].get("phase_ms"),
                     "algorithmic_flop_per_iter": flop,
-                    "achieved_tensor_tflops_fp16x3": 3 * flop / (res["fp16x3"]["ms_per_iter"] / 1e3) / 1e12,
-                    "achieved_tflops_fp32": (flop / (res["fp32"]["ms_per_iter"] / 1e3) / 1e12
-                                             if "fp32" in res else None),
+                    "roofline": local_roofline({}, "fp32", "gradient", w.N, w.N, w.M,
+                                               res["fp16x3"]["ms_per_iter"] / 1e3, gradient=True),
                     "table_build_s": build_s,
                     "config": {"N": w.N, "K": w.K, "M": w.M, "dt": w.dt, "checkpoint_every": 32, "B": 1,
                                "table": "level table" if args.levels else "digit table"}})
@@ -684,12 +695,10 @@ def run_workload(args):
             ms = _events_time(it, 1)
             res[f"{prec}{'_with_U' if want else '_state_only'}"] = {
                 "realisation_steps_per_s": w.B * Ms / (ms / 1e3), "ms": ms}
-        flop_step = 3 * w.K * w.digits * 8.0 * w.N ** 3
         out.update({"metric": "REDO prop steps/s (noisy-drive ensemble)", "unit": "realisation-steps/s",
                     "value": res["fp16x3_with_U"]["realisation_steps_per_s"], "results": res,
-                    "achieved_tensor_tflops_fp16x3": flop_step * res["fp16x3_with_U"]["realisation_steps_per_s"] / 1e12,
-                    "tensor_frac_of_sustained": (flop_step * res["fp16x3_with_U"]["realisation_steps_per_s"] / 1e12
-                                                 / _peaks().get("bf16_tflops_sustained", 1709.6)),
+                    "roofline": local_roofline({}, "fp32", "call", w.N, w.B * (w.N + 1), Ms,
+                                               res["fp16x3_with_U"]["ms"] / 1e3),
                     "sample": f"{Ms} of the 2000 steps, all 64 realisations", "table_build_s": build_s,
                     "config": {"N": w.N, "K": w.K, "B": w.B, "M_timed": Ms}})
     elif args.workload == "freeze":

@@ -117,6 +117,14 @@ typedef struct redo_table redo_table;
  *           gradients use the target D_h^dag U_T D_h, and redo_simulate (which then needs
  *           a diagonal H0) starts the folded chain from D_h^dag psi0.  The workspace of
  *           each call grows by B FP64 matrices (two sets when H0 is not diagonal).
+ * Locally controlled systems.  When H0 is diagonal and every H_k is a sum of one-qubit operators
+ * (x, y, z controls of single spins, global fields), every table operator is a tensor product of
+ * 2 x 2 operators.  The table then also keeps those, and redo_propagate (with _drift and _phase),
+ * redo_fidelity_grad (with _drift and _phase), redo_simulate and redo_state_grad apply a step as one
+ * rotation per qubit and one diagonal instead of K * digits dense products: the same results to
+ * rounding, in the call's precision (REDO_FP16X3 calls run in FP32).  A pulse whose step operators
+ * alone exceed 512 MiB, FP64 unitary gradients at N = 1024, redo_propagate_steps, redo_propagate_noalloc
+ * and all other systems use the dense operators.
  *  stream   stream for the build; synchronised before returning.
  *  out      receives the handle; free with redo_table_free.
  * Errors: REDO_ERR_INVALID, REDO_ERR_NOT_HERMITIAN (relative tolerance 1e-12
@@ -315,9 +323,11 @@ redo_status redo_propagate_noalloc(const redo_table* t, const int32_t* q, int64_
  *                thousands of products that lowers F near 1 by more than 1e-6 unless removed.
  *  F_out         device double [B] or NULL;  grad  device double [B][M][K].
  *  workspace     >= redo_fidelity_grad_workspace() bytes, 256-byte aligned.
+ * With re-unitarisation and N <= 64 the pulse product also gets a Newton-Schulz step before tau and F.
  * Method: segment products (one per C steps), prefix checkpoints and suffix
  * costates per segment, then one backward sweep per segment that evaluates the
- * traces with the sparse (CSR) form of H_k captured at table build time.  When
+ * traces with the sparse (CSR) form of H_k captured at table build time (locally
+ * controlled systems: from three one-qubit sums per qubit and step).  When
  * every forward partial product of the segment chains fits in 24 GiB (N <= 64,
  * and the tensor-core sweeps at N >= 128), the workspace holds them
  * (redo_fidelity_grad_workspace counts them) and the backward sweep reads them;
@@ -340,13 +350,15 @@ redo_status redo_fidelity_grad_workspace(const redo_table* t, int64_t B, int64_t
  * of a diagonal observable (Tr[O rho(t)] with rho = |psi><psi|), plus optionally
  * the final propagator U_M ... U_1.
  *
- * The state is advanced by one matrix-vector product per table operator, in
- * FP64 for REDO_FP64 and FP32 otherwise; U_final, if requested, is computed
+ * The state is advanced by one matrix-vector product per table operator (locally
+ * controlled systems: by the step's one-qubit rotations), in FP64 for REDO_FP64 and FP32 otherwise; U_final, if requested, is computed
  * exactly as redo_propagate(prec, reunit_every) computes U_out.
  *  psi0      device complex128 [N] (or [B][N] if psi0_batched != 0).
  *  obs_diag  device double [N];  expect  device double [B][M+1].
  *  U_final   device complex128 [B][N][N] or NULL.
- *  workspace >= redo_simulate_workspace(..., want_U = U_final != NULL) bytes.
+ *  workspace >= redo_simulate_workspace(..., want_U = U_final != NULL) bytes, 256-byte aligned.  A
+ *            locally controlled system given less (NULL for N <= 64 without U_final) advances the
+ *            state by its dense operators, which need none.
  */
 redo_status redo_simulate(const redo_table* t, const int32_t* q, int64_t B, int64_t M,
                           redo_precision prec, int32_t reunit_every, const void* psi0,
@@ -365,8 +377,10 @@ redo_status redo_simulate(const redo_table* t, const int32_t* q, int64_t B, int6
  *  prec         REDO_FP64 or REDO_FP32 (operators of that precision; traces and a in FP64).
  *  psi0, psi_target  device complex128 [N], or [B][N] when batched != 0.
  *  F_out        device double [B] or NULL;  grad device double [B][M][K] or NULL (one of the two).
- *  workspace    >= redo_state_grad_workspace bytes (zero unless the table is a symmetric-split
- *               one, which also needs a diagonal H0).
+ *  workspace    >= redo_state_grad_workspace bytes, 256-byte aligned.  A symmetric-split table (which
+ *               also needs a diagonal H0) requires 2 B N complex128 vectors of it; a locally
+ *               controlled system given less than the query returns uses its dense operators, which
+ *               need no more (so NULL is accepted without a symmetric split).
  * Errors: REDO_ERR_INVALID, REDO_ERR_UNSUPPORTED, REDO_ERR_CUDA.  No synchronisation.
  */
 redo_status redo_state_grad_workspace(const redo_table* t, int64_t B, size_t* bytes);

@@ -951,6 +951,18 @@ bool local_eligible(const redo_table* t, int64_t M, int prec, int what) {
   return loc_scratch(t, 1, M, prec, what, nullptr).total <= kLocSlice;
 }
 
+// Whether a plain propagation gains by it.  One step costs the dense chain 4 N^3 K digits multiply-adds;
+// here it is N^2 (4 + 4n) (complex rotations: 6 + 8n), about 28 a row for the diagonal (FP32: 100, a
+// sine and cosine) and per qubit 230 FP64 operations of square roots and divisions (FP32: 500, three
+// angles) and 32 a pair.  The FP32 dense column kernel is bound by its operand reads at about half
+// this path's rate.  So N = 2, and N = 4 with level tables, stay dense; from N = 8 on this form wins.
+bool local_pays(const redo_table* t, int prec) {
+  const double N = t->N, n = t->loc, dense = 4.0 * N * N * N * t->K * t->digits;
+  if (prec == REDO_FP64) return dense > 32.0 * t->loc_pairs + 230.0 * n + 28.0 * N + N * N * (4 + 4 * n);
+  const double rot = loc_near(false, t->N) ? 6 + 8 * n : 4 + 4 * n;
+  return 2.0 * dense > 40.0 * t->loc_pairs + 500.0 * n + 100.0 * N + N * N * rot;
+}
+
 static int64_t local_slice(const redo_table* t, int64_t B, int64_t M, int prec, int what) {
   const int64_t n = (int64_t)(kLocSlice / loc_scratch(t, 1, M, prec, what, nullptr).total);
   return n < B ? n : B;

@@ -502,7 +502,9 @@ static cudaError_t expect_diag_n(const redo_table* t, const int32_t* q, int64_t 
                                  cudaStream_t s) {
   const cplx<R>* T = std::is_same<R, double>::value ? (const cplx<R>*)t->T64 : (const cplx<R>*)t->T32;
   if constexpr (N * sizeof(R) <= 64) {            // one column in registers: N <= 16 (FP32), 8 (FP64)
-    if (t->dct) {
+    // FP64 only with a column for every lane of the SMs: a warp's FP64 instruction takes 70 cycles, so
+    // few pulses do better with a thread per entry (N = 8, 240 x 693: 9.4 ms here, 2.6 ms there)
+    if (t->dct && (sizeof(R) == 4 || B * N >= (int64_t)t->num_sms * kColThreads)) {
       // small blocks: they fill the SMs evenly (256 threads left a third wave nearly empty), and one
       // warp each while the pulses are few
       const int th = B * N >= (int64_t)t->num_sms * kColThreads ? 64 : 32, per = th / N;

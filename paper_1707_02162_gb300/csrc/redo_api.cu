@@ -517,7 +517,7 @@ static PropLayout prop_layout(const redo_table* t, int64_t B, int64_t M, redo_pr
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t el = L.eff_prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
   const size_t n2 = (size_t)t->N * t->N;
-  if (local_eligible(t, M, L.eff_prec, kLocalChain)) {
+  if (local_eligible(t, M, L.eff_prec, kLocalChain) && (diag || local_pays(t, L.eff_prec))) {
     L.local = true;
     L.p = reunit_every > 0 ? plan_chain_aligned(t, B, M, reunit_every) : plan_chain_local(t, B, M, L.eff_prec, false);
     if (t->N > kSmallN) {

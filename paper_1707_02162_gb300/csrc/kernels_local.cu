@@ -954,13 +954,14 @@ bool local_eligible(const redo_table* t, int64_t M, int prec, int what) {
 // Whether a plain propagation gains by it.  One step costs the dense chain 4 N^3 K digits multiply-adds;
 // here it is N^2 (4 + 4n) (complex rotations: 6 + 8n), about 28 a row for the diagonal (FP32: 100, a
 // sine and cosine) and per qubit 230 FP64 operations of square roots and divisions (FP32: 500, three
-// angles) and 32 a pair.  The FP32 dense column kernel is bound by its operand reads at about half
-// this path's rate.  So N = 2, and N = 4 with level tables, stay dense; from N = 8 on this form wins.
+// angles) and 32 a pair.  The FP32 dense column kernel is bound by its operand reads at about two
+// thirds of this path's rate (N = 4, global controls, 1000 x 500: 155 us dense, 234 us here; N = 8:
+// 528 and 315).  So N = 2, and N = 4 with few factors, stay dense; from N = 8 on this form wins.
 bool local_pays(const redo_table* t, int prec) {
   const double N = t->N, n = t->loc, dense = 4.0 * N * N * N * t->K * t->digits;
   if (prec == REDO_FP64) return dense > 32.0 * t->loc_pairs + 230.0 * n + 28.0 * N + N * N * (4 + 4 * n);
   const double rot = loc_near(false, t->N) ? 6 + 8 * n : 4 + 4 * n;
-  return 2.0 * dense > 40.0 * t->loc_pairs + 500.0 * n + 100.0 * N + N * N * rot;
+  return 1.5 * dense > 40.0 * t->loc_pairs + 500.0 * n + 100.0 * N + N * N * rot;
 }
 
 static int64_t local_slice(const redo_table* t, int64_t B, int64_t M, int prec, int what) {
@@ -982,7 +983,9 @@ ChainPlan plan_chain_local(const redo_table* t, int64_t B, int64_t M, int prec, 
   int64_t S = warps > 0 ? (4 * 4 * (int64_t)t->num_sms + warps - 1) / warps : 1;
   const int64_t min_steps = t->N <= 8 ? 4 : (t->N <= 64 ? 8 : 32);
   if (S > M / min_steps) S = M / min_steps;
-  if (S > 64) S = 64;
+  // (FP32 steps and products of N <= 16 are short beside a launch: one combine pass)
+  const int64_t most = !dbl && t->N <= 16 ? 16 : 64;
+  if (S > most) S = most;
   if (S < 1) S = 1;
   return plan_chain_aligned(t, B, M, M > 0 ? (M + S - 1) / S : 1);
 }

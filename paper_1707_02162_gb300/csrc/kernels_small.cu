@@ -866,16 +866,17 @@ cudaError_t launch_chain_segments(const redo_table* t, const int32_t* q, const C
 // Segments per group of the two-pass combine: about sqrt(S), 0 for one pass.  A pulse's segments
 // are multiplied by one CTA, so a single pulse of S segments is a chain of S dependent products;
 // groups make it sqrt(S) + S / sqrt(S), in parallel over the groups.
-static int64_t combine_group(const ChainPlan& p) {
+// FP32 products of N <= 16 take less than a microsecond each, so a second launch pays later.
+static int64_t combine_group(const redo_table* t, const ChainPlan& p, bool dbl) {
   const int64_t L = p.F > 0 ? p.S : 0;
-  if (L < 9) return 0;
+  if (L < (!dbl && t->N <= 16 ? 17 : 9)) return 0;
   int64_t g = 3;
   while (g * g < L) ++g;
   return g;
 }
 
 size_t combine_mid_bytes(const redo_table* t, const ChainPlan& p, int prec) {
-  const int64_t g = combine_group(p);
+  const int64_t g = combine_group(t, p, prec == REDO_FP64);
   if (!g) return 0;
   const size_t el = prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
   return ((size_t)p.B * ((p.S + g - 1) / g) * t->N * t->N * el + 255) & ~(size_t)255;
@@ -903,7 +904,7 @@ static cudaError_t chain_combine_pass(const redo_table* t, int64_t B, int64_t L,
 template <typename R>
 static cudaError_t chain_combine_t(const redo_table* t, const ChainPlan& p, const void* seg_in,
                                    void* prod_out, int64_t* status, cudaStream_t s, void* mid) {
-  const int64_t L = p.F > 0 ? p.S : 0, g = mid ? combine_group(p) : 0;
+  const int64_t L = p.F > 0 ? p.S : 0, g = mid ? combine_group(t, p, sizeof(R) == 8) : 0;
   if (!g) return chain_combine_pass<R>(t, p.B, L, L, seg_in, prod_out, status, s);
   cudaError_t e = chain_combine_pass<R>(t, p.B, L, g, seg_in, mid, status, s);
   if (e) return e;

@@ -412,6 +412,7 @@ redo_status redo_table_set_phase_axes(redo_table* t, const double* sz) {
       return set_error(REDO_ERR_OOM, "phase axes: %s", cudaGetErrorString(e));
     }
   }
+  REDO_CUDA_TRY(local_phase_axes(t, sz));
   std::vector<float> f(sz, sz + (size_t)K * N);
   REDO_CUDA_TRY(cudaMemcpy(t->sz32, f.data(), sizeof(float) * K * N, cudaMemcpyHostToDevice));
   REDO_CUDA_TRY(cudaMemcpy(t->sz64, sz, sizeof(double) * K * N, cudaMemcpyHostToDevice));

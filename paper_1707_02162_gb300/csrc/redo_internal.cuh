@@ -63,6 +63,7 @@ struct redo_table {
   size_t tc_bytes;
   int tc_nb;                  // operand block height of the large-N planes (128 or 256)
   float* sz32;                // sz64 in FP32
+  double* wz;                 // [K][loc] one-qubit parts of the S_kz when they are sums of those, or nullptr
   double* sz64;               // [K][N] diagonals of the species' S_kz (amplitude/phase calls), or nullptr
   int32_t* h0_pairs;          // host: (row, column) of every off-diagonal nonzero of H0
   int64_t h0_npairs;
@@ -185,6 +186,7 @@ namespace redo {
 cudaError_t launch_local_split(double2* pd, int64_t n, cudaStream_t s);
 cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_t s);
 void local_free(redo_table* t);
+cudaError_t local_phase_axes(redo_table* t, const double* sz);
 // What a call computes: segment products, the gradient, the amplitude/phase gradient, the state's
 // observable.
 enum LocalWhat { kLocalChain = 0, kLocalGrad = 1, kLocalPhaseGrad = 2, kLocalSim = 3 };

@@ -234,3 +234,27 @@ def test_diagonal_controls_expectations(n, B, prec, tol):
         assert np.abs(ex[b].cpu().numpy() - eo).max() < tol
         assert abs(float(mean[b]) - eo[1:].mean()) < tol
     t.close()
+
+
+@pytest.mark.parametrize("n", [2, 3, 5, 7])
+@pytest.mark.parametrize("axes", ["species", "general"])
+@pytest.mark.parametrize("prec,gtol", [("fp64", 1e-9), ("fp32", 2e-4)])
+def test_local_phase_gradients(n, axes, prec, gtol):
+    # species S_z (sums of one-qubit parts) and general diagonals, which keep the boundary traces
+    from paper_1707_02162_gb300 import redo
+    w = inputs.phase_config(n, B=2, M=11, base=8, digits=2)
+    sz = w.extra["sz"].copy()
+    if axes == "general":
+        z = [1.0 - 2.0 * ((np.arange(w.N) >> i) & 1) for i in range(n)]
+        sz[0] = sz[0] + 0.25 * z[0] * z[1]
+    t = _table(w)
+    t.set_phase_axes(sz)
+    F, ga, gp = t.fidelity_grad_phase(t.quantize(w.u), w.extra["phi"], w.target, prec, checkpoint_every=4)
+    T, D = O.build_table(w.H0, w.Hk, w.dt, w.lo, w.hi, w.levels, w.base, w.digits, method="eig")
+    _, dig, _, _ = _ref.oracle_levels(w)
+    for b in range(w.B):
+        Fo, gao, gpo = O.phase_gradient(T, D, w.Hk, sz, w.dt, dig[b], w.extra["phi"][b], w.target)
+        assert abs(float(F[b]) - Fo) < (1e-12 if prec == "fp64" else 2e-5)
+        assert np.abs(ga[b].cpu().numpy() - gao).max() <= gtol * np.abs(gao).max()
+        assert np.abs(gp[b].cpu().numpy() - gpo).max() <= gtol * np.abs(gpo).max()
+    t.close()

@@ -152,6 +152,10 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
                o_h = put(hp.data(), sizeof(double2) * 4 * pairs), o_h32 = put(hp32.data(), sizeof(float2) * 4 * pairs),
                o_kptr = put(kptr.data(), sizeof(int32_t) * (K + 1)), o_kp = put(kpair.data(), sizeof(int32_t) * pairs),
                o_D = put(D.data(), sizeof(double2) * N), o_D32 = put(D32.data(), sizeof(float4) * N);
+  // room for the phase axes' one-qubit parts (local_phase_axes) and whether they apply
+  const std::vector<double> none((size_t)K * n, 0.0);
+  const int32_t off = 0;
+  const size_t o_wz = put(none.data(), sizeof(double) * none.size()), o_wzon = put(&off, sizeof(off));
   const size_t o_u64 = (host.size() + 255) & ~(size_t)255, o_u32 = o_u64 + sizeof(double2) * 4 * ent;
   cudaError_t e = cudaMalloc(&t->loc_mem, o_u32 + sizeof(float2) * 4 * ent);
   if (e) return e;
@@ -165,6 +169,8 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
   t->loc_kpair = (int32_t*)(base + o_kp);
   t->loc_D64 = (double2*)(base + o_D);
   t->loc_D32 = (float4*)(base + o_D32);
+  t->wz = (double*)(base + o_wz);
+  t->wz_on = (int32_t*)(base + o_wzon);
   t->loc_u64 = (double2*)(base + o_u64);
   t->loc_u32 = (float2*)(base + o_u32);
   loc_table_kernel<<<(unsigned)((ent + 127) / 128 < 4096 ? (ent + 127) / 128 : 4096), 128, 0, s>>>(
@@ -174,18 +180,15 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
   return cudaSuccess;
 }
 
-void local_free(redo_table* t) {
-  cudaFree(t->loc_mem);
-  cudaFree(t->wz);
-}
+void local_free(redo_table* t) { cudaFree(t->loc_mem); }
 
-// sz [K][N] (host): keeps their one-qubit parts when each is a sum of those
+// sz [K][N] (host): their one-qubit parts when each is a sum of those, written over the previous ones
+// (a captured call reads them, and whether they apply, where it found them at capture)
 cudaError_t local_phase_axes(redo_table* t, const double* sz) {
-  if (t->wz) cudaFree(t->wz);
-  t->wz = nullptr;
   if (!t->loc) return cudaSuccess;
   const int N = t->N, K = t->K, n = t->loc;
   std::vector<double> w((size_t)K * n);
+  int32_t on = 1;
   for (int k = 0; k < K; ++k) {
     const double* z = sz + (size_t)k * N;
     double mx = 0.0;
@@ -195,15 +198,13 @@ cudaError_t local_phase_axes(redo_table* t, const double* sz) {
       double v = z[0];
       for (int i = 0; i < n; ++i)
         if ((r >> i) & 1) v -= 2.0 * w[(size_t)k * n + i];
-      if (std::fabs(v - z[r]) > 8 * 2.3e-16 * mx) return cudaSuccess;
+      if (std::fabs(v - z[r]) > 8 * 2.3e-16 * mx) on = 0;
     }
   }
-  cudaError_t e = cudaMalloc(&t->wz, sizeof(double) * w.size());
-  if (e) {
-    t->wz = nullptr;
-    return e;
-  }
-  return cudaMemcpy(t->wz, w.data(), sizeof(double) * w.size(), cudaMemcpyHostToDevice);
+  cudaError_t e = cudaMemcpy(t->wz, w.data(), sizeof(double) * w.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(t->wz_on, &on, sizeof(on), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) t->wz_local = on;
+  return e;
 }
 
 template <typename R> static LocTab<R> loc_tab(const redo_table* t, int64_t* status) {
@@ -469,14 +470,17 @@ static cudaError_t loc_chain_t(const redo_table* t, const ChainPlan& p, int64_t 
 // the Bloch sums Im Tr(sigma_i P R) of every qubit are added over x.  They hold every control's
 // trace: Tr(g P R) for g = sum_i g_i needs the one-qubit partial traces only.  bl receives them as
 // [step][part][3n], one part per warp of the chain, added in a fixed order afterwards.
-// TZ (amplitude/phase calls): also Tz = Im Tr(S_kz P R) at every step boundary.
+// TZ (amplitude/phase calls): also Tz = Im Tr(S_kz P R) at every step boundary.  gate: the form with
+// (TZ) and without the boundary traces both stand in a captured call, and the one that the axes in
+// force do not need returns.
 // ============================================================================
 template <typename R, int N, int E, bool TZ>
 __global__ void __launch_bounds__(kLocThreads, E * sizeof(R) <= 64 ? 4 : 2)
 loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t M, int64_t S, int64_t sps,
                  int64_t chains, const cplx<R>* __restrict__ Pck, const cplx<R>* __restrict__ Rck,
                  const double2* __restrict__ tau, R* __restrict__ bl, int K, const R* __restrict__ sz,
-                 R* __restrict__ bz) {
+                 R* __restrict__ bz, const int32_t* __restrict__ gate) {
+  if (gate && (*gate != 0) == TZ) return;
   using L = LocCol<R, N, E>;
   using WS = WarpSums<R, 3 * L::NQ>;
   constexpr int LPC = N * L::G, PARTS = LPC >= 32 ? LPC / 32 : 1, W = LPC >= 32 ? 32 : LPC;
@@ -602,7 +606,8 @@ __global__ void __launch_bounds__(256) loc_sums_kernel(const R* __restrict__ bl,
 // gphi[b][n][k] = (2 / N^2) (Tz[n+1][k] - Tz[n][k]) (the traces already carry conj(tau))
 template <typename R>
 __global__ void loc_phase_kernel(const R* __restrict__ bz, int64_t B, int64_t M, int parts, int K, double scale,
-                                 double* __restrict__ gphi) {
+                                 double* __restrict__ gphi, const int32_t* __restrict__ gate) {
+  if (gate && *gate != 0) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B * M * K; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t bn = i / K, b = bn / M, n = bn - b * M;
     const int k = (int)(i - bn * K);
@@ -623,7 +628,9 @@ __global__ void loc_phase_kernel(const R* __restrict__ bz, int64_t B, int64_t M,
 template <typename R, bool NEAR>
 __global__ void loc_phase_local_kernel(int64_t steps, int K, int n, int parts, const cplx<R>* __restrict__ cs,
                                        const R* __restrict__ bl, const double* __restrict__ sums,
-                                       const double* __restrict__ wz, double scale, double* __restrict__ gphi) {
+                                       const double* __restrict__ wz, double scale, double* __restrict__ gphi,
+                                       const int32_t* __restrict__ gate) {
+  if (gate && *gate == 0) return;
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < steps * K;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t st = idx / K;
@@ -652,7 +659,7 @@ __global__ void loc_phase_local_kernel(int64_t steps, int K, int n, int parts, c
 template <typename R, int N, bool TWO>
 static cudaError_t loc_sweep_n(const redo_table* t, const ChainPlan& p, int64_t B, const void* cs, const void* delta,
                                const void* Pck, const void* Rck, const double2* tau, void* bl, void* bz,
-                               cudaStream_t s) {
+                               const int32_t* gate, cudaStream_t s) {
   if constexpr (sizeof(R) == 8 && N > 512) {
     return cudaErrorInvalidValue;                    // not eligible: two columns do not fit the registers
   } else {
@@ -664,7 +671,7 @@ static cudaError_t loc_sweep_n(const redo_table* t, const ChainPlan& p, int64_t 
   kern<<<(unsigned)((warps + 3) / 4), kLocThreads, 0, s>>>(
       (const cplx<R>*)cs, (const cplx<R>*)delta, p.M, p.S, sps, chains, (const cplx<R>*)Pck, (const cplx<R>*)Rck, tau,
       (R*)bl, t->K,
-      sizeof(R) == 8 ? (const R*)t->sz64 : (const R*)t->sz32, (R*)bz);
+      sizeof(R) == 8 ? (const R*)t->sz64 : (const R*)t->sz32, (R*)bz, gate);
   return cudaGetLastError();
   }
 }
@@ -672,9 +679,9 @@ static cudaError_t loc_sweep_n(const redo_table* t, const ChainPlan& p, int64_t 
 template <typename R>
 static cudaError_t loc_sweep_t(const redo_table* t, const ChainPlan& p, int64_t B, const void* cs, const void* delta,
                                const void* Pck, const void* Rck, const double2* tau, void* bl, void* bz,
-                               cudaStream_t s) {
+                               const int32_t* gate, cudaStream_t s) {
   constexpr bool TWO = true;
-  LOC_DISPATCH(loc_sweep_n, t, p, B, cs, delta, Pck, Rck, tau, bl, bz, s)
+  LOC_DISPATCH(loc_sweep_n, t, p, B, cs, delta, Pck, Rck, tau, bl, bz, gate, s)
 }
 
 // ============================================================================
@@ -1098,25 +1105,45 @@ cudaError_t launch_local_chain(const redo_table* t, const int32_t* q, const Chai
   return cudaSuccess;
 }
 
+// Which form of the phase gradient a call launches.  The axes in force decide; a captured call is
+// replayed with the axes set by then, so it holds both forms behind the table's device flag (gate).
+struct PhaseForm {
+  bool sums = true, boundary = false;
+  const int32_t* gate = nullptr;
+};
+static PhaseForm phase_form(const redo_table* t, cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  PhaseForm f;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone) {
+    f.sums = t->wz_local != 0;
+    f.boundary = !f.sums;
+  } else {
+    f.boundary = true;
+    f.gate = t->wz_on;
+  }
+  return f;
+}
+
 template <typename R>
 static cudaError_t loc_finish_t(const redo_table* t, int64_t B, int64_t M, int64_t m0, int64_t T, int parts, double norm,
-                                const LocScratch& w, double* grad, double* gphi, cudaStream_t s) {
+                                const LocScratch& w, double* grad, double* gphi, const PhaseForm& f, cudaStream_t s) {
   const int64_t steps = B * T, gn = steps * t->K, gb = (gn + 127) / 128;
   if (w.sums)
     loc_sums_kernel<R><<<(unsigned)steps, 256, 0, s>>>((const R*)w.bl, parts, 3 * t->loc, w.sums);
   loc_grad_kernel<R><<<(unsigned)(gb < 16384 ? gb : 16384), 128, 0, s>>>(
       steps, t->K, t->loc, t->loc_pairs, parts, t->loc_kptr, t->loc_kpair, (const R*)w.g, (const R*)w.bl, w.sums, M, m0,
       T, 2.0 * t->dt / norm, grad);
-  if (gphi && t->wz) {
+  if (gphi && f.sums) {
     auto kern = loc_phase_local_kernel<R, false>;
     if constexpr (sizeof(R) == 4)
       if (loc_near(false, t->N)) kern = loc_phase_local_kernel<R, true>;
     kern<<<(unsigned)(gb < 16384 ? gb : 16384), 128, 0, s>>>(steps, t->K, t->loc, parts, (const cplx<R>*)w.cs,
-                                                             (const R*)w.bl, w.sums, t->wz, 2.0 / norm, gphi);
-  } else if (gphi) {
+                                                             (const R*)w.bl, w.sums, t->wz, 2.0 / norm, gphi, f.gate);
+  }
+  if (gphi && f.boundary) {
     const int64_t n = B * M * t->K, blocks = (n + 255) / 256;
     loc_phase_kernel<R><<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>((const R*)w.bz, B, M, parts, t->K,
-                                                                                  2.0 / norm, gphi);
+                                                                                  2.0 / norm, gphi, f.gate);
   }
   return cudaGetLastError();
 }
@@ -1132,20 +1159,24 @@ cudaError_t launch_local_grad(const redo_table* t, const int32_t* q, const Chain
   const int E = loc_entries(dbl, t->N, true), parts = loc_parts(t, dbl);
   const size_t mat = (size_t)t->N * t->N * (dbl ? sizeof(double2) : sizeof(float2));
   const double norm = (double)t->N * (double)t->N;
+  const PhaseForm f = what == kLocalPhaseGrad ? phase_form(t, s) : PhaseForm{};
   for (int64_t b0 = 0; b0 < p.B; b0 += slice) {
     const int64_t nb = b0 + slice < p.B ? slice : p.B - b0;
     cudaError_t e = cudaSuccess;
     if (slice < p.B && (e = loc_steps(t, q, nb, p.M, prec, E, pd, b0, w, status, s))) return e;
     const char* P = (const char*)Pck + (size_t)(b0 * p.S) * mat;
     const char* Q = (const char*)Rck + (size_t)(b0 * p.S) * mat;
-    void* bz = what == kLocalPhaseGrad && !t->wz ? w.bz : nullptr;
-    e = dbl ? loc_sweep_t<double>(t, p, nb, w.cs, w.delta, P, Q, tau + b0, w.bl, bz, s)
-            : loc_sweep_t<float>(t, p, nb, w.cs, w.delta, P, Q, tau + b0, w.bl, bz, s);
-    if (e) return e;
+    for (int tz = 0; tz < 2; ++tz) {
+      if (!(tz ? f.boundary : f.sums)) continue;
+      void* bz = tz ? w.bz : nullptr;
+      e = dbl ? loc_sweep_t<double>(t, p, nb, w.cs, w.delta, P, Q, tau + b0, w.bl, bz, f.gate, s)
+              : loc_sweep_t<float>(t, p, nb, w.cs, w.delta, P, Q, tau + b0, w.bl, bz, f.gate, s);
+      if (e) return e;
+    }
     const int64_t at = b0 * p.M * t->K;
     double* gp = gphi ? gphi + at : nullptr;
-    e = dbl ? loc_finish_t<double>(t, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, s)
-            : loc_finish_t<float>(t, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, s);
+    e = dbl ? loc_finish_t<double>(t, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, f, s)
+            : loc_finish_t<float>(t, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, f, s);
     if (e) return e;
   }
   return cudaSuccess;
@@ -1271,7 +1302,7 @@ static cudaError_t loc_state_t(const redo_table* t, const int32_t* q, int64_t B,
     if (e) return e;
     LOC_VEC(loc_state_kernel, (const cplx<R>*)w.cs, (const cplx<R>*)w.delta, B, M, m0, T, fwd, bk, psi0, psiT, batched,
             F_out, (R*)w.bl, (cplx<R>*)w.bz)
-    if (bk && (e = loc_finish_t<R>(t, B, M, m0, T, 1, 1.0, w, grad, nullptr, s))) return e;
+    if (bk && (e = loc_finish_t<R>(t, B, M, m0, T, 1, 1.0, w, grad, nullptr, PhaseForm{}, s))) return e;
   }
   return cudaGetLastError();
 }

@@ -63,7 +63,9 @@ struct redo_table {
   size_t tc_bytes;
   int tc_nb;                  // operand block height of the large-N planes (128 or 256)
   float* sz32;                // sz64 in FP32
-  double* wz;                 // [K][loc] one-qubit parts of the S_kz when they are sums of those, or nullptr
+  double* wz;                 // [K][loc] one-qubit parts of the S_kz (in loc_mem), for wz_local / *wz_on != 0:
+  int32_t* wz_on;             // every S_kz is a sum of those (device copy for captured calls)
+  int wz_local;
   double* sz64;               // [K][N] diagonals of the species' S_kz (amplitude/phase calls), or nullptr
   int32_t* h0_pairs;          // host: (row, column) of every off-diagonal nonzero of H0
   int64_t h0_npairs;

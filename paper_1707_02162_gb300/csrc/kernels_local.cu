@@ -15,15 +15,16 @@ namespace redo {
 // Detection and one-qubit tables (at table build)
 // ============================================================================
 
-// Digit operators u[pair][j][c] = exp(-i dt theta h) of a 2 x 2 Hermitian h = a0 I + v.sigma:
-// exp(-i t a0) (cos(t |v|) I - i sin(t |v|) / |v| v.sigma), theta as in the dense table.
-__global__ void loc_table_kernel(const double2* __restrict__ h, const int32_t* __restrict__ k, int pairs, int d,
-                                 int base, double dt, const double* __restrict__ lo, const double* __restrict__ delta,
+// Digit operators u[set][j][c] = exp(-i dt theta h) of a 2 x 2 Hermitian h = a0 I + v.sigma:
+// exp(-i t a0) (cos(t |v|) I - i sin(t |v|) / |v| v.sigma), theta as in the dense table; rep[set] is a
+// pair with these operators.
+__global__ void loc_table_kernel(const double2* __restrict__ h, const int32_t* __restrict__ k,
+                                 const int32_t* __restrict__ rep, int sets, int d, int base, double dt, const double* __restrict__ lo, const double* __restrict__ delta,
                                  double2* __restrict__ u64, float2* __restrict__ u32) {
-  const int64_t total = (int64_t)pairs * d * base;
+  const int64_t total = (int64_t)sets * d * base;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % base), j = (int)((e / base) % d), p = (int)(e / ((int64_t)base * d));
-    const int kk = k[p] & ~kLocFirst;
+    const int c = (int)(e % base), j = (int)((e / base) % d), p = rep[e / ((int64_t)base * d)];
+    const int kk = k[p] & 0xff;
     double bj = 1.0;
     for (int i = 0; i < j; ++i) bj *= (double)base;
     const double th = j == 0 ? __dadd_rn(lo[kk], __dmul_rn((double)c, delta[kk])) : __dmul_rn((double)c * bj, delta[kk]);
@@ -80,17 +81,16 @@ static bool split_local(const double* H, int N, int n, double2* h) {
   return true;
 }
 
-// h: host copies of H0 then H_0 .. H_{K-1}.  Leaves t->loc = 0 for any other system.
-cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_t s) {
-  t->loc = 0;
-  if (!t->h0_diagonal) return cudaSuccess;
+// h: host copies of H0 then H_0 .. H_{K-1}.  Leaves o.on false for any other system.
+void local_detect(redo_table* t, const std::vector<double>& h, TableArena& ar, LocalParts& o) {
+  if (!t->h0_diagonal) return;
   const int N = t->N, K = t->K;
   int n = 0;
   while ((1 << n) < N) ++n;
   const size_t n2 = (size_t)N * N;
   std::vector<double2> hk((size_t)K * n * 4);
   for (int k = 0; k < K; ++k)
-    if (!split_local(h.data() + 2 * n2 * (k + 1), N, n, hk.data() + (size_t)k * n * 4)) return cudaSuccess;
+    if (!split_local(h.data() + 2 * n2 * (k + 1), N, n, hk.data() + (size_t)k * n * 4)) return;
   std::vector<int32_t> ptr(n + 1), kk;
   std::vector<double2> hp;
   std::vector<char> seen(K, 0);
@@ -126,61 +126,81 @@ cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_
     const double a = t->dt * h[2 * ((size_t)r * N + r)], sh = std::sin(0.5 * a), x = -2.0 * sh * sh, y = -std::sin(a);
     D32[r] = make_float4((float)x, (float)y, (float)(x - (double)(float)x), (float)(y - (double)(float)y));
   }
+  // X controls of every qubit, or a global field's part on each, are one set of operators: N = 8 with six
+  // controls of 4096 levels keeps 0.8 MB, not 2.4 MB (which fits beside the dense table in one mapping: building the table takes
+  // 237 us for two global controls, 264 for six local ones; with an allocation, copy and wait of their own 318
+  // and 305, without one-qubit tables 270 and 299)
+  std::vector<int32_t> rep;
+  for (int p = 0; p < pairs; ++p) {
+    const int k = kk[p] & ~kLocFirst;
+    int set = 0;
+    for (; set < (int)rep.size(); ++set) {
+      const int r = rep[set], kr = kk[r] & 0xff;
+      if (std::memcmp(&hp[4 * p], &hp[4 * r], 4 * sizeof(double2)) == 0 && t->lo[k] == t->lo[kr] &&
+          t->delta[k] == t->delta[kr])
+        break;
+    }
+    if (set == (int)rep.size()) rep.push_back(p);
+    kk[p] |= set << 8;
+  }
   std::vector<float2> hp32(hp.size());
   for (size_t i = 0; i < hp.size(); ++i) hp32[i] = make_float2((float)hp[i].x, (float)hp[i].y);
   // one operator per level (no digit products per step) while the table stays small beside L2
-  const bool levels = t->levels <= 65536 && (double)pairs * t->levels * 96.0 <= 64e6;
+  const bool levels = t->levels <= 65536 && (double)rep.size() * t->levels * 96.0 <= 64e6;
   t->loc_d = levels ? 1 : t->digit_count;
   t->loc_base = levels ? (int)t->levels : t->digit_base;
   t->loc_pairs = pairs;
-  const size_t ent = (size_t)pairs * t->loc_d * t->loc_base;
+  o.entries = rep.size() * t->loc_d * t->loc_base;
+  o.rep = ar.put(rep.data(), sizeof(int32_t) * rep.size());
   std::vector<double2> D(N);
   for (int r = 0; r < N; ++r) {
     const double a = t->dt * h[2 * ((size_t)r * N + r)];
     const double sh = std::sin(0.5 * a);
     D[r] = make_double2(-2.0 * sh * sh, -std::sin(a));                // exp(-i a) - 1
   }
-  // one allocation and one copy for the small arrays, the tables behind them
-  std::vector<unsigned char> host;
-  auto put = [&](const void* src, size_t bytes) {
-    const size_t at = (host.size() + 255) & ~(size_t)255;
-    host.resize(at + bytes);
-    std::memcpy(host.data() + at, src, bytes);
-    return at;
-  };
-  const size_t o_ptr = put(ptr.data(), sizeof(int32_t) * (n + 1)), o_k = put(kk.data(), sizeof(int32_t) * pairs),
-               o_h = put(hp.data(), sizeof(double2) * 4 * pairs), o_h32 = put(hp32.data(), sizeof(float2) * 4 * pairs),
-               o_kptr = put(kptr.data(), sizeof(int32_t) * (K + 1)), o_kp = put(kpair.data(), sizeof(int32_t) * pairs),
-               o_D = put(D.data(), sizeof(double2) * N), o_D32 = put(D32.data(), sizeof(float4) * N);
-  // room for the phase axes' one-qubit parts (local_phase_axes) and whether they apply
+  o.ptr = ar.put(ptr.data(), sizeof(int32_t) * (n + 1));
+  o.k = ar.put(kk.data(), sizeof(int32_t) * pairs);
+  o.h = ar.put(hp.data(), sizeof(double2) * 4 * pairs);
+  o.h32 = ar.put(hp32.data(), sizeof(float2) * 4 * pairs);
+  o.kptr = ar.put(kptr.data(), sizeof(int32_t) * (K + 1));
+  o.kpair = ar.put(kpair.data(), sizeof(int32_t) * pairs);
+  o.D = ar.put(D.data(), sizeof(double2) * N);
+  o.D32 = ar.put(D32.data(), sizeof(float4) * N);
+  // the phase axes' one-qubit parts (local_phase_axes) and whether they apply
   const std::vector<double> none((size_t)K * n, 0.0);
   const int32_t off = 0;
-  const size_t o_wz = put(none.data(), sizeof(double) * none.size()), o_wzon = put(&off, sizeof(off));
-  const size_t o_u64 = (host.size() + 255) & ~(size_t)255, o_u32 = o_u64 + sizeof(double2) * 4 * ent;
-  cudaError_t e = cudaMalloc(&t->loc_mem, o_u32 + sizeof(float2) * 4 * ent);
-  if (e) return e;
-  char* base = (char*)t->loc_mem;
-  if ((e = cudaMemcpyAsync(base, host.data(), host.size(), cudaMemcpyHostToDevice, s))) return e;
-  t->loc_ptr = (int32_t*)(base + o_ptr);
-  t->loc_k = (int32_t*)(base + o_k);
-  t->loc_h = (double2*)(base + o_h);
-  t->loc_h32 = (float2*)(base + o_h32);
-  t->loc_kptr = (int32_t*)(base + o_kptr);
-  t->loc_kpair = (int32_t*)(base + o_kp);
-  t->loc_D64 = (double2*)(base + o_D);
-  t->loc_D32 = (float4*)(base + o_D32);
-  t->wz = (double*)(base + o_wz);
-  t->wz_on = (int32_t*)(base + o_wzon);
-  t->loc_u64 = (double2*)(base + o_u64);
-  t->loc_u32 = (float2*)(base + o_u32);
-  loc_table_kernel<<<(unsigned)((ent + 127) / 128 < 4096 ? (ent + 127) / 128 : 4096), 128, 0, s>>>(
-      t->loc_h, t->loc_k, pairs, t->loc_d, t->loc_base, t->dt, t->d_lo, t->d_delta, t->loc_u64, t->loc_u32);
-  if ((e = cudaGetLastError()) || (e = cudaStreamSynchronize(s))) return e;   // the host arrays end here
-  t->loc = n;
-  return cudaSuccess;
+  o.wz = ar.put(none.data(), sizeof(double) * none.size());
+  o.wz_on = ar.put(&off, sizeof(off));
+  o.on = true;
 }
 
-void local_free(redo_table* t) { cudaFree(t->loc_mem); }
+void local_room(const redo_table* t, TableArena& ar, LocalParts& o) {
+  if (!o.on) return;
+  o.u64 = ar.room(sizeof(double2) * 4 * o.entries);
+  o.u32 = ar.room(sizeof(float2) * 4 * o.entries);
+}
+
+cudaError_t local_build(redo_table* t, const LocalParts& o, char* base, cudaStream_t s) {
+  if (!o.on) return cudaSuccess;
+  t->loc_ptr = (int32_t*)(base + o.ptr);
+  t->loc_k = (int32_t*)(base + o.k);
+  t->loc_h = (double2*)(base + o.h);
+  t->loc_h32 = (float2*)(base + o.h32);
+  t->loc_kptr = (int32_t*)(base + o.kptr);
+  t->loc_kpair = (int32_t*)(base + o.kpair);
+  t->loc_D64 = (double2*)(base + o.D);
+  t->loc_D32 = (float4*)(base + o.D32);
+  t->wz = (double*)(base + o.wz);
+  t->wz_on = (int32_t*)(base + o.wz_on);
+  t->loc_u64 = (double2*)(base + o.u64);
+  t->loc_u32 = (float2*)(base + o.u32);
+  const size_t blocks = (o.entries + 127) / 128, sets = o.entries / ((size_t)t->loc_d * t->loc_base);
+  loc_table_kernel<<<(unsigned)(blocks < 4096 ? blocks : 4096), 128, 0, s>>>(t->loc_h, t->loc_k, (const int32_t*)(base + o.rep),
+                                                                            (int)sets, t->loc_d, t->loc_base, t->dt,
+                                                                            t->d_lo, t->d_delta, t->loc_u64, t->loc_u32);
+  while ((1 << t->loc) < t->N) ++t->loc;
+  return cudaGetLastError();
+}
 
 // sz [K][N] (host): their one-qubit parts when each is a sum of those, written over the previous ones
 // (a captured call reads them, and whether they apply, where it found them at capture)
@@ -286,7 +306,7 @@ __device__ __forceinline__ void loc_derivatives(const LocTab<R>& tab, const int3
     g[3 * p] = g01.x;
     g[3 * p + 1] = -g01.y;
     g[3 * p + 2] = R(0.5) * (gm.a.x - gm.e.x);
-    if (p > p0) w = mat2_mul<R>(w, loc_term<R>(tab, p, loc_level<R>(tab, qrow, tab.k[p], false)));
+    if (p > p0) w = mat2_mul<R>(w, loc_term<R>(tab, tab.k[p], loc_level<R>(tab, qrow, tab.k[p], false)));
   }
 }
 

@@ -373,34 +373,39 @@ __global__ void diag_ctl_kernel(const double* __restrict__ hd, const double2* __
   }
 }
 
-// h: host copies of H0 then H_0 .. H_{K-1}.  Leaves t->dct = 0 unless every control is diagonal, N <= 16
+// h: host copies of H0 then H_0 .. H_{K-1}.  Leaves o.on false unless every control is diagonal, N <= 16
 // and the factors fit shared memory.
-cudaError_t diag_ctl_build(redo_table* t, const std::vector<double>& h, cudaStream_t s) {
-  t->dct = 0;
+void diag_ctl_detect(const redo_table* t, const std::vector<double>& h, TableArena& ar, DiagParts& o) {
   const int N = t->N, K = t->K;
-  const size_t ent = (size_t)K * t->digit_count * t->digit_base * N;
-  if (N > 16 || (ent + N * N) * sizeof(double2) > 160 * 1024) return cudaSuccess;
+  o.entries = (size_t)K * t->digit_count * t->digit_base * N;
+  if (N > 16 || (o.entries + N * N) * sizeof(double2) > 160 * 1024) return;
   std::vector<double> hd((size_t)K * N);
   for (int k = 0; k < K; ++k) {
     const double* H = h.data() + 2 * (size_t)N * N * (k + 1);
     for (int r = 0; r < N; ++r)
       for (int c = 0; c < N; ++c) {
-        if (r != c && (H[2 * (r * N + c)] != 0.0 || H[2 * (r * N + c) + 1] != 0.0)) return cudaSuccess;
+        if (r != c && (H[2 * (r * N + c)] != 0.0 || H[2 * (r * N + c) + 1] != 0.0)) return;
         if (r == c) hd[(size_t)k * N + r] = H[2 * (r * N + c)];
       }
   }
-  const size_t tot = ent + (size_t)N * N;
-  cudaError_t e = cudaMalloc(&t->dct_u, tot * (sizeof(double2) + sizeof(float2)) + hd.size() * sizeof(double));
-  if (e) return e;
+  o.hd = ar.put(hd.data(), hd.size() * sizeof(double));
+  o.on = true;
+}
+
+void diag_ctl_room(const redo_table* t, TableArena& ar, DiagParts& o) {
+  if (o.on) o.u = ar.room((o.entries + (size_t)t->N * t->N) * (sizeof(double2) + sizeof(float2)));
+}
+
+cudaError_t diag_ctl_build(redo_table* t, const DiagParts& o, char* base, cudaStream_t s) {
+  if (!o.on) return cudaSuccess;
+  const size_t tot = o.entries + (size_t)t->N * t->N;
+  t->dct_u = (double2*)(base + o.u);
   t->dct_u32 = (float2*)(t->dct_u + tot);
-  double* dhd = (double*)(t->dct_u32 + tot);
-  if ((e = cudaMemcpyAsync(dhd, hd.data(), hd.size() * sizeof(double), cudaMemcpyHostToDevice, s))) return e;
-  diag_ctl_kernel<<<(unsigned)((tot + 127) / 128), 128, 0, s>>>(dhd, t->D64, N, K, t->digit_count, t->digit_base, t->dt,
-                                                                t->d_lo, t->d_delta, t->dct_u, t->dct_u32, t->dct_u + ent,
-                                                                t->dct_u32 + ent);
-  if ((e = cudaGetLastError()) || (e = cudaStreamSynchronize(s))) return e;
+  diag_ctl_kernel<<<(unsigned)((tot + 127) / 128), 128, 0, s>>>(
+      (const double*)(base + o.hd), t->D64, t->N, t->K, t->digit_count, t->digit_base, t->dt, t->d_lo, t->d_delta,
+      t->dct_u, t->dct_u32, t->dct_u + o.entries, t->dct_u32 + o.entries);
   t->dct = 1;
-  return cudaSuccess;
+  return cudaGetLastError();
 }
 
 template <typename R, int N>

@@ -36,8 +36,8 @@ template <typename R> __device__ __forceinline__ cplx<R> cmul_conj(cplx<R> a, cp
 template <typename R>
 struct LocTab {
   const int32_t* ptr;        // [n + 1] pairs of qubit i
-  const int32_t* k;          // [pairs] term (| kLocFirst)
-  const cplx<R>* u;          // [pairs][d][base][4] digit operators, row-major 2 x 2
+  const int32_t* k;          // [pairs] term | operator set << 8 (| kLocFirst)
+  const cplx<R>* u;          // [sets][d][base][4] digit operators, row-major 2 x 2
   int d, base, K;
   int64_t levels;
   int64_t* status;
@@ -68,19 +68,20 @@ template <typename R> __device__ __forceinline__ Mat2<R> loc_load(const LocTab<R
   return m;
 }
 
-// u_ki at level index qv: the product of its digit operators
-template <typename R> __device__ __forceinline__ Mat2<R> loc_term(const LocTab<R>& t, int pair, int32_t qv) {
-  Mat2<R> m = loc_load(t, (int64_t)pair * t.d * t.base + qv % t.base);
+// u_ki (kf: its entry of LocTab::k) at level index qv: the product of its digit operators
+template <typename R> __device__ __forceinline__ Mat2<R> loc_term(const LocTab<R>& t, int kf, int32_t qv) {
+  const int set = (kf & ~kLocFirst) >> 8;
+  Mat2<R> m = loc_load(t, (int64_t)set * t.d * t.base + qv % t.base);
   for (int j = 1; j < t.d; ++j) {
     qv /= t.base;
-    m = mat2_mul<R>(loc_load(t, ((int64_t)pair * t.d + j) * t.base + qv % t.base), m);
+    m = mat2_mul<R>(loc_load(t, ((int64_t)set * t.d + j) * t.base + qv % t.base), m);
   }
   return m;
 }
 
 template <typename R>
 __device__ __forceinline__ int32_t loc_level(const LocTab<R>& t, const int32_t* qrow, int kf, bool count) {
-  int32_t qv = qrow[kf & ~kLocFirst];
+  int32_t qv = qrow[kf & 0xff];
   if (qv < 0 || qv >= t.levels) {
     if (count && (kf & kLocFirst) && t.status)
       atomicAdd((unsigned long long*)&t.status[REDO_STATUS_BADINDEX], (unsigned long long)t.bad_weight);
@@ -97,7 +98,8 @@ __device__ __forceinline__ Mat2<R> loc_step(const LocTab<R>& t, const int32_t* q
   v.b = v.c = cmake<R>(R(0), R(0));
   const int p0 = t.ptr[i], p1 = t.ptr[i + 1];
   for (int p = p0; p < p1; ++p) {
-    const Mat2<R> u = loc_term<R>(t, p, loc_level<R>(t, qrow, t.k[p], count));
+    const int kf = t.k[p];
+    const Mat2<R> u = loc_term<R>(t, kf, loc_level<R>(t, qrow, kf, count));
     v = p == p0 ? u : mat2_mul<R>(u, v);
   }
   return v;

@@ -163,9 +163,9 @@ redo_status redo_build_table(int32_t N, int32_t K, double dt, const void* H0, co
     return st;
   };
   cudaError_t e;
-  if ((e = cudaMalloc(&t->d_lo, sizeof(double) * K)) != cudaSuccess ||
-      (e = cudaMalloc(&t->d_delta, sizeof(double) * K)) != cudaSuccess ||
-      (e = cudaMalloc(&t->T64, sizeof(double2) * n2 * t->entries)) != cudaSuccess ||
+  TableArena ar;
+  const size_t o_lo = ar.put(t->lo, sizeof(double) * K), o_delta = ar.put(t->delta, sizeof(double) * K);
+  if ((e = cudaMalloc(&t->T64, sizeof(double2) * n2 * t->entries)) != cudaSuccess ||
       (e = cudaMalloc(&t->D64, sizeof(double2) * n2)) != cudaSuccess)
     return fail(set_error(REDO_ERR_OOM, "table allocation: %s", cudaGetErrorString(e)));
   if (flags & REDO_TABLE_STRANG) {
@@ -195,7 +195,8 @@ redo_status redo_build_table(int32_t N, int32_t K, double dt, const void* H0, co
   std::vector<int32_t> mono_m(K, 0);
   std::vector<double2> mono_h((size_t)K * N);
   std::vector<double> mono_a(K, 0.0);
-  bool mono_involutory = false;
+  bool mono_involutory = false, xr = false;
+  size_t o_ptr, o_col, o_row, o_val, o_xmask = 0, o_xval = 0;
   {
     // sparse (CSR) copy of the control operators for the gradient traces Tr(H_k W)
     std::vector<int32_t> ptr((size_t)K * (N + 1)), col, rowi;
@@ -216,18 +217,10 @@ redo_status redo_build_table(int32_t N, int32_t K, double dt, const void* H0, co
       ptr[(size_t)k * (N + 1) + N] = (int32_t)col.size();
     }
     t->hk_nnz = (int64_t)col.size();
-    const size_t nz = col.empty() ? 1 : col.size();
-    if ((e = cudaMalloc(&t->hk_ptr, sizeof(int32_t) * ptr.size())) != cudaSuccess ||
-        (e = cudaMalloc(&t->hk_col, sizeof(int32_t) * nz)) != cudaSuccess ||
-        (e = cudaMalloc(&t->hk_row, sizeof(int32_t) * nz)) != cudaSuccess ||
-        (e = cudaMalloc(&t->hk_val, sizeof(double2) * nz)) != cudaSuccess)
-      return fail(set_error(REDO_ERR_OOM, "operator CSR allocation: %s", cudaGetErrorString(e)));
-    if ((e = cudaMemcpy(t->hk_ptr, ptr.data(), sizeof(int32_t) * ptr.size(), cudaMemcpyHostToDevice)) ||
-        (!col.empty() &&
-         ((e = cudaMemcpy(t->hk_col, col.data(), sizeof(int32_t) * col.size(), cudaMemcpyHostToDevice)) ||
-          (e = cudaMemcpy(t->hk_row, rowi.data(), sizeof(int32_t) * rowi.size(), cudaMemcpyHostToDevice)) ||
-          (e = cudaMemcpy(t->hk_val, val.data(), sizeof(double2) * val.size(), cudaMemcpyHostToDevice)))))
-      return fail(cuda_error(e, "operator CSR upload"));
+    o_ptr = ar.put(ptr.data(), sizeof(int32_t) * ptr.size());
+    o_col = ar.put(col.data(), sizeof(int32_t) * col.size());
+    o_row = ar.put(rowi.data(), sizeof(int32_t) * rowi.size());
+    o_val = ar.put(val.data(), sizeof(double2) * val.size());
     // Operators with exactly one nonzero per row, at column r ^ m_k (every Pauli string:
     // X/Y flip bits, Z only sets phases) also get the compact form m_k, h_k[r] in FP32
     // that the tensor-core gradient's trace reads without gathering.
@@ -263,22 +256,43 @@ redo_status redo_build_table(int32_t N, int32_t K, double dt, const void* H0, co
         mono_a[k] = std::sqrt(a2);
       }
     }
-    const bool xr = mono && N > kSmallN;
+    xr = mono && N > kSmallN;
     if (xr) {
-      if ((e = cudaMalloc(&t->hk_xmask, sizeof(int32_t) * K)) != cudaSuccess ||
-          (e = cudaMalloc(&t->hk_xval, sizeof(float2) * K * N)) != cudaSuccess)
-        return fail(set_error(REDO_ERR_OOM, "operator allocation: %s", cudaGetErrorString(e)));
-      if ((e = cudaMemcpy(t->hk_xmask, xm.data(), sizeof(int32_t) * K, cudaMemcpyHostToDevice)) ||
-          (e = cudaMemcpy(t->hk_xval, xv.data(), sizeof(float2) * K * N, cudaMemcpyHostToDevice)))
-        return fail(cuda_error(e, "operator upload"));
+      o_xmask = ar.put(xm.data(), sizeof(int32_t) * K);
+      o_xval = ar.put(xv.data(), sizeof(float2) * K * N);
     }
   }
+  // one allocation and one upload for the small arrays, with the one-qubit and diagonal tables behind
+  // them; without room for those the table is built for the dense operators alone
+  LocalParts loc;
+  DiagParts dct;
+  local_detect(t, h, ar, loc);
+  diag_ctl_detect(t, h, ar, dct);
+  const size_t small = ar.total;
+  local_room(t, ar, loc);
+  diag_ctl_room(t, ar, dct);
+  if ((e = cudaMalloc(&t->mem, ar.total)) != cudaSuccess) {
+    loc.on = dct.on = false;
+    cudaGetLastError();
+    if ((e = cudaMalloc(&t->mem, small)) != cudaSuccess)
+      return fail(set_error(REDO_ERR_OOM, "table arrays: %s", cudaGetErrorString(e)));
+  }
+  char* mem = (char*)t->mem;
+  t->d_lo = (double*)(mem + o_lo);
+  t->d_delta = (double*)(mem + o_delta);
+  t->hk_ptr = (int32_t*)(mem + o_ptr);
+  t->hk_col = (int32_t*)(mem + o_col);
+  t->hk_row = (int32_t*)(mem + o_row);
+  t->hk_val = (double2*)(mem + o_val);
+  if (xr) {
+    t->hk_xmask = (int32_t*)(mem + o_xmask);
+    t->hk_xval = (float2*)(mem + o_xval);
+  }
+  if ((e = cudaMemcpyAsync(mem, ar.host.data(), ar.host.size(), cudaMemcpyHostToDevice, s)))
+    return fail(cuda_error(e, "table arrays"));
   if ((flags & (REDO_TABLE_FP32 | REDO_TABLE_FP16X3)) &&
       (e = cudaMalloc(&t->T32, sizeof(float2) * n2 * t->entries)) != cudaSuccess)
     return fail(set_error(REDO_ERR_OOM, "FP32 table allocation: %s", cudaGetErrorString(e)));
-  if ((e = cudaMemcpyAsync(t->d_lo, t->lo, sizeof(double) * K, cudaMemcpyHostToDevice, s)) ||
-      (e = cudaMemcpyAsync(t->d_delta, t->delta, sizeof(double) * K, cudaMemcpyHostToDevice, s)))
-    return fail(cuda_error(e, "copy lo/delta"));
   if (N <= kSmallN) {
     if ((e = launch_table_expm(t, (const double2*)H0, (const double2*)Hk, s)) != cudaSuccess)
       return fail(cuda_error(e, "table exponentials"));
@@ -353,8 +367,8 @@ redo_status redo_build_table(int32_t N, int32_t K, double dt, const void* H0, co
     e = N > kSmallN ? launch_build_tc_large_planes(t, s) : launch_build_tc_planes(t, s);
     if (e != cudaSuccess) return fail(cuda_error(e, "FP16x3 planes"));
   }
-  if ((e = local_build(t, h, s)) != cudaSuccess) return fail(cuda_error(e, "one-qubit tables"));
-  if ((e = diag_ctl_build(t, h, s)) != cudaSuccess) return fail(cuda_error(e, "diagonal controls"));
+  if ((e = local_build(t, loc, mem, s)) != cudaSuccess) return fail(cuda_error(e, "one-qubit tables"));
+  if ((e = diag_ctl_build(t, dct, mem, s)) != cudaSuccess) return fail(cuda_error(e, "diagonal controls"));
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(cuda_error(e, "table build"));
   *out = t;
   return REDO_OK;
@@ -363,23 +377,14 @@ redo_status redo_build_table(int32_t N, int32_t K, double dt, const void* H0, co
 redo_status redo_table_free(redo_table* t) {
   if (!t) return REDO_OK;
   if (t->build_stream) cudaStreamSynchronize(t->build_stream);
-  cudaFree(t->d_lo);
-  cudaFree(t->d_delta);
+  cudaFree(t->mem);
   cudaFree(t->T64);
   cudaFree(t->D64);
   cudaFree(t->Dh64);
   cudaFree(t->T32);
   cudaFree(t->tc_planes);
-  cudaFree(t->hk_ptr);
-  cudaFree(t->hk_col);
-  cudaFree(t->hk_row);
-  cudaFree(t->hk_val);
-  cudaFree(t->hk_xmask);
-  cudaFree(t->hk_xval);
   cudaFree(t->sz64);
   cudaFree(t->sz32);
-  local_free(t);
-  cudaFree(t->dct_u);
   std::free(t->h0_pairs);
   std::free(t);
   return REDO_OK;

@@ -44,6 +44,7 @@ struct redo_table {
   int64_t entries;            // K * digits * base
   double dt;
   double lo[redo::kMaxK], hi[redo::kMaxK], delta[redo::kMaxK];
+  void* mem;                  // the one allocation of the small arrays and one-qubit tables (TableArena)
   double* d_lo;               // device copies [K]
   double* d_delta;            // [K]
   double2* T64;               // [entries][N][N], term 0 digit 0 folded with D
@@ -63,7 +64,7 @@ struct redo_table {
   size_t tc_bytes;
   int tc_nb;                  // operand block height of the large-N planes (128 or 256)
   float* sz32;                // sz64 in FP32
-  double* wz;                 // [K][loc] one-qubit parts of the S_kz (in loc_mem), for wz_local / *wz_on != 0:
+  double* wz;                 // [K][loc] one-qubit parts of the S_kz, for wz_local / *wz_on != 0:
   int32_t* wz_on;             // every S_kz is a sum of those (device copy for captured calls)
   int wz_local;
   double* sz64;               // [K][N] diagonals of the species' S_kz (amplitude/phase calls), or nullptr
@@ -73,14 +74,14 @@ struct redo_table {
   // one-qubit operators or the drift is not diagonal
   int loc;
   int loc_pairs, loc_d, loc_base;
-  void* loc_mem;              // the one allocation that the following arrays lie in
   int32_t* loc_ptr;           // [loc + 1] (term, qubit) pairs of each qubit
-  int32_t* loc_k;             // [pairs] term, flagged at the first pair of a term
+  int32_t* loc_k;             // [pairs] term | operator set << 8, flagged at the first pair of a term
   double2* loc_h;             // [pairs][4] one-qubit part of the term's operator
   float2* loc_h32;
   int32_t* loc_kptr;          // [K + 1] and
   int32_t* loc_kpair;         // [pairs]: the pairs of each term (pair | qubit << 20)
-  double2* loc_u64;           // [pairs][loc_d][loc_base][4] digit (or level) operators
+  double2* loc_u64;           // [sets][loc_d][loc_base][4] digit (or level) operators, a set for every
+                              // distinct (one-qubit part, coefficient grid)
   float2* loc_u32;
   double2* loc_D64;           // [N] diagonal of the drift step minus 1
   float4* loc_D32;            // the same as FP32 hi + lo
@@ -183,11 +184,41 @@ struct LocalDiag {
   int64_t sb, sn;
 };
 }  // namespace redo
+#include <cstring>
 #include <vector>
 namespace redo {
+// The small arrays of a table under construction: copied in by put() (one upload), then space for the
+// tables that kernels fill.  Offsets become pointers once the allocation stands.
+struct TableArena {
+  std::vector<unsigned char> host;
+  size_t total = 0;
+  size_t put(const void* src, size_t bytes) {
+    const size_t at = (host.size() + 255) & ~(size_t)255;
+    host.resize(at + bytes);
+    if (bytes > 0) std::memcpy(host.data() + at, src, bytes);
+    total = host.size();
+    return at;
+  }
+  size_t room(size_t bytes) {                        // after the last put()
+    const size_t at = (total + 255) & ~(size_t)255;
+    total = at + bytes;
+    return at;
+  }
+};
 cudaError_t launch_local_split(double2* pd, int64_t n, cudaStream_t s);
-cudaError_t local_build(redo_table* t, const std::vector<double>& h, cudaStream_t s);
-void local_free(redo_table* t);
+// One-qubit tables and diagonal factors: host parts into the arena, room for the tables, and, once
+// the table's operators stand, the pointers into base and the kernels.
+struct LocalParts {
+  bool on = false;
+  size_t ptr, k, h, h32, kptr, kpair, D, D32, wz, wz_on, rep, u64, u32, entries;
+};
+struct DiagParts {
+  bool on = false;
+  size_t hd, u, entries;
+};
+void local_detect(redo_table* t, const std::vector<double>& h, TableArena& ar, LocalParts& o);
+void local_room(const redo_table* t, TableArena& ar, LocalParts& o);
+cudaError_t local_build(redo_table* t, const LocalParts& o, char* base, cudaStream_t s);
 cudaError_t local_phase_axes(redo_table* t, const double* sz);
 // What a call computes: segment products, the gradient, the amplitude/phase gradient, the state's
 // observable.
@@ -256,7 +287,9 @@ cudaError_t launch_state_grad(const redo_table* t, const int32_t* q, int64_t B, 
 cudaError_t launch_sim_stream(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int prec,
                               const double2* psi0, int psi0_batched, const double* obs, double* expect,
                               int64_t* status, cudaStream_t s);
-cudaError_t diag_ctl_build(redo_table* t, const std::vector<double>& h, cudaStream_t s);
+void diag_ctl_detect(const redo_table* t, const std::vector<double>& h, TableArena& ar, DiagParts& o);
+void diag_ctl_room(const redo_table* t, TableArena& ar, DiagParts& o);
+cudaError_t diag_ctl_build(redo_table* t, const DiagParts& o, char* base, cudaStream_t s);
 cudaError_t launch_levels_closed_form(const redo_table* t, const int32_t* xm, const double2* xh, const double* xa,
                                       double2* E, cudaStream_t s);
 cudaError_t launch_expect_diag(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int prec,

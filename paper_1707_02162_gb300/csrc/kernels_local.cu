@@ -487,7 +487,8 @@ static cudaError_t loc_chain_t(const redo_table* t, const ChainPlan& p, int64_t 
 // ============================================================================
 // GRAPE gradient: reverse sweep of the segments.  A column x of P and row x of R stay with the
 // same lanes, so undoing a step (P <- U^dag P, R <- R U) and the traces are local to them; only
-// the Bloch sums Im Tr(sigma_i P R) of every qubit are added over x.  They hold every control's
+// the Bloch sums Im Tr(sigma_i P R) of every qubit are added over x.  (R is taken times conj(tau), in
+// FP32 times 2^-exp_of(tau), which the gradients make up for.)  They hold every control's
 // trace: Tr(g P R) for g = sum_i g_i needs the one-qubit partial traces only.  bl receives them as
 // [step][part][3n], one part per warp of the chain, added in a fixed order afterwards.
 // TZ (amplitude/phase calls): also Tz = Im Tr(S_kz P R) at every step boundary.  gate: the form with
@@ -515,7 +516,11 @@ loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
   const cplx<R>* r = cs + b * M * L::CS;
   cplx<R> p[E], w[E];
   {
-    const double2 tb = tau[b];
+    double2 tb = tau[b];
+    if constexpr (sizeof(R) == 4) {
+      const double f = pow2(-exp_of(tb));
+      tb = make_double2(tb.x * f, tb.y * f);
+    }
     const cplx<R>* P = Pck + g * N * N + x;
     const cplx<R>* Q = Rck + g * N * N + (int64_t)x * N + l * E;
 #pragma unroll
@@ -578,10 +583,16 @@ loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
 
 // dF/du_kn = (2 dt / N^2) sum_i (gx X_i + gy Y_i + gz Z_i), a thread per (step, term): its pairs are
 // kpair[kptr[k] ..] (pair | qubit << 20), the Bloch sums bl [step][part][3n] or, already added, sums.
+// The sums are those of scaled vectors in FP32: times 2^exp_of(tau[b]), or times amp[b].
+template <typename R> __device__ __forceinline__ double loc_scale(const double2* tau, const double* amp, int64_t b) {
+  if (sizeof(R) == 8) return 1.0;
+  return amp ? amp[b] : pow2(exp_of(tau[b]));
+}
 template <typename R>
 __global__ void loc_grad_kernel(int64_t steps, int K, int n, int pairs, int parts, const int32_t* __restrict__ kptr,
                                 const int32_t* __restrict__ kpair, const R* __restrict__ g, const R* __restrict__ bl,
                                 const double* __restrict__ sums, int64_t M, int64_t w0, int64_t T, double scale,
+                                const double2* __restrict__ tau, const double* __restrict__ amp,
                                 double* __restrict__ grad) {
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < steps * K;
        idx += (int64_t)gridDim.x * blockDim.x) {
@@ -601,7 +612,7 @@ __global__ void loc_grad_kernel(int64_t steps, int K, int n, int pairs, int part
         acc += (double)gp[c] * v;
       }
     }
-    grad[(b * M + w0 + st - b * T) * K + k] = scale * acc;
+    grad[(b * M + w0 + st - b * T) * K + k] = scale * (acc * loc_scale<R>(tau, amp, b));
   }
 }
 
@@ -626,7 +637,7 @@ __global__ void __launch_bounds__(256) loc_sums_kernel(const R* __restrict__ bl,
 // gphi[b][n][k] = (2 / N^2) (Tz[n+1][k] - Tz[n][k]) (the traces already carry conj(tau))
 template <typename R>
 __global__ void loc_phase_kernel(const R* __restrict__ bz, int64_t B, int64_t M, int parts, int K, double scale,
-                                 double* __restrict__ gphi, const int32_t* __restrict__ gate) {
+                                 const double2* __restrict__ tau, double* __restrict__ gphi, const int32_t* __restrict__ gate) {
   if (gate && *gate != 0) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B * M * K; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t bn = i / K, b = bn / M, n = bn - b * M;
@@ -636,7 +647,7 @@ __global__ void loc_phase_kernel(const R* __restrict__ bz, int64_t B, int64_t M,
       a += (double)bz[((b * (M + 1) + n) * parts + p) * K + k];
       c += (double)bz[((b * (M + 1) + n + 1) * parts + p) * K + k];
     }
-    gphi[i] = scale * (c - a);
+    gphi[i] = scale * ((c - a) * loc_scale<R>(tau, nullptr, b));
   }
 }
 
@@ -646,9 +657,10 @@ __global__ void loc_phase_kernel(const R* __restrict__ bz, int64_t B, int64_t M,
 // ones. Bound by reading the Bloch sums once. N = 64, 16 x 200, FP32: error of the outputs against 64
 // bits 2.4e-6 -> 4.7e-7, time of the whole gradient 0.286 -> 0.288 ms (the scan bounds it).
 template <typename R, bool NEAR>
-__global__ void loc_phase_local_kernel(int64_t steps, int K, int n, int parts, const cplx<R>* __restrict__ cs,
+__global__ void loc_phase_local_kernel(int64_t steps, int64_t M, int K, int n, int parts, const cplx<R>* __restrict__ cs,
                                        const R* __restrict__ bl, const double* __restrict__ sums,
-                                       const double* __restrict__ wz, double scale, double* __restrict__ gphi,
+                                       const double* __restrict__ wz, double scale,
+                                       const double2* __restrict__ tau, double* __restrict__ gphi,
                                        const int32_t* __restrict__ gate) {
   if (gate && *gate == 0) return;
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < steps * K;
@@ -672,7 +684,7 @@ __global__ void loc_phase_local_kernel(int64_t steps, int K, int n, int parts, c
       }
       acc += w * (2.0 * (sx * sx + sy * sy) * v[2] - 2.0 * c * (sx * v[0] + sy * v[1]));
     }
-    gphi[idx] = scale * acc;
+    gphi[idx] = scale * (acc * loc_scale<R>(tau, nullptr, st / M));
   }
 }
 
@@ -880,12 +892,14 @@ __global__ void loc_expect_kernel(const cplx<R>* __restrict__ part, int64_t n, i
 // F_S = |<psi_T|U|psi_0>|^2 and the Bloch sums of its gradient: forward over the steps, then back
 // with the state undone and the costate <psi_T| U_M ... carried along (trace_undo).  One launch
 // covers the steps [m0, m0 + T): forward (fwd), at the chain's end the overlap, and back (back);
-// between launches both vectors rest in st[b][2][N].
+// between launches both vectors rest in st[b][2][N].  FP32 vectors are scaled by powers of two (psi_0
+// to entries near 1, the costate likewise), whose product goes to amp[b] for the gradient.
 template <typename R, int N>
 __global__ void __launch_bounds__(32)
 loc_state_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t B, int64_t M, int64_t m0,
                  int64_t T, int fwd, int back, const double2* __restrict__ psi0, const double2* __restrict__ psiT,
-                 int batched, double* __restrict__ F_out, R* __restrict__ bl, cplx<R>* __restrict__ st) {
+                 int batched, double* __restrict__ F_out, R* __restrict__ bl, cplx<R>* __restrict__ st,
+                 double* __restrict__ amp) {
   constexpr int E = loc_vec_entries(N);
   using L = LocCol<R, N, E>;
   using WS = WarpSums<R, 3 * L::NQ>;
@@ -897,11 +911,23 @@ loc_state_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
   const cplx<R>* r = cs + b * T * L::CS;
   cplx<R>* sp = st + b * 2 * N + l * E;
   cplx<R> p[E], w[E], dn[E], cn[L::CS];
+  // exponent of the largest entry of a vector (this lane's E entries at v)
+  auto top = [&](const double2* v) -> int {
+    int x = -200;
+#pragma unroll
+    for (int e = 0; e < E; ++e) x = max(x, exp_of(v[e]));
+#pragma unroll
+    for (int off = L::C; off < 32; off *= 2) x = max(x, __shfl_xor_sync(0xffffffffu, x, off));
+    return x;
+  };
+  const double2 *z0 = psi0 + (batched ? b * N : 0) + l * E, *zT = psiT + (batched ? b * N : 0) + l * E;
+  const int e0 = sizeof(R) == 4 && fwd ? top(z0) : 0;
   if (fwd) {
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const double2 z = m0 == 0 ? psi0[(batched ? b * N : 0) + l * E + e] : make_double2(0.0, 0.0);
-      p[e] = m0 == 0 ? cmake<R>((R)z.x, (R)z.y) : sp[e];
+      const double2 z = m0 == 0 ? z0[e] : make_double2(0.0, 0.0);
+      const double f = pow2(-e0);
+      p[e] = m0 == 0 ? cmake<R>((R)(z.x * f), (R)(z.y * f)) : sp[e];
     }
     L::load_diag(dn, d, l);
     if (T > 0) L::load_cs(cn, r);
@@ -927,7 +953,7 @@ loc_state_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
     double tx = 0.0, ty = 0.0;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      const double2 z = psiT[(batched ? b * N : 0) + l * E + e];
+      const double2 z = zT[e];
       const cplx<R> u = plus_mul<R, L::NEAR>(p[e], dn[e]);
       tx = fma(z.x, (double)u.x, tx); tx = fma(z.y, (double)u.y, tx);
       ty = fma(z.x, (double)u.y, ty); ty = fma(-z.y, (double)u.x, ty);
@@ -937,11 +963,21 @@ loc_state_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
       tx += __shfl_xor_sync(0xffffffffu, tx, off);
       ty += __shfl_xor_sync(0xffffffffu, ty, off);
     }
-    if (F_out && on && l == 0) F_out[b] = tx * tx + ty * ty;
+    if (F_out && on && l == 0) {
+      const double f = pow2(e0), x = tx * f, y = ty * f;
+      F_out[b] = x * x + y * y;
+    }
+    if constexpr (sizeof(R) == 4) {
+      const int eT = top(zT), et = exp_of(make_double2(tx, ty));
+      const double f = pow2(-eT - et);
+      tx *= f;
+      ty *= f;
+      if (on && l == 0) amp[b] = pow2(2 * e0 + eT + et);
+    }
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       // conj(psi_T) conj(tau), then the closing diagonal
-      const double2 z = psiT[(batched ? b * N : 0) + l * E + e];
+      const double2 z = zT[e];
       w[e] = plus_mul<R, L::NEAR>(cmake<R>((R)(z.x * tx - z.y * ty), (R)(-z.y * tx - z.x * ty)), dn[e]);
     }
   }
@@ -1146,24 +1182,26 @@ static PhaseForm phase_form(const redo_table* t, cudaStream_t s) {
 
 template <typename R>
 static cudaError_t loc_finish_t(const redo_table* t, int64_t B, int64_t M, int64_t m0, int64_t T, int parts, double norm,
-                                const LocScratch& w, double* grad, double* gphi, const PhaseForm& f, cudaStream_t s) {
+                                const LocScratch& w, double* grad, double* gphi, const PhaseForm& f,
+                                const double2* tau, const double* amp, cudaStream_t s) {
   const int64_t steps = B * T, gn = steps * t->K, gb = (gn + 127) / 128;
   if (w.sums)
     loc_sums_kernel<R><<<(unsigned)steps, 256, 0, s>>>((const R*)w.bl, parts, 3 * t->loc, w.sums);
   loc_grad_kernel<R><<<(unsigned)(gb < 16384 ? gb : 16384), 128, 0, s>>>(
       steps, t->K, t->loc, t->loc_pairs, parts, t->loc_kptr, t->loc_kpair, (const R*)w.g, (const R*)w.bl, w.sums, M, m0,
-      T, 2.0 * t->dt / norm, grad);
+      T, 2.0 * t->dt / norm, tau, amp, grad);
   if (gphi && f.sums) {
     auto kern = loc_phase_local_kernel<R, false>;
     if constexpr (sizeof(R) == 4)
       if (loc_near(false, t->N)) kern = loc_phase_local_kernel<R, true>;
-    kern<<<(unsigned)(gb < 16384 ? gb : 16384), 128, 0, s>>>(steps, t->K, t->loc, parts, (const cplx<R>*)w.cs,
-                                                             (const R*)w.bl, w.sums, t->wz, 2.0 / norm, gphi, f.gate);
+    kern<<<(unsigned)(gb < 16384 ? gb : 16384), 128, 0, s>>>(steps, M, t->K, t->loc, parts, (const cplx<R>*)w.cs,
+                                                             (const R*)w.bl, w.sums, t->wz, 2.0 / norm, tau, gphi,
+                                                             f.gate);
   }
   if (gphi && f.boundary) {
     const int64_t n = B * M * t->K, blocks = (n + 255) / 256;
     loc_phase_kernel<R><<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>((const R*)w.bz, B, M, parts, t->K,
-                                                                                  2.0 / norm, gphi, f.gate);
+                                                                                  2.0 / norm, tau, gphi, f.gate);
   }
   return cudaGetLastError();
 }
@@ -1195,8 +1233,8 @@ cudaError_t launch_local_grad(const redo_table* t, const int32_t* q, const Chain
     }
     const int64_t at = b0 * p.M * t->K;
     double* gp = gphi ? gphi + at : nullptr;
-    e = dbl ? loc_finish_t<double>(t, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, f, s)
-            : loc_finish_t<float>(t, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, f, s);
+    e = dbl ? loc_finish_t<double>(t, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, f, tau + b0, nullptr, s)
+            : loc_finish_t<float>(t, nb, p.M, 0, p.M, parts, norm, w, grad + at, gp, f, tau + b0, nullptr, s);
     if (e) return e;
   }
   return cudaSuccess;
@@ -1310,6 +1348,8 @@ static cudaError_t loc_state_t(const redo_table* t, const int32_t* q, int64_t B,
   const unsigned blocks = (unsigned)((B + cols - 1) / cols);
   const int64_t nw = M > 0 ? (M + win - 1) / win : 1;
   const bool back = grad && M > 0;
+  // (sized for FP64 vectors: behind the FP32 ones there is room for their scales)
+  double* amp = sizeof(R) == 4 ? (double*)((char*)w.bz + (size_t)B * 2 * t->N * sizeof(cplx<R>)) : nullptr;
   LocScratch fo = w;                                 // forward only: no derivative operators
   fo.g = nullptr;
   // windows 0 .. nw - 1 forward, the last one also back, then nw - 2 .. 0 back
@@ -1321,8 +1361,8 @@ static cudaError_t loc_state_t(const redo_table* t, const int32_t* q, int64_t B,
                                    bk ? w : fo, fwd ? status : nullptr, s);
     if (e) return e;
     LOC_VEC(loc_state_kernel, (const cplx<R>*)w.cs, (const cplx<R>*)w.delta, B, M, m0, T, fwd, bk, psi0, psiT, batched,
-            F_out, (R*)w.bl, (cplx<R>*)w.bz)
-    if (bk && (e = loc_finish_t<R>(t, B, M, m0, T, 1, 1.0, w, grad, nullptr, PhaseForm{}, s))) return e;
+            F_out, (R*)w.bl, (cplx<R>*)w.bz, amp)
+    if (bk && (e = loc_finish_t<R>(t, B, M, m0, T, 1, 1.0, w, grad, nullptr, PhaseForm{}, nullptr, amp, s))) return e;
   }
   return cudaGetLastError();
 }

@@ -32,6 +32,16 @@ template <typename R> __device__ __forceinline__ cplx<R> cmul_conj(cplx<R> a, cp
   return cmake<R>(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, -(a.x * b.y)));
 }
 
+// Powers of two that keep FP32 sums of products in range whatever the length of the vectors and
+// targets that they come from: the exponent of a value (clamped so that a few of them add up within
+// FP64), 2^e, and the exponent of the larger part.  Scaling by them rounds nothing.
+__device__ __forceinline__ int exp_of(double x) {
+  const int e = (int)((__double_as_longlong(x) >> 52) & 0x7ff) - 1023;
+  return e < -200 ? -200 : (e > 200 ? 200 : e);
+}
+__device__ __forceinline__ int exp_of(double2 z) { return max(exp_of(z.x), exp_of(z.y)); }
+__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
+
 // One-qubit tables of a local system: pairs (term k, qubit i) in order of qubit, then term.
 template <typename R>
 struct LocTab {

@@ -758,18 +758,46 @@ template <int E> __device__ __forceinline__ double2 lane_expect(const double2 (&
   return make_double2(acc, 0.0);
 }
 
+// FP32 pairs serve observables and states whose products stay in FP32's range; others (a largest
+// weight outside 2^-60 .. 2^60, or a largest entry of psi_0 outside 2^-60 .. 2^30) are summed in
+// FP64, with the weights read again.  A pulse's flag tells loc_expect_kernel what its parts hold.  (The step loop
+// stands once for each: with the choice inside, a step took 15 % longer.)
+template <int E> __device__ __forceinline__ int2 lane_top(const double2* psi, const double* obs) {
+  int2 t = make_int2(-200, -200);
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    t.x = max(t.x, exp_of(obs[e]));
+    t.y = max(t.y, exp_of(psi[e]));
+  }
+  return t;
+}
+__device__ __forceinline__ bool outside(int2 t) { return t.x < -60 || t.x > 60 || t.y < -60 || t.y > 30; }
+template <int E> __device__ __forceinline__ float2 lane_expect_wide(const float2 (&v)[E], const double* obs) {
+  double acc = 0.0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const double x = (double)v[e].x, y = (double)v[e].y;
+    acc = fma(obs[e], fma(x, x, y * y), acc);
+  }
+  return make_float2(__int_as_float(__double2hiint(acc)), __int_as_float(__double2loint(acc)));
+}
+template <typename R, int E, bool FP64SUM>
+__device__ __forceinline__ cplx<R> lane_part(const cplx<R> (&v)[E], const cplx<R> (&o)[E], const double* obs) {
+  if constexpr (sizeof(R) == 4 && FP64SUM) return lane_expect_wide<E>(v, obs);
+  else return lane_expect<E>(v, o);
+}
+
 // The same for N >= 512: a pulse per block of W warps, eight entries a lane (one warp would issue
 // 2500 instructions a step, one after another).  The qubits of the warp index pair the same lanes of
 // other warps through shared memory; two of them share one exchange, and the buffers alternate so
 // that one barrier a step is enough.
-template <typename R, int N>
-__global__ void __launch_bounds__(N / 8)
-loc_sim_wide_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t M,
-                    const double2* __restrict__ psi0, int batched, const double* __restrict__ obs,
-                    cplx<R>* __restrict__ part) {
+template <typename R, int N, bool FP64SUM>
+__device__ __forceinline__ void
+loc_sim_wide_steps(cplx<R> (*ex)[8][N / 8], const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t M,
+                   const double2* __restrict__ psi0, int batched, const double* __restrict__ obs,
+                   cplx<R>* __restrict__ part) {
   constexpr int E = 8, W = N / 256, LANES = 32 * W, NQ = Log2<N>::v;
   using L = LocCol<R, 256, E>;                       // the qubits within a warp
-  __shared__ cplx<R> ex[2][E][LANES];
   const int lane = threadIdx.x & 31, l = threadIdx.x, wp = threadIdx.x >> 5;
   const int64_t b = blockIdx.x;
   const cplx<R>* d = delta + b * (M + 1) * N;
@@ -799,7 +827,7 @@ loc_sim_wide_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ 
     const double ov = obs[l * E + e];
     w[e] = cmake<R>((R)ov, (R)(ov - (double)(R)ov));
   }
-  o[0] = lane_expect<E>(v, w);
+  o[0] = lane_part<R, E, FP64SUM>(v, w, obs + l * E);
   if (M > 0) load(0);
 #pragma unroll 1
   for (int64_t m = 0; m < M; ++m) {
@@ -824,15 +852,38 @@ loc_sim_wide_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ 
         v[e] = rot_one<R, false>(v[e], p, c9.x, (wp & 2) ? c9.y : -c9.y, R(0));
       }
     }
-    o[(m + 1) * LANES] = lane_expect<E>(v, w);
+    o[(m + 1) * LANES] = lane_part<R, E, FP64SUM>(v, w, obs + l * E);
   }
+}
+template <typename R, int N>
+__global__ void __launch_bounds__(N / 8)
+loc_sim_wide_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t M,
+                    const double2* __restrict__ psi0, int batched, const double* __restrict__ obs,
+                    cplx<R>* __restrict__ part, int32_t* __restrict__ flags) {
+  constexpr int E = 8;
+  __shared__ cplx<R> ex[2][E][N / 8];
+  if constexpr (sizeof(R) == 4) {
+    const int l = threadIdx.x;
+    const int2 t = lane_top<E>(psi0 + (batched ? (int64_t)blockIdx.x * N : 0) + l * E, obs + l * E);
+    int* top = reinterpret_cast<int*>(ex);           // (free until the first step)
+    if (l == 0) top[0] = top[1] = -200;
+    __syncthreads();
+    atomicMax(top, t.x);
+    atomicMax(top + 1, t.y);
+    __syncthreads();
+    const bool far = outside(make_int2(top[0], top[1]));
+    __syncthreads();
+    if (l == 0) flags[blockIdx.x] = far;
+    if (far) return loc_sim_wide_steps<R, N, true>(ex, cs, delta, M, psi0, batched, obs, part);
+  }
+  loc_sim_wide_steps<R, N, false>(ex, cs, delta, M, psi0, batched, obs, part);
 }
 
 // part[b][n][l]: lane l's part of <O> after n steps
-template <typename R, int N>
-__global__ void __launch_bounds__(32)
-loc_sim_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t B, int64_t M,
-               const double2* __restrict__ psi0, int batched, const double* __restrict__ obs, cplx<R>* __restrict__ part) {
+template <typename R, int N, bool FP64SUM>
+__device__ __forceinline__ void
+loc_sim_steps(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t B, int64_t M,
+              const double2* __restrict__ psi0, int batched, const double* __restrict__ obs, cplx<R>* __restrict__ part) {
   constexpr int E = loc_vec_entries(N);
   using L = LocCol<R, N, E>;
   const int lane = threadIdx.x, l = lane / L::C;
@@ -850,7 +901,7 @@ loc_sim_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta
     const double ov = obs[l * E + e];
     w[e] = cmake<R>((R)ov, (R)(ov - (double)(R)ov));
   }
-  cplx<R> a = lane_expect<E>(v, w);
+  cplx<R> a = lane_part<R, E, FP64SUM>(v, w, obs + l * E);
   if (on) o[0] = a;
   if (M > 0) {
     L::load_diag(dn, d, l);
@@ -867,22 +918,48 @@ loc_sim_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta
     L::load_diag(dn, d + nx * N, l);
     L::load_cs(cn, r + nx * L::CS);
     L::rotate(v, c, l);
-    a = lane_expect<E>(v, w);                        // |v|^2: the trailing phases do not enter
+    a = lane_part<R, E, FP64SUM>(v, w, obs + l * E); // |v|^2: the trailing phases do not enter
     if (on) o[(m + 1) * L::G] = a;
   }
 }
+// A warp's pulses are summed alike; each one's flag is the warp's.
+template <typename R, int N>
+__global__ void __launch_bounds__(32)
+loc_sim_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t B, int64_t M,
+               const double2* __restrict__ psi0, int batched, const double* __restrict__ obs, cplx<R>* __restrict__ part,
+               int32_t* __restrict__ flags) {
+  constexpr int E = loc_vec_entries(N);
+  using L = LocCol<R, N, E>;
+  if constexpr (sizeof(R) == 4) {
+    const int lane = threadIdx.x, l = lane / L::C;
+    const int64_t b_raw = (int64_t)blockIdx.x * L::C + lane % L::C, b = b_raw < B ? b_raw : B - 1;
+    int2 t = lane_top<E>(psi0 + (batched ? b * N : 0) + l * E, obs + l * E);
+#pragma unroll
+    for (int off = L::C; off < 32; off *= 2)
+      t = make_int2(max(t.x, __shfl_xor_sync(0xffffffffu, t.x, off)), max(t.y, __shfl_xor_sync(0xffffffffu, t.y, off)));
+    const bool far = __any_sync(0xffffffffu, outside(t));
+    if (b_raw < B && l == 0) flags[b] = far;
+    if (far) return loc_sim_steps<R, N, true>(cs, delta, B, M, psi0, batched, obs, part);
+  }
+  loc_sim_steps<R, N, false>(cs, delta, B, M, psi0, batched, obs, part);
+}
 
-// expect[i] = sum of its G parts, min(G, 32) lanes an item
+// expect[i] = sum of its G parts, min(G, 32) lanes an item (per items a pulse)
 template <typename R>
-__global__ void loc_expect_kernel(const cplx<R>* __restrict__ part, int64_t n, int G, double* __restrict__ expect) {
+__global__ void loc_expect_kernel(const cplx<R>* __restrict__ part, int64_t n, int64_t items, int G,
+                                  const int32_t* __restrict__ flags, double* __restrict__ expect) {
   const int w = G < 32 ? G : 32, l = threadIdx.x % w;
   const int64_t per = blockDim.x / w;
   for (int64_t i0 = blockIdx.x * per; i0 < n; i0 += gridDim.x * per) {
     const int64_t i = i0 + threadIdx.x / w;
     double a = 0.0;
+    const bool wide = sizeof(R) == 4 && i < n && flags[i / items] != 0;
     for (int q = l; q < G && i < n; q += w) {
       const cplx<R> p = part[i * G + q];
-      a += (double)p.x + (double)p.y;
+      if constexpr (sizeof(R) == 4)
+        a += wide ? __hiloint2double(__float_as_int(p.x), __float_as_int(p.y)) : (double)p.x + (double)p.y;
+      else
+        a += p.x;
     }
     for (int off = w / 2; off >= 1; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
     if (l == 0 && i < n) expect[i] = a;
@@ -1045,6 +1122,7 @@ static int loc_parts(const redo_table* t, bool dbl) {
 // sums, the boundary traces or the lanes' parts of the observable.
 struct LocScratch {
   void *delta, *cs, *bl, *bz, *g;
+  int32_t* flags;                                    // [pulses], observables only
   double* sums;
   size_t total;
 };
@@ -1068,6 +1146,7 @@ static LocScratch loc_scratch(const redo_table* t, int64_t nb, int64_t M, int pr
   w.bz = take(what == kLocalPhaseGrad ? (size_t)nb * (M + 1) * parts * t->K * el : 0);
   w.g = grad ? take((size_t)nb * M * t->loc_pairs * 3 * el) : nullptr;
   w.sums = grad && parts >= kLocSumParts ? (double*)take((size_t)nb * M * 3 * t->loc * sizeof(double)) : nullptr;
+  w.flags = what == kLocalSim ? (int32_t*)take((size_t)nb * sizeof(int32_t)) : nullptr;
   w.total = off;
   return w;
 }
@@ -1263,20 +1342,21 @@ static cudaError_t loc_sim_t(const redo_table* t, int64_t B, int64_t M, const do
   const cplx<R>*cs = (const cplx<R>*)w.cs, *delta = (const cplx<R>*)w.delta;
   cplx<R>* part = (cplx<R>*)w.bl;
   switch (t->N) {
-    case 2: loc_sim_kernel<R, 2><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
-    case 4: loc_sim_kernel<R, 4><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
-    case 8: loc_sim_kernel<R, 8><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
-    case 16: loc_sim_kernel<R, 16><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
-    case 32: loc_sim_kernel<R, 32><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
-    case 64: loc_sim_kernel<R, 64><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
-    case 128: loc_sim_kernel<R, 128><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
-    case 256: loc_sim_kernel<R, 256><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part); break;
-    case 512: loc_sim_wide_kernel<R, 512><<<blocks, 64, 0, s>>>(cs, delta, M, psi0, batched, obs, part); break;
-    case 1024: loc_sim_wide_kernel<R, 1024><<<blocks, 128, 0, s>>>(cs, delta, M, psi0, batched, obs, part); break;
+    case 2: loc_sim_kernel<R, 2><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part, w.flags); break;
+    case 4: loc_sim_kernel<R, 4><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part, w.flags); break;
+    case 8: loc_sim_kernel<R, 8><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part, w.flags); break;
+    case 16: loc_sim_kernel<R, 16><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part, w.flags); break;
+    case 32: loc_sim_kernel<R, 32><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part, w.flags); break;
+    case 64: loc_sim_kernel<R, 64><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part, w.flags); break;
+    case 128: loc_sim_kernel<R, 128><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part, w.flags); break;
+    case 256: loc_sim_kernel<R, 256><<<blocks, 32, 0, s>>>(cs, delta, B, M, psi0, batched, obs, part, w.flags); break;
+    case 512: loc_sim_wide_kernel<R, 512><<<blocks, 64, 0, s>>>(cs, delta, M, psi0, batched, obs, part, w.flags); break;
+    case 1024: loc_sim_wide_kernel<R, 1024><<<blocks, 128, 0, s>>>(cs, delta, M, psi0, batched, obs, part, w.flags); break;
     default: return cudaErrorInvalidValue;
   }
   const int64_t n = B * (M + 1), per = 128 / (lanes < 32 ? lanes : 32), nb = (n + per - 1) / per;
-  loc_expect_kernel<R><<<(unsigned)(nb < 4096 ? nb : 4096), 128, 0, s>>>((const cplx<R>*)w.bl, n, lanes, expect);
+  loc_expect_kernel<R><<<(unsigned)(nb < 4096 ? nb : 4096), 128, 0, s>>>((const cplx<R>*)w.bl, n, M + 1, lanes,
+                                                                     w.flags, expect);
   return cudaGetLastError();
 }
 
@@ -1332,6 +1412,7 @@ static LocScratch loc_state_scratch(const redo_table* t, const LocStatePlan& p, 
   w.g = c;
   c += up256(nb * T * 3 * t->loc_pairs * sizeof(double));
   w.sums = nullptr;
+  w.flags = nullptr;
   w.total = (size_t)(c - (char*)base);
   return w;
 }

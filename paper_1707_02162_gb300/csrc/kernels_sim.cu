@@ -8,7 +8,7 @@
 // registers while the current one is applied.  Thread (row r, part p) owns the
 // N/P entries A[r][p*N/P ...] of every operator; the P partial sums of a row
 // are combined with warp shuffles.
-#include "redo_internal.cuh"
+#include "local_ops.cuh"
 
 #include <type_traits>
 #include <vector>
@@ -408,32 +408,49 @@ cudaError_t diag_ctl_build(redo_table* t, const DiagParts& o, char* base, cudaSt
   return cudaGetLastError();
 }
 
-template <typename R, int N>
-__global__ void __launch_bounds__(kColThreads)
-expect_diagctl_kernel(const cplx<R>* __restrict__ U, int64_t entries, const int32_t* __restrict__ q, int64_t B, int64_t M,
-                      int K, int d, int base, int64_t levels, const double* __restrict__ rho,
-                      const double* __restrict__ obs, double* __restrict__ expect, double* __restrict__ mean,
-                      int64_t* status) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  cplx<R>* us = reinterpret_cast<cplx<R>*>(smem_raw);    // the factors, then D - 1
-  for (int64_t i = threadIdx.x; i < entries + N * N; i += blockDim.x) us[i] = U[i];
+// How a step's N terms o_r |u_r|^2 are added: kPlain rounds the weights to R.  The CTA-per-pulse kernel,
+// which a few pulses would take, does not: in its place (PAIRS) weights that FP32 does not hold are kept
+// as FP32 hi + lo (kPairs), and with a largest weight outside 2^-60 .. 2^60 the terms are added in FP64
+// (kFar).  (The terms of the other two are added in FP32: in FP64 pairs the mean was no nearer 64 bits,
+// 4.7e-7 both at N = 8, 50 x 300, and a call took 2.5 times as long; with the choice in the loop likewise.)
+enum { kPlain = 0, kPairs = 1, kFar = 2 };
+// FEW: a bad level index counts once per digit and not once per lane (as the kernel in whose place).
+template <typename R, int N, int SUM, bool FEW>
+__device__ __forceinline__ void
+expect_diagctl_body(const cplx<R>* us, int64_t entries, const int32_t* __restrict__ q, int64_t B, int64_t M, int K, int d,
+                    int base, int64_t levels, const double* __restrict__ rho, const double* __restrict__ obs,
+                    double* __restrict__ expect, double* __restrict__ mean, int64_t* status, int bad_weight) {
   const cplx<R>* D = us + entries;
-  __syncthreads();
   const int c = threadIdx.x % N;
   const int64_t b_raw = (int64_t)blockIdx.x * (blockDim.x / N) + threadIdx.x / N;
   const bool active = b_raw < B;
   const int64_t b = active ? b_raw : B - 1;        // idle lanes follow the last pulse, write nothing
-  R o[N];
+  R o[N], olo[SUM == kPairs ? N : 1];
 #pragma unroll
-  for (int r = 0; r < N; ++r) o[r] = (R)obs[r];
+  for (int r = 0; r < N; ++r) {
+    o[r] = (R)obs[r];
+    if constexpr (SUM == kPairs) olo[r] = (R)(obs[r] - (double)o[r]);
+  }
   const double rc = rho[c];
   cplx<R> u[N];
 #pragma unroll
   for (int r = 0; r < N; ++r) u[r] = cmake<R>(r == c ? R(1) : R(0), R(0));
-  auto part = [&]() -> R {
-    R v = R(0);
+  using V = typename std::conditional<SUM == kFar, double, R>::type;
+  V plo = V(0);                                    // what the weights' second parts add (kPairs)
+  auto part = [&]() -> V {
+    V v = V(0);
+    if constexpr (SUM == kPairs) plo = V(0);
 #pragma unroll
-    for (int r = 0; r < N; ++r) v = fma(o[r], fma(u[r].x, u[r].x, u[r].y * u[r].y), v);
+    for (int r = 0; r < N; ++r) {
+      if constexpr (SUM == kFar) {
+        const double x = (double)u[r].x, y = (double)u[r].y;
+        v = fma(obs[r], fma(x, x, y * y), v);
+      } else {
+        const R s = fma(u[r].x, u[r].x, u[r].y * u[r].y);
+        v = fma(o[r], s, v);
+        if constexpr (SUM == kPairs) plo = fma(olo[r], s, plo);
+      }
+    }
     return v;
   };
   auto group_sum = [&](double v) -> double {
@@ -441,10 +458,15 @@ expect_diagctl_kernel(const cplx<R>* __restrict__ U, int64_t entries, const int3
     for (int off = N / 2; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off, N);
     return v;
   };
-  const double e0 = group_sum(rc * (double)part());
+  auto value = [&](V v) -> double {
+    if constexpr (SUM == kPairs) return (double)v + (double)plo;
+    return (double)v;
+  };
+  const V p0 = part();
+  const double e0 = group_sum(rc * value(p0));
   if (expect && active && c == 0) expect[b * (M + 1)] = e0;
   const uint32_t recip = (uint32_t)((((uint64_t)1 << 32) + base - 1) / base);
-  R acc = R(0), lo = R(0);                         // the steps' sum as a pair: an FP32 step needs no FP64
+  V acc = V(0), lo = V(0);                         // the steps' sum as a pair: an FP32 step needs no FP64
   const int32_t* qb = q + b * M * K;
   int32_t qn = M > 0 ? qb[0] : 0;
   for (int64_t n = 0; n < M; ++n) {
@@ -474,7 +496,8 @@ expect_diagctl_kernel(const cplx<R>* __restrict__ U, int64_t entries, const int3
       // next coefficient's level, loaded while this one is applied
       qn = (k + 1 < K) ? qrow[k + 1] : (n + 1 < M ? qrow[K] : 0);
       if (qv < 0 || qv >= levels) {
-        if (status && active) atomicAdd((unsigned long long*)&status[REDO_STATUS_BADINDEX], 1ull);
+        if (status && active && (!FEW || c == 0))
+          atomicAdd((unsigned long long*)&status[REDO_STATUS_BADINDEX], FEW ? (unsigned long long)bad_weight : 1ull);
         qv = 0;
       }
       for (int j = 0; j < d; ++j) {
@@ -489,16 +512,46 @@ expect_diagctl_kernel(const cplx<R>* __restrict__ U, int64_t entries, const int3
         }
       }
     }
-    const R pv = part(), t = acc + pv, z = t - acc;
+    const V pv = part(), t = acc + pv, z = t - acc;
     lo += (acc - (t - z)) + (pv - z);
+    if constexpr (SUM == kPairs) lo += plo;
     acc = t;
     if (expect) {
-      const double ev = group_sum(rc * (double)pv);
+      const double ev = group_sum(rc * value(pv));
       if (active && c == 0) expect[b * (M + 1) + n + 1] = ev;
     }
   }
   const double tot = group_sum(rc * ((double)acc + (double)lo));
   if (mean && active && c == 0) mean[b] = M > 0 ? tot / (double)M : e0;
+}
+
+template <typename R, int N, bool PAIRS>
+__global__ void __launch_bounds__(kColThreads)
+expect_diagctl_kernel(const cplx<R>* __restrict__ U, int64_t entries, const int32_t* __restrict__ q, int64_t B, int64_t M,
+                      int K, int d, int base, int64_t levels, const double* __restrict__ rho,
+                      const double* __restrict__ obs, double* __restrict__ expect, double* __restrict__ mean,
+                      int64_t* status, int bad_weight) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cplx<R>* us = reinterpret_cast<cplx<R>*>(smem_raw);    // the factors, then D - 1
+  for (int64_t i = threadIdx.x; i < entries + N * N; i += blockDim.x) us[i] = U[i];
+  __syncthreads();
+  if constexpr (PAIRS) {
+    int top = -200;
+    bool held = true;
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      top = max(top, exp_of(obs[r]));
+      held = held && (double)(R)obs[r] == obs[r];
+    }
+    if (top < -60 || top > 60)
+      return expect_diagctl_body<R, N, kFar, true>(us, entries, q, B, M, K, d, base, levels, rho, obs, expect, mean,
+                                                   status, bad_weight);
+    if (!held)
+      return expect_diagctl_body<R, N, kPairs, true>(us, entries, q, B, M, K, d, base, levels, rho, obs, expect, mean,
+                                                     status, bad_weight);
+  }
+  expect_diagctl_body<R, N, kPlain, PAIRS>(us, entries, q, B, M, K, d, base, levels, rho, obs, expect, mean, status,
+                                           bad_weight);
 }
 
 template <typename R, int N>
@@ -507,6 +560,10 @@ static cudaError_t expect_diag_n(const redo_table* t, const int32_t* q, int64_t 
                                  cudaStream_t s) {
   const cplx<R>* T = std::is_same<R, double>::value ? (const cplx<R>*)t->T64 : (const cplx<R>*)t->T32;
   if constexpr (N * sizeof(R) <= 64) {            // one column in registers: N <= 16 (FP32), 8 (FP64)
+    const size_t table_smem = (size_t)t->entries * N * N * sizeof(cplx<R>);
+    // a column per thread: worth it once every SM gets a full CTA (256 / N pulses); fewer pulses keep
+    // one CTA each
+    const bool cols = table_smem <= 200 * 1024 && B * N >= (int64_t)t->num_sms * kColThreads;
     // FP64 only with a column for every lane of the SMs: a warp's FP64 instruction takes 70 cycles, so
     // few pulses do better with a thread per entry (N = 8, 240 x 693: 9.4 ms here, 2.6 ms there)
     if (t->dct && (sizeof(R) == 4 || B * N >= (int64_t)t->num_sms * kColThreads)) {
@@ -515,17 +572,16 @@ static cudaError_t expect_diag_n(const redo_table* t, const int32_t* q, int64_t 
       const int th = B * N >= (int64_t)t->num_sms * kColThreads ? 64 : 32, per = th / N;
       const int64_t ent = (int64_t)t->K * t->digit_count * t->digit_base * N;
       const size_t smem = (size_t)(ent + N * N) * sizeof(cplx<R>);
-      cudaError_t e = cudaFuncSetAttribute(expect_diagctl_kernel<R, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem);
+      const bool pairs = sizeof(R) == 4 && !cols;
+      auto kern = pairs ? expect_diagctl_kernel<R, N, sizeof(R) == 4> : expect_diagctl_kernel<R, N, false>;
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
-      expect_diagctl_kernel<R, N><<<(unsigned)((B + per - 1) / per), th, smem, s>>>(
+      kern<<<(unsigned)((B + per - 1) / per), th, smem, s>>>(
           std::is_same<R, double>::value ? (const cplx<R>*)t->dct_u : (const cplx<R>*)t->dct_u32, ent, q, B, M, t->K,
-          t->digit_count, t->digit_base, t->levels, rho, obs, expect, mean, status);
+          t->digit_count, t->digit_base, t->levels, rho, obs, expect, mean, status, pairs ? t->digits : 1);
       return cudaGetLastError();
     }
-    const size_t table_smem = (size_t)t->entries * N * N * sizeof(cplx<R>);
-    // worth it once every SM gets a full CTA (256 / N pulses); fewer pulses keep one CTA each
-    if (table_smem <= 200 * 1024 && B * N >= (int64_t)t->num_sms * kColThreads) {
+    if (cols) {
       cudaError_t e = cudaFuncSetAttribute(expect_cols_kernel<R, N>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)table_smem);
       if (e != cudaSuccess) return e;

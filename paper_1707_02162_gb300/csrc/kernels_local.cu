@@ -412,11 +412,11 @@ loc_steps_kernel(LocTab<R> tab, const int32_t* __restrict__ q, int64_t M, int64_
 // ============================================================================
 constexpr int kLocThreads = 128;
 
-template <typename R, int N, int E>
+template <typename R, int N, int E, bool NEAR>
 __global__ void __launch_bounds__(kLocThreads)
 loc_chain_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ delta, int64_t M, int64_t S, int64_t sps,
                  int64_t chains, cplx<R>* __restrict__ out) {
-  using L = LocCol<R, N, E>;
+  using L = LocCol<R, N, E, NEAR>;
   static_assert(L::G == 1 || N >= L::C, "lanes of one warp share a chain when they exchange");
   const int lane = threadIdx.x & 31, l = lane / L::C;
   const int64_t col = ((int64_t)blockIdx.x * (kLocThreads / 32) + (threadIdx.x >> 5)) * L::C + lane % L::C;
@@ -452,13 +452,16 @@ __host__ __device__ constexpr int loc_entries(bool dbl, int N, bool two) {
 }
 
 template <typename R, int N, bool TWO>
-static cudaError_t loc_chain_n(const redo_table* t, const ChainPlan& p, int64_t B, const void* cs, const void* delta,
-                               void* out, cudaStream_t s) {
+static cudaError_t loc_chain_n(const redo_table* t, const ChainPlan& p, int64_t B, bool near, const void* cs,
+                               const void* delta, void* out, cudaStream_t s) {
   constexpr int E = loc_entries(sizeof(R) == 8, N, TWO);
   const int64_t fps = (int64_t)t->K * t->digits, chains = B * p.S, sps = p.seg_len / fps;
   const int64_t warps = (chains * N * (N / E) + 31) / 32;
   if (warps == 0) return cudaSuccess;
-  loc_chain_kernel<R, N, E><<<(unsigned)((warps + 3) / 4), kLocThreads, 0, s>>>(
+  auto kern = loc_chain_kernel<R, N, E, loc_near(sizeof(R) == 8, N)>;
+  if constexpr (sizeof(R) == 4 && !TWO)
+    if (near) kern = loc_chain_kernel<R, N, E, true>;
+  kern<<<(unsigned)((warps + 3) / 4), kLocThreads, 0, s>>>(
       (const cplx<R>*)cs, (const cplx<R>*)delta, p.M, p.S, sps > 0 ? sps : 1, chains, (cplx<R>*)out);
   return cudaGetLastError();
 }
@@ -479,9 +482,9 @@ static cudaError_t loc_chain_n(const redo_table* t, const ChainPlan& p, int64_t 
   }
 
 template <typename R, bool TWO>
-static cudaError_t loc_chain_t(const redo_table* t, const ChainPlan& p, int64_t B, const void* cs, const void* delta,
-                               void* out, cudaStream_t s) {
-  LOC_DISPATCH(loc_chain_n, t, p, B, cs, delta, out, s)
+static cudaError_t loc_chain_t(const redo_table* t, const ChainPlan& p, int64_t B, bool near, const void* cs,
+                               const void* delta, void* out, cudaStream_t s) {
+  LOC_DISPATCH(loc_chain_n, t, p, B, near, cs, delta, out, s)
 }
 
 // ============================================================================
@@ -1127,6 +1130,7 @@ struct LocScratch {
   size_t total;
 };
 constexpr size_t kLocSumParts = 8;                   // from here on the parts are added by a kernel of their own
+static bool loc_near_of(const redo_table* t, bool dbl, int what) { return what == kLocalChainFine || loc_near(dbl, t->N); }
 static LocScratch loc_scratch(const redo_table* t, int64_t nb, int64_t M, int prec, int what, void* base) {
   const size_t el = prec == REDO_FP64 ? sizeof(double) : sizeof(float);
   const bool grad = what == kLocalGrad || what == kLocalPhaseGrad;
@@ -1141,7 +1145,7 @@ static LocScratch loc_scratch(const redo_table* t, int64_t nb, int64_t M, int pr
     return at;
   };
   w.delta = take((size_t)nb * (M + 1) * t->N * 2 * el);
-  w.cs = take((size_t)nb * M * t->loc * 2 * el * (loc_near(prec == REDO_FP64, t->N) ? 2 : 1));
+  w.cs = take((size_t)nb * M * t->loc * 2 * el * (loc_near_of(t, prec == REDO_FP64, what) ? 2 : 1));
   w.bl = take(grad ? (size_t)nb * M * parts * 3 * t->loc * el : (size_t)nb * (M + 1) * lanes * 2 * el);
   w.bz = take(what == kLocalPhaseGrad ? (size_t)nb * (M + 1) * parts * t->K * el : 0);
   w.g = grad ? take((size_t)nb * M * t->loc_pairs * 3 * el) : nullptr;
@@ -1168,6 +1172,16 @@ bool local_pays(const redo_table* t, int prec) {
   if (prec == REDO_FP64) return dense > 32.0 * t->loc_pairs + 230.0 * n + 28.0 * N + N * N * (4 + 4 * n);
   const double rot = loc_near(false, t->N) ? 6 + 8 * n : 4 + 4 * n;
   return 1.5 * dense > 40.0 * t->loc_pairs + 500.0 * n + 100.0 * N + N * N * rot;
+}
+
+// Which chain form a call takes.  FP32 products of controls that act on one qubit each have two nonzeros
+// a row, so the dense chain rounds twice a product, and the real rotations' error was up to 1.4 times its
+// (U, N = 64, 12 controls, 200 steps: 7.9e-7 dense, 1.0e-6); rotations near the identity, twice the
+// multiply-adds, give 4.4e-7 (N = 32: 6.3e-7, 9.1e-7, 3.6e-7; N = 128: 5.1e-7, 6.6e-7, 3.1e-7).  Split
+// FP16 was 5 times less exact (5.5e-6) and takes the real rotations; controls on several qubits at once
+// (global fields) have dense rows, whose error was larger (N = 64: 1.7e-6, 1.0e-6 with the real rotations).
+int local_chain_form(const redo_table* t, int prec_asked) {
+  return prec_asked == REDO_FP32 && t->loc_pairs <= t->K && t->N > 16 ? kLocalChainFine : kLocalChain;
 }
 
 static int64_t local_slice(const redo_table* t, int64_t B, int64_t M, int prec, int what) {
@@ -1198,13 +1212,14 @@ ChainPlan plan_chain_local(const redo_table* t, int64_t B, int64_t M, int prec, 
 
 template <typename R>
 static cudaError_t loc_steps_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int64_t m0, int64_t T, int E,
+                               bool near,
                                const LocalDiag& pd, int64_t b0, const LocScratch& w, int64_t* status,
                                cudaStream_t s) {
   const int ts = B * (T + 1) >= (int64_t)t->num_sms * 8 * kPrepSteps ? kPrepSteps : 8;
   const int64_t tiles = (T + 1 + ts - 1) / ts;
   auto kern = loc_steps_kernel<R, false>;
   if constexpr (sizeof(R) == 4)
-    if (loc_near(false, t->N)) kern = loc_steps_kernel<R, true>;
+    if (near) kern = loc_steps_kernel<R, true>;
   kern<<<(unsigned)(B * tiles), kPrepThreads, 0, s>>>(
       loc_tab<R>(t, status), q + b0 * M * t->K, M, m0, T, t->loc, t->N, E, tiles, ts,
       sizeof(R) == 8 ? (const typename DiagOf<R>::T*)t->loc_D64 : (const typename DiagOf<R>::T*)t->loc_D32,
@@ -1213,28 +1228,30 @@ static cudaError_t loc_steps_t(const redo_table* t, const int32_t* q, int64_t B,
   return cudaGetLastError();
 }
 
-static cudaError_t loc_steps(const redo_table* t, const int32_t* q, int64_t nb, int64_t M, int prec, int E,
+static cudaError_t loc_steps(const redo_table* t, const int32_t* q, int64_t nb, int64_t M, int prec, int what, int E,
                              const LocalDiag& pd, int64_t b0, const LocScratch& w, int64_t* status, cudaStream_t s) {
-  return prec == REDO_FP64 ? loc_steps_t<double>(t, q, nb, M, 0, M, E, pd, b0, w, status, s)
-                           : loc_steps_t<float>(t, q, nb, M, 0, M, E, pd, b0, w, status, s);
+  const bool near = loc_near_of(t, prec == REDO_FP64, what);
+  return prec == REDO_FP64 ? loc_steps_t<double>(t, q, nb, M, 0, M, E, near, pd, b0, w, status, s)
+                           : loc_steps_t<float>(t, q, nb, M, 0, M, E, near, pd, b0, w, status, s);
 }
 
 cudaError_t launch_local_chain(const redo_table* t, const int32_t* q, const ChainPlan& p, int prec, int what,
                                const LocalDiag& pd, void* ops, void* seg_out, int64_t* status, cudaStream_t s) {
-  const bool dbl = prec == REDO_FP64, two = what != kLocalChain;
+  const bool dbl = prec == REDO_FP64, two = what == kLocalGrad || what == kLocalPhaseGrad;
+  const bool near = loc_near_of(t, dbl, what);
   const int64_t slice = local_slice(t, p.B, p.M, prec, what);
   const LocScratch w = loc_scratch(t, slice, p.M, prec, what, ops);
   const int E = loc_entries(dbl, t->N, two);
   const size_t mat = (size_t)t->N * t->N * (dbl ? sizeof(double2) : sizeof(float2));
   for (int64_t b0 = 0; b0 < p.B; b0 += slice) {
     const int64_t nb = b0 + slice < p.B ? slice : p.B - b0;
-    cudaError_t e = loc_steps(t, q, nb, p.M, prec, E, pd, b0, w, status, s);
+    cudaError_t e = loc_steps(t, q, nb, p.M, prec, what, E, pd, b0, w, status, s);
     if (e) return e;
     void* out = (char*)seg_out + (size_t)(b0 * p.S) * mat;
-    e = dbl ? (two ? loc_chain_t<double, true>(t, p, nb, w.cs, w.delta, out, s)
-                   : loc_chain_t<double, false>(t, p, nb, w.cs, w.delta, out, s))
-            : (two ? loc_chain_t<float, true>(t, p, nb, w.cs, w.delta, out, s)
-                   : loc_chain_t<float, false>(t, p, nb, w.cs, w.delta, out, s));
+    e = dbl ? (two ? loc_chain_t<double, true>(t, p, nb, near, w.cs, w.delta, out, s)
+                   : loc_chain_t<double, false>(t, p, nb, near, w.cs, w.delta, out, s))
+            : (two ? loc_chain_t<float, true>(t, p, nb, near, w.cs, w.delta, out, s)
+                   : loc_chain_t<float, false>(t, p, nb, near, w.cs, w.delta, out, s));
     if (e) return e;
   }
   return cudaSuccess;
@@ -1300,7 +1317,7 @@ cudaError_t launch_local_grad(const redo_table* t, const int32_t* q, const Chain
   for (int64_t b0 = 0; b0 < p.B; b0 += slice) {
     const int64_t nb = b0 + slice < p.B ? slice : p.B - b0;
     cudaError_t e = cudaSuccess;
-    if (slice < p.B && (e = loc_steps(t, q, nb, p.M, prec, E, pd, b0, w, status, s))) return e;
+    if (slice < p.B && (e = loc_steps(t, q, nb, p.M, prec, what, E, pd, b0, w, status, s))) return e;
     const char* P = (const char*)Pck + (size_t)(b0 * p.S) * mat;
     const char* Q = (const char*)Rck + (size_t)(b0 * p.S) * mat;
     for (int tz = 0; tz < 2; ++tz) {
@@ -1366,7 +1383,7 @@ cudaError_t launch_local_sim(const redo_table* t, const int32_t* q, int64_t B, i
   const LocScratch w = loc_scratch(t, slice, M, prec, kLocalSim, ops);
   for (int64_t b0 = 0; b0 < B; b0 += slice) {
     const int64_t nb = b0 + slice < B ? slice : B - b0;
-    cudaError_t e = loc_steps(t, q, nb, M, prec, loc_sim_entries(t->N), LocalDiag{nullptr, 0, 0}, b0, w, status, s);
+    cudaError_t e = loc_steps(t, q, nb, M, prec, kLocalSim, loc_sim_entries(t->N), LocalDiag{nullptr, 0, 0}, b0, w, status, s);
     if (e) return e;
     const double2* p0 = psi0 + (batched ? b0 * t->N : 0);
     double* ex = expect + b0 * (M + 1);
@@ -1438,7 +1455,7 @@ static cudaError_t loc_state_t(const redo_table* t, const int32_t* q, int64_t B,
     const bool fwd = i < nw;
     const int64_t k = fwd ? i : 2 * nw - 2 - i, m0 = k * win, T = m0 + win < M ? win : M - m0;
     const int bk = back && i >= nw - 1;
-    cudaError_t e = loc_steps_t<R>(t, q, B, M, m0, T, loc_vec_entries(t->N), LocalDiag{nullptr, 0, 0}, 0,
+    cudaError_t e = loc_steps_t<R>(t, q, B, M, m0, T, loc_vec_entries(t->N), loc_near(sizeof(R) == 8, t->N), LocalDiag{nullptr, 0, 0}, 0,
                                    bk ? w : fo, fwd ? status : nullptr, s);
     if (e) return e;
     LOC_VEC(loc_state_kernel, (const cplx<R>*)w.cs, (const cplx<R>*)w.delta, B, M, m0, T, fwd, bk, psi0, psiT, batched,

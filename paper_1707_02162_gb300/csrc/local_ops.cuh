@@ -232,8 +232,8 @@ __host__ __device__ __forceinline__ int loc_pos(int r, int E, int G) {   // E >=
   return ((e >> 1) * G + l) * 2 + (e & 1);
 }
 
-template <typename R, int N, int E> struct LocCol {
-  static constexpr bool NEAR = loc_near(sizeof(R) == 8, N);
+template <typename R, int N, int E, bool NR = loc_near(sizeof(R) == 8, N)> struct LocCol {
+  static constexpr bool NEAR = NR;
   static constexpr int G = N / E, C = 32 / G, NQ = Log2<N>::v, EB = Log2<E>::v;
   static constexpr int CS = NQ * (NEAR ? 2 : 1);     // (c - 1, s) of every qubit, then (sy, 0)
   static_assert(G * E == N && G <= 32, "column layout");

@@ -486,6 +486,7 @@ struct PropLayout {
   size_t pd_off, zf_off, phout_off;     // amplitude/phase calls
   size_t mid_off;                       // group products of the two-pass combine (N <= 64)
   bool local;                           // locally controlled system: kernels_local.cu forms the segments
+  int what;                             // in this form
   size_t ops_off;                       // its step operators
 };
 
@@ -523,7 +524,8 @@ static PropLayout prop_layout(const redo_table* t, int64_t B, int64_t M, redo_pr
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t el = L.eff_prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
   const size_t n2 = (size_t)t->N * t->N;
-  if (local_eligible(t, M, L.eff_prec, kLocalChain) && (diag || local_pays(t, L.eff_prec))) {
+  L.what = local_chain_form(t, prec);
+  if (local_eligible(t, M, L.eff_prec, L.what) && (diag || local_pays(t, L.eff_prec))) {
     L.local = true;
     L.p = reunit_every > 0 ? plan_chain_aligned(t, B, M, reunit_every) : plan_chain_local(t, B, M, L.eff_prec, false);
     if (t->N > kSmallN) {
@@ -537,7 +539,7 @@ static PropLayout prop_layout(const redo_table* t, int64_t B, int64_t M, redo_pr
       L.total = L.prod64_off + (reunit_every > 0 ? up((size_t)B * n2 * sizeof(double2)) : 0);
     }
     L.ops_off = L.total;
-    L.total += local_ops_bytes(t, B, M, L.eff_prec, kLocalChain);
+    L.total += local_ops_bytes(t, B, M, L.eff_prec, L.what);
     add_strang(t, B, L.total, L.strang_off, L.strang_tmp_off);
     if (diag) add_phase(t, B, diag == 1 ? M : 1, L.total, L.pd_off, L.zf_off, L.phout_off);
     return L;
@@ -645,7 +647,7 @@ static redo_status propagate_core(const redo_table* t, const int32_t* q, const d
   if (L.local) {
     ProfScope ps(2, s);
     const LocalDiag pd{L.p.pd, phase ? M * t->N : t->N, phase ? t->N : 0};
-    if ((e = launch_local_chain(t, q, p, eff, kLocalChain, pd, (char*)workspace + L.ops_off, seg, dev_status, s)) !=
+    if ((e = launch_local_chain(t, q, p, eff, L.what, pd, (char*)workspace + L.ops_off, seg, dev_status, s)) !=
         cudaSuccess)
       return cuda_error(e, "local chains");
   }

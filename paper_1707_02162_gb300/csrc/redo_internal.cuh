@@ -221,8 +221,9 @@ void local_room(const redo_table* t, TableArena& ar, LocalParts& o);
 cudaError_t local_build(redo_table* t, const LocalParts& o, char* base, cudaStream_t s);
 cudaError_t local_phase_axes(redo_table* t, const double* sz);
 // What a call computes: segment products, the gradient, the amplitude/phase gradient, the state's
-// observable.
-enum LocalWhat { kLocalChain = 0, kLocalGrad = 1, kLocalPhaseGrad = 2, kLocalSim = 3 };
+// observable.  kLocalChainFine: segment products by rotations near the identity at every N (local_chain_form).
+enum LocalWhat { kLocalChain = 0, kLocalGrad = 1, kLocalPhaseGrad = 2, kLocalSim = 3, kLocalChainFine = 4 };
+int local_chain_form(const redo_table* t, int prec_asked);
 bool local_eligible(const redo_table* t, int64_t M, int prec, int what);
 bool local_pays(const redo_table* t, int prec);
 size_t local_ops_bytes(const redo_table* t, int64_t B, int64_t M, int prec, int what);

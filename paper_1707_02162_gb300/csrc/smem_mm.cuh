@@ -97,8 +97,8 @@ struct SmemMM {
   // Q = (I - A^dag A) / 2 written to Q, computing only half of the Hermitian Gram matrix: the
   // T(T+1)/2 tiles (ty <= tx) of a square tiling go to the first threads (whole warps), each writes
   // its entries and, off the tile diagonal ty == tx, their conjugate mirrors (tile (ty, tx) and
-  // tile (tx, ty) hold transposed entries).  Its diagonal is left to ns_diag.  Returns after the
-  // caller's barrier is due.
+  // tile (tx, ty) hold transposed entries).  In FP32 its diagonal is left to ns_diag.  Returns after
+  // the caller's barrier is due.
   __device__ __forceinline__ static void ns_half_gram(const cplx<R>* __restrict__ A, cplx<R>* __restrict__ Q,
                                                       int lt) {
     static_assert(TY == TX && TM == TN, "square tiling");
@@ -135,12 +135,16 @@ struct SmemMM {
 #pragma unroll
       for (int c = 0; c < TN; ++c) {
         const int r = ty + TY * a, col = tx + TX * c;
-        if (r != col) Q[r * N + col] = cmake<R>(-R(0.5) * Y[a][c].x, -R(0.5) * Y[a][c].y);
+        if (r != col || !kDiagApart)
+          Q[r * N + col] = cmake<R>((r == col ? R(0.5) : R(0)) - R(0.5) * Y[a][c].x, -R(0.5) * Y[a][c].y);
         if (ty != tx) Q[col * N + r] = cmake<R>(-R(0.5) * Y[a][c].x, R(0.5) * Y[a][c].y);
       }
   }
   // Q[c][c] = (1 - sum_r |A[r][c]|^2) / 2.  A nearly unitary FP32 matrix has this near 1e-8, the
-  // rounding of the plain sum: products are split by fma and added with compensation.
+  // rounding of the plain sum: products are split by fma and added with compensation.  (FP64 takes
+  // the plain sum: N threads with N dependent FP64 steps each made 512 matrices of N = 8 take 14.6 us
+  // in place of 8.9.)
+  static constexpr bool kDiagApart = sizeof(R) == 4;
   __device__ __forceinline__ static void ns_diag(const cplx<R>* __restrict__ A, cplx<R>* __restrict__ Q, int lt) {
     for (int c = lt; c < N; c += THREADS) {
       R s = R(-1), lo = R(0);
@@ -171,10 +175,11 @@ struct SmemMM {
 #pragma unroll
         for (int c = 0; c < TN; ++c) {
           const int r = ty + TY * a, col = tx + TX * c;
-          if (r != col) Q[r * N + col] = cmake<R>(-R(0.5) * Y[a][c].x, -R(0.5) * Y[a][c].y);
+          if (r != col || !kDiagApart)
+            Q[r * N + col] = cmake<R>((r == col ? R(0.5) : R(0)) - R(0.5) * Y[a][c].x, -R(0.5) * Y[a][c].y);
         }
     }
-    ns_diag(A, Q, THREADS - 1 - lt);                       // (the last threads have no half-Gram tile)
+    if constexpr (kDiagApart) ns_diag(A, Q, THREADS - 1 - lt);   // (the last threads have no half-Gram tile)
   }
   // Y = diag(p) X (a row scaling, p in FP64)
   __device__ __forceinline__ static void scale_rows(const double2* __restrict__ p,

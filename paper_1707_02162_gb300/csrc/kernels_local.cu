@@ -1203,8 +1203,16 @@ ChainPlan plan_chain_local(const redo_table* t, int64_t B, int64_t M, int prec, 
   int64_t S = warps > 0 ? (4 * 4 * (int64_t)t->num_sms + warps - 1) / warps : 1;
   const int64_t min_steps = t->N <= 8 ? 4 : (t->N <= 64 ? 8 : 32);
   if (S > M / min_steps) S = M / min_steps;
-  // (FP32 steps and products of N <= 16 are short beside a launch: one combine pass)
-  const int64_t most = !dbl && t->N <= 16 ? 16 : 64;
+  // M / S dependent steps, then 2 sqrt(S) dependent products when the segments are multiplied (in
+  // groups): best near S = (M / r)^(2/3), r the time of a product beside that of a step.  One pulse,
+  // M = 1e5, N = 8: FP64 2.7 ms with 64 segments, 0.57 ms with 1024 (dense plan 3.1 ms); FP32 3.8 ms with
+  // 16, 0.17 ms with 1024 (dense 0.77).  r as measured over M = 500 .. 1e5 (N = 64 FP64: 64 segments are
+  // best at every length).  Short FP32 pulses of N <= 16 stay with one combine pass.
+  const double r = t->N <= 16 ? 1.0 : (t->N == 32 ? 2.0 : (dbl ? 16.0 : 6.0));
+  int64_t most = (int64_t)std::cbrt(((double)M / r) * ((double)M / r));
+  if (most > 1024) most = 1024;
+  const int64_t least = !dbl && t->N <= 16 ? 16 : 64;
+  if (most < least || M < 400) most = least;
   if (S > most) S = most;
   if (S < 1) S = 1;
   return plan_chain_aligned(t, B, M, M > 0 ? (M + S - 1) / S : 1);

@@ -1442,8 +1442,13 @@ static LocScratch loc_state_scratch(const redo_table* t, const LocStatePlan& p, 
   return w;
 }
 
+// A bound of loc_state_scratch that never falls with B (the windows are rounded to whole steps): scratch
+// asked for a batch serves every smaller one.
 size_t local_state_bytes(const redo_table* t, int64_t B) {
-  return t->loc > 0 && B > 0 ? loc_state_scratch(t, loc_state_plan(t, B), nullptr).total : 0;
+  if (t->loc == 0 || B <= 0) return 0;
+  const size_t nb = (size_t)loc_state_plan(t, B).pulses, step = nb * loc_state_step(t), cap = (size_t)64 << 20;
+  const size_t steps = 64 * step > cap ? 64 * step : (4096 * step < cap ? 4096 * step : cap);
+  return up256(steps + nb * t->N * 3 * sizeof(double2) + 5 * 256);
 }
 
 template <typename R>

@@ -591,31 +591,54 @@ template <typename R> __device__ __forceinline__ double loc_scale(const double2*
   if (sizeof(R) == 8) return 1.0;
   return amp ? amp[b] : pow2(exp_of(tau[b]));
 }
+// The phase gradients when every S_kz is a sum of one-qubit parts (wz [K][n], half the difference of a
+// qubit's two values; the species' S_z are): the change of Z_i over a step's rotation follows from the
+// Bloch sums as 2 |s|^2 Z - 2 c (sx X + sy Y), without the boundary traces and the difference of two
+// nearly equal ones (N = 64, 16 x 200, FP32: error against 64 bits 2.4e-6 -> 4.7e-7).  Formed beside the
+// amplitudes' gradients: a launch of its own was 3 of the 66 us of N = 8, 10 x 41.  gphi nullptr: none.
+template <typename R> struct LocPhaseOut {
+  const cplx<R>* cs;
+  const double* wz;
+  const int32_t* gate;
+  double scale;
+  double* gphi;
+  int cs_step;               // entries of cs per step: n, or 2n with the rotations' second parts
+};
 template <typename R>
 __global__ void loc_grad_kernel(int64_t steps, int K, int n, int pairs, int parts, const int32_t* __restrict__ kptr,
                                 const int32_t* __restrict__ kpair, const R* __restrict__ g, const R* __restrict__ bl,
                                 const double* __restrict__ sums, int64_t M, int64_t w0, int64_t T, double scale,
                                 const double2* __restrict__ tau, const double* __restrict__ amp,
-                                double* __restrict__ grad) {
+                                double* __restrict__ grad, LocPhaseOut<R> ph) {
+  const bool phase = ph.gphi && !(ph.gate && *ph.gate == 0);
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < steps * K;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t st = idx / K, b = st / T;
     const int k = (int)(idx - st * K);
+    auto bloch = [&](int i, int c) -> double {
+      if (sums) return sums[st * 3 * n + 3 * i + c];
+      double v = 0.0;
+      for (int q = 0; q < parts; ++q) v += (double)bl[(st * parts + q) * 3 * n + 3 * i + c];
+      return v;
+    };
     double acc = 0.0;
     for (int e = kptr[k]; e < kptr[k + 1]; ++e) {
       const int p = kpair[e] & 0xfffff, i = kpair[e] >> 20;
       const R* gp = g + (st * pairs + p) * 3;
-      for (int c = 0; c < 3; ++c) {
-        double v = 0.0;
-        if (sums) {
-          v = sums[st * 3 * n + 3 * i + c];
-        } else {
-          for (int q = 0; q < parts; ++q) v += (double)bl[(st * parts + q) * 3 * n + 3 * i + c];
-        }
-        acc += (double)gp[c] * v;
-      }
+      for (int c = 0; c < 3; ++c) acc += (double)gp[c] * bloch(i, c);
     }
-    grad[(b * M + w0 + st - b * T) * K + k] = scale * (acc * loc_scale<R>(tau, amp, b));
+    const double f = loc_scale<R>(tau, amp, b);
+    grad[(b * M + w0 + st - b * T) * K + k] = scale * (acc * f);
+    if (!phase) continue;
+    acc = 0.0;
+    for (int i = 0; i < n; ++i) {
+      const double w = ph.wz[k * n + i];
+      if (w == 0.0) continue;
+      const cplx<R>* a = ph.cs + st * ph.cs_step + i;
+      const double c = 1.0 + (double)a->x, sx = (double)a->y, sy = ph.cs_step > n ? (double)a[n].x : 0.0;
+      acc += w * (2.0 * (sx * sx + sy * sy) * bloch(i, 2) - 2.0 * c * (sx * bloch(i, 0) + sy * bloch(i, 1)));
+    }
+    ph.gphi[idx] = ph.scale * (acc * f);
   }
 }
 
@@ -651,43 +674,6 @@ __global__ void loc_phase_kernel(const R* __restrict__ bz, int64_t B, int64_t M,
       c += (double)bz[((b * (M + 1) + n + 1) * parts + p) * K + k];
     }
     gphi[i] = scale * ((c - a) * loc_scale<R>(tau, nullptr, b));
-  }
-}
-
-// The same when every S_kz is a sum of one-qubit parts (wz [K][n], half the difference of a qubit's two
-// values; the species' S_z are): the change of Z_i over a step's rotation follows from the Bloch sums
-// as 2 |s|^2 Z - 2 c (sx X + sy Y), without the boundary traces and the difference of two nearly equal
-// ones. Bound by reading the Bloch sums once. N = 64, 16 x 200, FP32: error of the outputs against 64
-// bits 2.4e-6 -> 4.7e-7, time of the whole gradient 0.286 -> 0.288 ms (the scan bounds it).
-template <typename R, bool NEAR>
-__global__ void loc_phase_local_kernel(int64_t steps, int64_t M, int K, int n, int parts, const cplx<R>* __restrict__ cs,
-                                       const R* __restrict__ bl, const double* __restrict__ sums,
-                                       const double* __restrict__ wz, double scale,
-                                       const double2* __restrict__ tau, double* __restrict__ gphi,
-                                       const int32_t* __restrict__ gate) {
-  if (gate && *gate == 0) return;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < steps * K;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t st = idx / K;
-    const int k = (int)(idx - st * K);
-    double acc = 0.0;
-    for (int i = 0; i < n; ++i) {
-      const double w = wz[k * n + i];
-      if (w == 0.0) continue;
-      const cplx<R> a = cs[st * n * (NEAR ? 2 : 1) + i];
-      const double c = 1.0 + (double)a.x, sx = (double)a.y, sy = NEAR ? (double)cs[st * n * 2 + n + i].x : 0.0;
-      double v[3];
-      for (int d = 0; d < 3; ++d) {
-        v[d] = 0.0;
-        if (sums) {
-          v[d] = sums[st * 3 * n + 3 * i + d];
-        } else {
-          for (int q = 0; q < parts; ++q) v[d] += (double)bl[(st * parts + q) * 3 * n + 3 * i + d];
-        }
-      }
-      acc += w * (2.0 * (sx * sx + sy * sy) * v[2] - 2.0 * c * (sx * v[0] + sy * v[1]));
-    }
-    gphi[idx] = scale * (acc * loc_scale<R>(tau, nullptr, st / M));
   }
 }
 
@@ -1293,15 +1279,9 @@ static cudaError_t loc_finish_t(const redo_table* t, int64_t B, int64_t M, int64
     loc_sums_kernel<R><<<(unsigned)steps, 256, 0, s>>>((const R*)w.bl, parts, 3 * t->loc, w.sums);
   loc_grad_kernel<R><<<(unsigned)(gb < 16384 ? gb : 16384), 128, 0, s>>>(
       steps, t->K, t->loc, t->loc_pairs, parts, t->loc_kptr, t->loc_kpair, (const R*)w.g, (const R*)w.bl, w.sums, M, m0,
-      T, 2.0 * t->dt / norm, tau, amp, grad);
-  if (gphi && f.sums) {
-    auto kern = loc_phase_local_kernel<R, false>;
-    if constexpr (sizeof(R) == 4)
-      if (loc_near(false, t->N)) kern = loc_phase_local_kernel<R, true>;
-    kern<<<(unsigned)(gb < 16384 ? gb : 16384), 128, 0, s>>>(steps, M, t->K, t->loc, parts, (const cplx<R>*)w.cs,
-                                                             (const R*)w.bl, w.sums, t->wz, 2.0 / norm, tau, gphi,
-                                                             f.gate);
-  }
+      T, 2.0 * t->dt / norm, tau, amp, grad,
+      LocPhaseOut<R>{(const cplx<R>*)w.cs, t->wz, f.gate, 2.0 / norm, f.sums ? gphi : nullptr,
+                     t->loc * (loc_near(sizeof(R) == 8, t->N) ? 2 : 1)});
   if (gphi && f.boundary) {
     const int64_t n = B * M * t->K, blocks = (n + 255) / 256;
     loc_phase_kernel<R><<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>((const R*)w.bz, B, M, parts, t->K,

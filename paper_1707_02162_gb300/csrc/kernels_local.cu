@@ -267,13 +267,6 @@ __device__ __forceinline__ float4 loc_split(double2 d) {
   const float2 h = make_float2((float)d.x, (float)d.y);
   return make_float4(h.x, h.y, (float)(d.x - (double)h.x), (float)(d.y - (double)h.y));
 }
-// In place: a pulse's own diagonal (the same for all its steps) less 1, as FP32 hi + lo
-__global__ void loc_split_kernel(double2* p, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double2 v = p[i];
-    reinterpret_cast<float4*>(p)[i] = loc_split(make_double2(v.x - 1.0, v.y));
-  }
-}
 __device__ __forceinline__ double2 loc_times(double2 v, double2 d) {
   double2 o = make_double2(v.x + d.x, v.y + d.y);
   cfma<double>(o, v, d);
@@ -1473,13 +1466,6 @@ cudaError_t launch_local_state(const redo_table* t, const int32_t* q, int64_t B,
     if (e) return e;
   }
   return cudaSuccess;
-}
-
-cudaError_t launch_local_split(double2* pd, int64_t n, cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  const int64_t blocks = (n + 255) / 256;
-  loc_split_kernel<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(pd, n);
-  return cudaGetLastError();
 }
 
 }  // namespace redo

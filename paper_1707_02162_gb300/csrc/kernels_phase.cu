@@ -60,7 +60,7 @@ __global__ void phase_diag_kernel(const double* __restrict__ phi, const double* 
 constexpr int64_t kDriftSteps = 64;
 
 __global__ void drift_diag_kernel(const double* __restrict__ h, double dt, int64_t B, int64_t M, int N,
-                                  double2* __restrict__ pd, float2* __restrict__ pd32) {
+                                  double2* __restrict__ pd, float2* __restrict__ pd32, int split) {
   const int64_t runs = (M + kDriftSteps - 1) / kDriftSteps;
   for (int64_t w = blockIdx.x; w < B * runs; w += gridDim.x) {
     const int64_t b = w / runs, n0 = (w % runs) * kDriftSteps;
@@ -71,7 +71,11 @@ __global__ void drift_diag_kernel(const double* __restrict__ h, double dt, int64
       for (int64_t n = n0; n < n1; ++n) {
         if (pd32)
           pd32[(b * M + n) * N + a] = make_float2((float)cs, (float)-sn);
-        else
+        else if (split) {
+          const double x = cs - 1.0;
+          reinterpret_cast<float4*>(pd)[(b * M + n) * N + a] = make_float4(
+              (float)x, (float)-sn, (float)(x - (double)(float)x), (float)(-sn - (double)(float)-sn));
+        } else
           pd[(b * M + n) * N + a] = make_double2(cs, -sn);
       }
     }
@@ -236,11 +240,11 @@ cudaError_t launch_phase_diag(const redo_table* t, const double* phi, int64_t B,
 }
 
 cudaError_t launch_drift_diag(const redo_table* t, const double* h, int64_t B, int64_t M, double2* pd,
-                              float2* pd32, cudaStream_t s) {
+                              float2* pd32, cudaStream_t s, bool split) {
   const int64_t work = B * ((M + kDriftSteps - 1) / kDriftSteps);
   if (work == 0) return cudaSuccess;
   const int64_t blocks = work < (int64_t)t->num_sms * 16 ? work : (int64_t)t->num_sms * 16;
-  drift_diag_kernel<<<(unsigned)blocks, 128, 0, s>>>(h, t->dt, B, M, t->N, pd, pd32);
+  drift_diag_kernel<<<(unsigned)blocks, 128, 0, s>>>(h, t->dt, B, M, t->N, pd, pd32, split ? 1 : 0);
   return cudaGetLastError();
 }
 

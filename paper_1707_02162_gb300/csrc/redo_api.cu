@@ -622,8 +622,8 @@ static redo_status propagate_core(const redo_table* t, const int32_t* q, const d
     zf = (double2*)((char*)workspace + L.zf_off);
     const bool tc = !L.local && prec == REDO_FP16X3 && t->N <= kSmallN;     // the split-FP16 chains take FP32 diagonals
     e = phase ? launch_phase_diag(t, phi, B, M, tc ? nullptr : pd, tc ? (float2*)pd : nullptr, zf, s)
-              : launch_drift_diag(t, h, B, L.local ? (M > 0 ? 1 : 0) : M, tc ? nullptr : pd, tc ? (float2*)pd : nullptr, s);
-    if (e == cudaSuccess && L.local && !phase && L.eff_prec == REDO_FP32 && M > 0) e = launch_local_split(pd, B * t->N, s);
+              : launch_drift_diag(t, h, B, L.local ? (M > 0 ? 1 : 0) : M, tc ? nullptr : pd, tc ? (float2*)pd : nullptr, s,
+                                  L.local && L.eff_prec == REDO_FP32);
     if (e != cudaSuccess) return cuda_error(e, phase ? "phase diagonals" : "drift diagonals");
     if (tc)
       L.p.pd32 = (const float2*)pd;
@@ -1298,9 +1298,8 @@ redo_status redo_fidelity_grad_drift(const redo_table* t, const int32_t* q, cons
   const double2* ut = (const double2*)U_target;
   cudaError_t e;
   ProfScope ps(7, s);
-  if (M > 0 && (e = launch_drift_diag(t, h, B, L.g.local ? 1 : M, pd, nullptr, s)) != cudaSuccess)
-    return cuda_error(e, "drift diagonals");
-  if (M > 0 && L.g.local && L.g.eff_prec == REDO_FP32 && (e = launch_local_split(pd, B * t->N, s)) != cudaSuccess)
+  if (M > 0 && (e = launch_drift_diag(t, h, B, L.g.local ? 1 : M, pd, nullptr, s,
+                                      L.g.local && L.g.eff_prec == REDO_FP32)) != cudaSuccess)
     return cuda_error(e, "drift diagonals");
   L.g.p.pd = pd;
   if (L.g.local)

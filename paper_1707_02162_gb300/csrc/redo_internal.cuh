@@ -178,7 +178,7 @@ cudaError_t launch_polar_c128(int N, int prec_arith, const double2* in, double2*
 
 // Locally controlled systems (kernels_local.cu).  Step-opening diagonals of a call: p[b*sb + n*sn + r]
 // (nullptr: none).  sn = 0: the same for every step of a pulse; an FP32 call then holds the diagonals
-// as launch_local_split leaves them (less 1, FP32 hi + lo).
+// less 1 as FP32 hi + lo (launch_drift_diag with split).
 struct LocalDiag {
   const double2* p;
   int64_t sb, sn;
@@ -205,7 +205,6 @@ struct TableArena {
     return at;
   }
 };
-cudaError_t launch_local_split(double2* pd, int64_t n, cudaStream_t s);
 // One-qubit tables and diagonal factors: host parts into the arena, room for the tables, and, once
 // the table's operators stand, the pointers into base and the kernels.
 struct LocalParts {
@@ -389,9 +388,9 @@ cudaError_t launch_phase_diag(const redo_table* t, const double* phi, int64_t B,
                               float2* pd32, double2* zf, cudaStream_t s);
 // Per-pulse diagonal drift: pd[b][n][a] = exp(-i dt h[b][a]) for every step n (pd32 non-null:
 // FP32 there instead), the step-opening diagonals of a chain whose steps read
-// U_n = E_n D diag(exp(-i dt h_b)).
+// U_n = E_n D diag(exp(-i dt h_b)).  split: the diagonals less 1 as FP32 hi + lo (float4) at pd.
 cudaError_t launch_drift_diag(const redo_table* t, const double* h, int64_t B, int64_t M, double2* pd,
-                              float2* pd32, cudaStream_t s);
+                              float2* pd32, cudaStream_t s, bool split = false);
 // X_g <- P_n X_g in place for the chains g = (u, s) of a step-aligned plan, n = s*sps + i
 // (chains with n >= M untouched); X of precision prec.
 cudaError_t launch_phase_rows(int N, int prec, void* X, int64_t G, int64_t S, int64_t sps, int64_t i,

@@ -569,9 +569,15 @@ static cudaError_t expect_diag_n(const redo_table* t, const int32_t* q, int64_t 
     if (t->dct && (sizeof(R) == 4 || B * N >= (int64_t)t->num_sms * kColThreads)) {
       // small blocks: they fill the SMs evenly (256 threads left a third wave nearly empty), and one
       // warp each while the pulses are few
-      const int th = B * N >= (int64_t)t->num_sms * kColThreads ? 64 : 32, per = th / N;
       const int64_t ent = (int64_t)t->K * t->digit_count * t->digit_base * N;
       const size_t smem = (size_t)(ent + N * N) * sizeof(cplx<R>);
+      int th = B * N >= (int64_t)t->num_sms * kColThreads ? 64 : 32;
+      // every block stages the factors: where few fit an SM beside each other (227 KB), larger blocks
+      // keep it busy (N = 8, two controls of 256^2 levels, FP64, 5000 x 200: 17.1 ms in blocks of 64, 13.1 so,
+      // 15.3 with the dense kernels; N = 16, 128^2, FP32, 20 000 x 200: 4.84 and 4.19)
+      const int64_t fit = 227 * 1024 / (int64_t)(smem + 1024);
+      while (th < kColThreads && fit * th < kColThreads && B * N > (int64_t)t->num_sms * fit * th) th *= 2;
+      const int per = th / N;
       const bool pairs = sizeof(R) == 4 && !cols;
       auto kern = pairs ? expect_diagctl_kernel<R, N, sizeof(R) == 4> : expect_diagctl_kernel<R, N, false>;
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -1,5 +1,5 @@
 """Expectations of a few FP32 pulses under diagonal controls: weights of any length and not rounded, bad
-levels counted once per digit, as in the general kernel."""
+levels counted once per digit, as in the general kernel; and factor tables that fill shared memory."""
 import numpy as np
 import pytest
 
@@ -60,4 +60,25 @@ def test_few_pulse_expectations_count_bad_levels_once_per_digit():
     st = redo.new_status()
     t.expect_diag(q, rho, obs, "fp32", status=st)
     assert int(st[3]) == 2 * w.digits
+    t.close()
+
+
+@pytest.mark.parametrize("n,base,prec,B", [(4, 128, "fp32", 3), (4, 128, "fp32", 700), (4, 128, "fp32", 2500),
+                                           (3, 256, "fp64", 4900), (3, 100, "fp32", 4870)])
+def test_large_factor_tables(n, base, prec, B):
+    # two controls of base^2 levels: one to three blocks an SM, in blocks of 32 to 256 threads; every
+    # pulse as one of a few is
+    rng = np.random.default_rng(n)
+    N, M, K = 2 ** n, 9, 2
+    A = rng.normal(size=(N, N)) + 1j * rng.normal(size=(N, N))
+    Hk = np.stack([np.diag(rng.normal(size=N)) for _ in range(K)]).astype(np.complex128)
+    t = redo.Table((A + A.conj().T) / 2, Hk, 0.1, -np.ones(K), np.ones(K), base, 2, fp32=True)
+    q = torch.randint(0, base * base, (B, M, K), dtype=torch.int32, device="cuda",
+                      generator=torch.Generator(device="cuda").manual_seed(7))
+    rho, obs = rng.uniform(-1, 1, N), rng.uniform(-1, 1, N)
+    e, m = t.expect_diag(q, rho, obs, prec)
+    tol = 1e-12 if prec == "fp64" else 2e-5
+    for b in sorted({0, B // 2, B - 1}):
+        e1, m1 = t.expect_diag(q[b:b + 1].contiguous(), rho, obs, "fp64")
+        assert (e[b] - e1[0]).abs().max().item() < tol and abs(float(m[b] - m1[0])) < tol
     t.close()

@@ -1140,17 +1140,30 @@ bool local_eligible(const redo_table* t, int64_t M, int prec, int what) {
   return loc_scratch(t, 1, M, prec, what, nullptr).total <= kLocSlice;
 }
 
-// Whether a plain propagation gains by it.  One step costs the dense chain 4 N^3 K digits multiply-adds;
-// here it is N^2 (4 + 4n) (complex rotations: 6 + 8n), about 28 a row for the diagonal (FP32: 100, a
-// sine and cosine) and per qubit 230 FP64 operations of square roots and divisions (FP32: 500, three
-// angles) and 32 a pair.  The FP32 dense column kernel is bound by its operand reads at about two
-// thirds of this path's rate (N = 4, global controls, 1000 x 500: 155 us dense, 234 us here; N = 8:
-// 528 and 315).  So N = 2, and N = 4 with few factors, stay dense; from N = 8 on this form wins.
-bool local_pays(const redo_table* t, int prec) {
-  const double N = t->N, n = t->loc, dense = 4.0 * N * N * N * t->K * t->digits;
-  if (prec == REDO_FP64) return dense > 32.0 * t->loc_pairs + 230.0 * n + 28.0 * N + N * N * (4 + 4 * n);
-  const double rot = loc_near(false, t->N) ? 6 + 8 * n : 4 + 4 * n;
-  return 1.5 * dense > 40.0 * t->loc_pairs + 500.0 * n + 100.0 * N + N * N * rot;
+// Whether a call gains by it (systems of a few levels; the others always do).  Multiply-adds of a step:
+// dense 4 N^3 (a state: 4 N^2) K digits; here 32 a pair, per qubit 230 FP64 operations of square roots
+// and divisions (FP32: 500, three angles), 28 a row for the diagonal (FP32: 100, a sine and cosine), and
+// 4 + 4n an entry (complex rotations: 6 + 8n).
+// FP64, by measurement over B = 1 .. 3000, N = 2 .. 16: while the pulses leave SMs idle a call waits for
+// its dependent products and this form is ahead from N = 4 on (N = 4, two controls, 40 x 200: 158 us dense,
+// 101 here) and level at N = 2; once they fill the GPU its serial one-qubit work runs at half the rate of
+// the dense columns (N = 4, 300 x 100: 126 us dense, 195 here), a state's at the same rate (N = 8,
+// 300 x 100: 261 and 351; N = 16 the other way).
+// FP32: the dense column kernel is bound by its operand reads at about two thirds of this path's rate
+// (N = 4, global controls, 1000 x 500: 155 us dense, 234 us here; N = 8: 528 and 315), so plain
+// propagations at N = 2, and at N = 4 and 8 with few factors, stay dense; with a step-opening diagonal, for
+// gradients and for states this form is level or ahead at every size, and several times more exact.
+bool local_pays(const redo_table* t, int64_t B, int prec, int what, bool diag) {
+  const double N = t->N, n = t->loc, kd = (double)t->K * t->digits;
+  const bool dbl = prec == REDO_FP64, full = B >= t->num_sms;
+  const double prep = dbl ? 32.0 * t->loc_pairs + 230.0 * n + 28.0 * N : 40.0 * t->loc_pairs + 500.0 * n + 100.0 * N;
+  const double rot = loc_near(dbl, t->N) ? 6 + 8 * n : 4 + 4 * n;
+  if (what == kLocalSim) return !dbl || !full || N > 8 || kd > 2;
+  if (what == kLocalGrad) return !dbl || diag || N > 2 || !full;
+  if (what == kLocalPhaseGrad) return true;
+  const double dense = 4.0 * N * N * N * kd + (diag ? 4.0 * N * N : 0.0), here = prep + N * N * rot;
+  if (dbl) return N > 2 && (!full || dense > 2.0 * here);
+  return diag || 1.5 * dense > here;
 }
 
 // Which chain form a call takes.  FP32 products of controls that act on one qubit each have two nonzeros

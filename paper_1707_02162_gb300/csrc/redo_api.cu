@@ -525,7 +525,7 @@ static PropLayout prop_layout(const redo_table* t, int64_t B, int64_t M, redo_pr
   const size_t el = L.eff_prec == REDO_FP64 ? sizeof(double2) : sizeof(float2);
   const size_t n2 = (size_t)t->N * t->N;
   L.what = local_chain_form(t, prec);
-  if (local_eligible(t, M, L.eff_prec, L.what) && (diag || local_pays(t, L.eff_prec))) {
+  if (local_eligible(t, M, L.eff_prec, L.what) && local_pays(t, B, L.eff_prec, L.what, phase)) {
     L.local = true;
     L.p = reunit_every > 0 ? plan_chain_aligned(t, B, M, reunit_every) : plan_chain_local(t, B, M, L.eff_prec, false);
     if (t->N > kSmallN) {
@@ -948,9 +948,9 @@ struct GradLayout {
 // Locally controlled systems: segment products, checkpoints and costates as in the dense form, then
 // the step operators and the sweep's sums.
 static bool grad_layout_local(const redo_table* t, int64_t B, int64_t M, redo_precision prec, int32_t checkpoint_every,
-                              int what, GradLayout* L) {
+                              int what, bool diag, GradLayout* L) {
   L->eff_prec = prec == REDO_FP64 ? REDO_FP64 : REDO_FP32;
-  if (!local_eligible(t, M, L->eff_prec, what)) return false;
+  if (!local_eligible(t, M, L->eff_prec, what) || !local_pays(t, B, L->eff_prec, what, diag)) return false;
   L->local = true;
   L->p = checkpoint_every > 0 ? plan_chain_aligned(t, B, M, checkpoint_every)
                               : plan_chain_local(t, B, M, L->eff_prec, true);
@@ -1001,7 +1001,7 @@ static redo_status grad_local(const redo_table* t, const int32_t* q, const GradL
 static GradLayout grad_layout(const redo_table* t, int64_t B, int64_t M, redo_precision prec,
                               int32_t checkpoint_every) {
   GradLayout L;
-  if (grad_layout_local(t, B, M, prec, checkpoint_every, kLocalGrad, &L)) {
+  if (grad_layout_local(t, B, M, prec, checkpoint_every, kLocalGrad, false, &L)) {
     add_strang(t, B, L.total, L.strang_off, L.strang_tmp_off);
     return L;
   }
@@ -1129,7 +1129,7 @@ static PhaseGradLayout phase_grad_layout(const redo_table* t, int64_t B, int64_t
                                          int32_t checkpoint_every, bool phase = true) {
   PhaseGradLayout L;
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  if (grad_layout_local(t, B, M, prec, checkpoint_every, phase ? kLocalPhaseGrad : kLocalGrad, &L.g)) {
+  if (grad_layout_local(t, B, M, prec, checkpoint_every, phase ? kLocalPhaseGrad : kLocalGrad, true, &L.g)) {
     L.pd_off = L.g.total;
   } else if (t->N > kSmallN) {
     // lockstep SIMT sweeps on segments of whole steps (the diagonals fall between launches)
@@ -1326,6 +1326,12 @@ redo_status redo_fidelity_grad_drift(const redo_table* t, const int32_t* q, cons
   return REDO_OK;
 }
 
+// Whether simulate advances its states by the one-qubit operators (given the scratch)
+static bool sim_local(const redo_table* t, int64_t B, int64_t M, redo_precision prec) {
+  const int eff = prec == REDO_FP64 ? REDO_FP64 : REDO_FP32;
+  return local_eligible(t, M, eff, kLocalSim) && local_pays(t, B, eff, kLocalSim, false);
+}
+
 // Scratch of the state sweep: a local system's step operators, or the two state vectors of the
 // lockstep simulation (N > 64 with fewer pulses than SMs).
 static size_t sim_state_bytes(const redo_table* t, int64_t B, int64_t M, redo_precision prec, bool local) {
@@ -1342,9 +1348,7 @@ redo_status redo_simulate_workspace(const redo_table* t, int64_t B, int64_t M,
   if (B < 0 || M < 0 || reunit_every < 0) return set_error(REDO_ERR_INVALID, "negative size");
   redo_status st = check_prec(t, prec);
   if (st != REDO_OK) return st;
-  const size_t state = B > 0 ? sim_state_bytes(t, B, M, prec, local_eligible(t, M, prec == REDO_FP64 ? REDO_FP64
-                                                                                             : REDO_FP32, kLocalSim))
-                             : 0;
+  const size_t state = B > 0 ? sim_state_bytes(t, B, M, prec, sim_local(t, B, M, prec)) : 0;
   size_t prop = 0;
   if (want_U) {
     st = redo_propagate_workspace(t, B, M, prec, reunit_every, &prop);
@@ -1377,7 +1381,7 @@ redo_status redo_simulate(const redo_table* t, const int32_t* q, int64_t B, int6
     cudaError_t e;
     const int eff = prec == REDO_FP64 ? REDO_FP64 : REDO_FP32;
     // a caller that brings only the dense sweep's scratch (none at all for N <= 64) keeps that sweep
-    const bool local = local_eligible(t, M, eff, kLocalSim) && workspace && ((uintptr_t)workspace & 255) == 0 &&
+    const bool local = sim_local(t, B, M, prec) && workspace && ((uintptr_t)workspace & 255) == 0 &&
                        workspace_bytes >= sim_state_bytes(t, B, M, prec, true);
     const bool lockstep = !local && t->N > kSmallN && B < t->num_sms;
     const size_t need_state =

@@ -224,7 +224,7 @@ cudaError_t local_phase_axes(redo_table* t, const double* sz);
 enum LocalWhat { kLocalChain = 0, kLocalGrad = 1, kLocalPhaseGrad = 2, kLocalSim = 3, kLocalChainFine = 4 };
 int local_chain_form(const redo_table* t, int prec_asked);
 bool local_eligible(const redo_table* t, int64_t M, int prec, int what);
-bool local_pays(const redo_table* t, int prec);
+bool local_pays(const redo_table* t, int64_t B, int prec, int what, bool diag);
 size_t local_ops_bytes(const redo_table* t, int64_t B, int64_t M, int prec, int what);
 ChainPlan plan_chain_local(const redo_table* t, int64_t B, int64_t M, int prec, bool two);
 cudaError_t launch_local_chain(const redo_table* t, const int32_t* q, const ChainPlan& p, int prec, int what,

@@ -514,8 +514,8 @@ loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
   {
     double2 tb = tau[b];
     if constexpr (sizeof(R) == 4) {
-      const double f = pow2(-exp_of(tb));
-      tb = make_double2(tb.x * f, tb.y * f);
+      const int et = exp_of(tb);
+      tb = make_double2(down2(tb.x, et), down2(tb.y, et));
     }
     const cplx<R>* P = Pck + g * N * N + x;
     const cplx<R>* Q = Rck + g * N * N + (int64_t)x * N + l * E;
@@ -580,15 +580,17 @@ loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
 // dF/du_kn = (2 dt / N^2) sum_i (gx X_i + gy Y_i + gz Z_i), a thread per (step, term): its pairs are
 // kpair[kptr[k] ..] (pair | qubit << 20), the Bloch sums bl [step][part][3n] or, already added, sums.
 // The sums are those of scaled vectors in FP32: times 2^exp_of(tau[b]), or times amp[b].
-template <typename R> __device__ __forceinline__ double loc_scale(const double2* tau, const double* amp, int64_t b) {
-  if (sizeof(R) == 8) return 1.0;
-  return amp ? amp[b] : pow2(exp_of(tau[b]));
+template <typename R>
+__device__ __forceinline__ double loc_scaled(double x, const double2* tau, const double* amp, int64_t b) {
+  if (sizeof(R) == 8) return x;
+  return amp ? x * amp[b] : down2(x, -exp_of(tau[b]));
 }
 // The phase gradients when every S_kz is a sum of one-qubit parts (wz [K][n], half the difference of a
 // qubit's two values; the species' S_z are): the change of Z_i over a step's rotation follows from the
 // Bloch sums as 2 |s|^2 Z - 2 c (sx X + sy Y), without the boundary traces and the difference of two
 // nearly equal ones (N = 64, 16 x 200, FP32: error against 64 bits 2.4e-6 -> 4.7e-7).  Formed beside the
-// amplitudes' gradients: a launch of its own was 3 of the 66 us of N = 8, 10 x 41.  gphi nullptr: none.
+// amplitudes' gradients (PH): a launch of its own was 3 of the 66 us of N = 8, 10 x 41.  (A form apart:
+// with the choice at run time the other gradients' took 66 us, not 49, at N = 32, 256 x 500.)
 template <typename R> struct LocPhaseOut {
   const cplx<R>* cs;
   const double* wz;
@@ -597,13 +599,13 @@ template <typename R> struct LocPhaseOut {
   double* gphi;
   int cs_step;               // entries of cs per step: n, or 2n with the rotations' second parts
 };
-template <typename R>
+template <typename R, bool PH>
 __global__ void loc_grad_kernel(int64_t steps, int K, int n, int pairs, int parts, const int32_t* __restrict__ kptr,
                                 const int32_t* __restrict__ kpair, const R* __restrict__ g, const R* __restrict__ bl,
                                 const double* __restrict__ sums, int64_t M, int64_t w0, int64_t T, double scale,
                                 const double2* __restrict__ tau, const double* __restrict__ amp,
                                 double* __restrict__ grad, LocPhaseOut<R> ph) {
-  const bool phase = ph.gphi && !(ph.gate && *ph.gate == 0);
+  const bool phase = PH && !(ph.gate && *ph.gate == 0);
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < steps * K;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t st = idx / K, b = st / T;
@@ -620,9 +622,8 @@ __global__ void loc_grad_kernel(int64_t steps, int K, int n, int pairs, int part
       const R* gp = g + (st * pairs + p) * 3;
       for (int c = 0; c < 3; ++c) acc += (double)gp[c] * bloch(i, c);
     }
-    const double f = loc_scale<R>(tau, amp, b);
-    grad[(b * M + w0 + st - b * T) * K + k] = scale * (acc * f);
-    if (!phase) continue;
+    grad[(b * M + w0 + st - b * T) * K + k] = scale * loc_scaled<R>(acc, tau, amp, b);
+    if (!PH || !phase) continue;
     acc = 0.0;
     for (int i = 0; i < n; ++i) {
       const double w = ph.wz[k * n + i];
@@ -631,7 +632,7 @@ __global__ void loc_grad_kernel(int64_t steps, int K, int n, int pairs, int part
       const double c = 1.0 + (double)a->x, sx = (double)a->y, sy = ph.cs_step > n ? (double)a[n].x : 0.0;
       acc += w * (2.0 * (sx * sx + sy * sy) * bloch(i, 2) - 2.0 * c * (sx * bloch(i, 0) + sy * bloch(i, 1)));
     }
-    ph.gphi[idx] = ph.scale * (acc * f);
+    ph.gphi[idx] = ph.scale * loc_scaled<R>(acc, tau, amp, b);
   }
 }
 
@@ -666,7 +667,7 @@ __global__ void loc_phase_kernel(const R* __restrict__ bz, int64_t B, int64_t M,
       a += (double)bz[((b * (M + 1) + n) * parts + p) * K + k];
       c += (double)bz[((b * (M + 1) + n + 1) * parts + p) * K + k];
     }
-    gphi[i] = scale * ((c - a) * loc_scale<R>(tau, nullptr, b));
+    gphi[i] = scale * loc_scaled<R>(c - a, tau, nullptr, b);
   }
 }
 
@@ -850,8 +851,11 @@ loc_sim_wide_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ 
     int* top = reinterpret_cast<int*>(ex);           // (free until the first step)
     if (l == 0) top[0] = top[1] = -200;
     __syncthreads();
-    atomicMax(top, t.x);
-    atomicMax(top + 1, t.y);
+    const int x = __reduce_max_sync(0xffffffffu, t.x), y = __reduce_max_sync(0xffffffffu, t.y);
+    if ((l & 31) == 0) {
+      atomicMax(top, x);
+      atomicMax(top + 1, y);
+    }
     __syncthreads();
     const bool far = outside(make_int2(top[0], top[1]));
     __syncthreads();
@@ -985,8 +989,7 @@ loc_state_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const double2 z = m0 == 0 ? z0[e] : make_double2(0.0, 0.0);
-      const double f = pow2(-e0);
-      p[e] = m0 == 0 ? cmake<R>((R)(z.x * f), (R)(z.y * f)) : sp[e];
+      p[e] = m0 == 0 ? cmake<R>((R)down2(z.x, e0), (R)down2(z.y, e0)) : sp[e];
     }
     L::load_diag(dn, d, l);
     if (T > 0) L::load_cs(cn, r);
@@ -1028,9 +1031,8 @@ loc_state_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
     }
     if constexpr (sizeof(R) == 4) {
       const int eT = top(zT), et = exp_of(make_double2(tx, ty));
-      const double f = pow2(-eT - et);
-      tx *= f;
-      ty *= f;
+      tx = down2(tx, eT + et);
+      ty = down2(ty, eT + et);
       if (on && l == 0) amp[b] = pow2(2 * e0 + eT + et);
     }
 #pragma unroll
@@ -1283,10 +1285,11 @@ static cudaError_t loc_finish_t(const redo_table* t, int64_t B, int64_t M, int64
   const int64_t steps = B * T, gn = steps * t->K, gb = (gn + 127) / 128;
   if (w.sums)
     loc_sums_kernel<R><<<(unsigned)steps, 256, 0, s>>>((const R*)w.bl, parts, 3 * t->loc, w.sums);
-  loc_grad_kernel<R><<<(unsigned)(gb < 16384 ? gb : 16384), 128, 0, s>>>(
+  auto kern = gphi && f.sums ? loc_grad_kernel<R, true> : loc_grad_kernel<R, false>;
+  kern<<<(unsigned)(gb < 16384 ? gb : 16384), 128, 0, s>>>(
       steps, t->K, t->loc, t->loc_pairs, parts, t->loc_kptr, t->loc_kpair, (const R*)w.g, (const R*)w.bl, w.sums, M, m0,
       T, 2.0 * t->dt / norm, tau, amp, grad,
-      LocPhaseOut<R>{(const cplx<R>*)w.cs, t->wz, f.gate, 2.0 / norm, f.sums ? gphi : nullptr,
+      LocPhaseOut<R>{(const cplx<R>*)w.cs, t->wz, f.gate, 2.0 / norm, gphi,
                      t->loc * (loc_near(sizeof(R) == 8, t->N) ? 2 : 1)});
   if (gphi && f.boundary) {
     const int64_t n = B * M * t->K, blocks = (n + 255) / 256;

@@ -122,9 +122,13 @@ typedef struct redo_table redo_table;
  * 2 x 2 operators.  The table then also keeps those, and redo_propagate (with _drift and _phase),
  * redo_fidelity_grad (with _drift and _phase), redo_simulate and redo_state_grad apply a step as one
  * rotation per qubit and one diagonal instead of K * digits dense products: the same results to
- * rounding, in the call's precision (REDO_FP16X3 calls run in FP32).  A pulse whose step operators
- * alone exceed 512 MiB, FP64 unitary gradients at N = 1024, redo_propagate_steps, redo_propagate_noalloc
- * and all other systems use the dense operators.
+ * rounding, in the call's precision (REDO_FP16X3 calls run in FP32).  Their step operators take scratch, in
+ * slices of pulses of at most 512 MiB (state transfer: about 64 MiB, 256 MiB for large batches).  The dense
+ * operators remain for all other systems; for a pulse whose step operators alone exceed 512 MiB, FP64 unitary
+ * gradients at N = 1024, redo_propagate_steps and redo_propagate_noalloc; and where they are faster: FP32
+ * propagations at N = 2 (and at N = 4 and 8 with few factors a step), FP64 propagations at N = 2, and, with at
+ * least one pulse per SM, FP64 propagations with few factors, gradients at N = 2, and simulations at N <= 8 with
+ * at most two factors a step.
  *  stream   stream for the build; synchronised before returning.
  *  out      receives the handle; free with redo_table_free.
  * Errors: REDO_ERR_INVALID, REDO_ERR_NOT_HERMITIAN (relative tolerance 1e-12
@@ -188,9 +192,11 @@ redo_status redo_quantize(const redo_table* t, const double* u, int64_t B, int64
  *  reunit_every  R >= 0.  R = 0: no re-unitarisation.  R > 0: segments are cut
  *              at every R-th time step and each segment product -- the
  *              propagator of R consecutive steps -- is replaced by its unitary
- *              polar factor (one Newton-Schulz step P <- P(3I - P^dag P)/2 in
+ *              polar factor (one Newton-Schulz step P <- P + P(I - P^dag P)/2 in
  *              the chain precision), and each pulse product gets one more
- *              Newton-Schulz step in FP64 before the fidelity.  This removes
+ *              Newton-Schulz step with an FP64 result before the fidelity (of FP32
+ *              products: I - P^dag P to about 48 bits in FP32 pairs, the small
+ *              correction in FP32, the sum in FP64; unitary to 1e-12).  This removes
  *              the norm drift of reduced-precision chains; R > M acts as R = M.
  *  U_out       device complex128 [B][N][N]; receives U_b.  May be NULL if F is wanted only.
  *  U_target    device complex128 [N][N] or NULL.
@@ -313,7 +319,9 @@ redo_status redo_propagate_noalloc(const redo_table* t, const int32_t* q, int64_
  *  q, B, M       as for redo_propagate.
  *  U_target      device complex128 [N][N], or [B][N][N] if target_batched != 0.
  *  prec          REDO_FP64 or REDO_FP32, or REDO_FP16X3 for N >= 128 (products;
- *                traces and tau in FP64).
+ *                tau and F in FP64, and the traces: of locally controlled systems in
+ *                FP32 their terms are added in FP32 within a warp, with a power of two
+ *                taken out so that U_target may be of any length, and in FP64 across).
  *  checkpoint_every  C > 0: forward checkpoints every C steps; 0: automatic.
  *  reunit_every  R >= 0.  R = 0: none.  R > 0 (requires R = checkpoint_every): every
  *                checkpoint segment product, the propagator of R consecutive steps, is
@@ -351,14 +359,16 @@ redo_status redo_fidelity_grad_workspace(const redo_table* t, int64_t B, int64_t
  * the final propagator U_M ... U_1.
  *
  * The state is advanced by one matrix-vector product per table operator (locally
- * controlled systems: by the step's one-qubit rotations), in FP64 for REDO_FP64 and FP32 otherwise; U_final, if requested, is computed
- * exactly as redo_propagate(prec, reunit_every) computes U_out.
+ * controlled systems: by the step's one-qubit rotations), in FP64 for REDO_FP64 and FP32
+ * otherwise; the expectation is added in FP64 (locally controlled systems in FP32: in FP32
+ * pairs of about 48 bits, or in FP64 when obs_diag or psi0 leave their range); U_final, if
+ * requested, is computed exactly as redo_propagate(prec, reunit_every) computes U_out.
  *  psi0      device complex128 [N] (or [B][N] if psi0_batched != 0).
  *  obs_diag  device double [N];  expect  device double [B][M+1].
  *  U_final   device complex128 [B][N][N] or NULL.
  *  workspace >= redo_simulate_workspace(..., want_U = U_final != NULL) bytes, 256-byte aligned.  A
  *            locally controlled system given less (NULL for N <= 64 without U_final) advances the
- *            state by its dense operators, which need none.
+ *            state by its dense operators, which need none for N <= 64.
  */
 redo_status redo_simulate(const redo_table* t, const int32_t* q, int64_t B, int64_t M,
                           redo_precision prec, int32_t reunit_every, const void* psi0,
@@ -374,7 +384,9 @@ redo_status redo_simulate(const redo_table* t, const int32_t* q, int64_t B, int6
  * Costs O(N^2) per factor (matrix-vector products, forward and then reverse, undoing each
  * unitary factor on both vectors), so it is the cheap form of GRAPE for large N.
  *  q            device int32 [B][M][K] levels.
- *  prec         REDO_FP64 or REDO_FP32 (operators of that precision; traces and a in FP64).
+ *  prec         REDO_FP64 or REDO_FP32 (operators of that precision; a in FP64, and the traces: of
+ *               locally controlled systems in FP32 added in FP32 per step, with powers of two taken
+ *               out so that psi0 and psi_target may be of any length).
  *  psi0, psi_target  device complex128 [N], or [B][N] when batched != 0.
  *  F_out        device double [B] or NULL;  grad device double [B][M][K] or NULL (one of the two).
  *  workspace    >= redo_state_grad_workspace bytes, 256-byte aligned.  A symmetric-split table (which
@@ -397,7 +409,10 @@ redo_status redo_state_grad(const redo_table* t, const int32_t* q, int64_t B, in
  * basis where rho(0) = O = sum_i I_ix are diagonal (the Hamiltonian terms passed to
  * redo_build_table are then given in that basis).  N <= 64.
  *  q            device int32 [B][M][K] levels from redo_quantize.
- *  prec         REDO_FP64 or REDO_FP32 (the latter needs REDO_TABLE_FP32); the reduction is FP64.
+ *  prec         REDO_FP64 or REDO_FP32 (the latter needs REDO_TABLE_FP32).  The sum over c and the mean
+ *               are FP64 (or pairs of that accuracy); in FP32 with N <= 16 the N terms of a column may
+ *               be added in FP32 (by the column kernels: always with one column per GPU lane or more,
+ *               and with every H_k diagonal).
  *  rho_diag     device double [N];  obs_diag device double [N].
  *  expect       device double [B][M+1] or NULL;  expect_mean device double [B] or NULL:
  *               the mean of e_1 .. e_M (e_0 when M = 0).  At least one of the two.

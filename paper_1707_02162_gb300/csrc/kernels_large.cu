@@ -138,7 +138,8 @@ static cudaError_t cgemm(const Ops& ops, int64_t batch, int N, R alpha, R diag, 
   const int64_t blocks = batch * (N / kT) * (N / kT);
   // up to two tiles of 64 per SM: 32 x 32 tiles spread them (10 products of N = 256: 50 -> 45 us; two
   // 29 -> 23 us); above, the larger tile reads its operands half as often
-  if (blocks <= 304)
+  constexpr int64_t kTwoPerSm = 2 * 152;            // (the products carry no table to ask for the SM count)
+  if (blocks <= kTwoPerSm)
     cgemm_kernel<R, ADJA, 32, Ops><<<(unsigned)(4 * blocks), 256, 0, s>>>(ops, N, alpha, diag);
   else
     cgemm_kernel<R, ADJA, kT, Ops><<<(unsigned)blocks, 256, 0, s>>>(ops, N, alpha, diag);

@@ -1171,7 +1171,8 @@ bool local_pays(const redo_table* t, int64_t B, int prec, int what, bool diag) {
 // Which chain form a call takes.  FP32 products of controls that act on one qubit each have two nonzeros
 // a row, so the dense chain rounds twice a product, and the real rotations' error was up to 1.4 times its
 // (U, N = 64, 12 controls, 200 steps: 7.9e-7 dense, 1.0e-6); rotations near the identity, twice the
-// multiply-adds, give 4.4e-7 (N = 32: 6.3e-7, 9.1e-7, 3.6e-7; N = 128: 5.1e-7, 6.6e-7, 3.1e-7).  Split
+// multiply-adds, give 4.4e-7 (N = 32: 6.3e-7, 9.1e-7, 3.6e-7; N = 128: 5.1e-7, 6.6e-7, 3.1e-7).  256 x
+// 2000 at N = 64, re-unitarised: 3.82 ms with the real rotations, 4.96 here, 232 dense.  Split
 // FP16 was 5 times less exact (5.5e-6) and takes the real rotations; controls on several qubits at once
 // (global fields) have dense rows, whose error was larger (N = 64: 1.7e-6, 1.0e-6 with the real rotations).
 int local_chain_form(const redo_table* t, int prec_asked) {

@@ -347,7 +347,7 @@ def ensemble_measure(redo, inputs, torch, peaks, M=2000):
             "realisation_steps_per_s": steps / (ms16 / 1e3), "ms_per_call": ms16,
             "products_per_step": w.K * (1 if levels else w.digits),
             "fp64_state_only": {"realisation_steps_per_s": steps / (ms64 / 1e3), "ms_per_call": ms64},
-            "max_abs_dZ1_fp16x3_vs_fp64": float((ex16 - ex64).abs().max()),
+            "max_abs_dZ1_vs_fp64": float((ex16 - ex64).abs().max()),
             "table_build_s": build_s}
         t.close()
         del ws16, ws64, Uf
@@ -768,7 +768,7 @@ def run_workload(args):
         steps = n_om * n_la * M
         out.update({"metric": "noisy exotic freezing Q(omega, lambda) map: pulse-steps/s", "unit": "pulse-steps/s",
                     "value": steps / (kern_ms / 1e3), "kernel_ms": kern_ms, "wall_s_with_drive_synthesis": wall,
-                    "precision": "fp32 chains, fp64 reductions", "pulses": n_om * n_la, "steps": M,
+                    "precision": "fp32 chains and step sums, means in fp32 pairs", "pulses": n_om * n_la, "steps": M,
                     "fp64_same_gpu": {"pulse_steps_per_s": fp64_rate, "sample": f"{n_la} pulses x {M} steps",
                                       "max_abs_dQ_fp32_vs_fp64": fp32_vs_fp64},
                     "lambda0_peaks_vs_bessel_roots": peaks,
@@ -777,7 +777,8 @@ def run_workload(args):
                                "lambdas": [0.0, 1.0, n_la], "T": Tw, "base": 100, "digits": 2}})
     elif args.workload == "state":
         # state-to-state GRAPE on the 8-qubit GRAPE system (N=256, K=16, M=1000, dt=2 us): fidelity +
-        # gradient per pulse by matrix-vector sweeps; one pulse and a batch of 152 (one CTA each)
+        # gradient per pulse by matrix-vector sweeps of the dense operators (no scratch given, so not the
+        # one-qubit form); one pulse and a batch of 152 (one CTA each)
         w = inputs.config(2, M=args.M if args.M != M_FULL else None)
         t = redo.Table(w.H0, w.Hk, w.dt, w.lo, w.hi, w.base, w.digits, fp32=True, levels=not args.digit_table)
         res = {}
@@ -805,8 +806,8 @@ def run_workload(args):
     elif args.workload == "phase":
         # Section III amplitude/phase drive: 6 qubits (N=64), each its own species (x-table of X_i/2,
         # levels on [0, Omega]), phases on [0, 2 pi), B=256 pulses x M=2000 steps, level table,
-        # split FP16 with re-unitarisation every 64 steps.  Against the same pulses in x/y form
-        # (coefficients A cos phi, A sin phi on 12 per-qubit x/y controls).
+        # requested in split FP16 (one-qubit operators: FP32) with re-unitarisation every 64 steps.
+        # Against the same pulses in x/y form (coefficients A cos phi, A sin phi on 12 per-qubit x/y controls).
         B = args.B if args.B != B_FULL else 256
         M = args.M if args.M != M_FULL else 2000
         w = inputs.phase_config(6, B=B, M=M, seed=1)
@@ -834,8 +835,8 @@ def run_workload(args):
         torch.cuda.synchronize()
         redo.redo_profile_enable(False)
         prof = redo.redo_profile_read()
-        tc_ms = prof.get("chain_tc", (0.0, 0))[0]
-        # FP64 on 16 pulses: accuracy of the split-FP16 result
+        chain_ms = prof["chain_segments"][0]             # step operators and chains
+        # FP64 on 16 pulses: accuracy of the result
         Bs = 16
         U64 = torch.empty((Bs, w.N, w.N), dtype=torch.complex128, device="cuda")
         F64 = torch.empty(Bs, dtype=torch.float64, device="cuda")
@@ -847,7 +848,7 @@ def run_workload(args):
                                                                ws64), 1)
         dF = float((F64 - F[:Bs]).abs().max())
         dU = float((U64 - U[:Bs]).abs().max())
-        # GRAPE gradient in amplitudes and phases (FP32 SIMT chains), all pulses
+        # GRAPE gradient in amplitudes and phases (FP32), all pulses
         gA = torch.empty((B, M, w.K), dtype=torch.float64, device="cuda")
         gP = torch.empty_like(gA)
         Fg = torch.empty(B, dtype=torch.float64, device="cuda")
@@ -883,30 +884,18 @@ def run_workload(args):
         msxy = _events_time(itxy, args.steps)
         txy.close()
         K = w.K
-        op_bytes = B * M * K * 32768.0
-        flop = B * M * K * 8.0 * w.N ** 3 * 3
-        pk = _peaks()
         out.update({"metric": "REDO prop steps/s (amplitude/phase controls)", "unit": "pulse-steps/s",
                     "value": B * M / (ms / 1e3), "ms_per_call": ms,
                     "xy_form_same_pulses": {"pulse_steps_per_s": B * M / (msxy / 1e3), "ms_per_call": msxy,
                                             "controls": 12},
                     "speedup_vs_xy_form": msxy / ms,
                     "fp64_same_gpu": {"pulse_steps_per_s": Bs * M / (ms64 / 1e3), "pulses": Bs,
-                                      "max_abs_dF_fp16x3_vs_fp64": dF, "max_abs_dU": dU},
+                                      "max_abs_dF_vs_fp64": dF, "max_abs_dU": dU},
                     "grape_gradient_fp32": {"instance_iters_per_s": B * 1e3 / msg, "ms_per_call": msg,
-                                            "what": "F, dF/dA and dF/dphi of all pulses, FP32 SIMT chains, "
+                                            "what": "F, dF/dA and dF/dphi of all pulses, FP32 one-qubit operators, "
                                                     "checkpoints every 64 steps"},
-                    "roofline": {"kernel": "chain_tc", "kernel_ms": tc_ms,
-                                 "hbm_achieved_gbs": op_bytes / (tc_ms / 1e3) / 1e9 if tc_ms else None,
-                                 "hbm_frac": (op_bytes / (tc_ms / 1e3) / 1e9 / pk.get("hbm_gbs", 6794.5)
-                                              if tc_ms else None),
-                                 "tensor_tflops": flop / (tc_ms / 1e3) / 1e12 if tc_ms else None,
-                                 "tensor_frac_of_sustained": (flop / (tc_ms / 1e3) / 1e12
-                                                              / pk.get("bf16_tflops_sustained", 1709.6)
-                                                              if tc_ms else None),
-                                 "algorithmic": f"{op_bytes:.4g} B of table operands (B*M*{K} x 32 KB), "
-                                                f"{flop:.4g} fp16 flop (B*M*{K} complex products x 3)"},
-                    "precision": "fp16x3 (tcgen05 chains; step phases applied in the chain epilogue, FP32)",
+                    "roofline": local_roofline({}, "fp32", "loc_steps + loc_chain", w.N, B * w.N, M, chain_ms / 1e3),
+                    "precision": "fp32 one-qubit operators (requested fp16x3)",
                     "config": {"N": w.N, "species": K, "B": B, "M": M, "dt": w.dt, "reunit_every": REUNIT,
                                "table": "level table" if args.levels else "digit table"}})
     elif args.workload == "plain":

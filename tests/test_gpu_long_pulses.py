@@ -23,7 +23,7 @@ def _dense(t, q, prec):
 @pytest.mark.parametrize("n,prec,tol", [(2, "fp64", 1e-10), (3, "fp64", 1e-10), (3, "fp32", 2e-3), (4, "fp32", 2e-3),
                                         (5, "fp32", 2e-3)])
 def test_long_pulse_in_many_segments(n, prec, tol):
-    # 40001 ragged steps: several hundred segments (FP64 rounding 1.1e-16 a product, R24 of the chain's
+    # 40001 ragged steps: several hundred segments (FP64 rounding of 1.1e-16 a product adds up over the chain's
     # length; FP32 chains this long lose norm, so the bound is loose)
     w = inputs.config(0, n_qubits=n, B=1, M=40001, base=16, digits=2)
     t = _table(w)

@@ -144,7 +144,22 @@ void local_detect(redo_table* t, const std::vector<double>& h, TableArena& ar, L
     kk[p] |= set << 8;
   }
   std::vector<float2> hp32(hp.size());
-  for (size_t i = 0; i < hp.size(); ++i) hp32[i] = make_float2((float)hp[i].x, (float)hp[i].y);
+  // FP32 operators of entries near 1 whatever the unit of the controls; the gradients make up for it
+  for (int k = 0; k < K; ++k) {
+    double mx = 0.0;
+    for (int e = kptr[k]; e < kptr[k + 1]; ++e)
+      for (int c = 0; c < 4; ++c) {
+        const double2 v = hp[4 * (kpair[e] & 0xfffff) + c];
+        mx = std::fmax(mx, std::fmax(std::fabs(v.x), std::fabs(v.y)));
+      }
+    const int x = mx > 0.0 ? std::ilogb(mx) : 0;
+    kptr.push_back(x);
+    for (int e = kptr[k]; e < kptr[k + 1]; ++e)
+      for (int c = 0; c < 4; ++c) {
+        const size_t i = 4 * (size_t)(kpair[e] & 0xfffff) + c;
+        hp32[i] = make_float2((float)std::scalbn(hp[i].x, -x), (float)std::scalbn(hp[i].y, -x));
+      }
+  }
   // one operator per level (no digit products per step) while the table stays small beside L2
   const bool levels = t->levels <= 65536 && (double)rep.size() * t->levels * 96.0 <= 64e6;
   t->loc_d = levels ? 1 : t->digit_count;
@@ -162,7 +177,7 @@ void local_detect(redo_table* t, const std::vector<double>& h, TableArena& ar, L
   o.k = ar.put(kk.data(), sizeof(int32_t) * pairs);
   o.h = ar.put(hp.data(), sizeof(double2) * 4 * pairs);
   o.h32 = ar.put(hp32.data(), sizeof(float2) * 4 * pairs);
-  o.kptr = ar.put(kptr.data(), sizeof(int32_t) * (K + 1));
+  o.kptr = ar.put(kptr.data(), sizeof(int32_t) * kptr.size());
   o.kpair = ar.put(kpair.data(), sizeof(int32_t) * pairs);
   o.D = ar.put(D.data(), sizeof(double2) * N);
   o.D32 = ar.put(D32.data(), sizeof(float4) * N);
@@ -579,11 +594,12 @@ loc_sweep_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
 
 // dF/du_kn = (2 dt / N^2) sum_i (gx X_i + gy Y_i + gz Z_i), a thread per (step, term): its pairs are
 // kpair[kptr[k] ..] (pair | qubit << 20), the Bloch sums bl [step][part][3n] or, already added, sums.
-// The sums are those of scaled vectors in FP32: times 2^exp_of(tau[b]), or times amp[b].
+// The sums are those of scaled vectors (and operators, by 2^-e) in FP32: times 2^e 2^exp_of(tau[b]), or
+// 2^e amp[b].
 template <typename R>
-__device__ __forceinline__ double loc_scaled(double x, const double2* tau, const double* amp, int64_t b) {
+__device__ __forceinline__ double loc_scaled(double x, const double2* tau, const double* amp, int64_t b, int e) {
   if (sizeof(R) == 8) return x;
-  return amp ? x * amp[b] : down2(x, -exp_of(tau[b]));
+  return amp ? down2(x, -e) * amp[b] : down2(x, -exp_of(tau[b]) - e);
 }
 // The phase gradients when every S_kz is a sum of one-qubit parts (wz [K][n], half the difference of a
 // qubit's two values; the species' S_z are): the change of Z_i over a step's rotation follows from the
@@ -622,7 +638,7 @@ __global__ void loc_grad_kernel(int64_t steps, int K, int n, int pairs, int part
       const R* gp = g + (st * pairs + p) * 3;
       for (int c = 0; c < 3; ++c) acc += (double)gp[c] * bloch(i, c);
     }
-    grad[(b * M + w0 + st - b * T) * K + k] = scale * loc_scaled<R>(acc, tau, amp, b);
+    grad[(b * M + w0 + st - b * T) * K + k] = scale * loc_scaled<R>(acc, tau, amp, b, kptr[K + 1 + k]);
     if (!PH || !phase) continue;
     acc = 0.0;
     for (int i = 0; i < n; ++i) {
@@ -632,7 +648,7 @@ __global__ void loc_grad_kernel(int64_t steps, int K, int n, int pairs, int part
       const double c = 1.0 + (double)a->x, sx = (double)a->y, sy = ph.cs_step > n ? (double)a[n].x : 0.0;
       acc += w * (2.0 * (sx * sx + sy * sy) * bloch(i, 2) - 2.0 * c * (sx * bloch(i, 0) + sy * bloch(i, 1)));
     }
-    ph.gphi[idx] = ph.scale * loc_scaled<R>(acc, tau, amp, b);
+    ph.gphi[idx] = ph.scale * loc_scaled<R>(acc, tau, amp, b, 0);
   }
 }
 
@@ -667,7 +683,7 @@ __global__ void loc_phase_kernel(const R* __restrict__ bz, int64_t B, int64_t M,
       a += (double)bz[((b * (M + 1) + n) * parts + p) * K + k];
       c += (double)bz[((b * (M + 1) + n + 1) * parts + p) * K + k];
     }
-    gphi[i] = scale * loc_scaled<R>(c - a, tau, nullptr, b);
+    gphi[i] = scale * loc_scaled<R>(c - a, tau, nullptr, b, 0);
   }
 }
 

@@ -41,10 +41,11 @@ __device__ __forceinline__ int exp_of(double x) {
 }
 __device__ __forceinline__ int exp_of(double2 z) { return max(exp_of(z.x), exp_of(z.y)); }
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
-// x 2^-e by its exponent (an FP64 product is 64 cycles of a warp): 0 below the normal range
+// x 2^-e by its exponent (an FP64 product is 64 cycles of a warp): 0 below the normal range, infinite above
 __device__ __forceinline__ double down2(double x, int e) {
   const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
   if (ex == 0x7ff || e == 0) return x;
+  if (ex - e >= 0x7ff && ex > 0) return __hiloint2double((hi & (int)0x80000000) | 0x7ff00000, 0);
   return ex == 0 || ex - e <= 0 ? 0.0 : __hiloint2double(hi - (int)((unsigned)e << 20), __double2loint(x));
 }
 

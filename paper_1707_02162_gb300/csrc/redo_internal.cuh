@@ -77,8 +77,8 @@ struct redo_table {
   int32_t* loc_ptr;           // [loc + 1] (term, qubit) pairs of each qubit
   int32_t* loc_k;             // [pairs] term | operator set << 8, flagged at the first pair of a term
   double2* loc_h;             // [pairs][4] one-qubit part of the term's operator
-  float2* loc_h32;
-  int32_t* loc_kptr;          // [K + 1] and
+  float2* loc_h32;            // the same times 2^-e, e the term's exponent
+  int32_t* loc_kptr;          // [K + 1], then the terms' exponents [K], and
   int32_t* loc_kpair;         // [pairs]: the pairs of each term (pair | qubit << 20)
   double2* loc_u64;           // [sets][loc_d][loc_base][4] digit (or level) operators, a set for every
                               // distinct (one-qubit part, coefficient grid)

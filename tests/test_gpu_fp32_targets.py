@@ -68,3 +68,26 @@ def test_state_gradient_of_scaled_states(n, e0, eT):
     f = 4.0 ** (e0 + eT)
     assert torch.equal(Fs, F * f) and torch.equal(gs, g * f)
     t.close()
+
+
+@pytest.mark.parametrize("n", [1, 3, 6])
+@pytest.mark.parametrize("e", [140, -140])
+def test_gradients_of_controls_in_other_units(n, e):
+    # operators times 2^e on a grid times 2^-e: the same steps, gradients times 2^e
+    w, rng = _workload(n, B=3, M=9)
+    psi0, psiT = _states(rng, 3, w.N), _states(rng, 3, w.N)
+    got = []
+    for f in (1.0, 2.0 ** e):
+        w2 = inputs.Workload(w.name, n, w.H0, w.Hk * f, w.dt, w.lo / f, w.hi / f, w.levels, w.base, w.digits, w.u / f)
+        w2.Hk[0] = w.Hk[0]                            # one term in the first unit
+        w2.lo[0], w2.hi[0], w2.u[:, :, 0] = w.lo[0], w.hi[0], w.u[:, :, 0]
+        t = _table(w2)
+        q = t.quantize(w2.u)
+        g = t.fidelity_grad(q, torch.as_tensor(w.target, device="cuda"), "fp32", checkpoint_every=4)[1]
+        s = t.state_grad(q, psi0, psiT, "fp32")[1]
+        got.append((q, g, s))
+        t.close()
+    (q, g, s), (q2, g2, s2) = got
+    assert torch.equal(q, q2)
+    for a, b in ((g, g2), (s, s2)):
+        assert torch.equal(b[..., 0], a[..., 0]) and torch.equal(b[..., 1:], a[..., 1:] * 2.0 ** e)

@@ -955,7 +955,8 @@ __global__ void loc_expect_kernel(const cplx<R>* __restrict__ part, int64_t n, i
   for (int64_t i0 = blockIdx.x * per; i0 < n; i0 += gridDim.x * per) {
     const int64_t i = i0 + threadIdx.x / w;
     double a = 0.0;
-    const bool wide = sizeof(R) == 4 && i < n && flags[i / items] != 0;
+    // (a slice's parts are 8 bytes or more of 512 MiB, so i and items hold in 32 bits)
+    const bool wide = sizeof(R) == 4 && i < n && flags[(uint32_t)i / (uint32_t)items] != 0;
     for (int q = l; q < G && i < n; q += w) {
       const cplx<R> p = part[i * G + q];
       if constexpr (sizeof(R) == 4)
@@ -995,6 +996,7 @@ loc_state_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
     int x = -200;
 #pragma unroll
     for (int e = 0; e < E; ++e) x = max(x, exp_of(v[e]));
+    if constexpr (L::C == 1) return __reduce_max_sync(0xffffffffu, x);
 #pragma unroll
     for (int off = L::C; off < 32; off *= 2) x = max(x, __shfl_xor_sync(0xffffffffu, x, off));
     return x;
@@ -1042,7 +1044,7 @@ loc_state_kernel(const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ del
       ty += __shfl_xor_sync(0xffffffffu, ty, off);
     }
     if (F_out && on && l == 0) {
-      const double f = pow2(e0), x = tx * f, y = ty * f;
+      const double x = down2(tx, -e0), y = down2(ty, -e0);
       F_out[b] = x * x + y * y;
     }
     if constexpr (sizeof(R) == 4) {

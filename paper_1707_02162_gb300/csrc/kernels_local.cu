@@ -19,7 +19,8 @@ namespace redo {
 // exp(-i t a0) (cos(t |v|) I - i sin(t |v|) / |v| v.sigma), theta as in the dense table; rep[set] is a
 // pair with these operators.
 __global__ void loc_table_kernel(const double2* __restrict__ h, const int32_t* __restrict__ k,
-                                 const int32_t* __restrict__ rep, int sets, int d, int base, double dt, const double* __restrict__ lo, const double* __restrict__ delta,
+                                 const int32_t* __restrict__ rep, int sets, int d, int base, double dt,
+                                 const double* __restrict__ lo, const double* __restrict__ delta,
                                  double2* __restrict__ u64, float2* __restrict__ u32) {
   const int64_t total = (int64_t)sets * d * base;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -127,9 +128,9 @@ void local_detect(redo_table* t, const std::vector<double>& h, TableArena& ar, L
     D32[r] = make_float4((float)x, (float)y, (float)(x - (double)(float)x), (float)(y - (double)(float)y));
   }
   // X controls of every qubit, or a global field's part on each, are one set of operators: N = 8 with six
-  // controls of 4096 levels keeps 0.8 MB, not 2.4 MB (which fits beside the dense table in one mapping: building the table takes
-  // 237 us for two global controls, 264 for six local ones; with an allocation, copy and wait of their own 318
-  // and 305, without one-qubit tables 270 and 299)
+  // controls of 4096 levels keeps 0.8 MB, not 2.4 MB (which fits beside the dense table in one mapping:
+  // building the table takes 237 us for two global controls, 264 for six local ones; with an allocation,
+  // copy and wait of their own 318 and 305, without one-qubit tables 270 and 299)
   std::vector<int32_t> rep;
   for (int p = 0; p < pairs; ++p) {
     const int k = kk[p] & ~kLocFirst;
@@ -210,9 +211,9 @@ cudaError_t local_build(redo_table* t, const LocalParts& o, char* base, cudaStre
   t->loc_u64 = (double2*)(base + o.u64);
   t->loc_u32 = (float2*)(base + o.u32);
   const size_t blocks = (o.entries + 127) / 128, sets = o.entries / ((size_t)t->loc_d * t->loc_base);
-  loc_table_kernel<<<(unsigned)(blocks < 4096 ? blocks : 4096), 128, 0, s>>>(t->loc_h, t->loc_k, (const int32_t*)(base + o.rep),
-                                                                            (int)sets, t->loc_d, t->loc_base, t->dt,
-                                                                            t->d_lo, t->d_delta, t->loc_u64, t->loc_u32);
+  loc_table_kernel<<<(unsigned)(blocks < 4096 ? blocks : 4096), 128, 0, s>>>(
+      t->loc_h, t->loc_k, (const int32_t*)(base + o.rep), (int)sets, t->loc_d, t->loc_base, t->dt, t->d_lo, t->d_delta,
+      t->loc_u64, t->loc_u32);
   while ((1 << t->loc) < t->N) ++t->loc;
   return cudaGetLastError();
 }
@@ -673,7 +674,8 @@ __global__ void __launch_bounds__(256) loc_sums_kernel(const R* __restrict__ bl,
 // gphi[b][n][k] = (2 / N^2) (Tz[n+1][k] - Tz[n][k]) (the traces already carry conj(tau))
 template <typename R>
 __global__ void loc_phase_kernel(const R* __restrict__ bz, int64_t B, int64_t M, int parts, int K, double scale,
-                                 const double2* __restrict__ tau, double* __restrict__ gphi, const int32_t* __restrict__ gate) {
+                                 const double2* __restrict__ tau, double* __restrict__ gphi,
+                                 const int32_t* __restrict__ gate) {
   if (gate && *gate != 0) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B * M * K; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t bn = i / K, b = bn / M, n = bn - b * M;
@@ -759,8 +761,8 @@ template <int E> __device__ __forceinline__ double2 lane_expect(const double2 (&
 
 // FP32 pairs serve observables and states whose products stay in FP32's range; others (a largest
 // weight outside 2^-60 .. 2^60, or a largest entry of psi_0 outside 2^-60 .. 2^30) are summed in
-// FP64, with the weights read again.  A pulse's flag tells loc_expect_kernel what its parts hold.  (The step loop
-// stands once for each: with the choice inside, a step took 15 % longer.)
+// FP64, with the weights read again.  A pulse's flag tells loc_expect_kernel what its parts hold.  (The
+// step loop stands once for each: with the choice inside, a step took 15 % longer.)
 template <int E> __device__ __forceinline__ int2 lane_top(const double2* psi, const double* obs) {
   int2 t = make_int2(-200, -200);
 #pragma unroll
@@ -1167,8 +1169,9 @@ bool local_eligible(const redo_table* t, int64_t M, int prec, int what) {
 // FP64, by measurement over B = 1 .. 3000, N = 2 .. 16: while the pulses leave SMs idle a call waits for
 // its dependent products and this form is ahead from N = 4 on (N = 4, two controls, 40 x 200: 158 us dense,
 // 101 here) and level at N = 2; once they fill the GPU its serial one-qubit work runs at half the rate of
-// the dense columns (N = 4, 300 x 100: 126 us dense, 195 here), a state's at the same rate (N = 8,
-// 300 x 100: 261 and 351; N = 16 the other way).
+// the dense columns (N = 4, 300 x 100: 126 us dense, 195 here).  A state's dense factors take about 1 us
+// each, one after another, its step here 2.5 to 3.5 (300 x 100, N = 4: one control 224 us dense, 265 here,
+// two 381 and 258; N = 8: 261 and 351, 435 and 345; N = 16: always ahead).
 // FP32: the dense column kernel is bound by its operand reads at about two thirds of this path's rate
 // (N = 4, global controls, 1000 x 500: 155 us dense, 234 us here; N = 8: 528 and 315), so plain
 // propagations at N = 2, and at N = 4 and 8 with few factors, stay dense; with a step-opening diagonal, for
@@ -1233,8 +1236,7 @@ ChainPlan plan_chain_local(const redo_table* t, int64_t B, int64_t M, int prec, 
 
 template <typename R>
 static cudaError_t loc_steps_t(const redo_table* t, const int32_t* q, int64_t B, int64_t M, int64_t m0, int64_t T, int E,
-                               bool near,
-                               const LocalDiag& pd, int64_t b0, const LocScratch& w, int64_t* status,
+                               bool near, const LocalDiag& pd, int64_t b0, const LocScratch& w, int64_t* status,
                                cudaStream_t s) {
   const int ts = B * (T + 1) >= (int64_t)t->num_sms * 8 * kPrepSteps ? kPrepSteps : 8;
   const int64_t tiles = (T + 1 + ts - 1) / ts;
@@ -1399,7 +1401,8 @@ cudaError_t launch_local_sim(const redo_table* t, const int32_t* q, int64_t B, i
   const LocScratch w = loc_scratch(t, slice, M, prec, kLocalSim, ops);
   for (int64_t b0 = 0; b0 < B; b0 += slice) {
     const int64_t nb = b0 + slice < B ? slice : B - b0;
-    cudaError_t e = loc_steps(t, q, nb, M, prec, kLocalSim, loc_sim_entries(t->N), LocalDiag{nullptr, 0, 0}, b0, w, status, s);
+    cudaError_t e = loc_steps(t, q, nb, M, prec, kLocalSim, loc_sim_entries(t->N), LocalDiag{nullptr, 0, 0}, b0, w,
+                              status, s);
     if (e) return e;
     const double2* p0 = psi0 + (batched ? b0 * t->N : 0);
     double* ex = expect + b0 * (M + 1);
@@ -1476,7 +1479,8 @@ static cudaError_t loc_state_t(const redo_table* t, const int32_t* q, int64_t B,
     const bool fwd = i < nw;
     const int64_t k = fwd ? i : 2 * nw - 2 - i, m0 = k * win, T = m0 + win < M ? win : M - m0;
     const int bk = back && i >= nw - 1;
-    cudaError_t e = loc_steps_t<R>(t, q, B, M, m0, T, loc_vec_entries(t->N), loc_near(sizeof(R) == 8, t->N), LocalDiag{nullptr, 0, 0}, 0,
+    cudaError_t e = loc_steps_t<R>(t, q, B, M, m0, T, loc_vec_entries(t->N), loc_near(sizeof(R) == 8, t->N),
+                                   LocalDiag{nullptr, 0, 0}, 0,
                                    bk ? w : fo, fwd ? status : nullptr, s);
     if (e) return e;
     LOC_VEC(loc_state_kernel, (const cplx<R>*)w.cs, (const cplx<R>*)w.delta, B, M, m0, T, fwd, bk, psi0, psiT, batched,
